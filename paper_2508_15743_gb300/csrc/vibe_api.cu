@@ -349,7 +349,7 @@ Bounds bounds_over(const Tables* ts, int count) {
       b.x_warp_scratch = std::max(b.x_warp_scratch, t.x_warp_scratch);
     }
   }
-  if (b.engines & 2) b.x_warp_smem += vibe::bpx_ring_bytes(b.XD);
+  if (b.engines & 2) b.x_warp_smem += vibe::bpx_window_bytes();
   return b;
 }
 
@@ -456,7 +456,8 @@ struct vibe_handle {
   float* lam = nullptr;
   float* alpha_m = nullptr;
   void* msg_init = nullptr;
-  uint32_t *xcol = nullptr, *xrmap = nullptr;
+  uint32_t *cpos = nullptr, *soff = nullptr, *xlnk = nullptr, *xcolid = nullptr, *xrmap = nullptr;
+  int32_t* stepcnt = nullptr;
   uint2* xrec = nullptr;
   int32_t *layer_ptr = nullptr, *layer_chk = nullptr, *layer_vptr = nullptr, *layer_var = nullptr,
           *nlayer_d = nullptr;
@@ -480,7 +481,8 @@ struct vibe_handle {
     cudaFree(tmp_counters);
     cudaFree(rowptr); cudaFree(colidx); cudaFree(colptr); cudaFree(rowidx); cudaFree(lrowptr); cudaFree(lcolidx);
     cudaFree(nlev); cudaFree(csc_ent); cudaFree(sched); cudaFree(lvl_off); cudaFree(perm); cudaFree(lam); cudaFree(alpha_m);
-    cudaFree(msg_init); cudaFree(xcol); cudaFree(xrec); cudaFree(xrmap); cudaFree(xsum); cudaFree(d_desc);
+    cudaFree(msg_init); cudaFree(cpos); cudaFree(soff); cudaFree(stepcnt); cudaFree(xrec); cudaFree(xlnk); cudaFree(xcolid);
+    cudaFree(xrmap); cudaFree(xsum); cudaFree(d_desc);
     cudaFree(layer_ptr); cudaFree(layer_chk); cudaFree(layer_vptr); cudaFree(layer_var); cudaFree(nlayer_d);
     cudaSetDevice(prev);
   }
@@ -602,8 +604,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   t.n_layered = p->n_layered;
   vibe::bp_warp_smem_bytes(&t, p->msg_fp16);
   t.XD = vibe::bpx_degree_bucket(maxcol);
-  t.XP = (t.XD + 3) / 4 * 4;
-  vibe::bpx_layout(&t, p->msg_fp16);
+  t.SP = E + (int)std::count(coldeg.begin(), coldeg.end(), 0);
+  t.x_warp_smem = vibe::bpx_summary_bytes(m, p->msg_fp16);
   t.engine = p->bp_engine;
   if (t.engine == VIBE_ENGINE_SUMMARY && t.XD == 0)
     return bail(fail(VIBE_ERR_UNSUPPORTED, "the summary engine takes columns of at most 16 checks"));
@@ -624,8 +626,9 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   }
   const int Lnnz = L->rowptr[k];
   const size_t msg_bytes = (size_t)m * t.RP * (p->msg_fp16 ? 2 : 4);
-  const size_t lev_scratch = std::max<size_t>(std::max<size_t>(2 * (size_t)n + E, 2 * (size_t)m + 2),
-                                              (size_t)K * ((size_t)m + 3 * (size_t)n + 1));
+  const size_t lev_scratch =
+      std::max({2 * (size_t)n + E, 2 * (size_t)m + 2, (size_t)K * ((size_t)m + 3 * (size_t)n + 1),
+                vibe::step_scratch_ints(n, K)});
   int32_t* scratch = nullptr;
   cudaStream_t s = nullptr;
 #define VIBE_TRY(call, what) \
@@ -646,9 +649,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   VIBE_TRY(dalloc(&h->lam, n), "tables");
   VIBE_TRY(dalloc(&h->alpha_m, K), "tables");
   VIBE_TRY(cudaMalloc(&h->msg_init, std::max<size_t>(msg_bytes, 16)), "tables");
-  VIBE_TRY(dalloc(&h->xcol, (size_t)n * t.XP), "tables");
-  VIBE_TRY(dalloc(&h->xrec, t.XP ? (size_t)K * n : 0), "tables");
-  VIBE_TRY(dalloc(&h->xrmap, t.XP ? (size_t)K * E : 0), "tables");
+  VIBE_TRY(dalloc(&h->cpos, E), "tables");
+  VIBE_TRY(dalloc(&h->stepcnt, K), "tables");
   VIBE_TRY(dalloc(&h->xsum, m), "tables");
   VIBE_TRY(dalloc(&h->d_desc, 1), "tables");
   if (p->n_layered > 0) {
@@ -674,10 +676,27 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   } else {
     VIBE_TRY(vibe::seeded_schedules(h->perm, n, K, p->seed, s), "schedule kernel");
   }
-  VIBE_TRY(vibe::build_tables(h->rowptr, h->colidx, m, n, K, h->perm, t.RP, t.DP, t.XP, p->msg_fp16, h->lam,
-                              h->colptr, h->rowidx, h->csc_ent, h->msg_init, h->sched, h->lvl_off, h->nlev, h->xcol,
-                              h->xrec, h->xrmap, h->xsum, scratch, s),
+  VIBE_TRY(vibe::build_tables(h->rowptr, h->colidx, m, n, E, K, h->perm, t.RP, t.DP, p->msg_fp16, h->lam, h->colptr,
+                              h->rowidx, h->cpos, h->csc_ent, h->msg_init, h->sched, h->lvl_off, h->nlev, h->xsum,
+                              scratch, s),
            "graph builder");
+  if (t.XD > 0) {
+    std::vector<int32_t> cnt(K);
+    VIBE_TRY(vibe::build_steps(m, n, K, h->perm, h->colptr, h->cpos, h->stepcnt, scratch, s), "step builder");
+    VIBE_TRY(cudaMemcpyAsync(cnt.data(), h->stepcnt, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, s), "step builder");
+    VIBE_TRY(cudaStreamSynchronize(s), "step builder");
+    t.nstep = *std::max_element(cnt.begin(), cnt.end());
+    t.soff_pitch = t.nstep + vibe::kStepPad;
+    VIBE_TRY(dalloc(&h->soff, (size_t)K * t.soff_pitch), "tables");
+    VIBE_TRY(dalloc(&h->xrec, (size_t)K * t.SP + 4), "tables");   // copied in groups of four slots
+    VIBE_TRY(dalloc(&h->xlnk, (size_t)K * t.SP + 4), "tables");
+    VIBE_TRY(dalloc(&h->xcolid, (size_t)K * t.SP), "tables");
+    VIBE_TRY(dalloc(&h->xrmap, (size_t)K * E), "tables");
+    VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
+                              h->soff, h->xrec, h->xlnk, h->xcolid, h->xrmap, s),
+             "step builder");
+  }
+  vibe::bpx_layout(&t, p->msg_fp16);
   if (p->n_layered > 0) {
     VIBE_TRY(vibe::build_layers(h->rowptr, h->colidx, h->colptr, h->rowidx, m, h->layer_ptr, h->layer_chk,
                                 h->layer_vptr, h->layer_var, h->nlayer_d, scratch, s),
@@ -689,7 +708,7 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   t.rowptr = h->rowptr; t.colidx = h->colidx; t.colptr = h->colptr; t.rowidx = h->rowidx;
   t.csc_ent = h->csc_ent; t.lam = h->lam; t.alpha_m = h->alpha_m; t.msg_init = h->msg_init; t.sched = h->sched; t.lvl_off = h->lvl_off;
   t.nlev = h->nlev; t.lrowptr = h->lrowptr; t.lcolidx = h->lcolidx;
-  t.xcol = h->xcol; t.xrec = h->xrec; t.xrmap = h->xrmap; t.xsum = h->xsum;
+  t.stepcnt = h->stepcnt; t.soff = h->soff; t.xrec = h->xrec; t.xlnk = h->xlnk; t.xcolid = h->xcolid; t.xrmap = h->xrmap; t.xsum = h->xsum;
   VIBE_TRY(cudaMemcpyAsync(h->d_desc, &t, sizeof(Tables), cudaMemcpyHostToDevice, s), "upload");
   VIBE_TRY(cudaStreamSynchronize(s), "graph builder");
   cudaFree(scratch);

@@ -3,49 +3,50 @@
 // results as the image engine (vibe_bp.cu), which keeps a member's whole message image in shared
 // memory; a different layout.
 //
-// Why a warp per (shot, member). The wavefront levels of a random serial order on these graphs are
-// short: a column conflicts with every column of its ~4 checks (~600 others), so a sweep of the d=11
-// problem has ~1000 levels of ~32 columns. One warp matches that width and synchronises with
-// __syncwarp. In shot mode each warp decodes one shot at a time (persistent, shots from a global
+// Mapping: one warp per (shot, member), one lane per edge. A sweep runs the member's steps (k_steps in
+// vibe_graph.cu): up to 32 edges of columns that share no check, packed in the member's order. A lane
+// asks its check's summary for the check-to-variable message of its edge, the lanes of a column pass
+// each other these messages with shuffles, and every lane forms its own exclusion sum and updates its
+// own check. In shot mode each warp decodes one shot at a time (persistent, shots from a global
 // counter), running the members one after another with the iteration budget of the correction limit
 // (Sec. III.D.2); in pair mode each warp takes one (shot, member) pair at a time, and the last member
 // of a shot to finish runs the shot's selection and epilogue.
 //
-// Check-node state: a 16-byte summary per check in shared memory.
-//   x, y   the values m1 <= m2 held by up to two "holder" edges of the row (their positions p1, p2
-//          inside the check's CSR row, bits 0-7 and 8-15 of w; nh = number of valid holders, bits
-//          16-17; a row of fewer than two entries holds a phantom second holder, position 255, +inf)
-//   z      a floor F: every entry of the row that is not a holder has magnitude >= F, and the
-//          holders' magnitudes are <= F (after a rescan, F is the third smallest magnitude, or +inf)
-//   w      also carries the parity of the sign bits of the row's messages (bit 18), the syndrome bit
-//          (bit 19) and the check's parity (H e)_c XOR s_c (bit 20).
-// The minimum over the row without the edge at position p is then m2 if p == p1 and nh == 2, m1 if
-// p != p1 and nh >= 1, and +inf if F is +inf; otherwise (the only remaining holder asks, or no holder
-// is left) the row is rescanned first -- lazily, only when a column actually needs the answer. The
-// sign product without p is the sign parity XOR the sign of p's own message. Together these are
-// exactly the minimum and sign product that Algorithm 1's check update takes over N(c) \ v.
+// Check-node state: a summary per check in shared memory.
+//   m1 <= m2  the magnitudes of up to two "holder" edges of the row, with their positions p1, p2 inside
+//             the check's CSR row; an empty holder is position 255 with +inf
+//   F         a floor: every entry of the row that is not a holder has magnitude >= F, and the holders'
+//             magnitudes are <= F (after a rescan, F is the third smallest magnitude, or +inf)
+//   flags     the parity of the sign bits of the row's messages XOR the syndrome bit (bit 31 of the flag
+//             word), and the check's parity (H e)_c XOR s_c (bit 30).
+// The minimum over the row without the edge at position p is m2 if p == p1, else m1 -- unless that
+// value exceeds F, which only an empty holder's +inf above a finite floor does: then the row is
+// rescanned first -- lazily, only when a column actually needs the answer. The sign product without p,
+// syndrome included, is the flag XOR the sign of p's own message. Together these are exactly the
+// minimum and sign product that Algorithm 1's check update takes over N(c) \ v.
 //
-// Keeping the summary exact after the edge at position p gets the new magnitude x:
-//   p holds m1:   x <= m2: m1 = x;  m2 < x <= F: the holders swap;  x > F: p leaves (nh - 1)
-//   p holds m2:   x < m1: the holders swap;  x <= F: m2 = x;  x > F: p leaves
-//   otherwise:    x < F: p becomes a holder (an empty slot, or the larger holder is evicted and its
-//                 value becomes the floor, or x itself becomes the floor if x >= m2)
-// With the floor most holders that grow stay answerable; on circuit-level colour codes this needs
-// ~2.5x fewer row rescans per sweep than two holders without a floor (117 vs 296 at d=11).
+// Keeping the summary exact after the edge at position p gets the new magnitude x: p leaves the
+// holders if it is one; then, if x <= F, (x, p) is inserted into the sorted pair of holders and the value
+// that falls out, if any, becomes the floor (it is <= F). With the floor most holders that grow stay
+// answerable; on circuit-level colour codes this needs ~2.5x fewer row rescans per sweep than two
+// holders without a floor (117 vs 296 at d=11).
 //
-// Messages. A member's variable-to-check messages live in the warp's global scratch in the member's
-// schedule order: the columns of one level (and of one 32-column chunk) are consecutive, so a chunk's
-// messages form one contiguous block and its stores coalesce. The column update never reads its old
-// messages: it needs only their signs, kept with its previous decision in a 32-bit state word per
-// schedule position (bit k: sign of the message to its k-th check; bit 31: decision). Messages are
-// read only by rescans, through a per-member map from each CSR entry of H to its message slot.
+// Messages. A member's variable-to-check messages live in the warp's global scratch in step order: a
+// step's messages are contiguous, so its stores coalesce. A step never reads its old messages: it needs
+// only their signs, kept with the columns' previous decisions as two 32-bit words per step (bit l: lane
+// l's edge; the decision on the lane of the column's last edge). Messages are read only by rescans,
+// through a per-member map from each CSR entry of H to its message slot.
 //
-// Pipeline: each lane copies the column data (checks with row positions, prior, state word) into a
-// shared-memory ring one chunk ahead of its update, and the schedule records that locate it two
-// chunks ahead; none of it is written by the chunks in between.
+// What bounds it and what the mapping bought. The engine is bound by instruction issue and by the
+// dependent chain of a step (summary, shuffles, sums, update, next step), not by DRAM. The mapping it
+// replaces gave each lane a whole column and unrolled its checks: on levels of 4-30 columns most lanes
+// idled through ~750 instructions; a step of 32 edges takes ~170 with nearly every lane at work.
+// Measured (GB300): circuit-level d=5, FP16, K=32, 4096 shots 826 -> 174 ms; XYZ d=7, FP32, K=16, 2500
+// shots 616 -> 147 ms; circuit-level d=11, FP32, K=64, T=50, 32 shots 220 -> 156 ms.
 //
 // Arithmetic equals the oracle's bit for bit: same per-node operation order (__fadd_rn/__fmul_rn), min
 // and sign exact, FP16 storage with -0 stored as +0.
+#include <cstddef>
 #include <type_traits>
 
 #include "vibe_internal.cuh"
@@ -53,548 +54,448 @@
 namespace vibe {
 namespace {
 
+// Stored messages as bits: the rounding of a sum, its sign bit at bit 31, loads and stores.
 template <typename MT>
 struct XMsg;
 
 template <>
 struct XMsg<float> {
-  __device__ __forceinline__ static float load(const float* p) { return __ldcg(p); }
-  __device__ __forceinline__ static float value(float x) { return x; }
-  __device__ __forceinline__ static float round(float x) { return x; }
-  __device__ __forceinline__ static float from(float x) { return x; }
+  __device__ __forceinline__ static uint32_t round(float x) { return __float_as_uint(x); }
+  __device__ __forceinline__ static uint32_t sign31(uint32_t b) { return b; }
+  __device__ __forceinline__ static uint32_t load(const float* p) { return __float_as_uint(__ldcg(p)); }
+  __device__ __forceinline__ static void store(float* p, uint32_t b) { __stcs(p, __uint_as_float(b)); }
 };
 
 template <>
 struct XMsg<__half> {
-  __device__ __forceinline__ static __half load(const __half* p) {
-    return __ushort_as_half(__ldcg(reinterpret_cast<const unsigned short*>(p)));
+  __device__ __forceinline__ static uint32_t round(float x) {   // -0 as +0
+    const uint32_t h = (uint32_t)__half_as_ushort(__float2half_rn(x));
+    return h == 0x8000u ? 0u : h;
   }
-  __device__ __forceinline__ static float value(__half x) { return __half2float(x); }
-  // rounds to half, -0 as +0, and returns the stored value as a float
-  __device__ __forceinline__ static float round(float x) {
-    unsigned short h = __half_as_ushort(__float2half_rn(x));
-    if (h == 0x8000u) h = 0;
-    return __half2float(__ushort_as_half(h));
+  __device__ __forceinline__ static uint32_t sign31(uint32_t b) { return b << 16; }
+  __device__ __forceinline__ static uint32_t load(const __half* p) {
+    return (uint32_t)__ldcg(reinterpret_cast<const unsigned short*>(p));
   }
-  __device__ __forceinline__ static __half from(float x) { return __float2half_rn(x); }   // x already rounded
+  __device__ __forceinline__ static void store(__half* p, uint32_t b) {
+    __stcs(reinterpret_cast<unsigned short*>(p), (unsigned short)b);
+  }
 };
 
-template <typename MT>
-__device__ __forceinline__ void store_msg(MT* p, float x) {
-  if constexpr (std::is_same<MT, float>::value) __stcs(p, x);
-  else __stcs(reinterpret_cast<unsigned short*>(p), __half_as_ushort(__float2half_rn(x)));
+// Shared memory by 32-bit address: the sweep keeps a handful of addresses in registers instead of
+// forming each one from the window base.
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t a, uint2 v) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t a, uint4 v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
 constexpr uint32_t kInfBits = 0x7f800000u;
-constexpr uint32_t kDecBit = 1u << 31;   // decision bit of a column state word
 
-__device__ __forceinline__ uint32_t sign_bit(float x) { return __float_as_uint(x) >> 31; }
+constexpr uint32_t kSgnBit = 1u << 31, kParBit = 1u << 30;   // flags of a summary
 
-__device__ __forceinline__ bool is_finite_bits(float x) { return (__float_as_uint(x) & kInfBits) != kInfBits; }
-
-// Check summaries in registers: float4 {m1, m2, F, w}, w = p1 | p2 << 8 | nh << 16 | sign parity << 18 |
-// syndrome << 19 | parity << 20 (see the header comment).
-constexpr uint32_t kNhShift = 16, kSgnBit = 1u << 18, kSynBit = 1u << 19, kParBit = 1u << 20;
-
-// Minimum magnitude over the row without the edge at position p; false if the summary cannot answer.
-__device__ __forceinline__ bool xquery(const float4 s, uint32_t p, float& out) {
-  const uint32_t w = __float_as_uint(s.w);
-  const uint32_t nh = (w >> kNhShift) & 3u, p1 = w & 0xffu;
-  const bool mine = p == p1;
-  out = nh == 2u ? (mine ? s.y : s.x) : (nh == 1u && !mine ? s.x : s.z);
-  return nh == 2u || (nh == 1u && !mine) || __float_as_uint(s.z) == kInfBits;   // +inf floor: all others +inf
-}
-
-// Whether the edge at position p taking magnitude x can change more than the flags: it holds m1 or
-// m2, or it drops below the floor.
-__device__ __forceinline__ bool xslow(const float4 s, uint32_t p, float x) {
-  const uint32_t w = __float_as_uint(s.w);
-  const uint32_t nh = (w >> kNhShift) & 3u;
-  return (nh >= 1u && p == (w & 0xffu)) || (nh == 2u && p == ((w >> 8) & 0xffu)) || x < s.z;
-}
-
-// The summary after the edge at position p takes magnitude x (the case analysis in the header),
-// written as: take p out of the holder list, then put (x, p) back if it stays within the floor --
-// a former holder when x <= F, any other edge when x < F -- evicting the larger holder into the
-// floor when the list is full.
-__device__ __forceinline__ float4 xupdate(const float4 s, uint32_t p, float x) {
-  const uint32_t w = __float_as_uint(s.w);
-  const uint32_t nh0 = (w >> kNhShift) & 3u, q10 = w & 0xffu, q2 = (w >> 8) & 0xffu;
-  const bool is1 = nh0 >= 1u && p == q10, is2 = nh0 == 2u && p == q2;
-  const bool was = is1 || is2;
-  const float a1 = is1 ? s.y : s.x, a2 = s.y, F = s.z;
-  const uint32_t q1 = is1 ? q2 : q10;
-  const uint32_t k = nh0 - (was ? 1u : 0u);
-  const bool ins = was ? x <= F : x < F;
-  const bool lt1 = k == 0u || x < a1;
-  const bool lt2 = k <= 1u || x < a2;
-  const float n1 = ins && lt1 ? x : a1;
-  const uint32_t r1 = ins && lt1 ? p : q1;
-  const float n2 = ins ? (lt1 ? a1 : (lt2 ? x : a2)) : a2;
-  const uint32_t r2 = ins ? (lt1 ? q1 : (lt2 ? p : q2)) : q2;
-  const float nF = ins && k == 2u ? (lt2 ? a2 : x) : F;
-  const uint32_t nk = ins ? min(k + 1u, 2u) : k;
-  return make_float4(n1, n2, nF, __uint_as_float((w & ~0x3ffffu) | r1 | (r2 << 8) | (nk << kNhShift)));
-}
-
-// Shared-memory storage of the summaries. FP32 messages: the float4 itself (16 bytes per check).
-// FP16 messages: 8 bytes, {m1 | sign parity << 15 | m2 << 16 | syndrome << 31, F | parity << 15 |
-// p1 << 16 | p2 << 24} with every magnitude a binary16 (exact: the magnitudes are those of stored
-// binary16 messages) and position 255 for an empty holder slot, from which the holder count follows.
+// What a lane sees of its check: `ans`, the minimum magnitude of the row without the lane's edge;
+// `ok`, whether the summary holds it; `flags`. A check is addressed by its summary's shared address, an
+// edge by its record word (position in the row in bits 0-7).
+// Sum<float>: 16 bytes per check {m1, m2, F, p1 | p2 << 8 | flags}.
+// Sum<__half>: 8 bytes. Magnitudes are binary16 (exact: those of stored binary16 messages) and a holder
+// is one 23-bit key, magnitude << 8 | position, so that an integer comparison orders holders by
+// magnitude, then position. x: key 1 | low 9 bits of F << 23; y: high 6 bits of F | key 2 << 6 | flags.
 template <typename MT>
-struct SumIO;
+struct Sum;
 
 template <>
-struct SumIO<float> {
-  float4* v;
-  __device__ __forceinline__ float4 load(int c) const { return v[c]; }
-  __device__ __forceinline__ void store(int c, float4 s) const { v[c] = s; }
-  __device__ __forceinline__ void flip(int c, uint32_t bits) const { reinterpret_cast<uint32_t*>(v + c)[3] ^= bits; }
+struct Sum<float> {
+  static constexpr int kBytes = 16;
+  float m1, m2, F;
+  uint32_t w;
+  bool is1;
+  __device__ __forceinline__ void load(uint32_t addr, uint32_t rec) {
+    const uint4 q = lds128(addr);
+    m1 = __uint_as_float(q.x);
+    m2 = __uint_as_float(q.y);
+    F = __uint_as_float(q.z);
+    w = q.w;
+    is1 = ((w ^ rec) & 0xffu) == 0u;
+  }
+  __device__ __forceinline__ float ans() const { return is1 ? m2 : m1; }
+  __device__ __forceinline__ bool ok() const { return ans() <= F; }
+  __device__ __forceinline__ uint32_t flags() const { return w; }
+  // the edge takes the message with bits b; `toggle` flips flag bits. Stores only what changed.
+  __device__ __forceinline__ void update(uint32_t addr, uint32_t rec, uint32_t b, uint32_t toggle, bool act) const {
+    const float inf = __uint_as_float(kInfBits);
+    const float x = fabsf(__uint_as_float(b));
+    const uint32_t p1 = w & 0xffu, p2 = (w >> 8) & 0xffu;
+    const bool was = is1 || ((p2 ^ rec) & 0xffu) == 0u, ins = x <= F;
+    const float b1 = ans(), b2 = was ? inf : m2;
+    const uint32_t c1 = is1 ? p2 : p1, c2 = was ? 255u : p2;
+    const float y = ins ? x : inf;
+    const uint32_t py = ins ? (rec & 0xffu) : 255u;
+    const bool lt1 = y < b1;
+    const float n1 = fminf(y, b1), t = fmaxf(y, b1);
+    const uint32_t r1 = lt1 ? py : c1, tp = lt1 ? c1 : py;
+    const bool lt2 = t < b2;
+    const float n2 = fminf(t, b2), h = fmaxf(t, b2);
+    const uint32_t r2 = lt2 ? tp : c2;
+    if (act && (was || ins || toggle))
+      sts128(addr, make_uint4(__float_as_uint(n1), __float_as_uint(n2), __float_as_uint(fminf(F, h)),
+                              ((w ^ toggle) & 0xffff0000u) | r1 | (r2 << 8)));
+  }
+  __device__ __forceinline__ static void init(uint32_t addr, float4 s, uint32_t flip) {
+    sts128(addr, make_uint4(__float_as_uint(s.x), __float_as_uint(s.y), __float_as_uint(s.z), __float_as_uint(s.w) ^ flip));
+  }
+  // a message as the rescan orders it: the bits of its magnitude (unsigned order of non-negative floats)
+  __device__ __forceinline__ static uint32_t key(uint32_t b, uint32_t) { return b & 0x7fffffffu; }
+  static constexpr uint32_t kNone = kInfBits;
+  __device__ __forceinline__ static void rescanned(uint32_t addr, uint32_t k1, uint32_t k2, uint32_t k3, uint32_t p1,
+                                                   uint32_t p2) {
+    sts128(addr, make_uint4(k1, k2, k3, (lds32(addr + 12) & 0xffff0000u) | p1 | (p2 << 8)));
+  }
 };
 
 template <>
-struct SumIO<__half> {
-  uint2* v;
-  __device__ __forceinline__ static float hf(uint32_t b) { return __half2float(__ushort_as_half((unsigned short)b)); }
-  __device__ __forceinline__ static uint32_t hb(float x) { return (uint32_t)__half_as_ushort(__float2half_rn(x)); }
-  __device__ __forceinline__ float4 load(int c) const {
-    const uint2 a = v[c];
-    const uint32_t p1 = (a.y >> 16) & 0xffu, p2 = a.y >> 24;
-    const uint32_t nh = (p1 != 255u ? 1u : 0u) + (p2 != 255u ? 1u : 0u);
-    const uint32_t w = p1 | (p2 << 8) | (nh << kNhShift) | (((a.x >> 15) & 1u) << 18) | ((a.x >> 31) << 19) |
-                       (((a.y >> 15) & 1u) << 20);
-    return make_float4(hf(a.x & 0x7fffu), hf((a.x >> 16) & 0x7fffu), hf(a.y & 0x7fffu), __uint_as_float(w));
+struct Sum<__half> {
+  static constexpr int kBytes = 8;
+  static constexpr uint32_t kEmpty = 0x7c00ffu;   // +inf at position 255
+  static constexpr uint32_t kKey = 0x7fffffu;
+  uint2 q;
+  uint32_t k1, k2, F;
+  bool is1;
+  __device__ __forceinline__ void load(uint32_t addr, uint32_t rec) {
+    q = lds64(addr);
+    k1 = q.x & kKey;
+    k2 = (q.y >> 6) & kKey;
+    F = __funnelshift_r(q.x, q.y, 23) & 0x7fffu;
+    is1 = ((q.x ^ rec) & 0xffu) == 0u;
   }
-  __device__ __forceinline__ void store(int c, float4 s) const {
+  __device__ __forceinline__ uint32_t akey() const { return is1 ? k2 : k1; }
+  __device__ __forceinline__ float ans() const { return __half2float(__ushort_as_half((unsigned short)(akey() >> 8))); }
+  __device__ __forceinline__ bool ok() const { return (akey() >> 8) <= F; }
+  __device__ __forceinline__ uint32_t flags() const { return q.y; }
+  __device__ __forceinline__ static uint2 pack(uint32_t k1, uint32_t k2, uint32_t F, uint32_t flags) {
+    return make_uint2(k1 | (F << 23), (F >> 9) | (k2 << 6) | flags);
+  }
+  __device__ __forceinline__ void update(uint32_t addr, uint32_t rec, uint32_t b, uint32_t toggle, bool act) const {
+    const uint32_t xh = b & 0x7fffu;
+    const bool was = is1 || ((k2 ^ rec) & 0xffu) == 0u, ins = xh <= F;
+    const uint32_t b1 = akey(), b2 = was ? kEmpty : k2;
+    const uint32_t y = ins ? __byte_perm(xh, rec, 0x3104) : kEmpty;   // magnitude << 8 | position
+    const uint32_t t = max(y, b1), h = max(t, b2);
+    if (act && (was || ins || toggle))
+      sts64(addr, pack(min(y, b1), min(t, b2), min(F, h >> 8), (q.y ^ toggle) & (kSgnBit | kParBit)));
+  }
+  __device__ __forceinline__ static void init(uint32_t addr, float4 s, uint32_t flip) {
     const uint32_t w = __float_as_uint(s.w);
-    const uint32_t nh = (w >> kNhShift) & 3u;
-    const uint32_t p1 = nh >= 1u ? (w & 0xffu) : 255u, p2 = nh == 2u ? ((w >> 8) & 0xffu) : 255u;
-    v[c] = make_uint2(hb(s.x) | (((w >> 18) & 1u) << 15) | (hb(s.y) << 16) | (((w >> 19) & 1u) << 31),
-                      hb(s.z) | (((w >> 20) & 1u) << 15) | (p1 << 16) | (p2 << 24));
+    sts64(addr, pack(((uint32_t)__half_as_ushort(__float2half_rn(s.x)) << 8) | (w & 0xffu),
+                     ((uint32_t)__half_as_ushort(__float2half_rn(s.y)) << 8) | ((w >> 8) & 0xffu),
+                     (uint32_t)__half_as_ushort(__float2half_rn(s.z)), (w & kSgnBit) ^ flip));
   }
-  __device__ __forceinline__ void flip(int c, uint32_t bits) const {
-    if (bits & kSgnBit) v[c].x ^= 1u << 15;
-    if (bits & kParBit) v[c].y ^= 1u << 15;
-  }
-};
-
-// (value, position) pairs ordered by value, then position
-__device__ __forceinline__ bool before(float a, uint32_t ia, float b, uint32_t ib) {
-  return a < b || (a == b && ia < ib);
-}
-
-struct Top3 {
-  float a1, a2, a3;
-  uint32_t q1, q2;
-  __device__ __forceinline__ void init() {
-    a1 = a2 = a3 = __uint_as_float(kInfBits);
-    q1 = q2 = 255u;
-  }
-  __device__ __forceinline__ void insert(float x, uint32_t q) {
-    const bool b1 = before(x, q, a1, q1), b2 = before(x, q, a2, q2);
-    a3 = b2 ? a2 : fminf(a3, x);
-    a2 = b1 ? a1 : (b2 ? x : a2);
-    q2 = b1 ? q1 : (b2 ? q : q2);
-    a1 = b1 ? x : a1;
-    q1 = b1 ? q : q1;
+  __device__ __forceinline__ static uint32_t key(uint32_t b, uint32_t pos) { return ((b & 0x7fffu) << 8) | pos; }
+  static constexpr uint32_t kNone = kEmpty;
+  __device__ __forceinline__ static void rescanned(uint32_t addr, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t,
+                                                   uint32_t) {
+    sts64(addr, pack(a1, a2, a3 >> 8, lds32(addr + 4) & (kSgnBit | kParBit)));
   }
 };
 
-// Chunks of column data in flight ahead of the update (1 or 2); schedule records go one chunk further.
-constexpr int kAhead = 1;
-
+// Warp-cooperative rescan of the check with summary `addr`, whose CSR row is b .. b + d: the two smallest magnitudes with
+// their positions and the third smallest as the floor; the flags are kept. Each lane keeps the three
+// smallest of its entries; the warp minimum is then taken three times, its owner dropping its entry.
+// NaN messages (sums of +inf and -inf) are no candidates.
 template <typename MT>
-__device__ __forceinline__ SumIO<MT> sum_io(unsigned char* p);
-template <>
-__device__ __forceinline__ SumIO<float> sum_io<float>(unsigned char* p) { return SumIO<float>{reinterpret_cast<float4*>(p)}; }
-template <>
-__device__ __forceinline__ SumIO<__half> sum_io<__half>(unsigned char* p) { return SumIO<__half>{reinterpret_cast<uint2*>(p)}; }
-
-// Warp-cooperative rescan of check c, whose CSR row is b .. b + d: the two smallest magnitudes with
-// their positions and the third smallest as the floor; the flags are kept.
-template <typename MT>
-__device__ __forceinline__ void rescan_row(int c, int b, int d, const uint32_t* rmap, const MT* msg,
-                                           const SumIO<MT>& S, int lane) {
+__device__ __forceinline__ void rescan_row(uint32_t addr, int b, int d, const uint32_t* rmap, const MT* msg, int lane) {
   uint32_t loc[8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int q = lane + 32 * u;
     loc[u] = q < d ? __ldg(rmap + b + q) : 0u;
   }
-  Top3 T;
-  T.init();
+  uint32_t a1 = Sum<MT>::kNone, a2 = a1, a3 = a1, p1 = 255u, p2 = 255u;
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int q = lane + 32 * u;
-    if (q < d) T.insert(fabsf(XMsg<MT>::value(XMsg<MT>::load(msg + loc[u]))), (uint32_t)q);
+    if (32 * u < d) {
+      const uint32_t k = q < d ? Sum<MT>::key(XMsg<MT>::load(msg + loc[u]), (uint32_t)q) : 0xffffffffu;
+      const bool b1 = k < a1, b2 = k < a2;
+      a3 = b2 ? a2 : min(a3, k);
+      a2 = b1 ? a1 : (b2 ? k : a2);
+      p2 = b1 ? p1 : (b2 ? (uint32_t)q : p2);
+      a1 = b1 ? k : a1;
+      p1 = b1 ? (uint32_t)q : p1;
+    }
   }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) {
-    const float b1 = __shfl_xor_sync(kFull, T.a1, off), b2 = __shfl_xor_sync(kFull, T.a2, off);
-    const float b3 = __shfl_xor_sync(kFull, T.a3, off);
-    const uint32_t r1 = __shfl_xor_sync(kFull, T.q1, off), r2 = __shfl_xor_sync(kFull, T.q2, off);
-    T.insert(b1, r1);
-    T.insert(b2, r2);
-    T.insert(b3, 255u);
-  }
-  if (lane == 0) {
-    const uint32_t w = __float_as_uint(S.load(c).w);
-    S.store(c, make_float4(T.a1, T.a2, T.a3, __uint_as_float((w & ~0x3ffffu) | T.q1 | (T.q2 << 8) | (2u << kNhShift))));
-  }
+  const uint32_t r1 = __reduce_min_sync(kFull, a1);
+  const int o1 = __ffs(__ballot_sync(kFull, a1 == r1)) - 1;
+  const uint32_t f1 = __shfl_sync(kFull, p1, o1);
+  if (lane == o1) { a1 = a2; p1 = p2; a2 = a3; p2 = 255u; }
+  const uint32_t r2 = __reduce_min_sync(kFull, a1);
+  const int o2 = __ffs(__ballot_sync(kFull, a1 == r2)) - 1;
+  const uint32_t f2 = __shfl_sync(kFull, p1, o2);
+  if (lane == o2) a1 = a2;
+  const uint32_t r3 = __reduce_min_sync(kFull, a1);
+  if (lane == 0) Sum<MT>::rescanned(addr, r1, r2, r3, f1, f2);
 }
 
-// What a column update reads besides the check summaries: its schedule record (column, degree, first
-// message slot), its checks with their row positions, its prior and its state word. None of it is
-// written by the chunks in between, so it is copied into a shared-memory ring with cp.async ahead of
-// use: the records of chunk c+2 and the rest of chunk c+1 while chunk c is updated. The copies hold
-// no registers, so the warp waits for nothing it does not yet need.
-template <int DP>
-struct XRing {
-  static constexpr int XP = (DP + 3) / 4 * 4;   // words of a column record
-  static constexpr int kStwWords = 48;          // the 16-byte blocks covering 32 state words
-  static constexpr int kRecSlots = kAhead + 2;   // chunk q's records stay until its update
-  static constexpr int kStages = kAhead + 1;
-  static constexpr int kRecBytes = kRecSlots * 32 * 8;
-  static constexpr int kStageBytes = 32 * XP * 4 + 32 * 4 + kStwWords * 4;
-  static constexpr int kBytes = kRecBytes + kStages * kStageBytes;
-  unsigned char* base;
-  __device__ __forceinline__ uint2* rec(uint32_t q) { return reinterpret_cast<uint2*>(base) + (q % kRecSlots) * 32; }
-  __device__ __forceinline__ unsigned char* stage(uint32_t q) { return base + kRecBytes + (q % kStages) * kStageBytes; }
-  __device__ __forceinline__ uint32_t* xc(uint32_t q) { return reinterpret_cast<uint32_t*>(stage(q)); }
-  __device__ __forceinline__ float* lam(uint32_t q) { return reinterpret_cast<float*>(stage(q) + 32 * XP * 4); }
-  __device__ __forceinline__ uint32_t* stw(uint32_t q) {
-    return reinterpret_cast<uint32_t*>(stage(q) + 32 * XP * 4 + 32 * 4);
-  }
+// The part of a warp's shared memory that is not check summaries: what the steps near the current one
+// need. The edge records come in chunks of kChunk steps by cp.async, one chunk ahead; a 64-entry ring
+// holds the step offsets (two 32-step blocks, so that chunks can be fetched ahead across a block's end);
+// st has (signs, decisions, first slot of the next step) of the current block, read by all lanes of a
+// step at once.
+constexpr int kChunk = 4, kBufs = 2;
+constexpr int kChunkSlots = kChunk * 32 + 8;   // a chunk is copied in groups of four slots
+
+struct XWin {
+  uint4 st[32];
+  uint2 rec[kBufs][kChunkSlots];
+  uint32_t lnk[kBufs][kChunkSlots];
+  uint32_t off[64];
 };
+static_assert(sizeof(XWin) % 16 == 0 && kChunkSlots % 4 == 0, "cp.async blocks are 16 bytes");
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// cp.async in its plain form with the source size stated (equal to the copy size). Read-only tables
-// may be cached in L1 (.ca); the per-warp state words, written through L2 by earlier sweeps, are
-// copied with .cg so that no L1 line can be stale.
-__device__ __forceinline__ void cp_async_ca4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_ca8(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_cg16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+__device__ __forceinline__ void cp_async_cg16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// A chunk of a sweep: up to 32 consecutive schedule entries [cs, min(cs + 32, e)) of level l, whose
-// entries end at e. l == nl marks the end of the sweep.
-struct Chunk {
-  int l;
-  uint32_t cs, e;
-};
-
-// The member's level offsets lo[0 .. nl] as the chunk walker needs them, one level at a time: lane l
-// holds lo[32k + l] of the current window k and lo[32k + 32 + l] of the next one, loaded 32 levels
-// before it is needed, so that starting a level costs a shuffle instead of a dependent global load.
-struct LevelWin {
-  const uint32_t* lo;
-  int nl, k;
-  uint32_t cur, nxt;
-  __device__ __forceinline__ uint32_t load(int x, int lane) const {
-    return x + lane <= nl ? __ldg(lo + x + lane) : 0u;
+// Copies the records of the chunk of steps [s, s + kChunk) into buffer `buf` (one commit group, empty
+// past the last step). win: shared address of the window; first: the member's first slot in the tables.
+__device__ __forceinline__ void fetch_chunk(uint32_t win, int buf, int s, const uint2* rec, const uint32_t* lnk,
+                                            size_t first, int lane) {
+  const uint32_t off = win + (uint32_t)offsetof(XWin, off);
+  const size_t b = (first + lds32(off + 4 * (s & 63))) & ~(size_t)3, e = first + lds32(off + 4 * ((s + kChunk) & 63));
+  const uint32_t dr = win + (uint32_t)offsetof(XWin, rec) + (uint32_t)buf * (uint32_t)sizeof(XWin::rec[0]);
+  const uint32_t dl = win + (uint32_t)offsetof(XWin, lnk) + (uint32_t)buf * (uint32_t)sizeof(XWin::lnk[0]);
+  const int quads = (int)((e - b + 3) >> 2);
+  for (int q = lane; q < quads; q += 32) {
+    cp_async_cg16(dr + 32 * q, rec + b + 4 * q);
+    cp_async_cg16(dr + 32 * q + 16, rec + b + 4 * q + 2);
+    cp_async_cg16(dl + 16 * q, lnk + b + 4 * q);
   }
-  __device__ __forceinline__ void start(const uint32_t* lo_, int nl_, int lane) {
-    lo = lo_;
-    nl = nl_;
-    k = 0;
-    cur = load(0, lane);
-    nxt = load(32, lane);
-  }
-  // lo[x]; x never decreases and grows by at most one per call (warp-uniform)
-  __device__ __forceinline__ uint32_t get(int x, int lane) {
-    if (x >= 32 * (k + 1)) {
-      ++k;
-      cur = nxt;
-      nxt = load(32 * (k + 1), lane);
-    }
-    return __shfl_sync(kFull, cur, x - 32 * k);
-  }
-};
-
-__device__ __forceinline__ Chunk first_chunk(LevelWin& W, int lane) {
-  const uint32_t a = W.get(0, lane);
-  return Chunk{0, a, W.get(1, lane)};
+  cp_async_commit();
 }
 
-__device__ __forceinline__ Chunk next_chunk(const Chunk& c, LevelWin& W, int lane) {
-  if (c.l >= W.nl) return c;
-  if (c.cs + 32 < c.e) return Chunk{c.l, c.cs + 32, c.e};
-  return Chunk{c.l + 1, c.e, c.l + 1 < W.nl ? W.get(c.l + 2, lane) : c.e};
+__device__ __forceinline__ float add_if(float acc, float x, uint32_t cond) {
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p add.rn.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(x), "r"(cond));
+  return acc;
 }
 
-__device__ __forceinline__ bool in_chunk(const Chunk& c, int nl, int lane) {
-  return c.l < nl && c.cs + (uint32_t)lane < c.e;
-}
-
-// Per-warp views of the current pair's state.
-template <typename MT>
-struct XState {
-  SumIO<MT> S;       // shared: m check summaries
-  MT* msg;           // global: E messages in the member's schedule order
-  uint32_t* stw;     // global: n column state words in schedule order
-  uint32_t* dec;     // global: nw decision bits in column order
-  const uint2* rec;  // the member's schedule records
-  const uint32_t* rmap;   // the member's CSR-entry -> message-slot map
-};
-
-// Serial-V update of one chunk (lane's column d when active). Returns the lane's change of the number
-// of unsatisfied checks.
-// The lane's column as the update sees it (read from the ring).
-template <int DP>
-struct XCol {
-  uint32_t v, deg, spos, st;
-  float lam;
-  uint32_t ent[DP];   // (check << 8) | position in the check's row
-};
-
-template <typename MT, int DP>
-__device__ __forceinline__ int update_chunk(bool active, const XCol<DP>& d, uint32_t j, const Tables& t, float alpha,
-                                            const XState<MT>& X, float* lpost, int lane, uint32_t& my_rescans) {
-  // check-to-variable messages from the summaries (Algorithm 1's check update over N(c) \ v)
-  float mcv[DP];
-  uint32_t need = 0u;
-#pragma unroll
-  for (int k = 0; k < DP; ++k) {
-    mcv[k] = 0.0f;
-    if (active && (uint32_t)k < d.deg) {
-      const float4 s = X.S.load((int)(d.ent[k] >> 8));
-      float mn;
-      if (!xquery(s, d.ent[k] & 0xffu, mn)) need |= 1u << k;
-      const uint32_t w = __float_as_uint(s.w);
-      const float mag = __fmul_rn(alpha, mn);
-      mcv[k] = (((w >> 18) ^ (w >> 19) ^ (d.st >> k)) & 1u) ? -mag : mag;   // sign parity, syndrome, own sign
-    }
-  }
-  if (__any_sync(kFull, need != 0u)) {
-    // rescan every check whose summary could not answer (checks of one level are touched by one
-    // column each, so the rows are distinct), then ask again. Row bounds of all of them first.
-    int rb[DP], rd[DP];
-#pragma unroll
-    for (int k = 0; k < DP; ++k) {
-      rb[k] = 0;
-      rd[k] = 0;
-      if ((need >> k) & 1u) {
-        const int c = (int)(d.ent[k] >> 8);
-        rb[k] = __ldg(t.rowptr + c);
-        rd[k] = __ldg(t.rowptr + c + 1);
-      }
-    }
-    uint32_t pend = need;
-    while (__any_sync(kFull, pend != 0u)) {
-      const int k0 = __ffs(pend) - 1;
-      uint32_t csel = 0u;
-      int bsel = 0, esel = 0;
-#pragma unroll
-      for (int k = 0; k < DP; ++k) {
-        csel = k == k0 ? d.ent[k] >> 8 : csel;
-        bsel = k == k0 ? rb[k] : bsel;
-        esel = k == k0 ? rd[k] : esel;
-      }
-      uint32_t bal = __ballot_sync(kFull, pend != 0u);
-      while (bal) {
-        const int src = __ffs(bal) - 1;
-        bal &= bal - 1u;
-        const int b = __shfl_sync(kFull, bsel, src);
-        rescan_row<MT>((int)__shfl_sync(kFull, csel, src), b, __shfl_sync(kFull, esel, src) - b, X.rmap, X.msg,
-                       X.S, lane);
-        ++my_rescans;
-      }
-      pend &= pend - 1u;
+// One sweep of a member over its ns steps. win: shared address of the warp's window (the summaries follow it); stg: (signs, decisions) of every
+// step in global scratch; LP: the posteriors go to lp. Returns the lane's change of the number of
+// unsatisfied checks.
+template <typename MT, int DP, bool LP>
+__device__ __forceinline__ int sweep_x(const Tables& t, const uint32_t* soff, const int ns, const size_t first,
+                                       const uint32_t* rmap, const float alpha, const uint32_t win, MT* msg, uint2* stg,
+                                       float* lp, uint32_t& rescans, const int lane) {
+  const uint32_t sums = win + (uint32_t)sizeof(XWin), off = win + (uint32_t)offsetof(XWin, off);
+  const uint2* trec = t.xrec;
+  const uint32_t* tlnk = t.xlnk;
+  const int32_t* rowptr = t.rowptr;
+  const int pitch = t.soff_pitch;
+  int dpar = 0;
+  uint32_t coff = __ldg(soff + lane), noff = __ldg(soff + 32 + lane);   // offsets of this block's steps and the next's
+  uint2 cst = lane < ns ? stg[lane] : make_uint2(0u, 0u), nst = cst;
+  sts32(off + 4 * lane, coff);
+  uint32_t ol = (uint32_t)lane;   // slot of the lane's edge
+  int buf = 0;
+  for (int s0 = 0; s0 < ns; s0 += 32) {
+    // block of 32 steps: its states and the next block's offsets into the window, the loads for the next
+    sts32(off + 4 * (((s0 + 32) & 63) + lane), noff);
+    {
+      const uint32_t up = __shfl_down_sync(kFull, coff, 1), nx = __shfl_sync(kFull, noff, 0);
+      sts128(win + 16 * lane, make_uint4(cst.x, cst.y, lane == 31 ? nx : up, 0u));
     }
     __syncwarp();
+    if (s0 == 0) fetch_chunk(win, 0, 0, trec, tlnk, first, lane);
+    coff = noff;
+    if (s0 + 32 < ns) {
+      noff = s0 + 64 + lane < pitch ? __ldg(soff + s0 + 64 + lane) : 0u;
+      nst = s0 + 32 + lane < ns ? stg[s0 + 32 + lane] : make_uint2(0u, 0u);
+    }
+    uint32_t wst = win;   // the step's window entry
+    for (int s1 = s0; s1 < min(s0 + 32, ns); s1 += kChunk) {
+      // this chunk's records are here, the last one's buffer is free
+      cp_async_wait<0>();
+      __syncwarp();
+      fetch_chunk(win, buf ^ 1, s1 + kChunk, trec, tlnk, first, lane);
+      // addresses of slot 0's records if the buffer reached back that far
+      const uint32_t o0 = ol - (uint32_t)lane, sh = (((uint32_t)first + o0) & 3u) - o0;
+      const uint32_t ra = win + (uint32_t)offsetof(XWin, rec) + (uint32_t)buf * (uint32_t)sizeof(XWin::rec[0]) + 8u * sh;
+      const uint32_t la = win + (uint32_t)offsetof(XWin, lnk) + (uint32_t)buf * (uint32_t)sizeof(XWin::lnk[0]) + 4u * sh;
+      buf ^= 1;
+#pragma unroll 1
+      for (int u = 0; u < kChunk; ++u) {   // steps past the last one have no edges
+        const uint4 st = lds128(wst);
+        uint2 r = make_uint2(0u, 0u);
+        uint32_t ln = 0u;
+        if (ol < st.z) {
+          r = lds64(ra + 8u * ol);
+          ln = lds32(la + 4u * ol);
+        }
+        const bool act = (int)ln < 0;
+        const uint32_t sa = sums + (r.x >> 18) * (uint32_t)Sum<MT>::kBytes;
+        const uint32_t osg = st.x << (31 - lane);   // bit 31: sign of the edge's own old message
+        Sum<MT> S;
+        S.load(sa, r.x);
+        uint32_t bal = __ballot_sync(kFull, act && !S.ok());
+        if (bal) {
+          // rescan every check whose summary could not answer (the checks of a step are distinct), ask again
+          int rb = 0, rd = 0;
+          if ((bal >> lane) & 1u) {
+            rb = __ldg(rowptr + (r.x >> 18));
+            rd = __ldg(rowptr + (r.x >> 18) + 1) - rb;
+          }
+          while (bal) {
+            const int src = __ffs(bal) - 1;
+            bal &= bal - 1u;
+            rescan_row<MT>(__shfl_sync(kFull, sa, src), __shfl_sync(kFull, rb, src), __shfl_sync(kFull, rd, src), rmap,
+                           msg, lane);
+            ++rescans;
+          }
+          __syncwarp();
+          S.load(sa, r.x);
+        }
+        // check-to-variable message (Algorithm 1's check update over N(c) \ v): sign parity, syndrome, own
+        // sign; then the exclusion sum: lambda and the column's other messages in ascending check order
+        const uint32_t mcv = __float_as_uint(__fmul_rn(alpha, S.ans())) ^ ((S.flags() ^ osg) & kSgnBit);
+        float acc = __uint_as_float(r.y);
 #pragma unroll
-    for (int k = 0; k < DP; ++k)
-      if ((need >> k) & 1u) {
-        const float4 s = X.S.load((int)(d.ent[k] >> 8));
-        float mn;
-        xquery(s, d.ent[k] & 0xffu, mn);
-        const uint32_t w = __float_as_uint(s.w);
-        const float mag = __fmul_rn(alpha, mn);
-        mcv[k] = (((w >> 18) ^ (w >> 19) ^ (d.st >> k)) & 1u) ? -mag : mag;
-      }
-  }
-  if (!active) return 0;
-  const uint32_t deg = d.deg;
-  float L = d.lam;
-#pragma unroll
-  for (int k = 0; k < DP; ++k)
-    if ((uint32_t)k < deg) L = __fadd_rn(L, mcv[k]);
-  const uint32_t e_new = L <= 0.0f ? 1u : 0u;
-  const bool flip = e_new != ((d.st & kDecBit) ? 1u : 0u);
-  uint32_t st = e_new << 31;
-  int dpar = 0;
-  float pre = d.lam;   // lambda + m_0 + ... + m_{k-1}, the shared head of every exclusion sum
-  MT* out = X.msg + d.spos;
-#pragma unroll
-  for (int k = 0; k < DP; ++k) {
-    if ((uint32_t)k < deg) {
-      float a = pre;
-#pragma unroll
-      for (int k2 = k + 1; k2 < DP; ++k2)
-        if ((uint32_t)k2 < deg) a = __fadd_rn(a, mcv[k2]);
-      const float x = XMsg<MT>::round(a);
-      store_msg<MT>(out + k, x);   // streamed: read again only by rescans
-      pre = __fadd_rn(pre, mcv[k]);
-      const uint32_t sx = sign_bit(x);
-      st |= sx << k;
-      // this level's only reader and writer of the check: the full summary update for holders and
-      // for edges that drop below the floor, a flag update for the rest
-      const int c = (int)(d.ent[k] >> 8);
-      const uint32_t p = d.ent[k] & 0xffu;
-      const float4 s = X.S.load(c);
-      const float ax = fabsf(x);
-      const uint32_t fl = ((((d.st >> k) ^ sx) & 1u) ? kSgnBit : 0u) | (flip ? kParBit : 0u);
-      if (flip) dpar += (__float_as_uint(s.w) & kParBit) ? -1 : 1;
-      if (xslow(s, p, ax)) {
-        float4 u = xupdate(s, p, ax);
-        u.w = __uint_as_float(__float_as_uint(u.w) ^ fl);
-        X.S.store(c, u);
-      } else if (fl) {
-        X.S.flip(c, fl);
+        for (int j = 0; j < DP; ++j)
+          acc = add_if(acc, __uint_as_float(__shfl_sync(kFull, mcv, (int)ln + j)), ln & (32u << j));
+        const float L = __fadd_rn(acc, __uint_as_float(mcv));   // on the last edge's lane: the posterior
+        const uint32_t dec = __ballot_sync(kFull, (ln & kLnkLast) && L <= 0.0f);
+        const uint32_t xb = XMsg<MT>::round(acc), xs = XMsg<MT>::sign31(xb);
+        const uint32_t sg = __ballot_sync(kFull, (int)(xs & ln) < 0);
+        if (act) XMsg<MT>::store(msg + ol, xb);   // streamed: read again only by rescans
+        uint32_t toggle = (xs ^ osg) & kSgnBit;
+        const uint32_t ch = dec ^ st.y;
+        if (ch) {   // some column of the step changed its decision
+          if (act && ((ch >> ((ln >> kLnkLastLane) & 31u)) & 1u)) {
+            toggle |= kParBit;
+            dpar += (S.flags() & kParBit) ? -1 : 1;
+          }
+        }
+        S.update(sa, r.x, xb, toggle, act);
+        if (lane == 0) sts64(wst, make_uint2(sg, dec));
+        if (LP) {
+          if (ln & kLnkLast) lp[__ldg(t.xcolid + first + ol)] = L;
+          else if (ln == 0u && ol < st.z) lp[__ldg(t.xcolid + first + ol)] = __uint_as_float(r.y);   // no checks
+        }
+        ol = st.z + (uint32_t)lane;
+        wst += 16u;
+        __syncwarp();
       }
     }
+    if (s0 + lane < ns) stg[s0 + lane] = lds64(win + 16 * lane);
+    __syncwarp();
+    cst = nst;
   }
-  __stcs(X.stw + j, st);
-  if (flip) atomicXor(X.dec + (d.v >> 5), 1u << (d.v & 31));
-  if (lpost) lpost[d.v] = L;
+  cp_async_wait<0>();
   return dpar;
 }
 
-// Ring copies for chunk number q. Records: each active lane copies its own 8-byte schedule record.
-template <int DP>
-__device__ __forceinline__ void issue_rec(XRing<DP>& R, uint32_t q, const Chunk& c, int nl, int lane, const uint2* rec) {
-  if (in_chunk(c, nl, lane)) cp_async_ca8(R.rec(q) + lane, rec + c.cs + lane);
-}
-
-// Column data: each active lane copies its column's record and prior (its schedule record is in the
-// ring already); lanes 0..8 copy the 16-byte blocks that cover the chunk's state words.
-template <int DP>
-__device__ __forceinline__ void issue_data(XRing<DP>& R, uint32_t q, const Chunk& c, int nl, int lane, const Tables& t,
-                                           const uint32_t* stw) {
-  if (c.l >= nl) return;
-  if (in_chunk(c, nl, lane)) {
-    const uint32_t v = R.rec(q)[lane].x & 0xffffffu;
-    const uint32_t* src = t.xcol + (size_t)v * t.XP;
-    uint32_t* dst = R.xc(q) + lane * XRing<DP>::XP;
-#pragma unroll
-    for (int b = 0; b < XRing<DP>::XP / 4; ++b)
-      if (4 * b < t.XP) cp_async_cg16(dst + 4 * b, src + 4 * b);
-    cp_async_ca4(R.lam(q) + lane, t.lam + v);
-  }
-  const uint32_t first = c.cs & ~3u, end = min(c.cs + 32u, c.e);
-  if ((uint32_t)lane < (end - first + 3u) / 4u) cp_async_cg16(R.stw(q) + 4 * lane, stw + first + 4 * lane);
-}
-
-template <int DP>
-__device__ __forceinline__ void read_col(XRing<DP>& R, uint32_t q, const Chunk& c, int lane, bool act, XCol<DP>& d) {
-  if (!act) {
-    d.deg = 0u;
-    return;
-  }
-  const uint2 r = R.rec(q)[lane];
-  d.v = r.x & 0xffffffu;
-  d.deg = r.x >> 24;
-  d.spos = r.y;
-  d.lam = R.lam(q)[lane];
-  d.st = R.stw(q)[(c.cs & 3u) + lane];
-  const uint4* src = reinterpret_cast<const uint4*>(R.xc(q) + lane * XRing<DP>::XP);
-#pragma unroll
-  for (int b = 0; b < XRing<DP>::XP / 4; ++b) {
-    const uint4 x = src[b];
-    if (4 * b + 0 < DP) d.ent[4 * b + 0] = x.x;
-    if (4 * b + 1 < DP) d.ent[4 * b + 1] = x.y;
-    if (4 * b + 2 < DP) d.ent[4 * b + 2] = x.z;
-    if (4 * b + 3 < DP) d.ent[4 * b + 3] = x.w;
-  }
-}
+// What a member's run is told and what it reports.
+struct MemberRun {
+  const uint32_t* syn;   // the shot's syndrome words
+  int nsyn;              // its flipped checks
+  int budget;            // sweeps at most
+  bool soft, keep_last;  // the posterior after every sweep / after sweep T
+  const int* conv;       // pair mode: the shot's converged members (pair_should_stop), else NULL
+  int K, M;
+  // results
+  int ran;               // sweeps run
+  uint32_t rescans;
+};
 
 // One member (index i) on one shot: initialises the member's state and runs up to `budget` sweeps,
-// stopping at the first that leaves H e = s, or before sweep `it` when stop(it) holds. Returns the
-// converging sweep (0 if none) and in `ran` the sweeps run; leaves the decisions in X.dec and the
-// posterior of the last sweep in lpost when soft output is on or `keep_last` is set and the member
-// reached sweep T.
-template <typename MT, int DP, typename Stop>
-__device__ __forceinline__ int run_member_x(const BpArgs& a, const Tables& t, int i, const uint32_t* syn, int nsyn,
-                                            int budget, bool keep_last, XState<MT>& X, unsigned char* base,
-                                            float* lpost, int lane, uint32_t& my_iters, uint32_t& my_rescans,
-                                            int& ran, Stop stop) {
-  const int n = t.n, m = t.m, T = t.T, nw = t.nw;
-  X.rec = t.xrec + (size_t)i * n;
-  X.rmap = t.xrmap + (size_t)i * t.E;
-  // member init: prior summaries with this shot's syndrome (parity = s), prior messages in the
-  // member's schedule order, state words and decisions 0
-  for (int c = lane; c < m; c += 32) {
-    float4 s = __ldg(t.xsum + c);
-    const uint32_t sb = (__ldg(syn + (c >> 5)) >> (c & 31)) & 1u;
-    s.w = __uint_as_float(__float_as_uint(s.w) | (sb ? (kSynBit | kParBit) : 0u));
-    X.S.store(c, s);
-  }
-  for (int j = lane; j < n; j += 32) {
-    const uint2 r = __ldg(X.rec + j);
-    const float x = XMsg<MT>::round(__ldg(t.lam + (r.x & 0xffffffu)));
-    for (uint32_t k = 0; k < (r.x >> 24); ++k) store_msg<MT>(X.msg + r.y + k, x);
-    __stcg(X.stw + j, 0u);
-  }
-  for (int w = lane; w < nw; w += 32) __stcg(X.dec + w, 0u);
+// stopping at the first that leaves H e = s, or in pair mode before a sweep that no longer counts.
+// Returns the converging sweep (0 if none; its decisions are then in the warp's scratch, column order);
+// leaves the posterior of the last sweep in the scratch when soft output is on or `keep_last` is set
+// and the member reached sweep T. smem_off: the warp's shared memory; gs: its global scratch. Not
+// inlined: the sweep gets its own registers, whatever the caller keeps between members.
+template <typename MT, int DP>
+__device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, int smem_off, unsigned char* gs) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  // Both through a shuffle: the compiler would otherwise read the thread index again wherever the lane is
+  // used and keep the addresses in uniform registers, moving them over at each use (14 of the 184
+  // instructions of a step).
+  const int lane = __shfl_sync(kFull, (int)(threadIdx.x & 31), (int)(threadIdx.x & 31));
+  const uint32_t win = __shfl_sync(kFull, (uint32_t)__cvta_generic_to_shared(smem) + (uint32_t)smem_off, lane);
+  const uint32_t sums = win + (uint32_t)sizeof(XWin);
+  const int m = t.m, T = t.T, nw = t.nw;
+  MT* msg = reinterpret_cast<MT*>(gs + t.xg_msg);
+  uint2* stg = reinterpret_cast<uint2*>(gs + t.xg_st);   // (signs, decisions) of every step
+  const uint32_t* syn = R.syn;
+  uint32_t rescans = 0;
+  const size_t first = (size_t)i * t.SP;
+  const uint32_t* colid = t.xcolid + first;
+  const uint32_t* rmap = t.xrmap + (size_t)i * t.E;
+  const uint32_t* soff = t.soff + (size_t)i * t.soff_pitch;
+  const int ns = __ldg(t.stepcnt + i);
+  // member init: prior summaries with this shot's syndrome (parity = s), prior messages in step order,
+  // signs and decisions 0
+  for (int c = lane; c < m; c += 32)
+    Sum<MT>::init(sums + c * Sum<MT>::kBytes, __ldg(t.xsum + c),
+                  ((__ldg(syn + (c >> 5)) >> (c & 31)) & 1u) ? (kSgnBit | kParBit) : 0u);
+  for (int j = lane; j < t.SP; j += 32)
+    XMsg<MT>::store(msg + j, XMsg<MT>::round(__uint_as_float(__ldg(&t.xrec[first + j].y))));
+  for (int s = lane; s < ns; s += 32) stg[s] = make_uint2(0u, 0u);
   __syncwarp();
-  const uint32_t* lo = t.lvl_off + (size_t)i * (n + 1);
-  const int nl = __ldg(t.nlev + i);
-  XRing<DP> R{base};
   const float alpha = __ldg(t.alpha_m + i);   // member i's scaling factor
-  int unsat = nsyn;
-  int conv = 0;
-  ran = 0;
+  const int budget = R.budget;
+  int unsat = R.nsyn;
+  int conv = 0, ran = 0;
   for (int it = 1; it <= budget; ++it) {
-    if (stop(it)) break;
+    if (R.conv && pair_should_stop(R.conv, R.K, R.M, i, it, lane)) break;
     // the posterior is needed after the last possible sweep of a member that may end without
     // converging (LLR average) and, for soft output, after every sweep
-    float* lp = (a.want_soft || (it == T && keep_last)) ? lpost : nullptr;
-    // the sweep in chunks of up to 32 columns of one level, one column per lane, through the ring:
-    // q counts chunks; the records of chunk q+2 and the column data of chunk q+1 are in flight while
-    // chunk q is updated
-    LevelWin W;
-    W.start(lo, nl, lane);
-    Chunk c0 = first_chunk(W, lane);
-    Chunk c1 = next_chunk(c0, W, lane);
-    Chunk c2 = next_chunk(c1, W, lane);
-    issue_rec(R, 0u, c0, nl, lane, X.rec);
-    issue_rec(R, 1u, c1, nl, lane, X.rec);
-    cp_async_commit();
-    cp_async_wait<0>();
-    issue_data<DP>(R, 0u, c0, nl, lane, t, X.stw);
-    cp_async_commit();
-    int dpar = 0;
-    for (uint32_t q = 0; c0.l < nl; ++q) {
-      cp_async_wait<0>();   // chunk q's data and chunk q+1's records
-      __syncwarp();
-      issue_rec(R, q + 2u, c2, nl, lane, X.rec);
-      issue_data<DP>(R, q + 1u, c1, nl, lane, t, X.stw);
-      cp_async_commit();
-      const bool act = in_chunk(c0, nl, lane);
-      XCol<DP> d;
-      read_col<DP>(R, q, c0, lane, act, d);
-      dpar += update_chunk<MT, DP>(act, d, c0.cs + lane, t, alpha, X, lp, lane, my_rescans);
-      __syncwarp();
-      c0 = c1;
-      c1 = c2;
-      c2 = next_chunk(c2, W, lane);
-    }
-    cp_async_wait<0>();
+    int dpar;
+    float* lp = reinterpret_cast<float*>(gs + t.xg_lpost);
+    if (R.soft || (it == T && R.keep_last))
+      dpar = sweep_x<MT, DP, true>(t, soff, ns, first, rmap, alpha, win, msg, stg, lp, rescans, lane);
+    else
+      dpar = sweep_x<MT, DP, false>(t, soff, ns, first, rmap, alpha, win, msg, stg, lp, rescans, lane);
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) dpar += __shfl_xor_sync(kFull, dpar, off);
     unsat += dpar;
-    ++my_iters;
     ran = it;
     if (unsat == 0) { conv = it; break; }
+  }
+  R.ran = ran;
+  R.rescans = rescans;
+  if (conv) {   // decisions in column order
+    uint32_t* bits = reinterpret_cast<uint32_t*>(gs + t.xg_dec);
+    for (int w = lane; w < nw; w += 32) __stcg(bits + w, 0u);
+    __syncwarp();
+    for (int s = lane; s < ns; s += 32) {
+      uint32_t d = stg[s].y;
+      const uint32_t o = __ldg(soff + s);
+      while (d) {
+        const uint32_t v = __ldg(colid + o + (uint32_t)__ffs(d) - 1u);
+        atomicOr(bits + (v >> 5), 1u << (v & 31));
+        d &= d - 1u;
+      }
+    }
+    __syncwarp();
   }
   return conv;
 }
@@ -617,18 +518,14 @@ __device__ __forceinline__ float decision_weight(const Tables& t, const uint32_t
   return W;
 }
 
-// Decodes shot `shot` of problem t with one warp. base: the warp's shared memory; gs: its global
+// Decodes shot `shot` of problem t with one warp. smem_off: the warp's shared memory; gs: its global
 // scratch (messages, state words, decisions, posterior, LLR accumulator, candidate records).
 template <typename MT, int DP>
-__device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, uint32_t shot, unsigned char* base,
+__device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, uint32_t shot, int smem_off,
                                               unsigned char* gs, int lane, uint32_t& my_iters,
                                               uint32_t& my_shots, uint32_t& my_fail, uint32_t& my_rescans) {
   const int n = t.n, m = t.m, K = t.K, M = t.M, T = t.T, nw = t.nw, kw = t.kw, mw = t.mw;
-  XState<MT> X;
-  X.S = sum_io<MT>(base + XRing<DP>::kBytes);
-  X.msg = reinterpret_cast<MT*>(gs + t.xg_msg);
-  X.stw = reinterpret_cast<uint32_t*>(gs + t.xg_st);
-  X.dec = reinterpret_cast<uint32_t*>(gs + t.xg_dec);
+  const uint32_t* dec = reinterpret_cast<const uint32_t*>(gs + t.xg_dec);
   float* lpost = reinterpret_cast<float*>(gs + t.xg_lpost);
   float* acc = reinterpret_cast<float*>(gs + t.xg_acc);
   uint32_t* cand = reinterpret_cast<uint32_t*>(gs + t.xg_cand);
@@ -672,14 +569,15 @@ __device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, 
   for (int i = 0; i < K; ++i) {
     const int budget = ncand < M ? T : __shfl_sync(kFull, c_t, M - 1) - 1;
     if (budget <= 0) break;
-    int ran = 0;
-    const int conv = run_member_x<MT, DP>(a, t, i, syn, nsyn, budget, ncand == 0, X, base, lpost, lane, my_iters,
-                                          my_rescans, ran, [](int) { return false; });
+    MemberRun R{syn, nsyn, budget, a.want_soft != 0, ncand == 0, nullptr, K, M, 0, 0u};
+    const int conv = run_member_x<MT, DP>(t, i, R, smem_off, gs);
+    my_iters += (uint32_t)R.ran;
+    my_rescans += R.rescans;
     if (conv) {
       // insert (conv, i); i exceeds every member already listed, so it goes after equal iterations
       const int p = __popc(__ballot_sync(kFull, lane < ncand && c_t <= conv));
       const int slot = ncand < M ? ncand : __shfl_sync(kFull, c_slot, M - 1);
-      const float W = decision_weight(t, X.dec, cand + (size_t)slot * nw, lane);
+      const float W = decision_weight(t, dec, cand + (size_t)slot * nw, lane);
       if (a.want_soft) {
         float* dst = cpost + (size_t)slot * n;
         for (int v = lane; v < n; v += 32) dst[v] = lpost[v];
@@ -755,7 +653,7 @@ __device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, 
 // shot to finish writes the shot's outcome (pair_epilogue, vibe_internal.cuh).
 template <typename MT, int DP>
 __device__ __forceinline__ void decode_pair_x(const BpArgs& a, const Tables& t, uint32_t shot, int slot, int i,
-                                              unsigned char* base, unsigned char* gs, int lane, uint32_t& my_iters,
+                                              int smem_off, unsigned char* gs, int lane, uint32_t& my_iters,
                                               uint32_t& my_shots, uint32_t& my_fail, uint32_t& my_rescans) {
   const int K = t.K, M = t.M, T = t.T, n = t.n, m = t.m, mw = t.mw, nw = t.nw, kw = t.kw;
   if (i >= K) return;
@@ -788,26 +686,23 @@ __device__ __forceinline__ void decode_pair_x(const BpArgs& a, const Tables& t, 
     return;
   }
   if (i == 0) ++my_shots;
-  XState<MT> X;
-  X.S = sum_io<MT>(base + XRing<DP>::kBytes);
-  X.msg = reinterpret_cast<MT*>(gs + t.xg_msg);
-  X.stw = reinterpret_cast<uint32_t*>(gs + t.xg_st);
-  X.dec = reinterpret_cast<uint32_t*>(gs + t.xg_dec);
+  const uint32_t* dec = reinterpret_cast<const uint32_t*>(gs + t.xg_dec);
   float* lpost = reinterpret_cast<float*>(gs + t.xg_lpost);
   int* conv = a.pconv + (size_t)slot * a.pair_K;
-  int ran = 0;
-  const int cv = run_member_x<MT, DP>(a, t, i, syn, nsyn, T, true, X, base, lpost, lane, my_iters, my_rescans, ran,
-                                      [&](int it) { return pair_should_stop(conv, K, M, i, it, lane); });
+  MemberRun R{syn, nsyn, T, a.want_soft != 0, true, conv, K, M, 0, 0u};
+  const int cv = run_member_x<MT, DP>(t, i, R, smem_off, gs);
+  my_iters += (uint32_t)R.ran;
+  my_rescans += R.rescans;
   const size_t rec = (size_t)slot * a.pair_K + i;
   if (cv) {
-    const float W = decision_weight(t, X.dec, a.pbits + rec * a.bnd.nw, lane);
+    const float W = decision_weight(t, dec, a.pbits + rec * a.bnd.nw, lane);
     if (lane == 0) a.pW[rec] = W;
     if (a.want_soft)
       for (int v = lane; v < n; v += 32) a.ppost[rec * a.bnd.n + v] = lpost[v];
     __threadfence();
     __syncwarp();
     if (lane == 0) *reinterpret_cast<volatile int*>(conv + i) = cv;
-  } else if (ran == T) {
+  } else if (R.ran == T) {
     llr_term_add(lpost, a.pterms + rec * a.bnd.n, n, true, lane);
   }
   __syncwarp();
@@ -815,14 +710,15 @@ __device__ __forceinline__ void decode_pair_x(const BpArgs& a, const Tables& t, 
   __syncwarp();
 }
 
-// Blocks (one warp each) per SM the register budget targets.
+// Blocks (one warp each) per SM the register budget targets: 128 registers, with which the sweep spills
+// nothing. (24 blocks and 80 registers spill inside it and are no faster: the engine waits on latencies.)
 constexpr int kMinBlocksX = 16 / kBpxWarpsPerCta;
 
 // MIXED: shots name their problems (dem_of_shot); the descriptors are copied to shared memory after
 // the warps' regions and shots of image-engine problems are left to that kernel. Otherwise every shot
 // decodes a.one from the parameter space.
 template <typename MT, int DP, bool MIXED>
-__global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const BpArgs a) {
+__global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const __grid_constant__ BpArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int wcta = threadIdx.x >> 5;
@@ -835,7 +731,7 @@ __global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const
     for (int q = threadIdx.x; q < words; q += blockDim.x) dst[q] = __ldg(src + q);
     __syncthreads();
   }
-  unsigned char* base = smem + (size_t)wcta * a.bnd.x_warp_smem;
+  const int smem_off = wcta * a.bnd.x_warp_smem;
   unsigned char* gs = a.xscratch + gw * a.xscratch_pitch;
   uint32_t my_iters = 0, my_shots = 0, my_fail = 0, my_rescans = 0;   // flushed before they could wrap
 
@@ -867,9 +763,9 @@ __global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const
           continue;
         }
         if (sdem[di].engine != VIBE_ENGINE_SUMMARY) continue;   // left to the image engine
-        decode_pair_x<MT, DP>(a, sdem[di], shot, (int)shot, i, base, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+        decode_pair_x<MT, DP>(a, sdem[di], shot, (int)shot, i, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
       } else {
-        decode_pair_x<MT, DP>(a, a.one, shot, (int)shot, i, base, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+        decode_pair_x<MT, DP>(a, a.one, shot, (int)shot, i, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
       }
     }
   }
@@ -908,9 +804,9 @@ __global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const
         continue;
       }
       if (sdem[di].engine != VIBE_ENGINE_SUMMARY) continue;   // left to the image engine
-      decode_shot_x<MT, DP>(a, sdem[di], shot, base, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+      decode_shot_x<MT, DP>(a, sdem[di], shot, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
     } else {
-      decode_shot_x<MT, DP>(a, a.one, shot, base, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+      decode_shot_x<MT, DP>(a, a.one, shot, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
     }
   }
   if (lane == 0 && a.counters) {
@@ -990,22 +886,14 @@ int bpx_degree_bucket(int maxcol) {
   return maxcol <= 4 ? 4 : maxcol <= 6 ? 6 : maxcol <= 8 ? 8 : maxcol <= 16 ? 16 : 0;
 }
 
-int bpx_ring_bytes(int XD) {
-  switch (XD) {
-    case 4: return XRing<4>::kBytes;
-    case 6: return XRing<6>::kBytes;
-    case 8: return XRing<8>::kBytes;
-    case 16: return XRing<16>::kBytes;
-    default: return 0;
-  }
-}
+int bpx_window_bytes() { return (int)sizeof(XWin); }
+
+int bpx_summary_bytes(int m, int msg_fp16) { return (int)a16((msg_fp16 ? 8 : 16) * (size_t)m); }
 
 void bpx_layout(Tables* t, int msg_fp16) {
-  // the check summaries (16 or 8 bytes per check); the prefetch ring comes on top (bounds)
-  t->x_warp_smem = (int)a16((msg_fp16 ? 8 : 16) * (size_t)t->m);
   long long g = 0;
-  t->xg_msg = g;   g += (long long)a16((size_t)t->E * (msg_fp16 ? 2 : 4));
-  t->xg_st = g;    g += (long long)a16(4 * (size_t)t->n);
+  t->xg_msg = g;   g += (long long)a16((size_t)t->SP * (msg_fp16 ? 2 : 4));
+  t->xg_st = g;    g += (long long)a16(8 * (size_t)t->nstep);
   t->xg_dec = g;   g += (long long)a16(4 * (size_t)t->nw);
   t->xg_lpost = g; g += (long long)a16(4 * (size_t)t->n);
   t->xg_acc = g;   g += (long long)a16(4 * (size_t)t->n);

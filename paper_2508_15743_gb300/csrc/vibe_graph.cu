@@ -5,7 +5,8 @@
 // edge's column, +inf padding), and for every ensemble member the dependency wavefronts of its
 // serial schedule: level(v) = 1 + max{level(u) : u before v in the member's order, u and v share a
 // check}. Columns of one level touch disjoint checks, so updating a level in any order gives the
-// same floats as the serial order of Algorithm 1 (serial branch).
+// same floats as the serial order of Algorithm 1 (serial branch). For the summary engine each member's
+// order is also packed into steps of 32 edges (k_steps).
 #include "vibe_internal.cuh"
 
 namespace vibe {
@@ -54,12 +55,11 @@ __global__ void k_csc_fill(const int32_t* __restrict__ rowptr, const int32_t* __
   }
 }
 
-// Sort each column's entries by check (insertion sort, degree <= 32) and emit rowidx, csc_ent and the
-// summary engine's column records xcol (XP words per column: (check << 8) | position of the edge in
-// the check's CSR row, ascending check, zero padded; none when XP == 0).
-__global__ void k_csc_finish(int n, int DP, int RP, int spc, int XP, const int32_t* __restrict__ colptr,
+// Sort each column's entries by check (insertion sort, degree <= 32) in place and emit rowidx and
+// csc_ent.
+__global__ void k_csc_finish(int n, int DP, int RP, int spc, const int32_t* __restrict__ colptr,
                              uint32_t* __restrict__ packed, int32_t* __restrict__ rowidx,
-                             uint32_t* __restrict__ csc_ent, uint32_t* __restrict__ xcol) {
+                             uint32_t* __restrict__ csc_ent) {
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
     int b = colptr[v], d = colptr[v + 1] - b;
     for (int i = 1; i < d; ++i) {
@@ -73,7 +73,6 @@ __global__ void k_csc_finish(int n, int DP, int RP, int spc, int XP, const int32
       csc_ent[(size_t)v * DP + k] = k < d ? csc_entry(x >> 8, x & 0xffu, RP, spc) : 0u;
       if (k < d) rowidx[b + k] = (int32_t)(x >> 8);
     }
-    for (int k = 0; k < XP; ++k) xcol[(size_t)v * XP + k] = k < d ? packed[b + k] : 0u;
   }
 }
 
@@ -108,8 +107,8 @@ __device__ __forceinline__ float msg_magnitude<__half>(__half x) { return fabsf(
 
 // Summary engine: the summary of each check's prior messages -- the two smallest magnitudes (ordered by
 // value, then row position) with their positions, the third smallest as the floor (+inf when the row
-// is shorter; a missing second holder is position 255 with +inf), two valid holders, and the parity
-// of the messages' sign bits (bit 18). The syndrome and parity bits are set per shot by the kernel.
+// is shorter; a missing second holder is position 255 with +inf), and the parity of the messages' sign
+// bits (bit 31). The syndrome enters per shot in the kernel.
 template <typename MT>
 __global__ void k_xsum(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx, int m,
                        const float* __restrict__ lam, float4* __restrict__ out) {
@@ -126,7 +125,7 @@ __global__ void k_xsum(const int32_t* __restrict__ rowptr, const int32_t* __rest
       else if (a < a2 || (a == a2 && p < q2)) { a3 = a2; a2 = a; q2 = p; }
       else if (a < a3) a3 = a;
     }
-    out[c] = make_float4(a1, a2, a3, __uint_as_float(q1 | (q2 << 8) | (2u << 16) | (sg << 18)));
+    out[c] = make_float4(a1, a2, a3, __uint_as_float(q1 | (q2 << 8) | (sg << 31)));
   }
 }
 
@@ -177,47 +176,134 @@ __global__ void k_levels(const uint32_t* __restrict__ perm, int n, int m, int K,
   nlev[i] = nl;
 }
 
-// Summary engine: each member's schedule entries with the offset of the column's first message in the
-// member's schedule-ordered message array (exclusive prefix sum of the degrees). One CTA per member.
-__global__ void k_xrec(const uint32_t* __restrict__ sched, int n, uint2* __restrict__ rec) {
-  __shared__ uint32_t part[1024];
-  __shared__ uint32_t carry;
-  const uint32_t* sc = sched + (size_t)blockIdx.x * n;
-  uint2* out = rec + (size_t)blockIdx.x * n;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += 1024) {
-    const int j = base + threadIdx.x;
-    const uint32_t ent = j < n ? sc[j] : 0u;
-    const uint32_t d = ent >> 24;
-    part[threadIdx.x] = d;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-      const uint32_t add = threadIdx.x >= off ? part[threadIdx.x - off] : 0u;
-      __syncthreads();
-      part[threadIdx.x] += add;
-      __syncthreads();
+// The steps of every member's sweep (one warp per member): its columns, taken in the member's order,
+// are packed into steps of at most 32 edges, each column into the first step that (1) comes after the
+// steps of all earlier columns it shares a check with and (2) still has a lane for each of its checks
+// (one lane for a column without checks). Columns of one step therefore share no check, and two
+// columns that do keep their order, so a sweep that takes the steps one after another, one lane per
+// edge, computes the floats of the serial order.
+// Why steps and not the wavefront levels: a level is cut where the next column conflicts, whatever
+// its size, and rounding each level up to whole warps leaves lanes idle. On random orders of the d=9
+// phenomenological problem the levels make 79 warps of edges and the steps 62 (E / 32 = 60.8); on
+// circuit-level d=11 4887 and 4407 (4371).
+// slot[v] = step << 5 | first lane, nstep = number of steps, off[s] = edges before step s (s <= nstep).
+// The search looks at 64 windows of 32 steps; past them it opens a new step at the end, which bounds the
+// work per column. lo (lane d - 1: degree d) skips the steps known to have no room for that degree.
+constexpr int kStepWindows = 64;
+
+__global__ void k_steps(const uint32_t* __restrict__ perm, int n, int m, const int32_t* __restrict__ colptr,
+                        const uint32_t* __restrict__ cpos, int room_in_smem, uint32_t* __restrict__ slot,
+                        uint32_t* __restrict__ off, int32_t* __restrict__ nstep, uint8_t* __restrict__ room_g) {
+  extern __shared__ uint32_t sh[];
+  uint32_t* nxt = sh;                       // m: first step allowed at each check
+  uint32_t* stage = sh + m;                 // 32 x kMaxColDeg: checks of the 32 columns in work
+  uint8_t* room = room_in_smem ? reinterpret_cast<uint8_t*>(stage + 32 * kMaxColDeg)
+                               : room_g + (size_t)blockIdx.x * n;   // free lanes of each step
+  const int lane = threadIdx.x;
+  perm += (size_t)blockIdx.x * n;
+  slot += (size_t)blockIdx.x * n;
+  off += (size_t)blockIdx.x * (n + 1);
+  for (int c = lane; c < m; c += 32) nxt[c] = 0u;
+  uint32_t lo = 0u;
+  uint32_t ns = 0u;
+  for (int t0 = 0; t0 < n; t0 += 32) {
+    const int cnt = min(32, n - t0);
+    uint32_t v = 0u;
+    int d = 0;
+    __syncwarp();
+    if (lane < cnt) {
+      v = perm[t0 + lane];
+      const int b = colptr[v];
+      d = colptr[v + 1] - b;
+      for (int k = 0; k < d; ++k) stage[lane * kMaxColDeg + k] = cpos[b + k] >> 8;
     }
-    if (j < n) out[j] = make_uint2(ent, carry + part[threadIdx.x] - d);
-    __syncthreads();
-    if (threadIdx.x == 1023) carry += part[1023];
-    __syncthreads();
+    __syncwarp();
+    uint32_t mine = 0u;
+    for (int j = 0; j < cnt; ++j) {
+      const int dj = __shfl_sync(kFull, d, j);
+      const uint32_t need = (uint32_t)max(dj, 1);
+      const uint32_t c = lane < dj ? stage[j * kMaxColDeg + lane] : 0u;
+      const uint32_t s0 = __reduce_max_sync(kFull, lane < dj ? nxt[c] : 0u);
+      const uint32_t lod = __shfl_sync(kFull, lo, (int)need - 1);
+      uint32_t s = max(s0, lod);
+      bool found = false;
+      for (int w = 0; w < kStepWindows && !found; ++w) {
+        const uint32_t x = s + lane;
+        const uint32_t bal = __ballot_sync(kFull, x >= ns || room[x] >= need);
+        if (bal) {
+          s += (uint32_t)__ffs(bal) - 1u;
+          found = true;
+        } else {
+          s += 32u;
+        }
+      }
+      if (!found) s = ns;
+      else if (s0 <= lod && lane == (int)need - 1) lo = s;
+      const uint32_t r = s < ns ? room[s] : 32u;
+      if (lane == j) mine = (s << 5) | (32u - r);
+      __syncwarp();
+      if (lane == 0) room[s] = (uint8_t)(r - need);
+      ns = max(ns, s + 1u);
+      if (lane < dj) nxt[c] = s + 1u;
+      __syncwarp();
+    }
+    if (lane < cnt) slot[v] = mine;
+  }
+  uint32_t run = 0u;
+  for (uint32_t s0 = 0; s0 <= ns; s0 += 32) {
+    const uint32_t x = s0 + lane;
+    const uint32_t u = x < ns ? 32u - room[x] : 0u;
+    uint32_t inc = u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += y;
+    }
+    if (x <= ns) off[x] = run + inc - u;
+    run += __shfl_sync(kFull, inc, 31);
+  }
+  if (lane == 0) nstep[blockIdx.x] = (int32_t)ns;
+}
+
+// The step offsets with the common pitch of the resident table; the entries past a member's last step
+// repeat its total.
+__global__ void k_step_offsets(const uint32_t* __restrict__ tmp, int tmp_pitch, const int32_t* __restrict__ nstep, int K,
+                               int pitch, uint32_t* __restrict__ soff) {
+  const long long total = (long long)K * pitch;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
+       q += (long long)gridDim.x * blockDim.x) {
+    const int i = (int)(q / pitch), s = (int)(q % pitch);
+    soff[q] = tmp[(size_t)i * tmp_pitch + min(s, nstep[i])];
   }
 }
 
-// Summary engine: for every member and every CSR entry q = (check c, column v) of H, the slot of the
-// message v -> c in the member's schedule-ordered message array.
-__global__ void k_xrmap(const uint2* __restrict__ rec, long long total, int n, int E, int XP,
-                        const uint32_t* __restrict__ xcol, const int32_t* __restrict__ rowptr,
-                        uint32_t* __restrict__ rmap) {
+// The edge records of every member's steps, one thread per (member, column); see Tables::xrec. xcolid
+// names each slot's column, xrmap the message slot of each CSR entry of H.
+__global__ void k_step_fill(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ off, int off_pitch, int n,
+                            long long total, int E, int SP, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colptr,
+                            const uint32_t* __restrict__ cpos, const float* __restrict__ lam, uint2* __restrict__ xrec,
+                            uint32_t* __restrict__ xlnk, uint32_t* __restrict__ xcolid, uint32_t* __restrict__ xrmap) {
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
        q += (long long)gridDim.x * blockDim.x) {
     const long long i = q / n;
-    const uint2 r = rec[q];
-    const uint32_t v = r.x & 0xffffffu, d = r.x >> 24;
-    for (uint32_t k = 0; k < d; ++k) {
-      const uint32_t x = xcol[(size_t)v * XP + k];
-      rmap[(size_t)i * E + rowptr[x >> 8] + (x & 0xffu)] = r.y + k;
+    const uint32_t v = (uint32_t)(q % n);
+    const uint32_t sl = slot[q];
+    const uint32_t o = off[i * off_pitch + (sl >> 5)] + (sl & 31u);
+    const int b = colptr[v], d = colptr[v + 1] - b;
+    const uint32_t lv = __float_as_uint(lam[v]);
+    if (d == 0) {
+      xrec[i * SP + o] = make_uint2(0u, lv);
+      xlnk[i * SP + o] = 0u;
+      xcolid[i * SP + o] = v;
+    }
+    for (int k = 0; k < d; ++k) {
+      const uint32_t x = cpos[b + k];
+      const uint32_t others = ((2u << (d - 1)) - 1u) & ~(1u << k);   // the summary engine has d <= 16
+      xrec[i * SP + o + k] = make_uint2(((x >> 8) << 18) | (x & 0xffu), lv);
+      xlnk[i * SP + o + k] = (sl & 31u) | (others << 5) | (((sl & 31u) + (uint32_t)(d - 1)) << kLnkLastLane) |
+                             (k == d - 1 ? kLnkLast : 0u) | kLnkEdge;
+      xcolid[i * SP + o + k] = v;
+      xrmap[(size_t)i * E + rowptr[x >> 8] + (x & 0xffu)] = o + (uint32_t)k;
     }
   }
 }
@@ -324,25 +410,20 @@ __global__ void k_layers(const int32_t* __restrict__ rowptr, const int32_t* __re
   }
 }
 
-cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m, int n, int K, const uint32_t* d_perm,
-                         int RP, int DP, int XP, int msg_fp16, const float* d_lam, int32_t* d_colptr, int32_t* d_rowidx,
-                         uint32_t* d_csc_ent, void* d_msg_init, uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev,
-                         uint32_t* d_xcol, uint2* d_xrec, uint32_t* d_xrmap, float4* d_xsum, int32_t* d_scratch,
+cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m, int n, int E, int K,
+                         const uint32_t* d_perm, int RP, int DP, int msg_fp16, const float* d_lam, int32_t* d_colptr,
+                         int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init,
+                         uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, float4* d_xsum, int32_t* d_scratch,
                          cudaStream_t s) {
-  // scratch layout: cnt[n] | fill[n] | packed[E] ; later reused by k_levels (K*(m+3n+1))
-  int E = 0;
-  cudaError_t err = cudaMemcpyAsync(&E, d_rowptr + m, sizeof(int), cudaMemcpyDeviceToHost, s);
-  if (err != cudaSuccess) return err;
-  if ((err = cudaStreamSynchronize(s)) != cudaSuccess) return err;
+  // scratch layout: cnt[n] | fill[n]; later reused by k_levels (K*(m+3n+1))
+  cudaError_t err;
   int32_t* cnt = d_scratch;
   int32_t* fill = cnt + n;
-  uint32_t* packed = reinterpret_cast<uint32_t*>(fill + n);
   if ((err = cudaMemsetAsync(cnt, 0, sizeof(int32_t) * 2 * (size_t)n, s)) != cudaSuccess) return err;
   k_col_count<<<grid_for(E, 256), 256, 0, s>>>(d_colidx, E, cnt);
   k_scan_single<<<1, 1024, 0, s>>>(cnt, n, d_colptr);
-  k_csc_fill<<<grid_for(m, 128), 128, 0, s>>>(d_rowptr, d_colidx, m, d_colptr, fill, packed);
-  k_csc_finish<<<grid_for(n, 128), 128, 0, s>>>(n, DP, RP, msg_fp16 ? 8 : 4, XP, d_colptr, packed, d_rowidx,
-                                                 d_csc_ent, d_xcol);
+  k_csc_fill<<<grid_for(m, 128), 128, 0, s>>>(d_rowptr, d_colidx, m, d_colptr, fill, d_cpos);
+  k_csc_finish<<<grid_for(n, 128), 128, 0, s>>>(n, DP, RP, msg_fp16 ? 8 : 4, d_colptr, d_cpos, d_rowidx, d_csc_ent);
   if (msg_fp16) {
     k_xsum<__half><<<grid_for(m, 128), 128, 0, s>>>(d_rowptr, d_colidx, m, d_lam, d_xsum);
     k_msg_init<__half><<<grid_for((long long)m * RP, 256), 256, 0, s>>>(d_rowptr, d_colidx, m, RP, d_lam,
@@ -353,11 +434,36 @@ cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m
                                                                       static_cast<float*>(d_msg_init));
   }
   k_levels<<<(K + 31) / 32, 32, 0, s>>>(d_perm, n, m, K, d_colptr, d_rowidx, d_sched, d_lvl_off, d_nlev, d_scratch);
-  if (XP > 0) {
-    k_xrec<<<K, 1024, 0, s>>>(d_sched, n, d_xrec);
-    k_xrmap<<<grid_for((long long)K * n, 256), 256, 0, s>>>(d_xrec, (long long)K * n, n, E, XP, d_xcol, d_rowptr,
-                                                            d_xrmap);
-  }
+  return cudaGetLastError();
+}
+
+cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
+                        int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s) {
+  uint32_t* slot = reinterpret_cast<uint32_t*>(d_scratch);
+  uint32_t* off = slot + (size_t)K * n;
+  uint8_t* room = reinterpret_cast<uint8_t*>(off + (size_t)K * (n + 1));
+  // m <= 16384 checks take 64 KB at most; the free-lane bytes follow when they fit too
+  const size_t fixed = 4 * ((size_t)m + 32 * kMaxColDeg), bytes = (size_t)n;
+  const bool room_in_smem = fixed + bytes <= 160u * 1024u;
+  const size_t smem = fixed + (room_in_smem ? bytes : 0);
+  cudaError_t err = ensure_dyn_smem<k_steps>(smem);
+  if (err != cudaSuccess) return err;
+  k_steps<<<K, 32, smem, s>>>(d_perm, n, m, d_colptr, d_cpos, room_in_smem ? 1 : 0, slot, off, d_nstep, room);
+  return cudaGetLastError();
+}
+
+size_t step_scratch_ints(int n, int K) { return (size_t)K * (2 * (size_t)n + 1) + ((size_t)K * n + 3) / 4; }
+
+cudaError_t fill_steps(int n, int E, int SP, int K, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
+                       const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
+                       uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,
+                       cudaStream_t s) {
+  const uint32_t* slot = reinterpret_cast<const uint32_t*>(d_scratch);
+  const uint32_t* off = slot + (size_t)K * n;
+  const int off_pitch = n + 1;
+  k_step_offsets<<<grid_for((long long)K * pitch, 256), 256, 0, s>>>(off, off_pitch, d_nstep, K, pitch, d_soff);
+  k_step_fill<<<grid_for((long long)K * n, 256), 256, 0, s>>>(slot, off, off_pitch, n, (long long)K * n, E, SP, d_rowptr,
+                                                              d_colptr, d_cpos, d_lam, d_xrec, d_xlnk, d_xcolid, d_xrmap);
   return cudaGetLastError();
 }
 

@@ -19,6 +19,11 @@ constexpr int kMaxColDeg = 32;
 constexpr int kMaxDems = 64;        // decoding problems in one mixed launch
 constexpr int kMaxDevices = 64;
 constexpr uint32_t kFull = 0xffffffffu;
+// Edge links (Tables::xlnk): bits 0-4 the lane of the column's first edge, bit 5 + j set for the column's
+// j-th edge except the record's own, then the lane of its last edge; 0 for a column without checks.
+constexpr int kLnkLastLane = 21;
+constexpr uint32_t kLnkLast = 1u << 30, kLnkEdge = 1u << 31;   // the record is the last edge's; it has a check
+constexpr int kStepPad = 66;            // step offsets kept past a member's last step (the kernels look ahead)
 
 // Position of slot `slot` of check row c inside the message image. A row is RP slots stored as
 // 16-byte chunks of `spc` slots (4 for float, 8 for half). When the row has 2, 4 or 8 chunks their
@@ -54,9 +59,11 @@ struct Tables {
                  // members with FP16 storage), laid out like the message image; -1 when unused
   int engine;    // VIBE_ENGINE_IMAGE or VIBE_ENGINE_SUMMARY
   // summary engine: column-degree bound XD (4, 6, 8 or 16; 0 when a column has more than 16 checks and
-  // the engine cannot run the problem), xcol pitch XP, shared memory of one warp (the m check
-  // summaries, bytes) and the parts of one warp's global scratch (bytes, 16-aligned)
-  int XD, XP, x_warp_smem;   // x_warp_smem: the m check summaries only
+  // the engine cannot run the problem), shared memory of one warp (the m check summaries, bytes) and the
+  // parts of one warp's global scratch (bytes, 16-aligned)
+  int XD, x_warp_smem;   // x_warp_smem: the m check summaries only
+  int SP;                // edge slots of one member's sweep: E, and one per column without checks
+  int nstep, soff_pitch; // largest step count of a member; entries per member of soff
   // xg_cpost = x_warp_scratch: the M*n candidate posteriors (soft output only) follow the fixed part
   long long xg_msg, xg_st, xg_dec, xg_lpost, xg_acc, xg_cand, xg_cpost, x_warp_scratch;
   const int32_t* rowptr;   // H CSR
@@ -77,11 +84,16 @@ struct Tables {
   const int32_t* layer_chk;   // m checks grouped by layer, ascending within a layer
   const int32_t* layer_vptr;  // nlayer+1 offsets into layer_var
   const int32_t* layer_var;   // E: per layer, the columns of its checks in layer_chk order (each at most once)
-  // summary engine
-  const uint32_t* xcol;    // n*XP: (check << 8) | position of the edge in the check's CSR row, ascending check
-  const uint2* xrec;       // K*n: (sched entry, offset of the column's first message in the member's
-                           // schedule-ordered message array), same order as sched
-  const uint32_t* xrmap;   // K*E: per member, the message slot of each CSR entry of H
+  // summary engine: the steps of each member's sweep (k_steps). Step s of member i holds the edge slots
+  // soff[i][s] .. soff[i][s+1] (at most 32, one lane each; the checks of a step are distinct), the edges
+  // of a column in consecutive slots.
+  // xrec[i][slot] = (check << 18 | position of the edge in the check's CSR row, prior LLR), xlnk its links
+  const int32_t* stepcnt;  // K step counts
+  const uint32_t* soff;    // K * soff_pitch
+  const uint2* xrec;       // K * SP
+  const uint32_t* xlnk;    // K * SP
+  const uint32_t* xcolid;  // K * SP: column of each slot
+  const uint32_t* xrmap;   // K*E: per member, the slot of each CSR entry of H
   const float4* xsum;      // m: summaries of the prior messages (see vibe_bpx.cu)
 };
 
@@ -91,8 +103,8 @@ struct Bounds {
   int RP;          // common row pitch if all problems share it, else 0
   int warp_smem;   // largest BP per-warp layout
   int lsd_order;   // largest LSD order
-  int x_warp_smem;    // summary-engine shared memory per warp: the prefetch ring for XD and the largest
-                      // problem's check summaries (0 if no problem uses that engine)
+  int x_warp_smem;    // summary-engine shared memory per warp: the step window and the largest problem's
+                      // check summaries (0 if no problem uses that engine)
   long long x_warp_scratch;   // largest summary-engine global scratch per warp, bytes
   int engines;     // bit 0: some problem uses the image engine, bit 1: the summary engine
   int XD;          // largest summary-engine column-degree bound
@@ -343,12 +355,22 @@ cudaError_t ensure_dyn_smem(size_t smem) {
 }
 int set_error(int code, const char* msg);
 
-// K0: graph builder (vibe_graph.cu)
-cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m, int n, int K, const uint32_t* d_perm,
-                         int RP, int DP, int XP, int msg_fp16, const float* d_lam, int32_t* d_colptr, int32_t* d_rowidx,
-                         uint32_t* d_csc_ent, void* d_msg_init, uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev,
-                         uint32_t* d_xcol, uint2* d_xrec, uint32_t* d_xrmap, float4* d_xsum, int32_t* d_scratch,
+// K0: graph builder (vibe_graph.cu). d_cpos: the CSC entries of H as (check << 8) | position in the
+// check's CSR row.
+cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m, int n, int E, int K,
+                         const uint32_t* d_perm, int RP, int DP, int msg_fp16, const float* d_lam, int32_t* d_colptr,
+                         int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init,
+                         uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, float4* d_xsum, int32_t* d_scratch,
                          cudaStream_t s);
+// Packs each member's order into steps (K step counts in d_nstep); fill_steps then writes the resident
+// tables from the same scratch (step_scratch_ints).
+size_t step_scratch_ints(int n, int K);
+cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
+                        int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s);
+cudaError_t fill_steps(int n, int E, int SP, int K, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
+                       const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
+                       uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,
+                       cudaStream_t s);
 cudaError_t seeded_schedules(uint32_t* d_perm, int n, int K, uint64_t seed, cudaStream_t s);
 // Check layers of the layered schedule (greedy colouring in ascending check order) from the CSR and
 // CSC of H: layer_ptr (m+1 entries), layer_chk (m), layer_vptr (m+1), layer_var (E), the layer count in
@@ -367,8 +389,9 @@ cudaError_t bp_occupancy(const Bounds& b, int ndem, int msg_fp16, int* blocks_pe
 
 // K1': summary-engine BP + ensemble selection (vibe_bpx.cu)
 int bpx_degree_bucket(int maxcol);          // XD for a largest column degree (0: above 16)
-int bpx_ring_bytes(int XD);                  // per-warp shared-memory prefetch ring of a launch with bound XD
-void bpx_layout(Tables* t, int msg_fp16);   // fills t's x_warp_smem and xg_* fields
+int bpx_window_bytes();                      // per-warp shared memory of the step window
+int bpx_summary_bytes(int m, int msg_fp16);  // shared memory of one warp's check summaries
+void bpx_layout(Tables* t, int msg_fp16);    // fills t's xg_* fields
 size_t bpx_cta_smem_bytes(const Bounds& b, int ndem);
 cudaError_t launch_bpx(const BpArgs& a, int msg_fp16, int grid, cudaStream_t s);
 cudaError_t bpx_occupancy(const Bounds& b, int ndem, int msg_fp16, int* blocks_per_sm);

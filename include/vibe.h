@@ -68,8 +68,9 @@ typedef struct {
                         check-to-variable messages by member_alpha[i] instead of alpha, an ensemble
                         mixing heuristics (Sec. V); results, ranking and LLR average are otherwise
                         unchanged. Both engines, all schedules and storage precisions */
-  int32_t pair_mode; /* 0: one warp per shot runs the shot's members one after another (throughput);
-                        1: one warp per (shot, member) pair, so a shot's members run at the same time
+  int32_t pair_mode; /* 0: one warp per shot runs the shot's members one after another (throughput), except
+                        that a batch of at most eight shots per resident warp, whose members' records
+                        fit in 2 GiB, runs as in pair mode, which ends sooner; 1: one warp per (shot, member) pair, so a shot's members run at the same time
                         and its BP latency is that of its slowest member, not the sum (latency). The
                         outputs are identical; pair mode does more sweeps in total (members run until
                         they see M earlier candidates) and keeps every member's record per shot */
@@ -153,7 +154,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
  *   the normalised LLR average that ranked the columns;
  *   d_observables: B x ceil(k/32) true logical flips (may be NULL) -- with d_counters, counts
  *   shots whose L e differs; d_counters: VIBE_NUM_COUNTERS uint64 accumulators (may be NULL).
- *   The handle's workspace is allocated on the first call and grown when a larger batch needs it;
+ *   The handle's workspace is allocated on the first call and grown when a larger batch needs it (in shot
+ *   mode with up to 2 GiB of members' records; without that memory small batches run one warp per shot);
  *   calls with a batch no larger than an earlier one allocate nothing. Large batches run in chunks.
  *   Calls on one handle must not overlap in time (the workspace is shared); use one handle per stream.
  *   Errors: VIBE_ERR_INVALID (NULL handle/required pointer, B < 0), VIBE_ERR_NOMEM, VIBE_ERR_CUDA.
@@ -229,7 +231,7 @@ int vibe_profile_read(vibe_handle* h, double* bp_ms, double* lsd_ms, int64_t* bp
  *   Errors: VIBE_ERR_INVALID (NULL handle/pointers, B < 0, handle's device not current),
  *   VIBE_ERR_UNSUPPORTED (batch too large, or a handle on the summary engine, whose per-warp message
  *   arrays leave no useful grid in 64 MiB), VIBE_ERR_CUDA. B = 0 performs only the set-up above.
- *   Always runs one warp per shot, whatever the handle's pair_mode (same results).
+ *   Always runs one warp per shot, whatever the batch and the handle's pair_mode (same results).
  */
 int vibe_decode_noalloc(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, uint32_t* d_corrections,
                         uint32_t* d_logical, vibe_shot_stats* d_stats, void* stream);
@@ -257,7 +259,7 @@ int vibe_autotune(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, void* 
 /* Launch configuration of a handle or a batch (vibe_get_launch). */
 typedef struct {
   int32_t engines;           /* bit 0: the image engine's kernel runs, bit 1: the summary engine's */
-  int32_t pair_mode;         /* 1: one warp per (shot, member) pair; 0: one warp per shot */
+  int32_t pair_mode;         /* as vibe_params.pair_mode */
   int32_t bp_blocks_per_sm;  /* image-engine CTAs per SM of its persistent grid (0 if it does not run) */
   int32_t bpx_blocks_per_sm; /* summary-engine CTAs per SM (0 if it does not run) */
   int32_t lsd_blocks_per_sm; /* LSD CTAs per SM */

@@ -98,6 +98,19 @@ struct Launch {
   // keeps every warp busy across shots (a launch ends with its slowest pair) and a small one runs whole
   long long pair_chunk(bool soft) const { return std::max(1LL, kPairBytes / pair_shot_bytes(soft)); }
   static constexpr long long kPairBytes = 8LL << 30;
+  // Shots up to which a batch in shot mode runs as pairs all the same (same results). A batch of a few
+  // shots per warp ends with the warps whose shots reach LSD: each runs K * T sweeps one after another
+  // while the rest of the GPU is idle. Pairs spread those sweeps. Measured, shot against pair mode:
+  // circuit-level d=5 (K=32, FP16) 202 / 73 ms at 1.1 shots per resident warp, 358 / 281 ms at 4.5; the
+  // 4.8.8 d=9 phenomenological code (K=16) 46.3 / 40.7 ms at 4.5 and 157 / 155 ms at 18; the 6.6.6 one 99.6
+  // / 102 ms at 13 and 381 / 404 ms at 54. So the line is drawn at eight shots per warp, and where the
+  // members' records pass 2 GiB.
+  long long auto_pair_shots() const {
+    if (bnd.K < 2) return 0;
+    const long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta + (long long)bpx_grid() * vibe::kBpxWarpsPerCta;
+    return std::min(8 * warps, kAutoPairBytes / pair_shot_bytes(false));
+  }
+  static constexpr long long kAutoPairBytes = 2LL << 30;
 };
 
 // Device memory a decode uses besides its inputs and outputs; grown on demand, reused afterwards.
@@ -124,22 +137,35 @@ struct Workspace {
   float* ppost = nullptr;
   unsigned int* pdone = nullptr;
 
+  bool no_records = false;   // there was no memory for the records of shot mode's small batches
+
+  void release_records() {
+    cudaFree(pconv); cudaFree(pW); cudaFree(pbits); cudaFree(pterms); cudaFree(ppost); cudaFree(pdone);
+    pconv = nullptr; pW = nullptr; pbits = nullptr; pterms = nullptr; ppost = nullptr; pdone = nullptr;
+    pair_shots = 0; pair_soft = false; no_records = false;
+  }
+  // whether a batch of B shots runs as pairs
+  bool as_pairs(const Launch& L, long long B, bool soft) const {
+    return L.pair_mode || (B <= std::min(pair_shots, L.auto_pair_shots()) && (!soft || pair_soft));
+  }
   void release() {
+    release_records();
     cudaFree(ctrl); cudaFree(lsd_shots); cudaFree(lsd_soft); cudaFree(bp_scratch); cudaFree(bpx_scratch);
     cudaFree(lsd_scratch);
-    cudaFree(pconv); cudaFree(pW); cudaFree(pbits); cudaFree(pterms); cudaFree(ppost); cudaFree(pdone);
     ctrl = nullptr; lsd_shots = nullptr; lsd_soft = nullptr; bp_scratch = nullptr; bpx_scratch = nullptr;
     lsd_scratch = nullptr;
-    pconv = nullptr; pW = nullptr; pbits = nullptr; pterms = nullptr; ppost = nullptr; pdone = nullptr;
-    chunk = 0; bp_warps = 0; lsd_ctas = 0; bpx_bytes = 0; pair_shots = 0; pair_soft = false; lsd_words = 0;
+    chunk = 0; bp_warps = 0; lsd_ctas = 0; bpx_bytes = 0; lsd_words = 0;
   }
   int ensure(const Launch& L, long long need, bool soft) {
-    const long long ps = L.pair_mode ? std::min(need, L.pair_chunk(soft)) : 0;
+    // records of as many shots as a batch of this size or a smaller one runs as pairs. In shot mode a first
+    // soft output grows nothing: without the posteriors' records it runs one warp per shot
+    const long long ps = std::min(need, L.pair_mode ? L.pair_chunk(soft) : L.auto_pair_shots());
     const long long want = std::min(need, chunk_max);
     const int warps = L.bp_grid() * vibe::kBpWarpsPerCta;
     const long long xb = (long long)L.bpx_grid() * vibe::kBpxWarpsPerCta * L.bpx_pitch(soft);
-    const bool pair_ok = !L.pair_mode || (ps <= pair_shots && (!soft || pair_soft) && L.bnd.K * L.bnd.nw <= pk_nw &&
-                                          L.bnd.K * L.bnd.n <= pk_n);
+    const bool pair_ok = ps == 0 || (!L.pair_mode && no_records) ||
+                         (ps <= pair_shots && (!L.pair_mode || !soft || pair_soft) && L.bnd.K * L.bnd.nw <= pk_nw &&
+                          L.bnd.K * L.bnd.n <= pk_n);
     const bool lsd_ok = (long long)L.lsd_grid() * vibe::lsd_scratch_words(L.bnd, L.lsd_threads) <=
                         (long long)lsd_ctas * lsd_words;
     if (ctrl && want <= chunk && warps <= bp_warps && lsd_ok && xb <= bpx_bytes && pair_ok)
@@ -156,18 +182,26 @@ struct Workspace {
     VIBE_CUDA(dalloc(&lsd_scratch, (size_t)L.lsd_grid() * (size_t)vibe::lsd_scratch_words(b, L.lsd_threads)),
               "workspace");
     lsd_words = vibe::lsd_scratch_words(b, L.lsd_threads);
-    if (L.pair_mode) {
+    if (ps > 0) {
       const size_t S = (size_t)ps;
-      VIBE_CUDA(dalloc(&pconv, S * b.K), "workspace");
-      VIBE_CUDA(dalloc(&pW, S * b.K), "workspace");
-      VIBE_CUDA(dalloc(&pbits, S * b.K * (size_t)b.nw), "workspace");
-      VIBE_CUDA(dalloc(&pterms, S * b.K * (size_t)b.n), "workspace");
-      if (soft) VIBE_CUDA(dalloc(&ppost, S * b.K * (size_t)b.n), "workspace");
-      VIBE_CUDA(dalloc(&pdone, S), "workspace");
-      pair_shots = ps;
-      pair_soft = soft;
-      pk_nw = (long long)b.K * b.nw;
-      pk_n = (long long)b.K * b.n;
+      cudaError_t e = dalloc(&pconv, S * b.K);
+      if (e == cudaSuccess) e = dalloc(&pW, S * b.K);
+      if (e == cudaSuccess) e = dalloc(&pbits, S * b.K * (size_t)b.nw);
+      if (e == cudaSuccess) e = dalloc(&pterms, S * b.K * (size_t)b.n);
+      if (e == cudaSuccess && soft) e = dalloc(&ppost, S * b.K * (size_t)b.n);
+      if (e == cudaSuccess) e = dalloc(&pdone, S);
+      if (e == cudaSuccess) {
+        pair_shots = ps;
+        pair_soft = soft;
+        pk_nw = (long long)b.K * b.nw;
+        pk_n = (long long)b.K * b.n;
+      } else if (L.pair_mode) {
+        return cuda_fail(e, "workspace");
+      } else {   // shot mode does without them
+        cudaGetLastError();
+        release_records();
+        no_records = true;
+      }
     }
     chunk = c;
     bp_warps = warps;
@@ -221,13 +255,14 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
   int rc = ws.ensure(L, q.B, q.soft != nullptr);
   if (rc != VIBE_OK) return rc;
   const long long step = ws.chunk;
+  const bool pairs = ws.as_pairs(L, q.B, q.soft != nullptr);
   for (long long b0 = 0; b0 < q.B; b0 += step) {
     const long long nb = std::min(step, q.B - b0);
     VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, 8 * sizeof(unsigned int), s), "decode");
     cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
     if (prof.on) { e0 = prof.next(); e1 = prof.next(); e2 = prof.next(); }
     if (e0) cudaEventRecord(e0, s);
-    const long long sub = L.pair_mode ? std::min(nb, ws.pair_shots) : nb;
+    const long long sub = pairs ? std::min(nb, ws.pair_shots) : nb;
     for (long long s0 = 0; s0 < nb; s0 += sub) {
       const long long ns = std::min(sub, nb - s0);
       const long long o = b0 + s0;
@@ -235,7 +270,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
         VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, sizeof(unsigned int), s), "decode");
         VIBE_CUDA(cudaMemsetAsync(ws.ctrl + 3, 0, 3 * sizeof(unsigned int), s), "decode");
       }
-      if (L.pair_mode) {
+      if (pairs) {
         VIBE_CUDA(cudaMemsetAsync(ws.pconv, 0, sizeof(int) * (size_t)ns * L.bnd.K, s), "decode");
         VIBE_CUDA(cudaMemsetAsync(ws.pdone, 0, sizeof(unsigned int) * (size_t)ns, s), "decode");
       }
@@ -259,13 +294,13 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       a.xscratch = ws.bpx_scratch;
       a.xscratch_pitch = L.bpx_pitch(a.want_soft != 0);
       a.next_shot_x = ws.ctrl + 3;
-      a.pair_mode = L.pair_mode;
+      a.pair_mode = pairs;
       a.pair_K = L.bnd.K;
       a.pconv = ws.pconv; a.pW = ws.pW; a.pbits = ws.pbits; a.pterms = ws.pterms; a.ppost = ws.ppost;
       a.pdone = ws.pdone;
       a.next_pair = ws.ctrl + 4;
       a.next_pair_x = ws.ctrl + 5;
-      const long long units = L.pair_mode ? ns * L.bnd.K : ns;   // shots, or (shot, member) pairs
+      const long long units = pairs ? ns * L.bnd.K : ns;   // shots, or (shot, member) pairs
       if (L.warp_engine()) {
         const int grid =
             (int)std::min<long long>(L.bp_grid(), (units + vibe::kBpWarpsPerCta - 1) / vibe::kBpWarpsPerCta);

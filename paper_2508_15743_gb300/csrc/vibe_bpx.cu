@@ -81,34 +81,6 @@ struct XMsg<__half> {
   }
 };
 
-// Shared memory by 32-bit address: the sweep keeps a handful of addresses in registers instead of
-// forming each one from the window base.
-__device__ __forceinline__ uint32_t lds32(uint32_t a) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint2 lds64(uint32_t a) {
-  uint2 v;
-  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ uint4 lds128(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
-  return v;
-}
-__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
-  asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-__device__ __forceinline__ void sts64(uint32_t a, uint2 v) {
-  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
-}
-__device__ __forceinline__ void sts128(uint32_t a, uint4 v) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
-constexpr uint32_t kInfBits = 0x7f800000u;
 
 constexpr uint32_t kSgnBit = 1u << 31, kParBit = 1u << 30;   // flags of a summary
 
@@ -292,11 +264,6 @@ __device__ __forceinline__ void fetch_chunk(uint32_t win, int buf, int s, const 
     cp_async_cg16(dl + 16 * q, lnk + b + 4 * q);
   }
   cp_async_commit();
-}
-
-__device__ __forceinline__ float add_if(float acc, float x, uint32_t cond) {
-  asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p add.rn.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(x), "r"(cond));
-  return acc;
 }
 
 // One sweep of a member over its ns steps. win: shared address of the warp's window (the summaries follow it); stg: (signs, decisions) of every

@@ -19,6 +19,7 @@ constexpr int kMaxColDeg = 32;
 constexpr int kMaxDems = 64;        // decoding problems in one mixed launch
 constexpr int kMaxDevices = 64;
 constexpr uint32_t kFull = 0xffffffffu;
+constexpr uint32_t kInfBits = 0x7f800000u;
 // Edge links (Tables::xlnk): bits 0-4 the lane of the column's first edge, bit 5 + j set for the column's
 // j-th edge except the record's own, then the lane of its last edge; 0 for a column without checks.
 constexpr int kLnkLastLane = 21;
@@ -324,6 +325,39 @@ __device__ inline bool pair_epilogue(const BpArgs& a, const Tables& t, uint32_t 
     }
     return false;   // LSD decides, and counts, this shot
   }
+}
+
+// Shared memory by 32-bit address: the sweep keeps a handful of addresses in registers instead of
+// forming each one from the window base.
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint2 lds64(uint32_t a) {
+  uint2 v;
+  asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ uint4 lds128(uint32_t a) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
+  return v;
+}
+__device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t a, uint2 v) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t a, uint4 v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+
+// acc + x where cond is not 0
+__device__ __forceinline__ float add_if(float acc, float x, uint32_t cond) {
+  asm("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p add.rn.f32 %0, %0, %1;\n\t}" : "+f"(acc) : "f"(x), "r"(cond));
+  return acc;
 }
 
 // A handle's resident problem and launch configuration, as other host files see it (vibe_api.cu).

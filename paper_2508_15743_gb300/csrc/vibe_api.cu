@@ -177,7 +177,7 @@ struct Workspace {
     VIBE_CUDA(dalloc(&ctrl, 8), "workspace");
     VIBE_CUDA(dalloc(&lsd_shots, (size_t)c), "workspace");
     VIBE_CUDA(dalloc(&lsd_soft, (size_t)c * b.n), "workspace");
-    VIBE_CUDA(dalloc(&bp_scratch, (size_t)warps * (size_t)(2 + b.M) * b.n), "workspace");
+    VIBE_CUDA(dalloc(&bp_scratch, (size_t)warps * (size_t)(2 + b.global_st + b.M) * b.n), "workspace");
     VIBE_CUDA(dalloc(&bpx_scratch, (size_t)xkeep), "workspace");
     VIBE_CUDA(dalloc(&lsd_scratch, (size_t)L.lsd_grid() * (size_t)vibe::lsd_scratch_words(b, L.lsd_threads)),
               "workspace");
@@ -290,7 +290,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       a.next_shot = ws.ctrl; a.lsd_count = ws.ctrl + 1; a.lsd_shots = ws.lsd_shots; a.lsd_soft = ws.lsd_soft;
       a.lsd_shot_base = (uint32_t)s0;
       a.scratch = ws.bp_scratch;
-      a.scratch_pitch = (long long)(2 + L.bnd.M) * L.bnd.n;
+      a.scratch_pitch = (long long)(2 + L.bnd.global_st + L.bnd.M) * L.bnd.n;
       a.xscratch = ws.bpx_scratch;
       a.xscratch_pitch = L.bpx_pitch(a.want_soft != 0);
       a.next_shot_x = ws.ctrl + 3;
@@ -377,6 +377,7 @@ Bounds bounds_over(const Tables* ts, int count) {
       b.RP = first_warp ? t.RP : (b.RP == t.RP ? b.RP : 0);
       first_warp = false;
       b.warp_smem = std::max(b.warp_smem, t.warp_smem);
+      if (t.off_st < 0) b.global_st = 1;
     } else {
       b.engines |= 2;
       b.XD = std::max(b.XD, t.XD);
@@ -632,33 +633,18 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   h->L.pair_mode = p->pair_mode;
   Tables& t = h->t;
   t.m = m; t.n = n; t.k = k; t.E = E; t.K = K;
-  t.RP = std::max(8, (maxrow + 7) / 8 * 8);
+  const int spc = p->msg_fp16 ? 8 : 4;   // slots per 16-byte chunk of a row
+  t.RP = (maxrow + spc - 1) / spc * spc;
   t.DP = maxcol <= 4 ? 4 : maxcol <= 8 ? 8 : maxcol <= 16 ? 16 : 32;
   t.mw = (m + 31) / 32; t.nw = (n + 31) / 32; t.kw = (k + 31) / 32; t.W = t.mw;
   t.T = p->max_iter; t.M = p->M; t.lsd_order = p->lsd_order; t.alpha = p->alpha; t.n_flood = p->n_flood;
   t.n_layered = p->n_layered;
-  vibe::bp_warp_smem_bytes(&t, p->msg_fp16);
   t.XD = vibe::bpx_degree_bucket(maxcol);
   t.SP = E + (int)std::count(coldeg.begin(), coldeg.end(), 0);
   t.x_warp_smem = vibe::bpx_summary_bytes(m, p->msg_fp16);
   t.engine = p->bp_engine;
   if (t.engine == VIBE_ENGINE_SUMMARY && t.XD == 0)
     return bail(fail(VIBE_ERR_UNSUPPORTED, "the summary engine takes columns of at most 16 checks"));
-  if (t.engine == VIBE_ENGINE_AUTO) {
-    // the image engine when its per-warp image leaves at least 8 warps per SM, else the summary engine
-    int optin = 0, blocks = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    t.engine = VIBE_ENGINE_IMAGE;
-    const Bounds bw = bounds_over(&t, 1);
-    t.engine = VIBE_ENGINE_SUMMARY;
-    if (vibe::bp_cta_smem_bytes(bw, 0) <= (size_t)optin &&
-        vibe::bp_occupancy(bw, 0, p->msg_fp16, &blocks) == cudaSuccess &&
-        (blocks * vibe::kBpWarpsPerCta >= 8 || (other_schedules && blocks >= 1) || (t.XD == 0 && blocks >= 1)))
-      t.engine = VIBE_ENGINE_IMAGE;
-    if (other_schedules && t.engine != VIBE_ENGINE_IMAGE)
-      return bail(fail(VIBE_ERR_UNSUPPORTED,
-                       "flooding and layered members need the image engine; the message image does not fit"));
-  }
   const int Lnnz = L->rowptr[k];
   const size_t msg_bytes = (size_t)m * t.RP * (p->msg_fp16 ? 2 : 4);
   const size_t lev_scratch =
@@ -715,7 +701,7 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
                               h->rowidx, h->cpos, h->csc_ent, h->msg_init, h->sched, h->lvl_off, h->nlev, h->xsum,
                               scratch, s),
            "graph builder");
-  if (t.XD > 0) {
+  {
     std::vector<int32_t> cnt(K);
     VIBE_TRY(vibe::build_steps(m, n, K, h->perm, h->colptr, h->cpos, h->stepcnt, scratch, s), "step builder");
     VIBE_TRY(cudaMemcpyAsync(cnt.data(), h->stepcnt, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, s), "step builder");
@@ -726,12 +712,31 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     VIBE_TRY(dalloc(&h->xrec, (size_t)K * t.SP + 4), "tables");   // copied in groups of four slots
     VIBE_TRY(dalloc(&h->xlnk, (size_t)K * t.SP + 4), "tables");
     VIBE_TRY(dalloc(&h->xcolid, (size_t)K * t.SP), "tables");
-    VIBE_TRY(dalloc(&h->xrmap, (size_t)K * E), "tables");
-    VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
+    if (t.XD > 0) VIBE_TRY(dalloc(&h->xrmap, (size_t)K * E), "tables");
+    VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.DP, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
                               h->soff, h->xrec, h->xlnk, h->xcolid, h->xrmap, s),
              "step builder");
   }
   vibe::bpx_layout(&t, p->msg_fp16);
+  vibe::bp_warp_smem_bytes(&t, p->msg_fp16);
+  if (t.engine == VIBE_ENGINE_AUTO) {
+    // the image engine when its per-warp image leaves at least 8 warps per SM, else the summary engine
+    int optin = 0, blocks = 0;
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+    t.engine = VIBE_ENGINE_IMAGE;
+    const Bounds bw = bounds_over(&t, 1);
+    t.engine = VIBE_ENGINE_SUMMARY;
+    if (vibe::bp_cta_smem_bytes(bw, 0) <= (size_t)optin &&
+        vibe::bp_occupancy(bw, 0, p->msg_fp16, &blocks) == cudaSuccess &&
+        (blocks * vibe::kBpWarpsPerCta >= 8 || (other_schedules && blocks >= 1) || (t.XD == 0 && blocks >= 1)))
+      t.engine = VIBE_ENGINE_IMAGE;
+    if (other_schedules && t.engine != VIBE_ENGINE_IMAGE) {
+      cudaFree(scratch);
+      cudaStreamDestroy(s);
+      return bail(fail(VIBE_ERR_UNSUPPORTED,
+                       "flooding and layered members need the image engine; the message image does not fit"));
+    }
+  }
   if (p->n_layered > 0) {
     VIBE_TRY(vibe::build_layers(h->rowptr, h->colidx, h->colptr, h->rowidx, m, h->layer_ptr, h->layer_chk,
                                 h->layer_vptr, h->layer_var, h->nlayer_d, scratch, s),

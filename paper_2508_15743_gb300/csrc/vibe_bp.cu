@@ -2,8 +2,9 @@
 //
 // One warp decodes one shot at a time and pulls shots from a global counter until the batch is
 // done. For its shot the warp runs the K members one after another (Sec. III.D.2): member i keeps its
-// variable-to-check messages in the warp's slice of shared memory, sweeps its dependency wavefronts
-// (lanes = columns of one level, which share no check) and stops as soon as H e = s (Algorithm 1).
+// variable-to-check messages in the warp's slice of shared memory, sweeps its steps (k_steps in
+// vibe_graph.cu: up to 32 edges of columns that share no check, one lane per edge) and stops as soon
+// as H e = s (Algorithm 1).
 //
 // Correction limit (Sec. III.D.2 step 3). The candidates are the first M converged members in
 // (iteration, member) order. Running members in index order, member i can only enter that set by
@@ -19,6 +20,7 @@
 // Arithmetic is the oracle's to the bit: fixed per-node operation order, __fadd_rn/__fmul_rn (no
 // contraction), min and sign exact. Stored messages are never -0 (a sum that starts at lambda_v > 0
 // cannot round to -0 in FP32; FP16 stores map -0 to +0), so the sign bit of a message equals x < 0.
+#include <algorithm>
 #include <type_traits>
 
 #include "vibe_internal.cuh"
@@ -26,125 +28,82 @@
 namespace vibe {
 namespace {
 
+// A stored message in shared memory, and the row scan: |x| minimum with the XOR of the signs as its
+// sign over the 16-byte chunks of a row, as a float (min.xorsign.abs does both at once; a NaN -- the sum
+// of +inf and -inf -- never wins and has sign 0).
 template <typename MT>
 struct Msg;
 
+__device__ __forceinline__ float minx(float a, float b) {
+  float d;
+  asm("min.xorsign.abs.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ uint32_t minx2(uint32_t a, uint32_t b) {   // two halves
+  uint32_t d;
+  asm("min.xorsign.abs.f16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
+  return d;
+}
+
 template <>
 struct Msg<float> {
-  // Minimum magnitude (as a float) and XOR of the raw words over 8 slots starting at row8.
-  __device__ __forceinline__ static void scan8(const float* row8, float& mn, uint32_t& sg) {
-    const float4 a = reinterpret_cast<const float4*>(row8)[0];
-    const float4 b = reinterpret_cast<const float4*>(row8)[1];
-    const float m01 = fminf(fabsf(a.x), fabsf(a.y)), m23 = fminf(fabsf(a.z), fabsf(a.w));
-    const float m45 = fminf(fabsf(b.x), fabsf(b.y)), m67 = fminf(fabsf(b.z), fabsf(b.w));
-    mn = fminf(mn, fminf(fminf(m01, m23), fminf(m45, m67)));
-    sg ^= __float_as_uint(a.x) ^ __float_as_uint(a.y) ^ __float_as_uint(a.z) ^ __float_as_uint(a.w) ^
-          __float_as_uint(b.x) ^ __float_as_uint(b.y) ^ __float_as_uint(b.z) ^ __float_as_uint(b.w);
-  }
-  __device__ __forceinline__ static uint32_t sign(uint32_t sg) { return sg >> 31; }
-  __device__ __forceinline__ static void set_inf(float* p) { *p = __int_as_float(0x7f800000); }
+  static constexpr int kBytes = 4;
+  static constexpr int kSpc = 4;   // slots per 16-byte chunk of a row
+  static constexpr uint32_t kInf = kInfBits;
+  __device__ __forceinline__ static void store(uint32_t a, uint32_t b) { sts32(a, b); }
+  __device__ __forceinline__ static uint32_t round(float x) { return __float_as_uint(x); }
   __device__ __forceinline__ static void store(float* p, float x) { *p = x; }
   __device__ __forceinline__ static float value(float x) { return x; }
-  static constexpr int kSpc = 4;   // slots per 16-byte chunk of a row
+  template <int NCH>
+  __device__ __forceinline__ static float scan(uint32_t row, int nch) {
+    float v = __int_as_float(0x7f800000);
+    auto chunk = [&](uint32_t a) {
+      const uint4 q = lds128(a);
+      v = minx(v, minx(minx(__uint_as_float(q.x), __uint_as_float(q.y)), minx(__uint_as_float(q.z), __uint_as_float(q.w))));
+    };
+    if (NCH) {
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) chunk(row + 16 * i);
+    } else {
+      for (int i = 0; i < nch; ++i) chunk(row + 16 * i);
+    }
+    return v;
+  }
 };
 
 template <>
 struct Msg<__half> {
-  __device__ __forceinline__ static void scan8(const __half* row8, float& mn, uint32_t& sg) {
-    const uint4 q = *reinterpret_cast<const uint4*>(row8);
-    const __half2 h0 = __habs2(*reinterpret_cast<const __half2*>(&q.x));
-    const __half2 h1 = __habs2(*reinterpret_cast<const __half2*>(&q.y));
-    const __half2 h2 = __habs2(*reinterpret_cast<const __half2*>(&q.z));
-    const __half2 h3 = __habs2(*reinterpret_cast<const __half2*>(&q.w));
-    const __half2 hm = __hmin2(__hmin2(h0, h1), __hmin2(h2, h3));
-    mn = fminf(mn, __half2float(__hmin(__low2half(hm), __high2half(hm))));
-    const uint32_t x = q.x ^ q.y ^ q.z ^ q.w;
-    sg ^= x ^ (x >> 16);
+  static constexpr int kBytes = 2;
+  static constexpr int kSpc = 8;
+  static constexpr uint32_t kInf = 0x7c00u;
+  __device__ __forceinline__ static void store(uint32_t a, uint32_t b) { sts16(a, b); }
+  __device__ __forceinline__ static uint32_t round(float x) {   // -0 as +0
+    const uint32_t h = (uint32_t)__half_as_ushort(__float2half_rn(x));
+    return h == 0x8000u ? 0u : h;
   }
-  __device__ __forceinline__ static uint32_t sign(uint32_t sg) { return (sg >> 15) & 1u; }
-  __device__ __forceinline__ static void set_inf(__half* p) { *reinterpret_cast<unsigned short*>(p) = 0x7c00u; }
   __device__ __forceinline__ static void store(__half* p, float x) {
-    unsigned short h = __half_as_ushort(__float2half_rn(x));
-    if (h == 0x8000u) h = 0;
-    *reinterpret_cast<unsigned short*>(p) = h;
+    *reinterpret_cast<unsigned short*>(p) = (unsigned short)round(x);
   }
   __device__ __forceinline__ static float value(__half x) { return __half2float(x); }
-  static constexpr int kSpc = 8;
+  template <int NCH>
+  __device__ __forceinline__ static float scan(uint32_t row, int nch) {
+    uint32_t v = 0x7c007c00u;
+    auto chunk = [&](uint32_t a) {
+      const uint4 q = lds128(a);
+      v = minx2(v, minx2(minx2(q.x, q.y), minx2(q.z, q.w)));
+    };
+    if (NCH) {
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) chunk(row + 16 * i);
+    } else {
+      for (int i = 0; i < nch; ++i) chunk(row + 16 * i);
+    }
+    return __half2float(__ushort_as_half((unsigned short)minx2(v, v >> 16)));
+  }
 };
 
 __device__ __forceinline__ bool is_finite_bits(float x) {
   return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
-}
-
-// One serial-V column update (readings R2, R3 of the oracle): check-to-variable messages from the
-// current variable-to-check messages of the other columns, posterior, literal exclusion sums, decision.
-// RPC = row pitch in 8-slot chunks (0: read it from the tables).
-//
-// Exclusion of the column's own message from its check rows: a check is touched by exactly one
-// column per wavefront level, so the updating lane owns the row until the level ends. It overwrites
-// its own slot with +inf (magnitude that never wins a minimum, sign bit 0), takes the minimum
-// magnitude and the XOR of the sign bits over the whole row, and later stores its new message in
-// the same slot. Minimum and parity equal those over the other slots exactly.
-// DP is the launch's largest column pitch; dp the problem's own (dp <= DP).
-template <typename MT, int DP, int RPC>
-__device__ __forceinline__ void update_column(uint32_t v, int deg, const uint32_t* csc, int dp, const float* lam,
-                                              uint32_t rp, float alpha, MT* msgs, uint8_t* dec8, const uint8_t* s8,
-                                              uint8_t* par8, float* lpost) {
-  uint32_t ent[DP];
-  const uint4* ce = reinterpret_cast<const uint4*>(csc + (size_t)v * dp);
-#pragma unroll
-  for (int q = 0; q < DP / 4; ++q) {
-    uint4 x = make_uint4(0u, 0u, 0u, 0u);
-    if (4 * q < dp) x = __ldg(ce + q);
-    ent[4 * q + 0] = x.x; ent[4 * q + 1] = x.y; ent[4 * q + 2] = x.z; ent[4 * q + 3] = x.w;
-  }
-  const float lamv = __ldg(lam + v);
-  const uint32_t RP = RPC ? (uint32_t)RPC * 8u : rp;
-  float mcv[DP];
-#pragma unroll
-  for (int k = 0; k < DP; ++k) {
-    mcv[k] = 0.0f;
-    if (k < deg) {
-      const uint32_t c = ent[k] >> 9;
-      MT* row = msgs + c * RP;
-      Msg<MT>::set_inf(row + (ent[k] & 0xffu));
-      float mn = __int_as_float(0x7f800000);
-      uint32_t sg = 0;
-      if (RPC) {
-#pragma unroll
-        for (int ch = 0; ch < RPC; ++ch) Msg<MT>::scan8(row + 8 * ch, mn, sg);
-      } else {
-        for (uint32_t ch = 0; ch < RP; ch += 8) Msg<MT>::scan8(row + ch, mn, sg);
-      }
-      const uint32_t neg = Msg<MT>::sign(sg) ^ (uint32_t)s8[c];
-      const float mag = __fmul_rn(alpha, mn);
-      mcv[k] = neg ? -mag : mag;
-    }
-  }
-  float L = lamv;
-#pragma unroll
-  for (int k = 0; k < DP; ++k)
-    if (k < deg) L = __fadd_rn(L, mcv[k]);
-  float pre = lamv;  // lambda + m_0 + ... + m_{k-1}, the shared head of every exclusion sum
-#pragma unroll
-  for (int k = 0; k < DP; ++k) {
-    if (k < deg) {
-      float a = pre;
-#pragma unroll
-      for (int k2 = k + 1; k2 < DP; ++k2)
-        if (k2 < deg) a = __fadd_rn(a, mcv[k2]);
-      Msg<MT>::store(msgs + (ent[k] >> 9) * RP + (ent[k] & 0xffu), a);
-      pre = __fadd_rn(pre, mcv[k]);
-    }
-  }
-  const uint8_t e_new = L <= 0.0f;
-  if (e_new != dec8[v]) {
-#pragma unroll
-    for (int k = 0; k < DP; ++k)
-      if (k < deg) par8[ent[k] >> 9] ^= 1u;
-    dec8[v] = e_new;
-  }
-  if (lpost) lpost[v] = L;
 }
 
 // One parallel (flooding) iteration of Algorithm 1 on the warp's FP32 message image.
@@ -154,10 +113,13 @@ __device__ __forceinline__ void update_column(uint32_t v, int deg, const uint32_
 // slots: exactly the exclusion over N(c) \ v). Column pass: a lane takes whole columns and turns its
 // own slots into the new variable-to-check messages with the sums of the serial update. Every column
 // reads only its own slots, so the passes need no second image. Parity pass: (H e)_c XOR s_c from
-// the decisions (many columns touch a check in the column pass).
+// the decisions (many columns touch a check in the column pass); returns whether the lane met an
+// unsatisfied check.
+__device__ __forceinline__ uint32_t syn_bit(const uint32_t* s32, int c) { return (s32[c >> 5] >> (c & 31)) & 1u; }
+
 template <int DP>
-__device__ __forceinline__ void flood_sweep(const Tables& t, float alpha, float* msgs, uint8_t* dec8,
-                                            const uint8_t* s8, uint8_t* par8, float* lpost, int lane) {
+__device__ __forceinline__ bool flood_sweep(const Tables& t, float alpha, float* msgs, uint8_t* dec8,
+                                            const uint32_t* s32, float* lpost, int lane) {
   const int m = t.m, n = t.n;
   const uint32_t RP = (uint32_t)t.RP;
   for (int c = lane; c < m; c += 32) {
@@ -177,7 +139,7 @@ __device__ __forceinline__ void flood_sweep(const Tables& t, float alpha, float*
       const uint32_t pos = row_position((uint32_t)c, (uint32_t)j, (int)RP, 4);
       const float x = row[pos];
       const float mn = j == a1 ? m2 : m1;
-      const uint32_t neg = (sx ^ (__float_as_uint(x) >> 31) ^ (uint32_t)s8[c]) & 1u;
+      const uint32_t neg = (sx ^ (__float_as_uint(x) >> 31) ^ syn_bit(s32, c)) & 1u;
       const float mag = __fmul_rn(alpha, mn);
       row[pos] = neg ? -mag : mag;
     }
@@ -218,12 +180,14 @@ __device__ __forceinline__ void flood_sweep(const Tables& t, float alpha, float*
     if (lpost) lpost[v] = L;
   }
   __syncwarp();
+  bool bad = false;
   for (int c = lane; c < m; c += 32) {
-    uint32_t p = s8[c];
+    uint32_t p = syn_bit(s32, c);
     for (int e = __ldg(t.rowptr + c); e < __ldg(t.rowptr + c + 1); ++e) p ^= dec8[__ldg(t.colidx + e)];
-    par8[c] = (uint8_t)p;
+    bad |= p != 0u;
   }
   __syncwarp();
+  return bad;
 }
 
 // One iteration of a schedule over check layers, with the check-to-variable messages in their own
@@ -240,9 +204,8 @@ __device__ __forceinline__ void flood_sweep(const Tables& t, float alpha, float*
 // Then every posterior (lambda plus the column's cv entries in ascending check order), decision and
 // check parity. cv holds zeros when a layered member starts (init in run_member).
 template <typename MT, int DP>
-__device__ __forceinline__ void layer_sweep(const Tables& t, float alpha, bool flood, MT* msgs, float* cv,
-                                            uint8_t* dec8, const uint8_t* s8, uint8_t* par8, float* lpost,
-                                            int lane) {
+__device__ __forceinline__ bool layer_sweep(const Tables& t, float alpha, bool flood, MT* msgs, float* cv,
+                                            uint8_t* dec8, const uint32_t* s32, float* lpost, int lane) {
   const int m = t.m, n = t.n;
   const uint32_t RP = (uint32_t)t.RP;
   const int nl = flood ? 1 : t.nlayer;
@@ -266,7 +229,7 @@ __device__ __forceinline__ void layer_sweep(const Tables& t, float alpha, bool f
       for (int j = 0; j < deg; ++j) {
         const uint32_t pos = row_position((uint32_t)c, (uint32_t)j, (int)RP, Msg<MT>::kSpc);
         const float x = Msg<MT>::value(row[pos]);
-        const uint32_t neg = (sx ^ (__float_as_uint(x) >> 31) ^ (uint32_t)s8[c]) & 1u;
+        const uint32_t neg = (sx ^ (__float_as_uint(x) >> 31) ^ syn_bit(s32, c)) & 1u;
         const float mag = __fmul_rn(alpha, j == a1 ? m2 : m1);
         crow[pos] = neg ? -mag : mag;
       }
@@ -316,55 +279,167 @@ __device__ __forceinline__ void layer_sweep(const Tables& t, float alpha, bool f
     if (lpost) lpost[v] = L;
   }
   __syncwarp();
+  bool bad = false;
   for (int c = lane; c < m; c += 32) {
-    uint32_t p = s8[c];
+    uint32_t p = syn_bit(s32, c);
     for (int e = __ldg(t.rowptr + c); e < __ldg(t.rowptr + c + 1); ++e) p ^= dec8[__ldg(t.colidx + e)];
-    par8[c] = (uint8_t)p;
+    bad |= p != 0u;
   }
   __syncwarp();
+  return bad;
 }
 
-// Blocks per SM the register budget targets: FP16 states are small enough for 24 warps per SM,
-// FP32 states (twice the message bytes) fill shared memory at about 16-18.
-template <typename MT>
-struct MinBlocks { static constexpr int value = 16 / kBpWarpsPerCta; };
-template <>
-struct MinBlocks<__half> { static constexpr int value = 24 / kBpWarpsPerCta; };
+// Warps per SM the register budget targets. Shared-memory wavefronts bound the kernel, which this many
+// warps keep busy; the FP32 states of the d=9 phenomenological problem fill shared memory at 20.
+template <typename MT, int DP>
+struct MinBlocks { static constexpr int value = (DP <= 8 ? 20 : 16) / kBpWarpsPerCta; };
 
-// Decodes one shot of problem t with the warp (the body of the persistent loop below).
-// One member (index i) of the shot whose syndrome bytes are in the warp's shared memory: initialises
-// the member's message image and runs up to `budget` sweeps, stopping at the first that leaves
-// H e = s, or before sweep `it` when stop(it) holds. Returns the converging sweep (0 if none) and in
-// `ran` the sweeps run; leaves the decisions in the warp's decision bytes and the posterior of the
-// last sweep in lpost when soft output is on or `keep_last` is set and the member reached sweep T.
-template <typename MT, int DP, int RPC, bool MIXED, typename Stop>
-__device__ __forceinline__ int run_member(const Tables& t, int i, int budget, bool want_soft, bool keep_last,
-                                          unsigned char* base, float* lpost, int lane, unsigned long long& my_iters,
-                                          int& ran, Stop stop) {
-  const int n = t.n, m = t.m, T = t.T;
-  const int m4 = (m + 3) >> 2;
+// What a member's run is told and what it reports.
+struct ImageRun {
+  int budget;               // sweeps at most
+  bool soft, keep_last;     // the posterior after every sweep / after sweep T
+  const int* conv;          // pair mode: the shot's converged members (pair_should_stop), else NULL
+  float* lpost;             // global: n posteriors
+  uint32_t* st;             // the steps' decision words: shared (generic address) or global
+  int ran;                  // result: sweeps run
+};
+
+constexpr int kRecSteps = 2;   // steps fetched together, one group ahead
+
+// One serial sweep of a member over its ns steps on the message image at shared address msgs. A lane
+// holds one edge of a step (its check is no other lane's): it writes +inf into its own slot of the row
+// -- a magnitude that never wins a minimum, sign bit 0 -- so that the row scan gives the minimum and sign
+// product over the other slots exactly, gets the column's other messages from their lanes, forms its
+// exclusion sum in the order of Algorithm 1 and stores the new message in its slot. Decisions are one
+// word per step (on the lane of the column's last edge); check parities are flipped, and the word
+// stored, only when one changes.
+// What bounds it: shared-memory wavefronts (94 % of their peak). The lanes' rows are random, so a 16-byte
+// row load of 32 lanes takes ~9 wavefronts instead of 4. With one lane per column a sweep of the d=9
+// phenomenological problem took 42 chunks of 187 instructions and 2800 wavefronts; its 62 steps take 90
+// instructions each. Measured, 32768 shots of it (K=16, T=30): 96.7 -> 73.1 ms with FP32 messages, 78.1 ->
+// 51.2 ms with FP16; the 4.8.8 code, whose rows of 10 now take three chunks instead of four, 40 -> 16 ms.
+// NCH: 16-byte chunks of a row (0: from the tables). par32 holds the check parities.
+template <typename MT, int DP, int NCH, bool LP>
+__device__ __forceinline__ void step_sweep(const Tables& t, const uint32_t* soff, const int ns, const size_t first,
+                                           const float alpha, const uint32_t msgs, const uint32_t s32,
+                                           const uint32_t par32, uint32_t* st, float* lp, const int lane) {
+  const int nch = NCH ? NCH : t.RP / Msg<MT>::kSpc;
+  const uint32_t row_bytes = (uint32_t)nch * 16u;
+  // the chunk swizzle of row_position(): slot ^ ((check >> a) & (n - 1)) * slots per chunk
+  const uint32_t swz_mask = (nch == 2 || nch == 4 || nch == 8) ? (uint32_t)nch - 1u : 0u;
+  const int swz_shift = nch == 2 ? 2 : nch == 4 ? 1 : 0;
+  const uint2* trec = t.xrec + first + lane;
+  const uint32_t* tlnk = t.xlnk + first + lane;
+  const bool wide = DP > 16 && t.DP > 16;
+  uint32_t o[kRecSteps + 1], on[kRecSteps + 1];   // first slots of this group's steps and the next one's
+  uint2 r[kRecSteps], rn[kRecSteps];
+  uint32_t ln[kRecSteps], lnn[kRecSteps];
+  auto fetch = [&](const uint32_t (&off)[kRecSteps + 1], uint2 (&rec)[kRecSteps], uint32_t (&lnk)[kRecSteps]) {
+#pragma unroll
+    for (int u = 0; u < kRecSteps; ++u) {
+      rec[u] = make_uint2(0u, 0u);
+      lnk[u] = 0u;
+      if (off[u] + (uint32_t)lane < off[u + 1]) {
+        rec[u] = __ldg(trec + off[u]);
+        lnk[u] = __ldg(tlnk + off[u]);
+      }
+    }
+  };
+#pragma unroll
+  for (int u = 0; u <= kRecSteps; ++u) {
+    o[u] = __ldg(soff + u);
+    on[u] = __ldg(soff + kRecSteps + u);
+  }
+  fetch(o, r, ln);
+  for (int s0 = 0; s0 < ns; s0 += kRecSteps) {
+    fetch(on, rn, lnn);
+    uint32_t of[kRecSteps];   // the offsets after the next group's
+#pragma unroll
+    for (int u = 0; u < kRecSteps; ++u) of[u] = __ldg(soff + s0 + 2 * kRecSteps + 1 + u);
+#pragma unroll
+    for (int u = 0; u < kRecSteps; ++u) {
+      const uint32_t old = s0 + u < ns ? st[s0 + u] : 0u;
+      const uint32_t c = r[u].x >> 18;
+      const uint32_t row = msgs + c * row_bytes;
+      uint32_t pos = r[u].x & 0xffu;
+      if (NCH == 0 || NCH == 2 || NCH == 4 || NCH == 8) pos ^= ((c >> swz_shift) & swz_mask) * (uint32_t)Msg<MT>::kSpc;
+      const uint32_t own = row + pos * (uint32_t)Msg<MT>::kBytes;
+      const bool act = (int)ln[u] < 0;
+      if (act) Msg<MT>::store(own, Msg<MT>::kInf);
+      const uint32_t sw = lds32(s32 + ((c >> 5) << 2));
+      const float mn = Msg<MT>::template scan<NCH>(row, nch);
+      const uint32_t mcv = __float_as_uint(__fmul_rn(alpha, mn)) ^ (__funnelshift_l(0u, sw, ~c) & 0x80000000u);
+      float acc = __uint_as_float(r[u].y);
+      // links of columns of more than 16 checks: first lane | k << 5 | degree - 1 << 10
+      uint32_t incl = ln[u] >> 5, lastl = (ln[u] >> kLnkLastLane) & 31u;
+      if (wide) {
+        const uint32_t k = (ln[u] >> 5) & 31u, dm1 = (ln[u] >> 10) & 31u;
+        incl = ((2u << dm1) - 1u) & ~(1u << k);
+        lastl = (ln[u] + dm1) & 31u;
+      } else if (DP > 16) {
+        incl &= 0xffffu;
+      }
+#pragma unroll
+      for (int j = 0; j < DP; ++j)
+        acc = add_if(acc, __uint_as_float(__shfl_sync(kFull, mcv, (int)ln[u] + j)), incl & (1u << j));
+      const float L = __fadd_rn(acc, __uint_as_float(mcv));   // on the last edge's lane: the posterior
+      const uint32_t dec = __ballot_sync(kFull, (ln[u] & kLnkLast) && L <= 0.0f);
+      if (act) Msg<MT>::store(own, Msg<MT>::round(acc));
+      const uint32_t ch = dec ^ old;
+      if (ch) {   // some column of the step changed its decision
+        if (act && ((ch >> lastl) & 1u)) red_xor_shared(par32 + ((c >> 5) << 2), 1u << (c & 31));
+        if (lane == 0) st[s0 + u] = dec;
+      }
+      if (LP) {
+        if (ln[u] & kLnkLast) lp[__ldg(t.xcolid + first + o[u] + lane)] = L;
+        else if (ln[u] == 0u && o[u] + (uint32_t)lane < o[u + 1])   // column without checks
+          lp[__ldg(t.xcolid + first + o[u] + lane)] = __uint_as_float(r[u].y);
+      }
+      __syncwarp();
+    }
+#pragma unroll
+    for (int u = 0; u < kRecSteps; ++u) { r[u] = rn[u]; ln[u] = lnn[u]; }
+#pragma unroll
+    for (int u = 0; u <= kRecSteps; ++u) o[u] = on[u];
+    on[0] = on[kRecSteps];
+#pragma unroll
+    for (int u = 0; u < kRecSteps; ++u) on[u + 1] = of[u];
+  }
+}
+
+// One member (index i) of the shot whose syndrome words are in the warp's shared memory at byte offset
+// smem_off: initialises the member's message image and runs up to `budget` sweeps, stopping at the first
+// that leaves H e = s, or in pair mode before a sweep that no longer counts. Returns the converging sweep
+// (0 if none); leaves the decisions in the step words (serial member) or the decision bytes, and the
+// posterior of the last sweep in lpost when soft output is on or `keep_last` is set and the member
+// reached sweep T. Not inlined: the sweep gets its own registers, whatever the caller keeps.
+template <typename MT, int DP, int NCH>
+__device__ __noinline__ int run_member(const Tables& t, int i, int smem_off, ImageRun& R) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  unsigned char* base = smem + smem_off;
+  // through a shuffle: read once, and in a register of its own (the compiler would read it at each use)
+  const int lane = __shfl_sync(kFull, (int)(threadIdx.x & 31), (int)(threadIdx.x & 31));
+  const uint32_t sbase = __shfl_sync(kFull, (uint32_t)__cvta_generic_to_shared(smem) + (uint32_t)smem_off, lane);
+  const int n = t.n, m = t.m, T = t.T, mw = t.mw;
   const int n4 = (n + 3) >> 2;
   const int msg_vec = (int)(((size_t)m * t.RP * sizeof(MT)) / 16);
-  const uint32_t* csc = t.csc_ent;
-  const float* lam = t.lam;
-  const int dp = MIXED ? t.DP : DP;   // one problem: the pitch is the launch's
-  const uint32_t rp = (uint32_t)t.RP;
-  MT* msgs = reinterpret_cast<MT*>(base + t.off_msg);
-  uint8_t* dec8 = base + t.off_dec;
-  uint8_t* s8 = base + t.off_s;
-  uint8_t* par8 = base + t.off_par;
+  const uint32_t* s32 = reinterpret_cast<const uint32_t*>(base + t.off_s);
+  uint32_t* par = reinterpret_cast<uint32_t*>(base + t.off_par);
+  const bool flood = i < t.n_flood;
+  const bool layered = !flood && i < t.n_flood + t.n_layered;
+  const int ns = __ldg(t.stepcnt + i);
   // member init: messages from the prior image, decisions 0, parity = s
   {
     const uint4* src = reinterpret_cast<const uint4*>(t.msg_init);
-    uint4* dst = reinterpret_cast<uint4*>(msgs);
-    for (int q = lane; q < msg_vec; q += 32) dst[q] = __ldg(src + q);
-    uint32_t* d32 = reinterpret_cast<uint32_t*>(dec8);
-    for (int q = lane; q < n4; q += 32) d32[q] = 0u;
-    const uint32_t* s32 = reinterpret_cast<const uint32_t*>(s8);
-    uint32_t* p32 = reinterpret_cast<uint32_t*>(par8);
-    for (int q = lane; q < m4; q += 32) p32[q] = s32[q];
+    for (int q = lane; q < msg_vec; q += 32) sts128(sbase + t.off_msg + 16 * q, __ldg(src + q));
+    if (flood || layered) {
+      uint32_t* d32 = reinterpret_cast<uint32_t*>(base + t.off_dec);
+      for (int q = lane; q < n4; q += 32) d32[q] = 0u;
+    } else {
+      for (int q = lane; q < ns; q += 32) R.st[q] = 0u;
+    }
+    for (int q = lane; q < mw; q += 32) par[q] = s32[q];
   }
-  const bool layered = i >= t.n_flood && i < t.n_flood + t.n_layered;
   float* cv = t.off_cv >= 0 ? reinterpret_cast<float*>(base + t.off_cv) : nullptr;
   if (layered) {   // the layered member's check-to-variable messages start at zero
     uint4* c4 = reinterpret_cast<uint4*>(cv);
@@ -373,72 +448,107 @@ __device__ __forceinline__ int run_member(const Tables& t, int i, int budget, bo
   }
   __syncwarp();
 
-  const uint32_t* sch = t.sched + (size_t)i * n;
-  const uint32_t* lo = t.lvl_off + (size_t)i * (n + 1);
-  const int nl = __ldg(t.nlev + i);
+  const size_t first = (size_t)i * t.SP;
+  const uint32_t* soff = t.soff + (size_t)i * t.soff_pitch;
   const float alpha = __ldg(t.alpha_m + i);   // member i's scaling factor
-  int conv = 0;
-  ran = 0;
+  const int budget = R.budget;
+  int conv = 0, ran = 0;
   for (int it = 1; it <= budget; ++it) {
-    if (stop(it)) break;
+    if (R.conv && pair_should_stop(R.conv, t.K, t.M, i, it, lane)) break;
     // the posterior is needed after the last possible sweep of a member that may end without
     // converging (LLR average) and, for soft output, after every sweep
-    float* lp = (want_soft || (it == T && keep_last)) ? lpost : nullptr;
-    bool swept = false;   // by a schedule other than the member's serial one
-    if (i < t.n_flood) {   // parallel schedule
-      if constexpr (std::is_same<MT, float>::value) flood_sweep<DP>(t, alpha, msgs, dec8, s8, par8, lp, lane);
-      else layer_sweep<MT, DP>(t, alpha, true, msgs, cv, dec8, s8, par8, lp, lane);
-      swept = true;
-    } else if (layered) {
-      layer_sweep<MT, DP>(t, alpha, false, msgs, cv, dec8, s8, par8, lp, lane);
-      swept = true;
-    }
-    for (int l = 0; l < nl && !swept; ++l) {
-      const uint32_t b = __ldg(lo + l), e = __ldg(lo + l + 1);
-      for (uint32_t idx = b + lane; idx < e; idx += 32) {
-        const uint32_t ent = __ldg(sch + idx);
-        update_column<MT, DP, RPC>(ent & 0xffffffu, (int)(ent >> 24), csc, dp, lam, rp, alpha, msgs, dec8, s8,
-                                   par8, lp);
-      }
+    float* lp = (R.soft || (it == T && R.keep_last)) ? R.lpost : nullptr;
+    bool bad = false;
+    if (flood || layered) {
+      MT* msgs = reinterpret_cast<MT*>(base + t.off_msg);
+      uint8_t* dec8 = base + t.off_dec;
+      if (std::is_same<MT, float>::value && flood)
+        bad = flood_sweep<DP>(t, alpha, reinterpret_cast<float*>(msgs), dec8, s32, lp, lane);
+      else
+        bad = layer_sweep<MT, DP>(t, alpha, flood, msgs, cv, dec8, s32, lp, lane);
+    } else {
+      if (lp)
+        step_sweep<MT, DP, NCH, true>(t, soff, ns, first, alpha, sbase + t.off_msg, sbase + t.off_s, sbase + t.off_par,
+                                      R.st, lp, lane);
+      else
+        step_sweep<MT, DP, NCH, false>(t, soff, ns, first, alpha, sbase + t.off_msg, sbase + t.off_s, sbase + t.off_par,
+                                       R.st, nullptr, lane);
+      for (int q = lane; q < mw; q += 32) bad |= lds32(sbase + t.off_par + 4 * q) != 0u;
       __syncwarp();
     }
-    ++my_iters;
     ran = it;
-    uint32_t bad = 0;
-    const uint32_t* p32 = reinterpret_cast<const uint32_t*>(par8);
-    for (int q = lane; q < m4; q += 32) bad |= p32[q];
     if (!__any_sync(kFull, bad)) { conv = it; break; }
   }
+  R.ran = ran;
   return conv;
 }
 
-template <typename MT, int DP, int RPC, bool MIXED>
-__device__ __forceinline__ void decode_shot(const BpArgs& a, const Tables& t, uint32_t shot, unsigned char* base,
-                                            float* acc, float* lpost, float* cand_post, int lane,
-                                            unsigned long long& my_iters, unsigned long long& my_shots,
-                                            unsigned long long& my_fail) {
-  const int n = t.n, m = t.m, K = t.K, M = t.M, T = t.T, nw = t.nw, kw = t.kw;
-  const int m4 = (m + 3) >> 2;
-  const int n4 = (n + 3) >> 2;
-  const int msg_vec = (int)(((size_t)m * t.RP * sizeof(MT)) / 16);
-  const uint32_t* csc = t.csc_ent;
-  const float* lam = t.lam;
-  const int dp = MIXED ? t.DP : DP;   // one problem: the pitch is the launch's
-  const uint32_t rp = (uint32_t)t.RP;
-  MT* msgs = reinterpret_cast<MT*>(base + t.off_msg);
-  uint8_t* dec8 = base + t.off_dec;
-  uint8_t* s8 = base + t.off_s;
-  uint8_t* par8 = base + t.off_par;
-  uint32_t* cand = reinterpret_cast<uint32_t*>(base + t.off_cand);
-  const uint32_t* syn = a.syn + (size_t)shot * a.syn_stride;
-  uint32_t any = 0;
-  for (int c = lane; c < 4 * m4; c += 32) {
-    uint32_t b = c < m ? (__ldg(syn + (c >> 5)) >> (c & 31)) & 1u : 0u;
-    s8[c] = (uint8_t)b;
-    any |= b;
+// The decisions a converged member left, as bits in column order in shared memory, and W(e) = sum of
+// lambda_j over e_j = 1, ascending j.
+__device__ __forceinline__ float member_bits(const Tables& t, int i, unsigned char* base, const uint32_t* st,
+                                             uint32_t* bits, int lane) {
+  const int n = t.n, nw = t.nw;
+  if (i < t.n_flood + t.n_layered) {
+    const uint8_t* dec8 = base + t.off_dec;
+    for (int w = 0; w < nw; ++w) {
+      const int v = 32 * w + lane;
+      const uint32_t word = __ballot_sync(kFull, v < n && dec8[v] != 0);
+      if (lane == 0) bits[w] = word;
+    }
+  } else {
+    const uint32_t* soff = t.soff + (size_t)i * t.soff_pitch;
+    const uint32_t* colid = t.xcolid + (size_t)i * t.SP;
+    const int ns = __ldg(t.stepcnt + i);
+    for (int w = lane; w < nw; w += 32) bits[w] = 0u;
+    __syncwarp();
+    for (int s = lane; s < ns; s += 32) {
+      uint32_t d = st[s];
+      if (!d) continue;
+      const uint32_t o = __ldg(soff + s);
+      while (d) {
+        const uint32_t v = __ldg(colid + o + (uint32_t)__ffs(d) - 1u);
+        atomicOr(bits + (v >> 5), 1u << (v & 31));
+        d &= d - 1u;
+      }
+    }
   }
-  any = __any_sync(kFull, any);
   __syncwarp();
+  float W = 0.0f;
+  for (int w = 0; w < nw; ++w) {
+    uint32_t x = bits[w];
+    while (x) {
+      W = __fadd_rn(W, __ldg(t.lam + 32 * w + __ffs(x) - 1));
+      x &= x - 1;
+    }
+  }
+  return W;
+}
+
+// The syndrome of a shot as words in shared memory (bits past m cleared); returns whether it is not zero.
+__device__ __forceinline__ bool load_syndrome(const Tables& t, const uint32_t* syn, uint32_t* s32, int lane) {
+  uint32_t any = 0;
+  for (int w = lane; w < t.mw; w += 32) {
+    const int rem = t.m - 32 * w;
+    const uint32_t x = __ldg(syn + w) & (rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
+    s32[w] = x;
+    any |= x;
+  }
+  any = __any_sync(kFull, any != 0u);
+  __syncwarp();
+  return any != 0u;
+}
+
+// Decodes one shot of problem t with the warp (the body of the persistent loop below). smem_off: the
+// warp's shared memory; acc, lpost, cand_post, gst: its global scratch.
+template <typename MT, int DP, int NCH>
+__device__ __forceinline__ void decode_shot(const BpArgs& a, const Tables& t, uint32_t shot, unsigned char* base,
+                                            int smem_off, float* acc, float* lpost, float* cand_post, uint32_t* gst,
+                                            int lane, unsigned long long& my_iters, unsigned long long& my_shots,
+                                            unsigned long long& my_fail) {
+  const int n = t.n, K = t.K, M = t.M, T = t.T, nw = t.nw, kw = t.kw;
+  uint32_t* cand = reinterpret_cast<uint32_t*>(base + t.off_cand);
+  uint32_t* st = t.off_st >= 0 ? reinterpret_cast<uint32_t*>(base + t.off_st) : gst;
+  const bool any = load_syndrome(t, a.syn + (size_t)shot * a.syn_stride, reinterpret_cast<uint32_t*>(base + t.off_s), lane);
   ++my_shots;
   uint32_t* out_corr = a.corr + (size_t)shot * a.corr_stride;
 
@@ -470,26 +580,14 @@ __device__ __forceinline__ void decode_shot(const BpArgs& a, const Tables& t, ui
   for (int i = 0; i < K; ++i) {
     const int budget = ncand < M ? T : __shfl_sync(kFull, c_t, M - 1) - 1;
     if (budget <= 0) break;
-    int ran = 0;
-    const int conv = run_member<MT, DP, RPC, MIXED>(t, i, budget, a.want_soft != 0, ncand == 0, base, lpost, lane,
-                                                    my_iters, ran, [](int) { return false; });
+    ImageRun R{budget, a.want_soft != 0, ncand == 0, nullptr, lpost, st, 0};
+    const int conv = run_member<MT, DP, NCH>(t, i, smem_off, R);
+    my_iters += (unsigned long long)R.ran;
     if (conv) {
       // insert (conv, i); i exceeds every member already listed, so it goes after equal iterations
       const int p = __popc(__ballot_sync(kFull, lane < ncand && c_t <= conv));
       const int slot = ncand < M ? ncand : __shfl_sync(kFull, c_slot, M - 1);
-      uint32_t* bits = cand + (size_t)slot * nw;
-      float W = 0.0f;
-      for (int w = 0; w < nw; ++w) {
-        const int v = 32 * w + lane;
-        const uint32_t word = __ballot_sync(kFull, v < n && dec8[v] != 0);
-        if (lane == 0) bits[w] = word;
-        uint32_t x = word;
-        while (x) {
-          const int bpos = __ffs(x) - 1;
-          W = __fadd_rn(W, __ldg(lam + 32 * w + bpos));
-          x &= x - 1;
-        }
-      }
+      const float W = member_bits(t, i, base, st, cand + (size_t)slot * nw, lane);
       if (a.want_soft) {
         float* dst = cand_post + (size_t)slot * n;
         for (int v = lane; v < n; v += 32) dst[v] = lpost[v];
@@ -576,24 +674,15 @@ __device__ __forceinline__ void decode_shot(const BpArgs& a, const Tables& t, ui
 
 // Pair mode: member i of shot `shot` (slot `slot` of the chunk) with one warp; the last member of the
 // shot to finish writes the shot's outcome (pair_epilogue, vibe_internal.cuh).
-template <typename MT, int DP, int RPC, bool MIXED>
+template <typename MT, int DP, int NCH>
 __device__ __forceinline__ void decode_pair(const BpArgs& a, const Tables& t, uint32_t shot, int slot, int i,
-                                            unsigned char* base, float* lpost, int lane, unsigned long long& my_iters,
-                                            unsigned long long& my_shots, unsigned long long& my_fail) {
-  const int K = t.K, M = t.M, T = t.T, n = t.n, m = t.m, nw = t.nw, kw = t.kw;
+                                            unsigned char* base, int smem_off, float* lpost, uint32_t* gst, int lane,
+                                            unsigned long long& my_iters, unsigned long long& my_shots,
+                                            unsigned long long& my_fail) {
+  const int K = t.K, M = t.M, T = t.T, n = t.n, nw = t.nw, kw = t.kw;
   if (i >= K) return;
-  const int m4 = (m + 3) >> 2;
-  uint8_t* s8 = base + t.off_s;
-  const uint8_t* dec8 = base + t.off_dec;
-  const uint32_t* syn = a.syn + (size_t)shot * a.syn_stride;
-  uint32_t any = 0;
-  for (int c = lane; c < 4 * m4; c += 32) {
-    const uint32_t b = c < m ? (__ldg(syn + (c >> 5)) >> (c & 31)) & 1u : 0u;
-    s8[c] = (uint8_t)b;
-    any |= b;
-  }
-  any = __any_sync(kFull, any);
-  __syncwarp();
+  uint32_t* st = t.off_st >= 0 ? reinterpret_cast<uint32_t*>(base + t.off_st) : gst;
+  const bool any = load_syndrome(t, a.syn + (size_t)shot * a.syn_stride, reinterpret_cast<uint32_t*>(base + t.off_s), lane);
   if (!any && !a.want_soft) {
     // s = 0: every member converges in iteration 1 to e = 0; member 0 is chosen -- written by member 0
     if (i != 0) return;
@@ -616,32 +705,22 @@ __device__ __forceinline__ void decode_pair(const BpArgs& a, const Tables& t, ui
   }
   if (i == 0) ++my_shots;
   int* conv = a.pconv + (size_t)slot * a.pair_K;
-  int ran = 0;
-  const int cv = run_member<MT, DP, RPC, MIXED>(t, i, T, a.want_soft != 0, true, base, lpost, lane, my_iters, ran,
-                                                [&](int it) { return pair_should_stop(conv, K, M, i, it, lane); });
+  ImageRun R{T, a.want_soft != 0, true, conv, lpost, st, 0};
+  const int cv = run_member<MT, DP, NCH>(t, i, smem_off, R);
+  my_iters += (unsigned long long)R.ran;
   const size_t rec = (size_t)slot * a.pair_K + i;
   if (cv) {
-    // the correction's bits and W(e) = sum of lambda_j over e_j = 1, ascending j
-    uint32_t* bits = a.pbits + rec * a.bnd.nw;
-    float W = 0.0f;
-    for (int w = 0; w < nw; ++w) {
-      const int v = 32 * w + lane;
-      const uint32_t word = __ballot_sync(kFull, v < n && dec8[v] != 0);
-      if (lane == 0) bits[w] = word;
-      uint32_t x = word;
-      while (x) {
-        const int bpos = __ffs(x) - 1;
-        W = __fadd_rn(W, __ldg(t.lam + 32 * w + bpos));
-        x &= x - 1;
-      }
-    }
+    // the correction's bits and W(e)
+    uint32_t* bits = reinterpret_cast<uint32_t*>(base + t.off_cand);
+    const float W = member_bits(t, i, base, st, bits, lane);
+    for (int w = lane; w < nw; w += 32) a.pbits[rec * a.bnd.nw + w] = bits[w];
     if (lane == 0) a.pW[rec] = W;
     if (a.want_soft)
       for (int v = lane; v < n; v += 32) a.ppost[rec * a.bnd.n + v] = lpost[v];
     __threadfence();
     __syncwarp();
     if (lane == 0) *reinterpret_cast<volatile int*>(conv + i) = cv;
-  } else if (ran == T) {
+  } else if (R.ran == T) {
     llr_term_add(lpost, a.pterms + rec * a.bnd.n, n, true, lane);
   }
   __syncwarp();
@@ -652,8 +731,8 @@ __device__ __forceinline__ void decode_pair(const BpArgs& a, const Tables& t, ui
 // MIXED: the shots of the launch name their problems (dem_of_shot); the problems' descriptors are
 // copied to shared memory after the warps' regions. Otherwise every shot decodes a.one, which the
 // kernel reads from its parameter space.
-template <typename MT, int DP, int RPC, bool MIXED>
-__global__ void __launch_bounds__(kBpWarpsPerCta * 32, MinBlocks<MT>::value) k_bp(const BpArgs a) {
+template <typename MT, int DP, int NCH, bool MIXED>
+__global__ void __launch_bounds__(kBpWarpsPerCta * 32, MinBlocks<MT, DP>::value) k_bp(const __grid_constant__ BpArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
   const int wcta = threadIdx.x >> 5;
@@ -666,10 +745,12 @@ __global__ void __launch_bounds__(kBpWarpsPerCta * 32, MinBlocks<MT>::value) k_b
     for (int q = threadIdx.x; q < words; q += blockDim.x) dst[q] = __ldg(src + q);
     __syncthreads();
   }
-  unsigned char* base = smem + (size_t)wcta * a.bnd.warp_smem;
+  const int smem_off = wcta * a.bnd.warp_smem;
+  unsigned char* base = smem + smem_off;
   float* acc = a.scratch + gw * a.scratch_pitch;  // n floats: LLR average accumulator
   float* lpost = acc + a.bnd.n;                    // n floats: the member's posterior when needed
-  float* cand_post = lpost + a.bnd.n;              // M * n floats (only with want_soft)
+  uint32_t* gst = reinterpret_cast<uint32_t*>(lpost + a.bnd.n);   // n words with bnd.global_st: decision words
+  float* cand_post = lpost + (a.bnd.global_st ? 2 : 1) * (size_t)a.bnd.n;   // M * n floats (only with want_soft)
   unsigned long long my_iters = 0, my_shots = 0, my_fail = 0;
 
   if (a.pair_mode) {
@@ -698,9 +779,9 @@ __global__ void __launch_bounds__(kBpWarpsPerCta * 32, MinBlocks<MT>::value) k_b
           continue;
         }
         if (sdem[di].engine != VIBE_ENGINE_IMAGE) continue;   // left to the summary engine
-        decode_pair<MT, DP, RPC, true>(a, sdem[di], shot, (int)shot, i, base, lpost, lane, my_iters, my_shots, my_fail);
+        decode_pair<MT, DP, NCH>(a, sdem[di], shot, (int)shot, i, base, smem_off, lpost, gst, lane, my_iters, my_shots, my_fail);
       } else {
-        decode_pair<MT, DP, RPC, false>(a, a.one, shot, (int)shot, i, base, lpost, lane, my_iters, my_shots, my_fail);
+        decode_pair<MT, DP, NCH>(a, a.one, shot, (int)shot, i, base, smem_off, lpost, gst, lane, my_iters, my_shots, my_fail);
       }
     }
   }
@@ -730,10 +811,10 @@ __global__ void __launch_bounds__(kBpWarpsPerCta * 32, MinBlocks<MT>::value) k_b
         continue;
       }
       if (sdem[di].engine != VIBE_ENGINE_IMAGE) continue;   // left to the summary engine
-      decode_shot<MT, DP, RPC, true>(a, sdem[di], shot, base, acc, lpost, cand_post, lane, my_iters, my_shots,
+      decode_shot<MT, DP, NCH>(a, sdem[di], shot, base, smem_off, acc, lpost, cand_post, gst, lane, my_iters, my_shots,
                                      my_fail);
     } else {
-      decode_shot<MT, DP, RPC, false>(a, a.one, shot, base, acc, lpost, cand_post, lane, my_iters, my_shots,
+      decode_shot<MT, DP, NCH>(a, a.one, shot, base, smem_off, acc, lpost, cand_post, gst, lane, my_iters, my_shots,
                                       my_fail);
     }
   }
@@ -744,31 +825,35 @@ __global__ void __launch_bounds__(kBpWarpsPerCta * 32, MinBlocks<MT>::value) k_b
   }
 }
 
-// RPC: row pitch in 8-slot chunks when every problem of the launch has RP 8, 16 or 32, else 0.
-inline int rpc_of(const Bounds& b) { return (b.RP == 8 || b.RP == 16 || b.RP == 32) ? b.RP / 8 : 0; }
+// 16-byte chunks of a row when every problem of the launch has the same 1 to 4, else 0 (read per problem).
+inline int nch_of(const Bounds& b, int spc) {
+  const int c = b.RP / spc;
+  return b.RP > 0 && c <= 4 ? c : 0;
+}
 
 inline size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-template <typename MT, int DP, int RPC, bool MIXED>
+template <typename MT, int DP, int NCH, bool MIXED>
 cudaError_t launch_one(const BpArgs& a, int grid, size_t smem, cudaStream_t s) {
-  cudaError_t err = ensure_dyn_smem<k_bp<MT, DP, RPC, MIXED>>(smem);
+  cudaError_t err = ensure_dyn_smem<k_bp<MT, DP, NCH, MIXED>>(smem);
   if (err != cudaSuccess) return err;
-  k_bp<MT, DP, RPC, MIXED><<<grid, kBpWarpsPerCta * 32, smem, s>>>(a);
+  k_bp<MT, DP, NCH, MIXED><<<grid, kBpWarpsPerCta * 32, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-template <typename MT, int DP, int RPC, bool MIXED>
+template <typename MT, int DP, int NCH, bool MIXED>
 cudaError_t occupancy_one(size_t smem, int* out) {
-  cudaError_t err = ensure_dyn_smem<k_bp<MT, DP, RPC, MIXED>>(smem);
+  cudaError_t err = ensure_dyn_smem<k_bp<MT, DP, NCH, MIXED>>(smem);
   if (err != cudaSuccess) return err;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bp<MT, DP, RPC, MIXED>, kBpWarpsPerCta * 32, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bp<MT, DP, NCH, MIXED>, kBpWarpsPerCta * 32, smem);
 }
 
 template <typename Fn>
-cudaError_t by_rpc(int rpc, Fn&& f) {
-  switch (rpc) {
+cudaError_t by_nch(int nch, Fn&& f) {
+  switch (nch) {
     case 1: return f(std::integral_constant<int, 1>{});
     case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
     case 4: return f(std::integral_constant<int, 4>{});
     default: return f(std::integral_constant<int, 0>{});
   }
@@ -785,15 +870,15 @@ cudaError_t by_dp(int DP, Fn&& f) {
   }
 }
 
-// Mixed launches use the generic row scan (RPC 0) only, which keeps the number of instantiations down.
+// Mixed launches use the generic row scan (NCH 0) only, which keeps the number of instantiations down.
 template <typename MT>
 cudaError_t launch_mt(const BpArgs& a, int grid, cudaStream_t s) {
   const bool mixed = a.dem_of_shot != nullptr;
   const size_t smem = bp_cta_smem_bytes(a.bnd, mixed ? a.ndem : 0);
   return by_dp(a.bnd.DP, [&](auto dp) {
     if (mixed) return launch_one<MT, decltype(dp)::value, 0, true>(a, grid, smem, s);
-    return by_rpc(rpc_of(a.bnd), [&](auto rpc) {
-      return launch_one<MT, decltype(dp)::value, decltype(rpc)::value, false>(a, grid, smem, s);
+    return by_nch(nch_of(a.bnd, Msg<MT>::kSpc), [&](auto nch) {
+      return launch_one<MT, decltype(dp)::value, decltype(nch)::value, false>(a, grid, smem, s);
     });
   });
 }
@@ -803,8 +888,8 @@ cudaError_t occupancy_mt(const Bounds& b, int ndem, int* out) {
   const size_t smem = bp_cta_smem_bytes(b, ndem);
   return by_dp(b.DP, [&](auto dp) {
     if (ndem > 0) return occupancy_one<MT, decltype(dp)::value, 0, true>(smem, out);
-    return by_rpc(rpc_of(b), [&](auto rpc) {
-      return occupancy_one<MT, decltype(dp)::value, decltype(rpc)::value, false>(smem, out);
+    return by_nch(nch_of(b, Msg<MT>::kSpc), [&](auto nch) {
+      return occupancy_one<MT, decltype(dp)::value, decltype(nch)::value, false>(smem, out);
     });
   });
 }
@@ -812,16 +897,22 @@ cudaError_t occupancy_mt(const Bounds& b, int ndem, int* out) {
 }  // namespace
 
 size_t bp_warp_smem_bytes(Tables* t, int msg_fp16) {
+  const size_t words = 4 * (size_t)t->mw, dec = ((size_t)t->n + 3) / 4 * 4, steps = 4 * (size_t)t->nstep;
+  const bool bytes = t->n_flood > 0 || t->n_layered > 0;   // these members keep a byte per decision
   size_t o = 0;
   t->off_msg = (int)o;
   o = align16(o + (size_t)t->m * t->RP * (msg_fp16 ? 2 : 4));
-  t->off_dec = (int)o;
-  o = align16(o + ((size_t)t->n + 3) / 4 * 4);
-  const size_t m4 = ((size_t)t->m + 3) / 4 * 4;
   t->off_s = (int)o;
-  o = align16(o + m4);
+  o = align16(o + words);
   t->off_par = (int)o;
-  o = align16(o + m4);
+  o = align16(o + words);
+  // decision bytes and step words share their place: a member uses one of them. The words of a graph of
+  // long chains (few columns per step) that would take more than n + 2m bytes go to global scratch.
+  t->off_dec = t->off_st = (int)o;
+  size_t d = bytes ? dec : 0;
+  if (steps <= std::max<size_t>(d, (size_t)t->n + 2 * (size_t)t->m)) d = std::max(d, steps);
+  else t->off_st = -1;
+  o = align16(o + d);
   t->off_cand = (int)o;
   o = align16(o + (size_t)t->M * t->nw * 4);
   t->off_cv = -1;

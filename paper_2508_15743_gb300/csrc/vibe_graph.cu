@@ -5,8 +5,8 @@
 // edge's column, +inf padding), and for every ensemble member the dependency wavefronts of its
 // serial schedule: level(v) = 1 + max{level(u) : u before v in the member's order, u and v share a
 // check}. Columns of one level touch disjoint checks, so updating a level in any order gives the
-// same floats as the serial order of Algorithm 1 (serial branch). For the summary engine each member's
-// order is also packed into steps of 32 edges (k_steps).
+// same floats as the serial order of Algorithm 1 (serial branch). The kernels run each member's
+// order packed into steps of 32 edges (k_steps).
 #include "vibe_internal.cuh"
 
 namespace vibe {
@@ -282,7 +282,8 @@ __global__ void k_step_offsets(const uint32_t* __restrict__ tmp, int tmp_pitch, 
 __global__ void k_step_fill(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ off, int off_pitch, int n,
                             long long total, int E, int SP, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colptr,
                             const uint32_t* __restrict__ cpos, const float* __restrict__ lam, uint2* __restrict__ xrec,
-                            uint32_t* __restrict__ xlnk, uint32_t* __restrict__ xcolid, uint32_t* __restrict__ xrmap) {
+                            uint32_t* __restrict__ xlnk, uint32_t* __restrict__ xcolid, uint32_t* __restrict__ xrmap,
+                            bool wide) {
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
        q += (long long)gridDim.x * blockDim.x) {
     const long long i = q / n;
@@ -298,12 +299,13 @@ __global__ void k_step_fill(const uint32_t* __restrict__ slot, const uint32_t* _
     }
     for (int k = 0; k < d; ++k) {
       const uint32_t x = cpos[b + k];
-      const uint32_t others = ((2u << (d - 1)) - 1u) & ~(1u << k);   // the summary engine has d <= 16
+      const uint32_t others = ((2u << (d - 1)) - 1u) & ~(1u << k);
+      const uint32_t links = wide ? ((uint32_t)k << 5) | ((uint32_t)(d - 1) << 10)
+                                  : (others << 5) | (((sl & 31u) + (uint32_t)(d - 1)) << kLnkLastLane);
       xrec[i * SP + o + k] = make_uint2(((x >> 8) << 18) | (x & 0xffu), lv);
-      xlnk[i * SP + o + k] = (sl & 31u) | (others << 5) | (((sl & 31u) + (uint32_t)(d - 1)) << kLnkLastLane) |
-                             (k == d - 1 ? kLnkLast : 0u) | kLnkEdge;
+      xlnk[i * SP + o + k] = (sl & 31u) | links | (k == d - 1 ? kLnkLast : 0u) | kLnkEdge;
       xcolid[i * SP + o + k] = v;
-      xrmap[(size_t)i * E + rowptr[x >> 8] + (x & 0xffu)] = o + (uint32_t)k;
+      if (xrmap) xrmap[(size_t)i * E + rowptr[x >> 8] + (x & 0xffu)] = o + (uint32_t)k;
     }
   }
 }
@@ -454,7 +456,7 @@ cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32
 
 size_t step_scratch_ints(int n, int K) { return (size_t)K * (2 * (size_t)n + 1) + ((size_t)K * n + 3) / 4; }
 
-cudaError_t fill_steps(int n, int E, int SP, int K, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
+cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
                        const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
                        uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,
                        cudaStream_t s) {
@@ -463,7 +465,7 @@ cudaError_t fill_steps(int n, int E, int SP, int K, int pitch, const int32_t* d_
   const int off_pitch = n + 1;
   k_step_offsets<<<grid_for((long long)K * pitch, 256), 256, 0, s>>>(off, off_pitch, d_nstep, K, pitch, d_soff);
   k_step_fill<<<grid_for((long long)K * n, 256), 256, 0, s>>>(slot, off, off_pitch, n, (long long)K * n, E, SP, d_rowptr,
-                                                              d_colptr, d_cpos, d_lam, d_xrec, d_xlnk, d_xcolid, d_xrmap);
+                                                              d_colptr, d_cpos, d_lam, d_xrec, d_xlnk, d_xcolid, d_xrmap, DP > 16);
   return cudaGetLastError();
 }
 

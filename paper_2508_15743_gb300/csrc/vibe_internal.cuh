@@ -21,7 +21,8 @@ constexpr int kMaxDevices = 64;
 constexpr uint32_t kFull = 0xffffffffu;
 constexpr uint32_t kInfBits = 0x7f800000u;
 // Edge links (Tables::xlnk): bits 0-4 the lane of the column's first edge, bit 5 + j set for the column's
-// j-th edge except the record's own, then the lane of its last edge; 0 for a column without checks.
+// j-th edge except the record's own, then the lane of its last edge; 0 for a column without checks. Where
+// columns have more than 16 checks (DP 32, image engine only): first lane | k << 5 | degree - 1 << 10.
 constexpr int kLnkLastLane = 21;
 constexpr uint32_t kLnkLast = 1u << 30, kLnkEdge = 1u << 31;   // the record is the last edge's; it has a check
 constexpr int kStepPad = 66;            // step offsets kept past a member's last step (the kernels look ahead)
@@ -56,6 +57,7 @@ struct Tables {
   int nlayer;    // check layers of the layered schedule (0 unless n_layered > 0)
   float alpha;   // the shared factor (alpha_m holds the one each member uses)
   int off_msg, off_dec, off_s, off_par, off_cand, warp_smem;   // image engine: per-warp shared memory, bytes
+  int off_st;    // image engine: the steps' decision words; -1: in the warp's global scratch
   int off_cv;    // image engine: float image of check-to-variable messages (layered members, flooding
                  // members with FP16 storage), laid out like the message image; -1 when unused
   int engine;    // VIBE_ENGINE_IMAGE or VIBE_ENGINE_SUMMARY
@@ -85,7 +87,7 @@ struct Tables {
   const int32_t* layer_chk;   // m checks grouped by layer, ascending within a layer
   const int32_t* layer_vptr;  // nlayer+1 offsets into layer_var
   const int32_t* layer_var;   // E: per layer, the columns of its checks in layer_chk order (each at most once)
-  // summary engine: the steps of each member's sweep (k_steps). Step s of member i holds the edge slots
+  // the steps of each member's sweep (k_steps). Step s of member i holds the edge slots
   // soff[i][s] .. soff[i][s+1] (at most 32, one lane each; the checks of a step are distinct), the edges
   // of a column in consecutive slots.
   // xrec[i][slot] = (check << 18 | position of the edge in the check's CSR row, prior LLR), xlnk its links
@@ -107,6 +109,7 @@ struct Bounds {
   int x_warp_smem;    // summary-engine shared memory per warp: the step window and the largest problem's
                       // check summaries (0 if no problem uses that engine)
   long long x_warp_scratch;   // largest summary-engine global scratch per warp, bytes
+  int global_st;   // some image-engine problem keeps its step words in global scratch
   int engines;     // bit 0: some problem uses the image engine, bit 1: the summary engine
   int XD;          // largest summary-engine column-degree bound
   int K;           // largest ensemble size
@@ -347,6 +350,12 @@ __device__ __forceinline__ uint4 lds128(uint32_t a) {
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) {
   asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
+__device__ __forceinline__ void sts16(uint32_t a, uint32_t v) {
+  asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((unsigned short)v) : "memory");
+}
+__device__ __forceinline__ void red_xor_shared(uint32_t a, uint32_t v) {
+  asm volatile("red.shared.xor.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
 __device__ __forceinline__ void sts64(uint32_t a, uint2 v) {
   asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(v.x), "r"(v.y) : "memory");
 }
@@ -401,7 +410,7 @@ cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m
 size_t step_scratch_ints(int n, int K);
 cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
                         int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s);
-cudaError_t fill_steps(int n, int E, int SP, int K, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
+cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
                        const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
                        uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,
                        cudaStream_t s);

@@ -73,13 +73,13 @@ extern "C" int vibe_decode_noalloc(vibe_handle* h, const uint32_t* d_syndromes, 
   const vibe::Tables& t = v.t;
   if (t.engine != VIBE_ENGINE_IMAGE)
     return vibe::set_error(VIBE_ERR_UNSUPPORTED, "the static workspace serves warp-engine handles only");
-  // Fixed part: counters, two n-float rows per BP warp (LLR accumulator, posterior), one row set per
-  // LSD CTA. The LSD CTAs are capped at one per SM so the fixed part stays small; the rest holds the
+  // Fixed part: counters, two n-float rows per BP warp (LLR accumulator, posterior; a third where the
+  // step words do not fit in shared memory), one row set per LSD CTA. The LSD CTAs are capped at one per SM so the fixed part stays small; the rest holds the
   // LSD hand-off queue.
   const int bp_grid = v.bp_grid;
   const int lsd_grid = v.lsd_grid < v.num_sms ? v.lsd_grid : v.num_sms;
   const size_t ctrl_b = 256;
-  const size_t bp_b = up256((size_t)bp_grid * vibe::kBpWarpsPerCta * 2 * (size_t)t.n * sizeof(float));
+  const size_t bp_b = up256((size_t)bp_grid * vibe::kBpWarpsPerCta * (2 + v.bnd.global_st) * (size_t)t.n * sizeof(float));
   const size_t lsd_b = up256((size_t)lsd_grid * (size_t)vibe::lsd_scratch_words(v.bnd, vibe::kLsdThreads) * sizeof(uint32_t));
   const size_t fixed = ctrl_b + bp_b + lsd_b;
   const size_t per_shot = (size_t)t.n * sizeof(float) + sizeof(uint32_t);
@@ -113,7 +113,7 @@ extern "C" int vibe_decode_noalloc(vibe_handle* h, const uint32_t* d_syndromes, 
   a.soft = nullptr; a.soft_stride = t.n; a.obs = nullptr; a.counters = nullptr;
   a.next_shot = ctrl; a.lsd_count = ctrl + 1; a.lsd_shots = lsd_shots; a.lsd_soft = lsd_soft;
   a.scratch = bp_scratch;
-  a.scratch_pitch = 2LL * t.n;
+  a.scratch_pitch = (2LL + v.bnd.global_st) * t.n;
   const long long need_ctas = (B + vibe::kBpWarpsPerCta - 1) / vibe::kBpWarpsPerCta;
   const int grid = (int)(need_ctas < bp_grid ? need_ctas : bp_grid);
   if ((e = vibe::launch_bp(a, v.msg_fp16, grid, s)) != cudaSuccess) return vibe::set_error(VIBE_ERR_CUDA, cudaGetErrorString(e));

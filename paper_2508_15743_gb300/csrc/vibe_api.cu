@@ -370,7 +370,8 @@ Bounds bounds_over(const Tables* ts, int count) {
   for (int i = 0; i < count; ++i) {
     const Tables& t = ts[i];
     b.m = std::max(b.m, t.m); b.n = std::max(b.n, t.n); b.W = std::max(b.W, t.W); b.nw = std::max(b.nw, t.nw);
-    b.kw = std::max(b.kw, t.kw); b.M = std::max(b.M, t.M); b.DP = std::max(b.DP, t.DP); b.K = std::max(b.K, t.K);
+    b.kw = std::max(b.kw, t.kw); b.M = std::max(b.M, t.M); b.DP = std::max(b.DP, t.DP);
+    b.CD = std::max(b.CD, t.CD); b.K = std::max(b.K, t.K);
     b.lsd_order = std::max(b.lsd_order, t.lsd_order);
     if (t.engine == VIBE_ENGINE_IMAGE) {
       b.engines |= 1;
@@ -636,6 +637,7 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   const int spc = p->msg_fp16 ? 8 : 4;   // slots per 16-byte chunk of a row
   t.RP = (maxrow + spc - 1) / spc * spc;
   t.DP = maxcol <= 4 ? 4 : maxcol <= 8 ? 8 : maxcol <= 16 ? 16 : 32;
+  t.CD = maxcol <= 3 ? 3 : t.DP;
   t.mw = (m + 31) / 32; t.nw = (n + 31) / 32; t.kw = (k + 31) / 32; t.W = t.mw;
   t.T = p->max_iter; t.M = p->M; t.lsd_order = p->lsd_order; t.alpha = p->alpha; t.n_flood = p->n_flood;
   t.n_layered = p->n_layered;
@@ -713,6 +715,10 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     VIBE_TRY(dalloc(&h->xlnk, (size_t)K * t.SP + 4), "tables");
     VIBE_TRY(dalloc(&h->xcolid, (size_t)K * t.SP), "tables");
     if (t.XD > 0) VIBE_TRY(dalloc(&h->xrmap, (size_t)K * E), "tables");
+    // the lanes' order pays where the image engine runs (xcolid serves as its scratch: it is filled next)
+    if (msg_bytes <= 100 * 1024)
+      VIBE_TRY(vibe::order_steps(n, t.SP, K, t.nstep, h->colptr, h->cpos, h->stepcnt, scratch, h->xcolid, s),
+               "step builder");
     VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.DP, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
                               h->soff, h->xrec, h->xlnk, h->xcolid, h->xrmap, s),
              "step builder");

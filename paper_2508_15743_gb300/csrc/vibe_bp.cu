@@ -50,22 +50,27 @@ struct Msg<float> {
   static constexpr int kBytes = 4;
   static constexpr int kSpc = 4;   // slots per 16-byte chunk of a row
   static constexpr uint32_t kInf = kInfBits;
+  static constexpr bool kDrop = true;   // the scan leaves the own slot out itself (rows of known length)
   __device__ __forceinline__ static void store(uint32_t a, uint32_t b) { sts32(a, b); }
   __device__ __forceinline__ static uint32_t round(float x) { return __float_as_uint(x); }
   __device__ __forceinline__ static void store(float* p, float x) { *p = x; }
   __device__ __forceinline__ static float value(float x) { return x; }
   template <int NCH>
-  __device__ __forceinline__ static float scan(uint32_t row, int nch) {
+  __device__ __forceinline__ static float scan(uint32_t row, int nch, uint32_t pos) {
     float v = __int_as_float(0x7f800000);
-    auto chunk = [&](uint32_t a) {
+    auto chunk = [&](uint32_t a, uint32_t drop) {
       const uint4 q = lds128(a);
-      v = minx(v, minx(minx(__uint_as_float(q.x), __uint_as_float(q.y)), minx(__uint_as_float(q.z), __uint_as_float(q.w))));
+      const float inf = __uint_as_float(kInfBits);
+      const float x = (drop & 1u) ? inf : __uint_as_float(q.x), y = (drop & 2u) ? inf : __uint_as_float(q.y);
+      const float z = (drop & 4u) ? inf : __uint_as_float(q.z), w = (drop & 8u) ? inf : __uint_as_float(q.w);
+      v = minx(v, minx(minx(x, y), minx(z, w)));
     };
     if (NCH) {
+      const uint32_t own = 1u << pos;
 #pragma unroll
-      for (int i = 0; i < NCH; ++i) chunk(row + 16 * i);
+      for (int i = 0; i < NCH; ++i) chunk(row + 16 * i, own >> (4 * i));
     } else {
-      for (int i = 0; i < nch; ++i) chunk(row + 16 * i);
+      for (int i = 0; i < nch; ++i) chunk(row + 16 * i, 0u);
     }
     return v;
   }
@@ -76,6 +81,7 @@ struct Msg<__half> {
   static constexpr int kBytes = 2;
   static constexpr int kSpc = 8;
   static constexpr uint32_t kInf = 0x7c00u;
+  static constexpr bool kDrop = false;
   __device__ __forceinline__ static void store(uint32_t a, uint32_t b) { sts16(a, b); }
   __device__ __forceinline__ static uint32_t round(float x) {   // -0 as +0
     const uint32_t h = (uint32_t)__half_as_ushort(__float2half_rn(x));
@@ -86,7 +92,7 @@ struct Msg<__half> {
   }
   __device__ __forceinline__ static float value(__half x) { return __half2float(x); }
   template <int NCH>
-  __device__ __forceinline__ static float scan(uint32_t row, int nch) {
+  __device__ __forceinline__ static float scan(uint32_t row, int nch, uint32_t) {
     uint32_t v = 0x7c007c00u;
     auto chunk = [&](uint32_t a) {
       const uint4 q = lds128(a);
@@ -307,17 +313,21 @@ struct ImageRun {
 constexpr int kRecSteps = 2;   // steps fetched together, one group ahead
 
 // One serial sweep of a member over its ns steps on the message image at shared address msgs. A lane
-// holds one edge of a step (its check is no other lane's): it writes +inf into its own slot of the row
-// -- a magnitude that never wins a minimum, sign bit 0 -- so that the row scan gives the minimum and sign
-// product over the other slots exactly, gets the column's other messages from their lanes, forms its
-// exclusion sum in the order of Algorithm 1 and stores the new message in its slot. Decisions are one
+// holds one edge of a step (its check is no other lane's): it scans its row with +inf -- a magnitude that
+// never wins a minimum, sign bit 0 -- in the place of its own slot, which gives the minimum and sign
+// product over the other slots exactly (FP32 rows of up to four chunks put it in while scanning, which
+// saves the 3.5 wavefronts of a scattered store; FP16 rows, where the halves cost more instructions than
+// that, and longer rows have it written to the slot first), gets
+// the column's other messages from their lanes, forms its exclusion sum in the order of Algorithm 1 and
+// stores the new message in its slot. Decisions are one
 // word per step (on the lane of the column's last edge); check parities are flipped, and the word
 // stored, only when one changes.
-// What bounds it: shared-memory wavefronts (94 % of their peak). The lanes' rows are random, so a 16-byte
-// row load of 32 lanes takes ~9 wavefronts instead of 4. With one lane per column a sweep of the d=9
-// phenomenological problem took 42 chunks of 187 instructions and 2800 wavefronts; its 62 steps take 90
-// instructions each. Measured, 32768 shots of it (K=16, T=30): 96.7 -> 73.1 ms with FP32 messages, 78.1 ->
-// 51.2 ms with FP16; the 4.8.8 code, whose rows of 10 now take three chunks instead of four, 40 -> 16 ms.
+// What bounds it: shared-memory wavefronts (94 % of their peak). The lanes' rows are random; the order of a
+// step's columns (k_step_order) brings a 16-byte row load of 32 lanes from ~9.5 wavefronts to ~8 (ideal 4).
+// With one lane per column a sweep of the d=9 phenomenological problem took 42 chunks of 187 instructions
+// and 2800 wavefronts; its 62 steps take 90 instructions each. Measured, 32768 shots of it (K=16, T=30):
+// 96.7 -> 61.7 ms with FP32 messages (73.1 before the order and without the dropped slot), 78.1 -> 48.0 ms with
+// FP16; the 4.8.8 code, whose rows of 10 now take three chunks instead of four, 40 -> 13 ms.
 // NCH: 16-byte chunks of a row (0: from the tables). par32 holds the check parities.
 template <typename MT, int DP, int NCH, bool LP>
 __device__ __forceinline__ void step_sweep(const Tables& t, const uint32_t* soff, const int ns, const size_t first,
@@ -365,9 +375,9 @@ __device__ __forceinline__ void step_sweep(const Tables& t, const uint32_t* soff
       if (NCH == 0 || NCH == 2 || NCH == 4 || NCH == 8) pos ^= ((c >> swz_shift) & swz_mask) * (uint32_t)Msg<MT>::kSpc;
       const uint32_t own = row + pos * (uint32_t)Msg<MT>::kBytes;
       const bool act = (int)ln[u] < 0;
-      if (act) Msg<MT>::store(own, Msg<MT>::kInf);
+      if (!(Msg<MT>::kDrop && NCH) && act) Msg<MT>::store(own, Msg<MT>::kInf);
       const uint32_t sw = lds32(s32 + ((c >> 5) << 2));
-      const float mn = Msg<MT>::template scan<NCH>(row, nch);
+      const float mn = Msg<MT>::template scan<NCH>(row, nch, pos);
       const uint32_t mcv = __float_as_uint(__fmul_rn(alpha, mn)) ^ (__funnelshift_l(0u, sw, ~c) & 0x80000000u);
       float acc = __uint_as_float(r[u].y);
       // links of columns of more than 16 checks: first lane | k << 5 | degree - 1 << 10
@@ -862,6 +872,7 @@ cudaError_t by_nch(int nch, Fn&& f) {
 template <typename Fn>
 cudaError_t by_dp(int DP, Fn&& f) {
   switch (DP) {
+    case 3: return f(std::integral_constant<int, 3>{});
     case 4: return f(std::integral_constant<int, 4>{});
     case 8: return f(std::integral_constant<int, 8>{});
     case 16: return f(std::integral_constant<int, 16>{});
@@ -875,7 +886,7 @@ template <typename MT>
 cudaError_t launch_mt(const BpArgs& a, int grid, cudaStream_t s) {
   const bool mixed = a.dem_of_shot != nullptr;
   const size_t smem = bp_cta_smem_bytes(a.bnd, mixed ? a.ndem : 0);
-  return by_dp(a.bnd.DP, [&](auto dp) {
+  return by_dp(a.bnd.CD, [&](auto dp) {
     if (mixed) return launch_one<MT, decltype(dp)::value, 0, true>(a, grid, smem, s);
     return by_nch(nch_of(a.bnd, Msg<MT>::kSpc), [&](auto nch) {
       return launch_one<MT, decltype(dp)::value, decltype(nch)::value, false>(a, grid, smem, s);
@@ -886,7 +897,7 @@ cudaError_t launch_mt(const BpArgs& a, int grid, cudaStream_t s) {
 template <typename MT>
 cudaError_t occupancy_mt(const Bounds& b, int ndem, int* out) {
   const size_t smem = bp_cta_smem_bytes(b, ndem);
-  return by_dp(b.DP, [&](auto dp) {
+  return by_dp(b.CD, [&](auto dp) {
     if (ndem > 0) return occupancy_one<MT, decltype(dp)::value, 0, true>(smem, out);
     return by_nch(nch_of(b, Msg<MT>::kSpc), [&](auto nch) {
       return occupancy_one<MT, decltype(dp)::value, decltype(nch)::value, false>(smem, out);

@@ -265,6 +265,74 @@ __global__ void k_steps(const uint32_t* __restrict__ perm, int n, int m, const i
   if (lane == 0) nstep[blockIdx.x] = (int32_t)ns;
 }
 
+// Column of each edge slot (only the slots of first edges are written, and read).
+__global__ void k_step_columns(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ off, int off_pitch, int n,
+                               long long total, int SP, uint32_t* __restrict__ at) {
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < total;
+       q += (long long)gridDim.x * blockDim.x) {
+    const long long i = q / n;
+    const uint32_t sl = slot[q];
+    at[i * SP + off[i * off_pitch + (sl >> 5)] + (sl & 31u)] = (uint32_t)(q % n);
+  }
+}
+
+// Order of a step's columns over its lanes (one warp per step). A 16-byte row load is served in four
+// phases of eight lanes, and rows fall on the eight bank groups by their index mod 8 (row_position): a
+// phase takes as many wavefronts as its most frequent residue. The columns are placed one after another,
+// each time the one that adds least to its phases (ties: more checks first). On the d=9 phenomenological
+// problem a row load of a step takes 8.0 wavefronts so ordered instead of 9.5 (ideal 4).
+// cnt packs the current phase's counts, four bits per residue.
+__global__ void k_step_order(const uint32_t* __restrict__ off, int off_pitch, const int32_t* __restrict__ nstep, int K,
+                             int n, int SP, int per_member, const uint32_t* __restrict__ at,
+                             const int32_t* __restrict__ colptr, const uint32_t* __restrict__ cpos,
+                             uint32_t* __restrict__ slot) {
+  const int lane = threadIdx.x & 31;
+  const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+  const int i = (int)(w / per_member), s = (int)(w % per_member);
+  if (i >= K || s >= nstep[i]) return;
+  const uint32_t b = off[(size_t)i * off_pitch + s];
+  const int used = (int)(off[(size_t)i * off_pitch + s + 1] - b);
+  slot += (size_t)i * n;
+  // the step's columns, one per lane
+  uint32_t v = 0u;
+  int d = 0, cols = 0;
+  for (int p = 0; p < used;) {
+    const uint32_t u = at[(size_t)i * SP + b + p];
+    const int du = colptr[u + 1] - colptr[u];
+    if (lane == cols) { v = u; d = du; }
+    ++cols;
+    p += max(du, 1);
+  }
+  const int e0 = lane < cols ? colptr[v] : 0;
+  bool left = lane < cols;
+  int pos = 0;
+  uint32_t cnt = 0u, top = 0u;   // the current phase's counts and their maximum
+  for (int k = 0; k < cols; ++k) {
+    uint32_t cost = 0u, c = cnt, t = top, t0 = top;
+    if (left) {
+      for (int j = 0; j < d; ++j) {
+        if (((pos + j) & 7) == 0) { cost += t - t0; c = 0u; t = t0 = 0u; }
+        const uint32_t r = 4u * ((cpos[e0 + j] >> 8) & 7u);
+        c += 1u << r;
+        t = max(t, (c >> r) & 15u);
+      }
+      cost += t - t0;
+    }
+    // least added cost, then most checks, then the lowest lane
+    const uint32_t key = left ? (cost << 16) | ((uint32_t)(32 - d) << 8) | (uint32_t)lane : 0xffffffffu;
+    const int pick = (int)(__reduce_min_sync(kFull, key) & 31u);
+    if (lane == pick) {
+      slot[v] = ((uint32_t)s << 5) | (uint32_t)pos;
+      left = false;
+    }
+    const int dp = max(__shfl_sync(kFull, d, pick), 1);
+    cnt = __shfl_sync(kFull, c, pick);
+    top = __shfl_sync(kFull, t, pick);
+    pos += dp;
+    if ((pos & 7) == 0) cnt = top = 0u;
+  }
+}
+
 // The step offsets with the common pitch of the resident table; the entries past a member's last step
 // repeat its total.
 __global__ void k_step_offsets(const uint32_t* __restrict__ tmp, int tmp_pitch, const int32_t* __restrict__ nstep, int K,
@@ -455,6 +523,16 @@ cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32
 }
 
 size_t step_scratch_ints(int n, int K) { return (size_t)K * (2 * (size_t)n + 1) + ((size_t)K * n + 3) / 4; }
+
+cudaError_t order_steps(int n, int SP, int K, int nstep, const int32_t* d_colptr, const uint32_t* d_cpos,
+                        const int32_t* d_nstep, int32_t* d_scratch, uint32_t* d_tmp, cudaStream_t s) {
+  uint32_t* slot = reinterpret_cast<uint32_t*>(d_scratch);
+  const uint32_t* off = slot + (size_t)K * n;
+  k_step_columns<<<grid_for((long long)K * n, 256), 256, 0, s>>>(slot, off, n + 1, n, (long long)K * n, SP, d_tmp);
+  const long long blocks = ((long long)K * nstep + 3) / 4;   // four warps each
+  k_step_order<<<(unsigned)blocks, 128, 0, s>>>(off, n + 1, d_nstep, K, n, SP, nstep, d_tmp, d_colptr, d_cpos, slot);
+  return cudaGetLastError();
+}
 
 cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
                        const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,

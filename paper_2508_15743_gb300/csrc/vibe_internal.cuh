@@ -49,6 +49,7 @@ struct Tables {
   int m, n, k, E, K;
   int RP;        // row pitch of the padded message image: max row degree rounded up to 8
   int DP;        // column pitch of csc_ent: max column degree rounded up to 4 (4, 8, 16 or 32)
+  int CD;        // column-degree bound of the image engine: 3, or DP
   int mw, nw, kw;
   int W;         // words of a bit vector over the checks: ceil(m/32)
   int T, M, lsd_order;
@@ -102,7 +103,7 @@ struct Tables {
 
 // Sizes that bound every problem of a launch (shared-memory layouts, strides, scratch pitches).
 struct Bounds {
-  int m, n, W, nw, kw, M, DP;
+  int m, n, W, nw, kw, M, DP, CD;
   int RP;          // common row pitch if all problems share it, else 0
   int warp_smem;   // largest BP per-warp layout
   int lsd_order;   // largest LSD order
@@ -410,6 +411,10 @@ cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m
 size_t step_scratch_ints(int n, int K);
 cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
                         int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s);
+// Orders the columns of each step over its lanes against bank conflicts (slot and off in the scratch;
+// tmp: K * SP words).
+cudaError_t order_steps(int n, int SP, int K, int nstep, const int32_t* d_colptr, const uint32_t* d_cpos,
+                        const int32_t* d_nstep, int32_t* d_scratch, uint32_t* d_tmp, cudaStream_t s);
 cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
                        const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
                        uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,

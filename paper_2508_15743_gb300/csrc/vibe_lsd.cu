@@ -5,13 +5,23 @@
 // reliability order (the averaged soft value ascending, ties to the lower index) together with all
 // checks of that column; clusters that come to share a check merge (union-find, root = smallest
 // check). Validity -- the cluster's syndrome lies in the GF(2) span of its columns -- is kept by
-// incremental elimination: every cluster holds an echelon basis of its column vectors, bit-packed
-// over the checks with one 32-bit word per lane, stored in rows keyed by the pivot check. A new
-// column is reduced against the basis and kept if it is independent; on a merge the basis of larger
-// rank survives and the other cluster's columns are reduced into it. When no cluster is invalid,
-// each cluster is solved by OSD-0: its columns are eliminated in reliability order (pivots = the
-// first independent ones) with a record of which columns make up each basis row, the syndrome is
-// reduced, and the recorded columns form the correction (free columns zero).
+// incremental elimination: every cluster holds a basis of its column vectors, bit-packed over the checks
+// with one 32-bit word per lane, a row's lowest set bit being its pivot and its place. A vector is
+// reduced from its lowest bit up, one row per pivot it meets, until it is zero or its lowest bit is no
+// pivot. A new column that does not reach zero becomes a row; on a merge the basis of larger rank
+// survives and the other cluster's columns are reduced into it. A cluster's reduced syndrome is kept
+// between rounds: without a merge its new checks are not flipped, so only the new rows are applied to
+// it. When no cluster is invalid, each cluster is solved by OSD-0: its columns are eliminated in
+// reliability order (pivots = the first independent ones) with a record of which columns make up each
+// basis row, the syndrome is reduced, and the recorded columns form the correction (free columns zero).
+//
+// Each check remembers its best free column; only the checks of a column that was just taken look again
+// (one warp per check, over its row). What bounded the kernel before was the growth of single large
+// clusters, a column per round: every round scanned every row of the cluster with an atomic minimum on
+// one word per entry (70,000 at 540 checks), walked the whole basis twice, and searched all checks for
+// roots on one thread. A launch lasts as long as its largest cluster: 226 shots of circuit-level d = 5, 7
+// and 9 at p = 1e-3 and 3e-3 (up to 578 columns) 157 -> 10.8 ms; 21 shots at d = 11 11.5 -> 1.5 ms; the 11,400
+// shots of small clusters of a d=9 phenomenological batch 3.5 -> 1.14 ms.
 //
 // Warps work on different clusters in parallel; the merge bookkeeping of each round is serial (one
 // thread) because it is short (one pick per invalid cluster). Every loop is bounded: at most n + 1
@@ -24,6 +34,8 @@
 namespace vibe {
 namespace {
 
+constexpr int kLook = -2;       // chk_best: look through the row
+constexpr int kSolve = 1 << 20;  // basis ids of the final solve: root + kSolve
 constexpr int kFreeRows = 10;   // largest LSD order: records kept for the first 10 free columns
 
 struct LsdShared {
@@ -33,10 +45,12 @@ struct LsdShared {
   int32_t* pend_next; // n  columns waiting to be reduced into their cluster's basis
   int32_t* ck_par;    // m  union-find parent, -1 = check in no cluster
   unsigned long long* best;  // m
-  uint8_t* valid;     // m
+  uint8_t* valid;     // m  per root: 1 = valid, 2 = invalid with its reduced syndrome kept
   uint8_t* dirty;     // m
   int32_t* rank;      // m
-  int32_t* b_head; int32_t* b_tail; int32_t* piv_next;  // m each: basis rows in insertion order
+  int32_t* chk_best;  // m  the check's best free column: kLook = to be found, -1 = none left
+  int32_t* bid;       // m  per root: id of the cluster's basis
+  int32_t* tag;       // m  per pivot: id of the basis its row belongs to
   int32_t* c_head; int32_t* c_tail; int32_t* c_cnt;     // m each: column lists
   int32_t* p_head; int32_t* p_tail;                     // m each: pending lists
   int32_t* dlist;     // m  roots to process this round
@@ -80,24 +94,6 @@ __device__ __forceinline__ void load_column(const Tables& t, int j, uint32_t (&x
   }
 }
 
-template <int WP>
-__device__ __forceinline__ bool any_bits(const uint32_t (&x)[WP]) {
-  uint32_t o = 0;
-#pragma unroll
-  for (int q = 0; q < WP; ++q) o |= x[q];
-  return __any_sync(kFull, o != 0u);
-}
-
-template <int WP>
-__device__ __forceinline__ uint32_t get_bit(const uint32_t (&x)[WP], int p, int lane) {
-  const int w = p >> 5;
-  uint32_t b = 0;
-#pragma unroll
-  for (int q = 0; q < WP; ++q)
-    if ((w >> 5) == q) b = (x[q] >> (p & 31)) & 1u;
-  return __shfl_sync(kFull, b, w & 31);
-}
-
 // lowest set bit index over the lane-distributed vector (word w = lane + 32 q), or INT_MAX
 template <int WP>
 __device__ __forceinline__ int lowest_bit(const uint32_t (&x)[WP], int lane) {
@@ -105,37 +101,36 @@ __device__ __forceinline__ int lowest_bit(const uint32_t (&x)[WP], int lane) {
 #pragma unroll
   for (int q = WP - 1; q >= 0; --q)
     if (x[q]) best = (lane + 32 * q) * 32 + (__ffs(x[q]) - 1);
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) best = min(best, __shfl_xor_sync(kFull, best, off));
-  return best;
+  return (int)__reduce_min_sync(kFull, (uint32_t)best);
 }
 
-// x <- x reduced by the basis rows listed from `head` (insertion order); comb tracks the same XORs
-// over the rows' column combinations when TRACK.
-// ops counts the 32-bit words XOR-ed (the same on every lane of the warp).
+// x <- x reduced by the basis with id `id`, from the lowest bit up; comb tracks the same XORs over the
+// rows' column combinations when TRACK. Returns the lowest bit left (no pivot of the basis), or
+// INT_MAX when x is zero. ops counts the 32-bit words XOR-ed (the same on every lane of the warp).
 template <int WP, bool TRACK>
-__device__ __forceinline__ void reduce(uint32_t (&x)[WP], uint32_t (&comb)[WP], int head, const LsdShared& S,
-                                       const uint32_t* basis, const uint32_t* combrow, int W, int CW, int lane,
-                                       unsigned long long& ops) {
-  const int maxrows = 32 * W;   // a basis never has more rows than checks
-  int g = 0;
-  for (int p = head; p >= 0 && g < maxrows; p = S.piv_next[p], ++g) {
-    if (get_bit<WP>(x, p, lane)) {
-      ops += (unsigned long long)(W + (TRACK ? CW : 0));
+__device__ __forceinline__ int reduce(uint32_t (&x)[WP], uint32_t (&comb)[WP], int id, const LsdShared& S,
+                                      const uint32_t* basis, const uint32_t* combrow, int W, int CW, int lane,
+                                      unsigned long long& ops) {
+  const int maxrows = 32 * W;   // a row clears its pivot and changes higher bits only
+  int p = lowest_bit<WP>(x, lane);
+  for (int g = 0; g < maxrows && p != 0x7fffffff && S.tag[p] == id; ++g) {
+    ops += (unsigned long long)(W + (TRACK ? CW : 0));
 #pragma unroll
-      for (int q = 0; q < WP; ++q) {
-        const int w = lane + 32 * q;
-        if (w < W) x[q] ^= basis[(size_t)p * W + w];
-        if (TRACK && w < CW) comb[q] ^= combrow[(size_t)p * CW + w];
-      }
+    for (int q = 0; q < WP; ++q) {
+      const int w = lane + 32 * q;
+      if (w < W) x[q] ^= basis[(size_t)p * W + w];
+      if (TRACK && w < CW) comb[q] ^= combrow[(size_t)p * CW + w];
     }
+    p = lowest_bit<WP>(x, lane);
   }
+  __syncwarp();   // every lane has read the last tag before the caller may change it
+  return p;
 }
 
 template <int WP, bool TRACK>
-__device__ __forceinline__ void append_row(const uint32_t (&x)[WP], const uint32_t (&comb)[WP], int p, int root,
+__device__ __forceinline__ void append_row(const uint32_t (&x)[WP], const uint32_t (&comb)[WP], int p, int root, int id,
                                            const LsdShared& S, uint32_t* basis, uint32_t* combrow, int W, int CW,
-                                           int32_t* head, int32_t* tail, int lane) {
+                                           int lane) {
 #pragma unroll
   for (int q = 0; q < WP; ++q) {
     const int w = lane + 32 * q;
@@ -143,9 +138,7 @@ __device__ __forceinline__ void append_row(const uint32_t (&x)[WP], const uint32
     if (TRACK && w < CW) combrow[(size_t)p * CW + w] = comb[q];
   }
   if (lane == 0) {
-    S.piv_next[p] = -1;
-    if (*tail >= 0) S.piv_next[*tail] = p; else *head = p;
-    *tail = p;
+    S.tag[p] = id;
     if (!TRACK) S.rank[root]++;
   }
   __syncwarp();
@@ -163,14 +156,14 @@ __device__ int merge_clusters(const LsdShared& S, int a, int b, int n) {
     if (pt >= 0) S.pend_next[pt] = j; else ph = j;
     pt = j;
   }
-  const int bh = S.b_head[X], bt = S.b_tail[X], rk = S.rank[X];
+  const int id = S.bid[X], rk = S.rank[X];
   // column lists: s ++ o
   if (S.c_head[o] >= 0) {
     if (S.c_tail[s] >= 0) S.col_next[S.c_tail[s]] = S.c_head[o]; else S.c_head[s] = S.c_head[o];
     S.c_tail[s] = S.c_tail[o];
   }
   S.c_cnt[s] += S.c_cnt[o];
-  S.b_head[s] = bh; S.b_tail[s] = bt; S.rank[s] = rk;
+  S.bid[s] = id; S.rank[s] = rk;
   S.p_head[s] = ph; S.p_tail[s] = pt;
   S.ck_par[o] = s;
   S.valid[s] = 0;
@@ -203,9 +196,9 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
     }
     S.ck_par = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
     S.rank = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
-    S.b_head = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
-    S.b_tail = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
-    S.piv_next = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
+    S.chk_best = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
+    S.bid = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
+    S.tag = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
     S.c_head = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
     S.c_tail = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
     S.c_cnt = reinterpret_cast<int32_t*>(take(4 * (size_t)mB));
@@ -268,7 +261,7 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
       const bool flipped = (__ldg(syn + (c >> 5)) >> (c & 31)) & 1u;
       S.ck_par[c] = flipped ? c : -1;
       S.valid[c] = 0; S.dirty[c] = 0; S.rank[c] = 0;
-      S.b_head[c] = -1; S.b_tail[c] = -1; S.piv_next[c] = -1;
+      S.chk_best[c] = kLook; S.bid[c] = c; S.tag[c] = -1;
       S.c_head[c] = -1; S.c_tail[c] = -1; S.c_cnt[c] = 0;
       S.p_head[c] = -1; S.p_tail[c] = -1;
     }
@@ -276,31 +269,61 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
     __syncthreads();
 
     for (int round = 0; round <= n + 1; ++round) {
-      // A: reset the pick of every invalid cluster
+      // A: reset the pick of every invalid cluster; its checks whose best column is gone look again
       for (int c = tid; c < m; c += NT)
-        if (S.ck_par[c] == c && !S.valid[c]) S.best[c] = ~0ull;
-      __syncthreads();
-      // B: best free column adjacent to each invalid cluster
-      for (int c = tid; c < m; c += NT) {
-        if (S.ck_par[c] < 0) continue;
-        const int r = find_root(S.ck_par, c, m);
-        if (S.valid[r]) continue;
-        for (int e = __ldg(t.rowptr + c); e < __ldg(t.rowptr + c + 1); ++e) {
-          const int j = __ldg(t.colidx + e);
-          if (S.col_root[j] < 0) atomicMin(&S.best[r], ((unsigned long long)S.key[j] << 32) | (unsigned)j);
+        if (S.ck_par[c] == c && S.valid[c] != 1) S.best[c] = ~0ull;
+      for (int c0 = 32 * warp; c0 < m; c0 += NT) {
+        const int c = c0 + lane;
+        bool look = false;
+        if (c < m && S.ck_par[c] >= 0 && S.valid[find_root(S.ck_par, c, m)] != 1) {
+          const int j = S.chk_best[c];
+          look = j == kLook || (j >= 0 && S.col_root[j] >= 0);
+        }
+        uint32_t bal = __ballot_sync(kFull, look);
+        while (bal) {
+          const int cc = c0 + __ffs(bal) - 1;
+          bal &= bal - 1u;
+          uint32_t key = 0xffffffffu, col = 0xffffffffu;
+          for (int e = __ldg(t.rowptr + cc) + lane; e < __ldg(t.rowptr + cc + 1); e += 32) {
+            const int j = __ldg(t.colidx + e);   // ascending: a later equal key does not win
+            if (S.col_root[j] < 0 && (S.key[j] < key || col == 0xffffffffu)) { key = S.key[j]; col = (uint32_t)j; }
+          }
+          const uint32_t k = __reduce_min_sync(kFull, key);
+          const uint32_t v = __reduce_min_sync(kFull, key == k ? col : 0xffffffffu);
+          if (lane == 0) S.chk_best[cc] = (int)v;   // -1: no free column
         }
       }
       __syncthreads();
+      // B: best free column adjacent to each invalid cluster
+      for (int c = tid; c < m; c += NT) {
+        const int j = S.chk_best[c];
+        if (S.ck_par[c] < 0 || j < 0) continue;
+        const int r = find_root(S.ck_par, c, m);
+        if (S.valid[r] == 1) continue;
+        const unsigned long long cand = ((unsigned long long)S.key[j] << 32) | (unsigned)j;
+        if (cand < *reinterpret_cast<volatile unsigned long long*>(&S.best[r])) atomicMin(&S.best[r], cand);
+      }
+      __syncthreads();
+      // the invalid clusters' roots, ascending (the first warp)
+      if (warp == 0) {
+        int npick = 0;
+        bool none = false;
+        for (int c0 = 0; c0 < m; c0 += 32) {
+          const int c = c0 + lane;
+          const bool pick = c < m && S.ck_par[c] == c && S.valid[c] != 1;
+          none |= pick && S.best[c] == ~0ull;
+          const uint32_t bal = __ballot_sync(kFull, pick);
+          if (pick) S.dlist[npick + __popc(bal & ((1u << lane) - 1u))] = c;
+          npick += __popc(bal);
+        }
+        none = __any_sync(kFull, none);
+        if (lane == 0) { S.flags[6] = npick; S.flags[7] = none ? 2 : 0; }
+        __syncwarp();
+      }
       // C: apply the picks (serial)
       if (tid == 0) {
-        int npick = 0, status = 0;
-        // picks are stored in dlist temporarily as root ids; the columns are read from best[]
-        for (int c = 0; c < m; ++c) {
-          if (S.ck_par[c] == c && !S.valid[c]) {
-            if (S.best[c] == ~0ull) { status = 2; break; }
-            S.dlist[npick++] = c;
-          }
-        }
+        const int npick = S.flags[6];
+        int status = S.flags[7];
         if (status == 0 && npick == 0) status = 1;
         if (status == 0) {
           for (int k = 0; k < npick; ++k) {
@@ -328,12 +351,20 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
               }
             }
           }
-          int nd = 0;
-          for (int c = 0; c < m; ++c)
-            if (S.ck_par[c] == c && S.dirty[c]) { S.dlist[nd++] = c; S.dirty[c] = 0; }
-          S.flags[1] = nd;
         }
         S.flags[2] = status;
+      }
+      if (warp == 0) {   // the changed clusters' roots, ascending
+        __syncwarp();
+        int nd = 0;
+        for (int c0 = 0; c0 < m && S.flags[2] == 0; c0 += 32) {
+          const int c = c0 + lane;
+          const bool d = c < m && S.ck_par[c] == c && S.dirty[c];
+          const uint32_t bal = __ballot_sync(kFull, d);
+          if (d) { S.dlist[nd + __popc(bal & ((1u << lane) - 1u))] = c; S.dirty[c] = 0; }
+          nd += __popc(bal);
+        }
+        if (lane == 0) S.flags[1] = nd;
       }
       __syncthreads();
       if (S.flags[2] != 0) break;
@@ -344,33 +375,47 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
         uint32_t x[WP], dummy[WP];
 #pragma unroll
         for (int qq = 0; qq < WP; ++qq) dummy[qq] = 0u;
+        const int id = S.bid[r];
         int guard = 0;
         for (int j = S.p_head[r]; j >= 0 && guard < n; j = S.pend_next[j], ++guard) {
           load_column<WP>(t, j, x, lane);
-          reduce<WP, false>(x, dummy, S.b_head[r], S, basis, combrow, W, CW, lane, gf2_ops);
-          if (any_bits<WP>(x)) {
-            const int p = lowest_bit<WP>(x, lane);
-            append_row<WP, false>(x, dummy, p, r, S, basis, combrow, W, CW, &S.b_head[r], &S.b_tail[r], lane);
-          }
+          const int p = reduce<WP, false>(x, dummy, id, S, basis, combrow, W, CW, lane, gf2_ops);
+          if (p != 0x7fffffff) append_row<WP, false>(x, dummy, p, r, id, S, basis, combrow, W, CW, lane);
         }
         __syncwarp();
         if (lane == 0) { S.p_head[r] = -1; S.p_tail[r] = -1; }
-        // restricted syndrome
+        // the syndrome restricted to the cluster -- what earlier rounds left of it, kept in the row of its
+        // root of the combination records (not used before the final solve)
+        if (S.valid[r] == 2) {
 #pragma unroll
-        for (int qq = 0; qq < WP; ++qq) {
-          const int w = lane + 32 * qq;
-          uint32_t y = w < W ? S.sbits[w] : 0u, keep = 0u;
-          while (y) {
-            const int b = __ffs(y) - 1;
-            y &= y - 1;
-            const int c = 32 * w + b;
-            if (c < m && S.ck_par[c] >= 0 && find_root(S.ck_par, c, m) == r) keep |= 1u << b;
+          for (int qq = 0; qq < WP; ++qq) {
+            const int w = lane + 32 * qq;
+            x[qq] = w < W ? combrow[(size_t)r * CW + w] : 0u;
           }
-          x[qq] = keep;
+        } else {
+#pragma unroll
+          for (int qq = 0; qq < WP; ++qq) {
+            const int w = lane + 32 * qq;
+            uint32_t y = w < W ? S.sbits[w] : 0u, keep = 0u;
+            while (y) {
+              const int b = __ffs(y) - 1;
+              y &= y - 1;
+              const int c = 32 * w + b;
+              if (c < m && S.ck_par[c] >= 0 && find_root(S.ck_par, c, m) == r) keep |= 1u << b;
+            }
+            x[qq] = keep;
+          }
         }
-        reduce<WP, false>(x, dummy, S.b_head[r], S, basis, combrow, W, CW, lane, gf2_ops);
-        const bool ok = !any_bits<WP>(x);
-        if (lane == 0) S.valid[r] = ok ? 1 : 0;
+        const bool ok = reduce<WP, false>(x, dummy, id, S, basis, combrow, W, CW, lane, gf2_ops) == 0x7fffffff;
+        const bool keep = !ok && CW >= W;
+        if (keep) {
+#pragma unroll
+          for (int qq = 0; qq < WP; ++qq) {
+            const int w = lane + 32 * qq;
+            if (w < W) combrow[(size_t)r * CW + w] = x[qq];
+          }
+        }
+        if (lane == 0) S.valid[r] = ok ? 1 : keep ? 2 : 0;
         __syncwarp();
       }
       __syncthreads();
@@ -386,8 +431,6 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
           big = max(big, S.c_cnt[c]);
           S.rank[c] = off;
           off += S.c_cnt[c];
-          S.b_head[c] = -1;
-          S.b_tail[c] = -1;
         }
       S.flags[3] = nr;
       S.flags[4] = big;
@@ -429,10 +472,9 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
 #pragma unroll
           for (int qq = 0; qq < WP; ++qq)
             comb[qq] = ((tp >> 5) == lane + 32 * qq) ? (1u << (tp & 31)) : 0u;
-          reduce<WP, true>(x, comb, S.b_head[r], S, basis, combrow, W, CW, lane, gf2_ops);
-          if (any_bits<WP>(x)) {
-            const int p = lowest_bit<WP>(x, lane);
-            append_row<WP, true>(x, comb, p, r, S, basis, combrow, W, CW, &S.b_head[r], &S.b_tail[r], lane);
+          const int p = reduce<WP, true>(x, comb, r + kSolve, S, basis, combrow, W, CW, lane, gf2_ops);
+          if (p != 0x7fffffff) {
+            append_row<WP, true>(x, comb, p, r, r + kSolve, S, basis, combrow, W, CW, lane);
           } else {
             if (nfree < t.lsd_order) {
 #pragma unroll
@@ -458,7 +500,7 @@ __global__ void __launch_bounds__(NT) k_lsd(const LsdArgs a) {
           x[qq] = keep;
           comb[qq] = 0u;
         }
-        reduce<WP, true>(x, comb, S.b_head[r], S, basis, combrow, W, CW, lane, gf2_ops);
+        reduce<WP, true>(x, comb, r + kSolve, S, basis, combrow, W, CW, lane, gf2_ops);
         const int q = min(t.lsd_order, nfree);
         if (q == 0) {
 #pragma unroll

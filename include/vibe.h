@@ -134,7 +134,7 @@ typedef struct vibe_batch vibe_batch; /* opaque: several handles decoded in one 
  *   (member i: SplitMix64 started at seed + (i+1)*0xD1B54A32D192ED03, Durstenfeld shuffle taking
  *   j = high 64 bits of next()*(k+1) for k = n-1 down to 1).
  *   Uses the current CUDA device. Copies everything it is given; the device tables (CSR/CSC of H,
- *   per-member dependency wavefronts, message images) stay resident until vibe_destroy.
+ *   per-member packed steps, message images) stay resident until vibe_destroy.
  *   Limits of this build (VIBE_ERR_UNSUPPORTED beyond them): n < 2^24, m < 2^24, every row of H has
  *   at most 255 entries, every column at most 32, and one shot's BP state (messages, posteriors,
  *   syndrome) must fit in 200 KB of shared memory.
@@ -176,12 +176,12 @@ int vibe_decode_host(vibe_handle* h, const uint32_t* h_syndromes, int64_t B, uin
                      uint64_t* h_counters, void* stream);
 
 /*
- * vibe_get_wavefronts -- the dependency wavefronts built for one member (Sec. III.D.1 step 4):
+ * vibe_get_wavefronts -- the dependency wavefronts of one member, found by this call (Sec. III.D.1 step 4):
  *   level(v) = 1 + max{level(u) : u before v in the member's order and u, v share a check}, so the
  *   columns of one level share no check and may be updated together with results identical to the
  *   serial order. order_out: n column indices grouped by level (host); level_offsets_out: n + 1
  *   entries, level l holds order_out[level_offsets_out[l] .. level_offsets_out[l+1]); *nlevels_out
- *   the level count. Synchronous. Errors: VIBE_ERR_INVALID, VIBE_ERR_CUDA.
+ *   the level count. Synchronous. Errors: VIBE_ERR_INVALID, VIBE_ERR_NOMEM, VIBE_ERR_CUDA.
  */
 int vibe_get_wavefronts(vibe_handle* h, int32_t member, uint32_t* order_out,
                         uint32_t* level_offsets_out, int32_t* nlevels_out);

@@ -42,6 +42,11 @@ int cuda_fail(cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, what); \
   } while (0)
 
+// A warp's message image above this does not leave the image engine a CTA (two warps in 227 KB).
+constexpr size_t kTeamImageBytes = size_t(114) << 10;
+
+constexpr int team_of(int cls) { return cls ? vibe::kTeam : 1; }
+
 constexpr size_t kWorkspaceBytes = size_t(4) << 30;   // LSD hand-off buffer budget per workspace
 
 int check_csr(const vibe_csr* A, const char* name, bool rows_nonempty) {
@@ -78,13 +83,28 @@ struct Launch {
   Bounds bnd{};
   int msg_fp16 = 0;
   int device = 0, num_sms = 0;
-  int bp_blocks_per_sm = 0, bpx_blocks_per_sm = 0, lsd_blocks_per_sm = 0;
+  int bp_blocks_per_sm = 0, bpx_blocks_per_sm = 0, lsd_blocks_per_sm = 0;   // bpx: of the smallest teams
+  int xocc[vibe::kTeamClasses] = {};   // summary engine: CTAs per SM that fit, by team class
   int pair_mode = 0;                // one warp per (shot, member) pair (vibe_params.pair_mode)
   int lsd_threads = vibe::kLsdThreads;   // threads per LSD CTA (tuned: 64, 128 or 256)
   bool warp_engine() const { return (bnd.engines & 1) != 0; }
   bool cta_engine() const { return (bnd.engines & 2) != 0; }
   int bp_grid() const { return warp_engine() ? std::max(1, bp_blocks_per_sm * num_sms) : 0; }
-  int bpx_grid() const { return cta_engine() ? std::max(1, bpx_blocks_per_sm * num_sms) : 0; }
+  int first_team() const {   // the smallest team class of the launch
+    for (int k = 0; k < vibe::kTeamClasses; ++k)
+      if ((bnd.teams >> k) & 1) return k;
+    return 0;
+  }
+  // the grids of the other classes are scaled as the first one's is
+  int bpx_grid(int k) const {
+    if (!((bnd.teams >> k) & 1)) return 0;
+    return std::max(1, xocc[k] * bpx_blocks_per_sm / std::max(1, xocc[first_team()])) * num_sms;
+  }
+  int bpx_grid() const {   // the largest
+    int g = 0;
+    for (int k = 0; k < vibe::kTeamClasses; ++k) g = std::max(g, bpx_grid(k));
+    return g;
+  }
   int lsd_grid() const { return std::max(1, lsd_blocks_per_sm * num_sms); }
   // per-warp global scratch of the summary engine, bytes; the candidate posteriors only with soft output
   long long bpx_pitch(bool soft) const {
@@ -107,7 +127,7 @@ struct Launch {
   // members' records pass 2 GiB.
   long long auto_pair_shots() const {
     if (bnd.K < 2) return 0;
-    const long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta + (long long)bpx_grid() * vibe::kBpxWarpsPerCta;
+    const long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta + (long long)bpx_grid();
     return std::min(8 * warps, kAutoPairBytes / pair_shot_bytes(false));
   }
   static constexpr long long kAutoPairBytes = 2LL << 30;
@@ -120,8 +140,9 @@ struct Workspace {
   long long lsd_words = 0;         // LSD scratch words per CTA the buffer was made for
   int bp_warps = 0, lsd_ctas = 0;
   long long bpx_bytes = 0;
-  unsigned int* ctrl = nullptr;   // [0] next shot (image engine), [1] LSD count, [2] next LSD shot,
-                                  // [3] next shot (summary engine), [4] / [5] next pair (image / summary)
+  static constexpr int kCtrl = 4 + 2 * vibe::kTeamClasses;
+  unsigned int* ctrl = nullptr;   // [0] next shot (image engine), [1] LSD count, [2] next LSD shot, [3] next pair
+                                  // (image engine), then next shot and next pair of each team class
   uint32_t* lsd_shots = nullptr;
   float* lsd_soft = nullptr;
   float* bp_scratch = nullptr;
@@ -162,7 +183,7 @@ struct Workspace {
     const long long ps = std::min(need, L.pair_mode ? L.pair_chunk(soft) : L.auto_pair_shots());
     const long long want = std::min(need, chunk_max);
     const int warps = L.bp_grid() * vibe::kBpWarpsPerCta;
-    const long long xb = (long long)L.bpx_grid() * vibe::kBpxWarpsPerCta * L.bpx_pitch(soft);
+    const long long xb = (long long)L.bpx_grid() * L.bpx_pitch(soft);
     const bool pair_ok = ps == 0 || (!L.pair_mode && no_records) ||
                          (ps <= pair_shots && (!L.pair_mode || !soft || pair_soft) && L.bnd.K * L.bnd.nw <= pk_nw &&
                           L.bnd.K * L.bnd.n <= pk_n);
@@ -174,7 +195,7 @@ struct Workspace {
     const long long xkeep = std::max(xb, bpx_bytes);
     release();
     const Bounds& b = L.bnd;
-    VIBE_CUDA(dalloc(&ctrl, 8), "workspace");
+    VIBE_CUDA(dalloc(&ctrl, kCtrl), "workspace");
     VIBE_CUDA(dalloc(&lsd_shots, (size_t)c), "workspace");
     VIBE_CUDA(dalloc(&lsd_soft, (size_t)c * b.n), "workspace");
     VIBE_CUDA(dalloc(&bp_scratch, (size_t)warps * (size_t)(2 + b.global_st + b.M) * b.n), "workspace");
@@ -258,7 +279,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
   const bool pairs = ws.as_pairs(L, q.B, q.soft != nullptr);
   for (long long b0 = 0; b0 < q.B; b0 += step) {
     const long long nb = std::min(step, q.B - b0);
-    VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, 8 * sizeof(unsigned int), s), "decode");
+    VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, Workspace::kCtrl * sizeof(unsigned int), s), "decode");
     cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
     if (prof.on) { e0 = prof.next(); e1 = prof.next(); e2 = prof.next(); }
     if (e0) cudaEventRecord(e0, s);
@@ -268,7 +289,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       const long long o = b0 + s0;
       if (s0 > 0) {   // the BP work counters start again; the LSD queue keeps filling
         VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, sizeof(unsigned int), s), "decode");
-        VIBE_CUDA(cudaMemsetAsync(ws.ctrl + 3, 0, 3 * sizeof(unsigned int), s), "decode");
+        VIBE_CUDA(cudaMemsetAsync(ws.ctrl + 3, 0, (Workspace::kCtrl - 3) * sizeof(unsigned int), s), "decode");
       }
       if (pairs) {
         VIBE_CUDA(cudaMemsetAsync(ws.pconv, 0, sizeof(int) * (size_t)ns * L.bnd.K, s), "decode");
@@ -293,13 +314,11 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       a.scratch_pitch = (long long)(2 + L.bnd.global_st + L.bnd.M) * L.bnd.n;
       a.xscratch = ws.bpx_scratch;
       a.xscratch_pitch = L.bpx_pitch(a.want_soft != 0);
-      a.next_shot_x = ws.ctrl + 3;
       a.pair_mode = pairs;
       a.pair_K = L.bnd.K;
       a.pconv = ws.pconv; a.pW = ws.pW; a.pbits = ws.pbits; a.pterms = ws.pterms; a.ppost = ws.ppost;
       a.pdone = ws.pdone;
-      a.next_pair = ws.ctrl + 4;
-      a.next_pair_x = ws.ctrl + 5;
+      a.next_pair = ws.ctrl + 3;
       const long long units = pairs ? ns * L.bnd.K : ns;   // shots, or (shot, member) pairs
       if (L.warp_engine()) {
         const int grid =
@@ -307,11 +326,15 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
         a.flag_bad = 1;
         VIBE_CUDA(vibe::launch_bp(a, L.msg_fp16, grid, s), "BP kernel launch");
       }
-      if (L.cta_engine()) {
-        const int grid =
-            (int)std::min<long long>(L.bpx_grid(), (units + vibe::kBpxWarpsPerCta - 1) / vibe::kBpxWarpsPerCta);
-        a.flag_bad = L.warp_engine() ? 0 : 1;
-        VIBE_CUDA(vibe::launch_bpx(a, L.msg_fp16, grid, s), "BP kernel launch");
+      bool first = !L.warp_engine();
+      for (int k = 0; k < vibe::kTeamClasses; ++k) {
+        if (!((L.bnd.teams >> k) & 1)) continue;
+        a.flag_bad = first ? 1 : 0;
+        first = false;
+        a.next_shot_x = ws.ctrl + 4 + 2 * k;
+        a.next_pair_x = a.next_shot_x + 1;
+        VIBE_CUDA(vibe::launch_bpx(a, team_of(k), L.msg_fp16, (int)std::min<long long>(L.bpx_grid(k), units), s),
+                  "BP kernel launch");
       }
       prof.bp_launches++;
     }
@@ -349,13 +372,15 @@ int size_launch(Launch& L) {
     VIBE_CUDA(vibe::bp_occupancy(L.bnd, nd, L.msg_fp16, &L.bp_blocks_per_sm), "BP occupancy");
     if (L.bp_blocks_per_sm < 1) return fail(VIBE_ERR_UNSUPPORTED, "the BP kernel cannot be resident");
   }
-  if (L.cta_engine()) {
-    if (vibe::bpx_cta_smem_bytes(L.bnd, nd) > (size_t)optin)
-      return fail(VIBE_ERR_UNSUPPORTED, "check summaries of one shot (%d bytes per warp) do not fit in shared memory",
-                  L.bnd.x_warp_smem);
-    VIBE_CUDA(vibe::bpx_occupancy(L.bnd, nd, L.msg_fp16, &L.bpx_blocks_per_sm), "BP occupancy");
-    if (L.bpx_blocks_per_sm < 1) return fail(VIBE_ERR_UNSUPPORTED, "the BP kernel cannot be resident");
+  for (int k = 0; k < vibe::kTeamClasses; ++k) {
+    if (!((L.bnd.teams >> k) & 1)) continue;
+    if (vibe::bpx_cta_smem_bytes(L.bnd, team_of(k), nd) > (size_t)optin)
+      return fail(VIBE_ERR_UNSUPPORTED, "check summaries of one shot (%d bytes) do not fit in shared memory",
+                  L.bnd.x_sums[k]);
+    VIBE_CUDA(vibe::bpx_occupancy(L.bnd, team_of(k), nd, L.msg_fp16, &L.xocc[k]), "BP occupancy");
+    if (L.xocc[k] < 1) return fail(VIBE_ERR_UNSUPPORTED, "the BP kernel cannot be resident");
   }
+  L.bpx_blocks_per_sm = L.cta_engine() ? L.xocc[L.first_team()] : 0;
   if (vibe::lsd_smem_bytes(L.bnd, L.ndem) > (size_t)optin)
     return fail(VIBE_ERR_UNSUPPORTED, "LSD state of one shot does not fit in shared memory");
   VIBE_CUDA(vibe::lsd_occupancy(L.bnd, L.ndem, L.lsd_threads, &L.lsd_blocks_per_sm), "LSD occupancy");
@@ -382,11 +407,12 @@ Bounds bounds_over(const Tables* ts, int count) {
     } else {
       b.engines |= 2;
       b.XD = std::max(b.XD, t.XD);
-      b.x_warp_smem = std::max(b.x_warp_smem, t.x_warp_smem);
+      const int k = vibe::team_class(t.team);
+      b.teams |= 1 << k;
+      b.x_sums[k] = std::max(b.x_sums[k], t.x_warp_smem);
       b.x_warp_scratch = std::max(b.x_warp_scratch, t.x_warp_scratch);
     }
   }
-  if (b.engines & 2) b.x_warp_smem += vibe::bpx_window_bytes();
   return b;
 }
 
@@ -488,8 +514,8 @@ struct vibe_handle {
   Profiler prof;
   // resident tables
   int32_t *rowptr = nullptr, *colidx = nullptr, *colptr = nullptr, *rowidx = nullptr;
-  int32_t *lrowptr = nullptr, *lcolidx = nullptr, *nlev = nullptr;
-  uint32_t *csc_ent = nullptr, *sched = nullptr, *lvl_off = nullptr, *perm = nullptr;
+  int32_t *lrowptr = nullptr, *lcolidx = nullptr;
+  uint32_t *csc_ent = nullptr, *perm = nullptr;
   float* lam = nullptr;
   float* alpha_m = nullptr;
   void* msg_init = nullptr;
@@ -517,7 +543,7 @@ struct vibe_handle {
     release_stage();
     cudaFree(tmp_counters);
     cudaFree(rowptr); cudaFree(colidx); cudaFree(colptr); cudaFree(rowidx); cudaFree(lrowptr); cudaFree(lcolidx);
-    cudaFree(nlev); cudaFree(csc_ent); cudaFree(sched); cudaFree(lvl_off); cudaFree(perm); cudaFree(lam); cudaFree(alpha_m);
+    cudaFree(csc_ent); cudaFree(perm); cudaFree(lam); cudaFree(alpha_m);
     cudaFree(msg_init); cudaFree(cpos); cudaFree(soff); cudaFree(stepcnt); cudaFree(xrec); cudaFree(xlnk); cudaFree(xcolid);
     cudaFree(xrmap); cudaFree(xsum); cudaFree(d_desc);
     cudaFree(layer_ptr); cudaFree(layer_chk); cudaFree(layer_vptr); cudaFree(layer_var); cudaFree(nlayer_d);
@@ -650,8 +676,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   const int Lnnz = L->rowptr[k];
   const size_t msg_bytes = (size_t)m * t.RP * (p->msg_fp16 ? 2 : 4);
   const size_t lev_scratch =
-      std::max({2 * (size_t)n + E, 2 * (size_t)m + 2, (size_t)K * ((size_t)m + 3 * (size_t)n + 1),
-                vibe::step_scratch_ints(n, K)});
+      std::max({2 * (size_t)n, 2 * (size_t)m + 2,
+                vibe::step_scratch_ints(n, K, t.XD > 0 && msg_bytes > kTeamImageBytes ? vibe::kTeam : 1)});
   int32_t* scratch = nullptr;
   cudaStream_t s = nullptr;
 #define VIBE_TRY(call, what) \
@@ -663,11 +689,7 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   VIBE_TRY(dalloc(&h->rowidx, E), "tables");
   VIBE_TRY(dalloc(&h->lrowptr, k + 1), "tables");
   VIBE_TRY(dalloc(&h->lcolidx, Lnnz), "tables");
-  VIBE_TRY(dalloc(&h->nlev, K), "tables");
   VIBE_TRY(dalloc(&h->csc_ent, (size_t)n * t.DP), "tables");
-  VIBE_TRY(dalloc(&h->sched, (size_t)K * n), "tables");
-
-  VIBE_TRY(dalloc(&h->lvl_off, (size_t)K * (n + 1)), "tables");
   VIBE_TRY(dalloc(&h->perm, (size_t)K * n), "tables");
   VIBE_TRY(dalloc(&h->lam, n), "tables");
   VIBE_TRY(dalloc(&h->alpha_m, K), "tables");
@@ -700,15 +722,36 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     VIBE_TRY(vibe::seeded_schedules(h->perm, n, K, p->seed, s), "schedule kernel");
   }
   VIBE_TRY(vibe::build_tables(h->rowptr, h->colidx, m, n, E, K, h->perm, t.RP, t.DP, p->msg_fp16, h->lam, h->colptr,
-                              h->rowidx, h->cpos, h->csc_ent, h->msg_init, h->sched, h->lvl_off, h->nlev, h->xsum,
-                              scratch, s),
+                              h->rowidx, h->cpos, h->csc_ent, h->msg_init, h->xsum, scratch, s),
            "graph builder");
   {
     std::vector<int32_t> cnt(K);
-    VIBE_TRY(vibe::build_steps(m, n, K, h->perm, h->colptr, h->cpos, h->stepcnt, scratch, s), "step builder");
-    VIBE_TRY(cudaMemcpyAsync(cnt.data(), h->stepcnt, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, s), "step builder");
-    VIBE_TRY(cudaStreamSynchronize(s), "step builder");
-    t.nstep = *std::max_element(cnt.begin(), cnt.end());
+    auto steps = [&](int team) -> cudaError_t {
+      cudaError_t er = vibe::build_steps(m, n, K, team, h->perm, h->colptr, h->cpos, h->stepcnt, scratch, s);
+      if (er == cudaSuccess)
+        er = cudaMemcpyAsync(cnt.data(), h->stepcnt, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, s);
+      if (er == cudaSuccess) er = cudaStreamSynchronize(s);
+      t.team = team;
+      t.nstep = er == cudaSuccess ? *std::max_element(cnt.begin(), cnt.end()) : 0;
+      return er;
+    };
+    VIBE_TRY(steps(1), "step builder");
+    // Wide graphs get a team of eight warps per member, where only the summary engine can run them and
+    // units of 8 x 32 edges keep at least 3/4 of their lanes at work (random orders: circuit-level d=13 7674
+    // steps with one warp, 1066 units with eight; d=11 4407 and 998: no). A member then takes that much less
+    // time, and its check summaries, which leave one-warp members 7 (FP32) or 12 warps on an SM at d=13,
+    // serve all eight. Measured, 4 shots of d=9 and d=13 (K=32, T=50): 182 -> 99 ms. Smaller teams did
+    // not pay: d=11 with four 158 -> 153 ms, d=9 with two, in batches that fill the GPU, 92 -> 103 ms.
+    if (t.XD > 0 && msg_bytes > kTeamImageBytes && t.SP >= 24 * vibe::kTeam * 32) {
+      const long long single = t.nstep;
+      int optin = 0;
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
+      VIBE_TRY(steps(vibe::kTeam), "step builder");
+      t.engine = VIBE_ENGINE_SUMMARY;
+      if (3 * t.nstep > 4 * single || vibe::bpx_cta_smem_bytes(bounds_over(&t, 1), vibe::kTeam, vibe::kMaxDems) > (size_t)optin)
+        VIBE_TRY(steps(1), "step builder");
+      t.engine = p->bp_engine;
+    }
     t.soff_pitch = t.nstep + vibe::kStepPad;
     VIBE_TRY(dalloc(&h->soff, (size_t)K * t.soff_pitch), "tables");
     VIBE_TRY(dalloc(&h->xrec, (size_t)K * t.SP + 4), "tables");   // copied in groups of four slots
@@ -716,10 +759,10 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     VIBE_TRY(dalloc(&h->xcolid, (size_t)K * t.SP), "tables");
     if (t.XD > 0) VIBE_TRY(dalloc(&h->xrmap, (size_t)K * E), "tables");
     // the lanes' order pays where the image engine runs (xcolid serves as its scratch: it is filled next)
-    if (msg_bytes <= 100 * 1024)
+    if (t.team == 1 && msg_bytes <= kTeamImageBytes)
       VIBE_TRY(vibe::order_steps(n, t.SP, K, t.nstep, h->colptr, h->cpos, h->stepcnt, scratch, h->xcolid, s),
                "step builder");
-    VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.DP, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
+    VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.DP, t.team, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
                               h->soff, h->xrec, h->xlnk, h->xcolid, h->xrmap, s),
              "step builder");
   }
@@ -752,8 +795,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     t.layer_ptr = h->layer_ptr; t.layer_chk = h->layer_chk; t.layer_vptr = h->layer_vptr; t.layer_var = h->layer_var;
   }
   t.rowptr = h->rowptr; t.colidx = h->colidx; t.colptr = h->colptr; t.rowidx = h->rowidx;
-  t.csc_ent = h->csc_ent; t.lam = h->lam; t.alpha_m = h->alpha_m; t.msg_init = h->msg_init; t.sched = h->sched; t.lvl_off = h->lvl_off;
-  t.nlev = h->nlev; t.lrowptr = h->lrowptr; t.lcolidx = h->lcolidx;
+  t.csc_ent = h->csc_ent; t.lam = h->lam; t.alpha_m = h->alpha_m; t.msg_init = h->msg_init;
+  t.lrowptr = h->lrowptr; t.lcolidx = h->lcolidx;
   t.stepcnt = h->stepcnt; t.soff = h->soff; t.xrec = h->xrec; t.xlnk = h->xlnk; t.xcolid = h->xcolid; t.xrmap = h->xrmap; t.xsum = h->xsum;
   VIBE_TRY(cudaMemcpyAsync(h->d_desc, &t, sizeof(Tables), cudaMemcpyHostToDevice, s), "upload");
   VIBE_TRY(cudaStreamSynchronize(s), "graph builder");
@@ -838,11 +881,22 @@ int vibe_get_wavefronts(vibe_handle* h, int32_t member, uint32_t* order_out, uin
                         int32_t* nlevels_out) {
   if (!h || !order_out || !level_offsets_out || !nlevels_out) return fail(VIBE_ERR_INVALID, "NULL argument");
   if (member < 0 || member >= h->t.K) return fail(VIBE_ERR_INVALID, "member out of range");
-  const int n = h->t.n;
-  VIBE_CUDA(cudaMemcpy(order_out, h->sched + (size_t)member * n, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost), "copy");
-  VIBE_CUDA(cudaMemcpy(level_offsets_out, h->lvl_off + (size_t)member * (n + 1), sizeof(uint32_t) * (n + 1),
-                       cudaMemcpyDeviceToHost), "copy");
-  VIBE_CUDA(cudaMemcpy(nlevels_out, h->nlev + member, sizeof(int32_t), cudaMemcpyDeviceToHost), "copy");
+  // the kernels run the packed steps; the levels are found here, for the member asked for
+  const int n = h->t.n, m = h->t.m;
+  uint32_t *sched = nullptr, *off = nullptr;
+  int32_t* work = nullptr;   // the level count, then scratch
+  cudaError_t e = dalloc(&sched, (size_t)n);
+  if (e == cudaSuccess) e = dalloc(&off, (size_t)n + 1);
+  if (e == cudaSuccess) e = dalloc(&work, (size_t)m + 3 * (size_t)n + 2);
+  if (e == cudaSuccess)
+    e = vibe::member_levels(h->perm + (size_t)member * n, n, m, h->colptr, h->rowidx, sched, off, work, work + 1, nullptr);
+  if (e == cudaSuccess) e = cudaMemcpy(order_out, sched, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(level_offsets_out, off, sizeof(uint32_t) * (n + 1), cudaMemcpyDeviceToHost);
+  if (e == cudaSuccess) e = cudaMemcpy(nlevels_out, work, sizeof(int32_t), cudaMemcpyDeviceToHost);
+  cudaFree(sched);
+  cudaFree(off);
+  cudaFree(work);
+  if (e != cudaSuccess) return cuda_fail(e, "wavefronts");
   for (int j = 0; j < n; ++j) order_out[j] &= 0xffffffu;
   return VIBE_OK;
 }

@@ -3,14 +3,17 @@
 // results as the image engine (vibe_bp.cu), which keeps a member's whole message image in shared
 // memory; a different layout.
 //
-// Mapping: one warp per (shot, member), one lane per edge. A sweep runs the member's steps (k_steps in
-// vibe_graph.cu): up to 32 edges of columns that share no check, packed in the member's order. A lane
-// asks its check's summary for the check-to-variable message of its edge, the lanes of a column pass
-// each other these messages with shuffles, and every lane forms its own exclusion sum and updates its
-// own check. In shot mode each warp decodes one shot at a time (persistent, shots from a global
-// counter), running the members one after another with the iteration budget of the correction limit
-// (Sec. III.D.2); in pair mode each warp takes one (shot, member) pair at a time, and the last member
-// of a shot to finish runs the shot's selection and epilogue.
+// Mapping: one warp, or for wide graphs a team of 8 (a CTA either way), per (shot, member), one lane per
+// edge. A sweep runs the
+// member's steps (k_steps in vibe_graph.cu): up to 32 edges per warp of columns that share no check, packed
+// in the member's order. A lane asks its check's summary for the check-to-variable message of its edge,
+// the lanes of a column pass each other these messages with shuffles, and every lane forms its own
+// exclusion sum and updates its own check. A team takes a unit of as many steps as it has warps at a
+// time, no two of which share a check, with a barrier after each unit. In shot mode each team decodes one
+// shot at a time (persistent, shots from a global counter), running the members one after another with
+// the iteration budget of the correction limit (Sec. III.D.2); in pair mode each team takes one (shot,
+// member) pair at a time, and the last member of a shot to finish runs the shot's selection and
+// epilogue. The first warp of a team runs that control flow and calls the others for each member.
 //
 // Check-node state: a summary per check in shared memory.
 //   m1 <= m2  the magnitudes of up to two "holder" edges of the row, with their positions p1, p2 inside
@@ -226,21 +229,37 @@ __device__ __forceinline__ void rescan_row(uint32_t addr, int b, int d, const ui
   if (lane == 0) Sum<MT>::rescanned(addr, r1, r2, r3, f1, f2);
 }
 
-// The part of a warp's shared memory that is not check summaries: what the steps near the current one
-// need. The edge records come in chunks of kChunk steps by cp.async, one chunk ahead; a 64-entry ring
-// holds the step offsets (two 32-step blocks, so that chunks can be fetched ahead across a block's end);
-// st has (signs, decisions, first slot of the next step) of the current block, read by all lanes of a
-// step at once.
-constexpr int kChunk = 4, kBufs = 2;
-constexpr int kChunkSlots = kChunk * 32 + 8;   // a chunk is copied in groups of four slots
+// What a warp's steps near the current one need: a window in shared memory. Its first 32 entries of 16
+// bytes are (signs, decisions, first slot of the step, end of its slots) of the warp's current block of
+// 32 steps, read by all lanes of a step at once. Then two buffers of edge records, which come in chunks of
+// four steps by cp.async, one chunk ahead, and two of their links. (Two steps per chunk cost 6 % and are
+// taken only where the window would not fit beside the summaries.) A chunk is copied in groups of four
+// slots.
+constexpr int kChunk = kStepChunk;
 
-struct XWin {
-  uint4 st[32];
-  uint2 rec[kBufs][kChunkSlots];
-  uint32_t lnk[kBufs][kChunkSlots];
-  uint32_t off[64];
+__host__ __device__ constexpr uint32_t chunk_slots(int chunk) { return (uint32_t)chunk * 32u + 8u; }
+__host__ __device__ constexpr uint32_t rec_at(int chunk, int buf) { return 512u + (uint32_t)buf * chunk_slots(chunk) * 8u; }
+__host__ __device__ constexpr uint32_t lnk_at(int chunk, int buf) {
+  return 512u + 2u * chunk_slots(chunk) * 8u + (uint32_t)buf * chunk_slots(chunk) * 4u;
+}
+__host__ __device__ constexpr uint32_t window_bytes(int chunk) { return lnk_at(chunk, 2); }
+static_assert(window_bytes(4) % 16 == 0 && window_bytes(2) % 16 == 0, "cp.async blocks are 16 bytes");
+
+// What the first warp of a team tells the others, and their common sums. It precedes the windows of the
+// team's warps in shared memory; the check summaries follow them.
+struct alignas(16) TeamCmd {
+  const Tables* t;
+  const uint32_t* syn;
+  const int* conv;
+  int go, i, nsyn, budget, soft, keep_last, K, M;
+  int stop;
+  int sum[kTeam];
 };
-static_assert(sizeof(XWin) % 16 == 0 && kChunkSlots % 4 == 0, "cp.async blocks are 16 bytes");
+
+__device__ __forceinline__ void team_sync(int W) {
+  if (W == 1) __syncwarp();
+  else __syncthreads();
+}
 
 __device__ __forceinline__ void cp_async_cg16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, 16;" ::"r"(dst), "l"(src) : "memory");
@@ -249,15 +268,13 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// Copies the records of the chunk of steps [s, s + kChunk) into buffer `buf` (one commit group, empty
-// past the last step). win: shared address of the window; first: the member's first slot in the tables.
-__device__ __forceinline__ void fetch_chunk(uint32_t win, int buf, int s, const uint2* rec, const uint32_t* lnk,
-                                            size_t first, int lane) {
-  const uint32_t off = win + (uint32_t)offsetof(XWin, off);
-  const size_t b = (first + lds32(off + 4 * (s & 63))) & ~(size_t)3, e = first + lds32(off + 4 * ((s + kChunk) & 63));
-  const uint32_t dr = win + (uint32_t)offsetof(XWin, rec) + (uint32_t)buf * (uint32_t)sizeof(XWin::rec[0]);
-  const uint32_t dl = win + (uint32_t)offsetof(XWin, lnk) + (uint32_t)buf * (uint32_t)sizeof(XWin::lnk[0]);
-  const int quads = (int)((e - b + 3) >> 2);
+// Copies the records of slots [sb, se) of a member into buffer `buf` (one commit group; none if empty).
+// win: shared address of the warp's window; first: the member's first slot in the tables.
+__device__ __forceinline__ void fetch_chunk(uint32_t win, int chunk, int buf, uint32_t sb, uint32_t se, const uint2* rec,
+                                            const uint32_t* lnk, size_t first, int lane) {
+  const size_t b = (first + sb) & ~(size_t)3, e = first + se;
+  const uint32_t dr = win + rec_at(chunk, buf), dl = win + lnk_at(chunk, buf);
+  const int quads = se > sb ? (int)((e - b + 3) >> 2) : 0;
   for (int q = lane; q < quads; q += 32) {
     cp_async_cg16(dr + 32 * q, rec + b + 4 * q);
     cp_async_cg16(dr + 32 * q + 16, rec + b + 4 * q + 2);
@@ -266,60 +283,76 @@ __device__ __forceinline__ void fetch_chunk(uint32_t win, int buf, int s, const 
   cp_async_commit();
 }
 
-// One sweep of a member over its ns steps. win: shared address of the warp's window (the summaries follow it); stg: (signs, decisions) of every
-// step in global scratch; LP: the posteriors go to lp. Returns the lane's change of the number of
-// unsatisfied checks.
-template <typename MT, int DP, bool LP>
+// One sweep of a member over its ns steps by warp w of a team of W. Of every kChunk * W consecutive steps
+// the warp has the kChunk from kChunk * w on; the j-th steps of all warps form a unit. win: shared address of the
+// warp's window; sums: of the summaries; stg: (signs, decisions) of every step in global scratch; LP: the
+// posteriors go to lp. Returns the lane's change of the number of unsatisfied checks.
+template <typename MT, int DP, bool LP, int chunk>
 __device__ __forceinline__ int sweep_x(const Tables& t, const uint32_t* soff, const int ns, const size_t first,
-                                       const uint32_t* rmap, const float alpha, const uint32_t win, MT* msg, uint2* stg,
-                                       float* lp, uint32_t& rescans, const int lane) {
-  const uint32_t sums = win + (uint32_t)sizeof(XWin), off = win + (uint32_t)offsetof(XWin, off);
+                                       const uint32_t* rmap, const float alpha, const uint32_t win, const uint32_t sums,
+                                       MT* msg, uint2* stg, float* lp, uint32_t& rescans, const int lane, const int W,
+                                       const int w) {
   const uint2* trec = t.xrec;
   const uint32_t* tlnk = t.xlnk;
   const int32_t* rowptr = t.rowptr;
-  const int pitch = t.soff_pitch;
+  const int J = ns / W;   // the warp's steps (with W > 1 ns is a multiple of kChunk * W)
   int dpar = 0;
-  uint32_t coff = __ldg(soff + lane), noff = __ldg(soff + 32 + lane);   // offsets of this block's steps and the next's
-  uint2 cst = lane < ns ? stg[lane] : make_uint2(0u, 0u), nst = cst;
-  sts32(off + 4 * lane, coff);
-  uint32_t ol = (uint32_t)lane;   // slot of the lane's edge
+  auto place = [&](int j) { return j / kChunk * kChunk * W + kChunk * w + j % kChunk; };
+  auto entry = [&](int j) {
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (j < J) {
+      const int q = place(j);
+      const uint2 x = stg[q];
+      v = make_uint4(x.x, x.y, __ldg(soff + q), __ldg(soff + q + 1));
+    }
+    return v;
+  };
+  uint4 cur = entry(lane), nxt = cur;
   int buf = 0;
-  for (int s0 = 0; s0 < ns; s0 += 32) {
-    // block of 32 steps: its states and the next block's offsets into the window, the loads for the next
-    sts32(off + 4 * (((s0 + 32) & 63) + lane), noff);
-    {
-      const uint32_t up = __shfl_down_sync(kFull, coff, 1), nx = __shfl_sync(kFull, noff, 0);
-      sts128(win + 16 * lane, make_uint4(cst.x, cst.y, lane == 31 ? nx : up, 0u));
-    }
+  for (int j0 = 0; j0 < J; j0 += 32) {
+    // block of 32 of the warp's steps
+    sts128(win + 16 * lane, cur);
     __syncwarp();
-    if (s0 == 0) fetch_chunk(win, 0, 0, trec, tlnk, first, lane);
-    coff = noff;
-    if (s0 + 32 < ns) {
-      noff = s0 + 64 + lane < pitch ? __ldg(soff + s0 + 64 + lane) : 0u;
-      nst = s0 + 32 + lane < ns ? stg[s0 + 32 + lane] : make_uint2(0u, 0u);
-    }
+    if (j0 == 0) fetch_chunk(win, chunk, 0, lds32(win + 8), lds32(win + 16 * (min(chunk, J) - 1) + 12), trec, tlnk, first, lane);
+    if (j0 + 32 < J) nxt = entry(j0 + 32 + lane);
+    const int jb = min(32, J - j0);
     uint32_t wst = win;   // the step's window entry
-    for (int s1 = s0; s1 < min(s0 + 32, ns); s1 += kChunk) {
+    for (int j1 = 0; j1 < jb; j1 += chunk) {
       // this chunk's records are here, the last one's buffer is free
       cp_async_wait<0>();
       __syncwarp();
-      fetch_chunk(win, buf ^ 1, s1 + kChunk, trec, tlnk, first, lane);
+      {
+        const int jn = j1 + chunk, left = J - j0 - jn;   // the next chunk and the steps from it on
+        const int le = min(chunk, left) - 1;
+        uint32_t sb = 0u, se = 0u;
+        if (left > 0) {
+          if (jn < 32) {
+            sb = lds32(win + 16 * jn + 8);
+            se = lds32(win + 16 * (jn + le) + 12);
+          } else {
+            sb = __shfl_sync(kFull, nxt.z, 0);
+            se = __shfl_sync(kFull, nxt.w, le);
+          }
+        }
+        fetch_chunk(win, chunk, buf ^ 1, sb, se, trec, tlnk, first, lane);
+      }
       // addresses of slot 0's records if the buffer reached back that far
-      const uint32_t o0 = ol - (uint32_t)lane, sh = (((uint32_t)first + o0) & 3u) - o0;
-      const uint32_t ra = win + (uint32_t)offsetof(XWin, rec) + (uint32_t)buf * (uint32_t)sizeof(XWin::rec[0]) + 8u * sh;
-      const uint32_t la = win + (uint32_t)offsetof(XWin, lnk) + (uint32_t)buf * (uint32_t)sizeof(XWin::lnk[0]) + 4u * sh;
+      const uint32_t o0 = lds32(wst + 8), sh = (((uint32_t)first + o0) & 3u) - o0;
+      const uint32_t ra = win + rec_at(chunk, buf) + 8u * sh, la = win + lnk_at(chunk, buf) + 4u * sh;
       buf ^= 1;
 #pragma unroll 1
-      for (int u = 0; u < kChunk; ++u) {   // steps past the last one have no edges
+      for (int u = 0; u < chunk; ++u) {   // steps past the last one have no edges
         const uint4 st = lds128(wst);
+        const uint32_t ol = st.z + (uint32_t)lane;   // slot of the lane's edge
         uint2 r = make_uint2(0u, 0u);
         uint32_t ln = 0u;
-        if (ol < st.z) {
+        if (ol < st.w) {
           r = lds64(ra + 8u * ol);
           ln = lds32(la + 4u * ol);
         }
         const bool act = (int)ln < 0;
-        const uint32_t sa = sums + (r.x >> 18) * (uint32_t)Sum<MT>::kBytes;
+        // lanes without an edge read their own window (a check could be another warp's in this unit)
+        const uint32_t sa = act ? sums + (r.x >> 18) * (uint32_t)Sum<MT>::kBytes : win;
         const uint32_t osg = st.x << (31 - lane);   // bit 31: sign of the edge's own old message
         Sum<MT> S;
         S.load(sa, r.x);
@@ -365,16 +398,15 @@ __device__ __forceinline__ int sweep_x(const Tables& t, const uint32_t* soff, co
         if (lane == 0) sts64(wst, make_uint2(sg, dec));
         if (LP) {
           if (ln & kLnkLast) lp[__ldg(t.xcolid + first + ol)] = L;
-          else if (ln == 0u && ol < st.z) lp[__ldg(t.xcolid + first + ol)] = __uint_as_float(r.y);   // no checks
+          else if (ln == 0u && ol < st.w) lp[__ldg(t.xcolid + first + ol)] = __uint_as_float(r.y);   // no checks
         }
-        ol = st.z + (uint32_t)lane;
         wst += 16u;
-        __syncwarp();
+        team_sync(W);
       }
     }
-    if (s0 + lane < ns) stg[s0 + lane] = lds64(win + 16 * lane);
+    if (j0 + lane < J) stg[place(j0 + lane)] = lds64(win + 16 * lane);
     __syncwarp();
-    cst = nst;
+    cur = nxt;
   }
   cp_async_wait<0>();
   return dpar;
@@ -388,6 +420,7 @@ struct MemberRun {
   bool soft, keep_last;  // the posterior after every sweep / after sweep T
   const int* conv;       // pair mode: the shot's converged members (pair_should_stop), else NULL
   int K, M;
+  int chunk;             // steps per chunk of records
   // results
   int ran;               // sweeps run
   uint32_t rescans;
@@ -397,17 +430,21 @@ struct MemberRun {
 // stopping at the first that leaves H e = s, or in pair mode before a sweep that no longer counts.
 // Returns the converging sweep (0 if none; its decisions are then in the warp's scratch, column order);
 // leaves the posterior of the last sweep in the scratch when soft output is on or `keep_last` is set
-// and the member reached sweep T. smem_off: the warp's shared memory; gs: its global scratch. Not
-// inlined: the sweep gets its own registers, whatever the caller keeps between members.
+// and the member reached sweep T. Called by all warps of the team (the block); gs: its global scratch.
+// Not inlined: the sweep gets its own registers, whatever the caller keeps between members.
 template <typename MT, int DP>
-__device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, int smem_off, unsigned char* gs) {
+__device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, unsigned char* gs) {
   extern __shared__ __align__(16) unsigned char smem[];
   // Both through a shuffle: the compiler would otherwise read the thread index again wherever the lane is
   // used and keep the addresses in uniform registers, moving them over at each use (14 of the 184
   // instructions of a step).
   const int lane = __shfl_sync(kFull, (int)(threadIdx.x & 31), (int)(threadIdx.x & 31));
-  const uint32_t win = __shfl_sync(kFull, (uint32_t)__cvta_generic_to_shared(smem) + (uint32_t)smem_off, lane);
-  const uint32_t sums = win + (uint32_t)sizeof(XWin);
+  const int W = (int)(blockDim.x >> 5), w = __shfl_sync(kFull, (int)(threadIdx.x >> 5), lane);
+  const int tid = 32 * w + lane, nt = 32 * W;
+  TeamCmd* cmd = reinterpret_cast<TeamCmd*>(smem);
+  const uint32_t wins = __shfl_sync(kFull, (uint32_t)__cvta_generic_to_shared(smem) + (uint32_t)sizeof(TeamCmd), lane);
+  const uint32_t win = wins + (uint32_t)w * window_bytes(R.chunk);
+  const uint32_t sums = wins + (uint32_t)W * window_bytes(R.chunk);
   const int m = t.m, T = t.T, nw = t.nw;
   MT* msg = reinterpret_cast<MT*>(gs + t.xg_msg);
   uint2* stg = reinterpret_cast<uint2*>(gs + t.xg_st);   // (signs, decisions) of every step
@@ -420,29 +457,55 @@ __device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, i
   const int ns = __ldg(t.stepcnt + i);
   // member init: prior summaries with this shot's syndrome (parity = s), prior messages in step order,
   // signs and decisions 0
-  for (int c = lane; c < m; c += 32)
+  for (int c = tid; c < m; c += nt)
     Sum<MT>::init(sums + c * Sum<MT>::kBytes, __ldg(t.xsum + c),
                   ((__ldg(syn + (c >> 5)) >> (c & 31)) & 1u) ? (kSgnBit | kParBit) : 0u);
-  for (int j = lane; j < t.SP; j += 32)
+  for (int j = tid; j < t.SP; j += nt)
     XMsg<MT>::store(msg + j, XMsg<MT>::round(__uint_as_float(__ldg(&t.xrec[first + j].y))));
-  for (int s = lane; s < ns; s += 32) stg[s] = make_uint2(0u, 0u);
-  __syncwarp();
+  for (int s = tid; s < ns; s += nt) stg[s] = make_uint2(0u, 0u);
+  team_sync(W);
   const float alpha = __ldg(t.alpha_m + i);   // member i's scaling factor
   const int budget = R.budget;
   int unsat = R.nsyn;
   int conv = 0, ran = 0;
   for (int it = 1; it <= budget; ++it) {
-    if (R.conv && pair_should_stop(R.conv, R.K, R.M, i, it, lane)) break;
+    if (R.conv) {   // one answer for the team: other members converge meanwhile
+      bool stop;
+      if (W == 1) {
+        stop = pair_should_stop(R.conv, R.K, R.M, i, it, lane);
+      } else {
+        if (w == 0) {
+          stop = pair_should_stop(R.conv, R.K, R.M, i, it, lane);
+          if (lane == 0) cmd->stop = stop;
+        }
+        __syncthreads();
+        stop = cmd->stop != 0;
+      }
+      if (stop) break;
+    }
     // the posterior is needed after the last possible sweep of a member that may end without
     // converging (LLR average) and, for soft output, after every sweep
     int dpar;
     float* lp = reinterpret_cast<float*>(gs + t.xg_lpost);
-    if (R.soft || (it == T && R.keep_last))
-      dpar = sweep_x<MT, DP, true>(t, soff, ns, first, rmap, alpha, win, msg, stg, lp, rescans, lane);
+    auto sweep = [&](auto with_lp, auto chunk) {
+      return sweep_x<MT, DP, decltype(with_lp)::value, decltype(chunk)::value>(t, soff, ns, first, rmap, alpha, win, sums,
+                                                                              msg, stg, lp, rescans, lane, W, w);
+    };
+    const bool with_lp = R.soft || (it == T && R.keep_last);
+    if (R.chunk == kChunk)
+      dpar = with_lp ? sweep(std::true_type{}, std::integral_constant<int, kChunk>{})
+                     : sweep(std::false_type{}, std::integral_constant<int, kChunk>{});
     else
-      dpar = sweep_x<MT, DP, false>(t, soff, ns, first, rmap, alpha, win, msg, stg, lp, rescans, lane);
+      dpar = with_lp ? sweep(std::true_type{}, std::integral_constant<int, 2>{})
+                     : sweep(std::false_type{}, std::integral_constant<int, 2>{});
 #pragma unroll
     for (int off = 16; off >= 1; off >>= 1) dpar += __shfl_xor_sync(kFull, dpar, off);
+    if (W > 1) {
+      if (lane == 0) cmd->sum[w] = dpar;
+      __syncthreads();
+      dpar = 0;
+      for (int q = 0; q < W; ++q) dpar += cmd->sum[q];
+    }
     unsat += dpar;
     ran = it;
     if (unsat == 0) { conv = it; break; }
@@ -451,9 +514,9 @@ __device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, i
   R.rescans = rescans;
   if (conv) {   // decisions in column order
     uint32_t* bits = reinterpret_cast<uint32_t*>(gs + t.xg_dec);
-    for (int w = lane; w < nw; w += 32) __stcg(bits + w, 0u);
-    __syncwarp();
-    for (int s = lane; s < ns; s += 32) {
+    for (int q = tid; q < nw; q += nt) __stcg(bits + q, 0u);
+    team_sync(W);
+    for (int s = tid; s < ns; s += nt) {
       uint32_t d = stg[s].y;
       const uint32_t o = __ldg(soff + s);
       while (d) {
@@ -462,9 +525,39 @@ __device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, i
         d &= d - 1u;
       }
     }
-    __syncwarp();
   }
+  team_sync(W);
   return conv;
+}
+
+// run_member_x by the team's first warp: hands the call to the others first.
+template <typename MT, int DP>
+__device__ __forceinline__ int team_member(const Tables& t, int i, MemberRun& R, unsigned char* gs) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  if (blockDim.x > 32) {
+    if (threadIdx.x == 0) {
+      TeamCmd* c = reinterpret_cast<TeamCmd*>(smem);
+      c->t = &t; c->syn = R.syn; c->conv = R.conv; c->go = 1; c->i = i; c->nsyn = R.nsyn; c->budget = R.budget;
+      c->soft = R.soft; c->keep_last = R.keep_last; c->K = R.K; c->M = R.M;
+    }
+    __syncthreads();
+  }
+  return run_member_x<MT, DP>(t, i, R, gs);
+}
+
+// The other warps of a team: run members until the first warp is done. Returns the rescans they made.
+template <typename MT, int DP>
+__device__ __forceinline__ uint32_t team_serve(unsigned char* gs) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const TeamCmd* c = reinterpret_cast<const TeamCmd*>(smem);
+  uint32_t rescans = 0;
+  for (;;) {
+    __syncthreads();
+    if (!c->go) return rescans;
+    MemberRun R{c->syn, c->nsyn, c->budget, c->soft != 0, c->keep_last != 0, c->conv, c->K, c->M, kChunk, 0, 0u};
+    run_member_x<MT, DP>(*c->t, c->i, R, gs);
+    rescans += R.rescans;
+  }
 }
 
 // W(e) = sum of lambda_j over e_j = 1, ascending j, of the decisions in dec (every lane folds the same
@@ -485,11 +578,11 @@ __device__ __forceinline__ float decision_weight(const Tables& t, const uint32_t
   return W;
 }
 
-// Decodes shot `shot` of problem t with one warp. smem_off: the warp's shared memory; gs: its global
+// Decodes shot `shot` of problem t with the team, driven by its first warp. gs: the team's global
 // scratch (messages, state words, decisions, posterior, LLR accumulator, candidate records).
 template <typename MT, int DP>
-__device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, uint32_t shot, int smem_off,
-                                              unsigned char* gs, int lane, uint32_t& my_iters,
+__device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, uint32_t shot, unsigned char* gs, int lane,
+                                              uint32_t& my_iters,
                                               uint32_t& my_shots, uint32_t& my_fail, uint32_t& my_rescans) {
   const int n = t.n, m = t.m, K = t.K, M = t.M, T = t.T, nw = t.nw, kw = t.kw, mw = t.mw;
   const uint32_t* dec = reinterpret_cast<const uint32_t*>(gs + t.xg_dec);
@@ -536,8 +629,8 @@ __device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, 
   for (int i = 0; i < K; ++i) {
     const int budget = ncand < M ? T : __shfl_sync(kFull, c_t, M - 1) - 1;
     if (budget <= 0) break;
-    MemberRun R{syn, nsyn, budget, a.want_soft != 0, ncand == 0, nullptr, K, M, 0, 0u};
-    const int conv = run_member_x<MT, DP>(t, i, R, smem_off, gs);
+    MemberRun R{syn, nsyn, budget, a.want_soft != 0, ncand == 0, nullptr, K, M, a.x_chunk, 0, 0u};
+    const int conv = team_member<MT, DP>(t, i, R, gs);
     my_iters += (uint32_t)R.ran;
     my_rescans += R.rescans;
     if (conv) {
@@ -616,11 +709,11 @@ __device__ __forceinline__ void decode_shot_x(const BpArgs& a, const Tables& t, 
   __syncwarp();
 }
 
-// Pair mode: member i of shot `shot` (slot `slot` of the chunk) with one warp; the last member of the
+// Pair mode: member i of shot `shot` (slot `slot` of the chunk) with the team; the last member of the
 // shot to finish writes the shot's outcome (pair_epilogue, vibe_internal.cuh).
 template <typename MT, int DP>
 __device__ __forceinline__ void decode_pair_x(const BpArgs& a, const Tables& t, uint32_t shot, int slot, int i,
-                                              int smem_off, unsigned char* gs, int lane, uint32_t& my_iters,
+                                              unsigned char* gs, int lane, uint32_t& my_iters,
                                               uint32_t& my_shots, uint32_t& my_fail, uint32_t& my_rescans) {
   const int K = t.K, M = t.M, T = t.T, n = t.n, m = t.m, mw = t.mw, nw = t.nw, kw = t.kw;
   if (i >= K) return;
@@ -656,8 +749,8 @@ __device__ __forceinline__ void decode_pair_x(const BpArgs& a, const Tables& t, 
   const uint32_t* dec = reinterpret_cast<const uint32_t*>(gs + t.xg_dec);
   float* lpost = reinterpret_cast<float*>(gs + t.xg_lpost);
   int* conv = a.pconv + (size_t)slot * a.pair_K;
-  MemberRun R{syn, nsyn, T, a.want_soft != 0, true, conv, K, M, 0, 0u};
-  const int cv = run_member_x<MT, DP>(t, i, R, smem_off, gs);
+  MemberRun R{syn, nsyn, T, a.want_soft != 0, true, conv, K, M, a.x_chunk, 0, 0u};
+  const int cv = team_member<MT, DP>(t, i, R, gs);
   my_iters += (uint32_t)R.ran;
   my_rescans += R.rescans;
   const size_t rec = (size_t)slot * a.pair_K + i;
@@ -677,20 +770,17 @@ __device__ __forceinline__ void decode_pair_x(const BpArgs& a, const Tables& t, 
   __syncwarp();
 }
 
-// Blocks (one warp each) per SM the register budget targets: 128 registers, with which the sweep spills
-// nothing. (24 blocks and 80 registers spill inside it and are no faster: the engine waits on latencies.)
-constexpr int kMinBlocksX = 16 / kBpxWarpsPerCta;
-
 // MIXED: shots name their problems (dem_of_shot); the descriptors are copied to shared memory after
-// the warps' regions and shots of image-engine problems are left to that kernel. Otherwise every shot
-// decodes a.one from the parameter space.
+// the team's region, and shots of image-engine problems or of another team size are left to their
+// launches. Otherwise every shot decodes a.one from the parameter space. The register budget is 128, with
+// which the sweep spills nothing. (80 registers spill inside it and are no faster: the engine waits on
+// latencies.)
 template <typename MT, int DP, bool MIXED>
-__global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const __grid_constant__ BpArgs a) {
+__global__ void __launch_bounds__(kTeam * 32, 2) k_bpx(const __grid_constant__ BpArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31;
-  const int wcta = threadIdx.x >> 5;
-  const long long gw = (long long)blockIdx.x * kBpxWarpsPerCta + wcta;
-  Tables* sdem = reinterpret_cast<Tables*>(smem + (size_t)kBpxWarpsPerCta * a.bnd.x_warp_smem);
+  const int W = (int)(blockDim.x >> 5);
+  Tables* sdem = reinterpret_cast<Tables*>(smem + (size_t)a.x_team_smem);
   if (MIXED) {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(a.dems);
     uint32_t* dst = reinterpret_cast<uint32_t*>(sdem);
@@ -698,9 +788,13 @@ __global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const
     for (int q = threadIdx.x; q < words; q += blockDim.x) dst[q] = __ldg(src + q);
     __syncthreads();
   }
-  const int smem_off = wcta * a.bnd.x_warp_smem;
-  unsigned char* gs = a.xscratch + gw * a.xscratch_pitch;
+  unsigned char* gs = a.xscratch + (long long)blockIdx.x * a.xscratch_pitch;
   uint32_t my_iters = 0, my_shots = 0, my_fail = 0, my_rescans = 0;   // flushed before they could wrap
+  if (threadIdx.x >= 32) {
+    my_rescans = team_serve<MT, DP>(gs);
+    if (lane == 0 && a.counters && my_rescans) atomicAdd(a.counters + VIBE_CNT_RESCANS, (unsigned long long)my_rescans);
+    return;
+  }
 
   if (a.pair_mode) {
     const unsigned long long npairs = (unsigned long long)a.nshots * (unsigned long long)a.pair_K;
@@ -729,10 +823,10 @@ __global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const
           }
           continue;
         }
-        if (sdem[di].engine != VIBE_ENGINE_SUMMARY) continue;   // left to the image engine
-        decode_pair_x<MT, DP>(a, sdem[di], shot, (int)shot, i, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+        if (sdem[di].engine != VIBE_ENGINE_SUMMARY || sdem[di].team != W) continue;   // left to another launch
+        decode_pair_x<MT, DP>(a, sdem[di], shot, (int)shot, i, gs, lane, my_iters, my_shots, my_fail, my_rescans);
       } else {
-        decode_pair_x<MT, DP>(a, a.one, shot, (int)shot, i, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+        decode_pair_x<MT, DP>(a, a.one, shot, (int)shot, i, gs, lane, my_iters, my_shots, my_fail, my_rescans);
       }
     }
   }
@@ -770,11 +864,15 @@ __global__ void __launch_bounds__(kBpxWarpsPerCta * 32, kMinBlocksX) k_bpx(const
         }
         continue;
       }
-      if (sdem[di].engine != VIBE_ENGINE_SUMMARY) continue;   // left to the image engine
-      decode_shot_x<MT, DP>(a, sdem[di], shot, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+      if (sdem[di].engine != VIBE_ENGINE_SUMMARY || sdem[di].team != W) continue;   // left to another launch
+      decode_shot_x<MT, DP>(a, sdem[di], shot, gs, lane, my_iters, my_shots, my_fail, my_rescans);
     } else {
-      decode_shot_x<MT, DP>(a, a.one, shot, smem_off, gs, lane, my_iters, my_shots, my_fail, my_rescans);
+      decode_shot_x<MT, DP>(a, a.one, shot, gs, lane, my_iters, my_shots, my_fail, my_rescans);
     }
+  }
+  if (W > 1) {
+    if (lane == 0) reinterpret_cast<TeamCmd*>(smem)->go = 0;
+    __syncthreads();
   }
   if (lane == 0 && a.counters) {
     atomicAdd(a.counters + VIBE_CNT_SHOTS, (unsigned long long)my_shots);
@@ -799,22 +897,22 @@ cudaError_t prefer_shared() {
 }
 
 template <typename MT, int DP, bool MIXED>
-cudaError_t launch_x(const BpArgs& a, int grid, size_t smem, cudaStream_t s) {
+cudaError_t launch_x(const BpArgs& a, int grid, int team, size_t smem, cudaStream_t s) {
   cudaError_t err = prefer_shared<MT, DP, MIXED>();
   if (err != cudaSuccess) return err;
   err = ensure_dyn_smem<k_bpx<MT, DP, MIXED>>(smem);
   if (err != cudaSuccess) return err;
-  k_bpx<MT, DP, MIXED><<<grid, kBpxWarpsPerCta * 32, smem, s>>>(a);
+  k_bpx<MT, DP, MIXED><<<grid, team * 32, smem, s>>>(a);
   return cudaGetLastError();
 }
 
 template <typename MT, int DP, bool MIXED>
-cudaError_t occupancy_x(size_t smem, int* out) {
+cudaError_t occupancy_x(size_t smem, int team, int* out) {
   cudaError_t err = prefer_shared<MT, DP, MIXED>();
   if (err != cudaSuccess) return err;
   err = ensure_dyn_smem<k_bpx<MT, DP, MIXED>>(smem);
   if (err != cudaSuccess) return err;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bpx<MT, DP, MIXED>, kBpxWarpsPerCta * 32, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bpx<MT, DP, MIXED>, team * 32, smem);
 }
 
 template <typename Fn>
@@ -829,21 +927,21 @@ cudaError_t by_xd(int XD, Fn&& f) {
 }
 
 template <typename MT>
-cudaError_t launch_x_mt(const BpArgs& a, int grid, cudaStream_t s) {
+cudaError_t launch_x_mt(const BpArgs& a, int grid, int team, cudaStream_t s) {
   const bool mixed = a.dem_of_shot != nullptr;
-  const size_t smem = bpx_cta_smem_bytes(a.bnd, mixed ? a.ndem : 0);
+  const size_t smem = bpx_cta_smem_bytes(a.bnd, team, mixed ? a.ndem : 0);
   return by_xd(a.bnd.XD, [&](auto dp) {
-    if (mixed) return launch_x<MT, decltype(dp)::value, true>(a, grid, smem, s);
-    return launch_x<MT, decltype(dp)::value, false>(a, grid, smem, s);
+    if (mixed) return launch_x<MT, decltype(dp)::value, true>(a, grid, team, smem, s);
+    return launch_x<MT, decltype(dp)::value, false>(a, grid, team, smem, s);
   });
 }
 
 template <typename MT>
-cudaError_t occupancy_x_mt(const Bounds& b, int ndem, int* out) {
-  const size_t smem = bpx_cta_smem_bytes(b, ndem);
+cudaError_t occupancy_x_mt(const Bounds& b, int team, int ndem, int* out) {
+  const size_t smem = bpx_cta_smem_bytes(b, team, ndem);
   return by_xd(b.XD, [&](auto dp) {
-    if (ndem > 0) return occupancy_x<MT, decltype(dp)::value, true>(smem, out);
-    return occupancy_x<MT, decltype(dp)::value, false>(smem, out);
+    if (ndem > 0) return occupancy_x<MT, decltype(dp)::value, true>(smem, team, out);
+    return occupancy_x<MT, decltype(dp)::value, false>(smem, team, out);
   });
 }
 
@@ -852,8 +950,6 @@ cudaError_t occupancy_x_mt(const Bounds& b, int ndem, int* out) {
 int bpx_degree_bucket(int maxcol) {
   return maxcol <= 4 ? 4 : maxcol <= 6 ? 6 : maxcol <= 8 ? 8 : maxcol <= 16 ? 16 : 0;
 }
-
-int bpx_window_bytes() { return (int)sizeof(XWin); }
 
 int bpx_summary_bytes(int m, int msg_fp16) { return (int)a16((msg_fp16 ? 8 : 16) * (size_t)m); }
 
@@ -869,16 +965,29 @@ void bpx_layout(Tables* t, int msg_fp16) {
   t->x_warp_scratch = g;
 }
 
-size_t bpx_cta_smem_bytes(const Bounds& b, int ndem) {
-  return (size_t)kBpxWarpsPerCta * b.x_warp_smem + a16((size_t)ndem * sizeof(Tables));
+static size_t team_smem(const Bounds& b, int team, int chunk) {
+  return sizeof(TeamCmd) + (size_t)team * window_bytes(chunk) + (size_t)b.x_sums[team_class(team)];
 }
 
-cudaError_t launch_bpx(const BpArgs& a, int msg_fp16, int grid, cudaStream_t s) {
-  return msg_fp16 ? launch_x_mt<__half>(a, grid, s) : launch_x_mt<float>(a, grid, s);
+// Steps per chunk: kChunk, or for single warps 2 where only that fits beside the summaries and descriptors.
+static int bpx_chunk(const Bounds& b, int team, int ndem) {
+  const size_t limit = 227u * 1024u;   // shared memory of a CTA on sm_103a
+  return team == 1 && team_smem(b, team, kChunk) + a16((size_t)ndem * sizeof(Tables)) > limit ? 2 : kChunk;
 }
 
-cudaError_t bpx_occupancy(const Bounds& b, int ndem, int msg_fp16, int* blocks_per_sm) {
-  return msg_fp16 ? occupancy_x_mt<__half>(b, ndem, blocks_per_sm) : occupancy_x_mt<float>(b, ndem, blocks_per_sm);
+size_t bpx_cta_smem_bytes(const Bounds& b, int team, int ndem) {
+  return team_smem(b, team, bpx_chunk(b, team, ndem)) + a16((size_t)ndem * sizeof(Tables));
+}
+
+cudaError_t launch_bpx(const BpArgs& a0, int team, int msg_fp16, int grid, cudaStream_t s) {
+  BpArgs a = a0;
+  a.x_chunk = bpx_chunk(a.bnd, team, a.dem_of_shot ? a.ndem : 0);
+  a.x_team_smem = (int)team_smem(a.bnd, team, a.x_chunk);
+  return msg_fp16 ? launch_x_mt<__half>(a, grid, team, s) : launch_x_mt<float>(a, grid, team, s);
+}
+
+cudaError_t bpx_occupancy(const Bounds& b, int team, int ndem, int msg_fp16, int* blocks_per_sm) {
+  return msg_fp16 ? occupancy_x_mt<__half>(b, team, ndem, blocks_per_sm) : occupancy_x_mt<float>(b, team, ndem, blocks_per_sm);
 }
 
 }  // namespace vibe

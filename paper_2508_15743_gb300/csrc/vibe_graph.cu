@@ -1,12 +1,12 @@
 // K0 -- Tanner-graph builder (offline setup, Sec. III.D.1).
 //
 // From the CSR of H it builds, on the device: the CSC of H (checks ascending per column), the packed
-// per-column edge table csc_ent used by the BP kernel, the padded message image (prior LLR of each
-// edge's column, +inf padding), and for every ensemble member the dependency wavefronts of its
-// serial schedule: level(v) = 1 + max{level(u) : u before v in the member's order, u and v share a
-// check}. Columns of one level touch disjoint checks, so updating a level in any order gives the
-// same floats as the serial order of Algorithm 1 (serial branch). The kernels run each member's
-// order packed into steps of 32 edges (k_steps).
+// per-column edge table csc_ent of the flooding and layered sweeps, the padded message image (prior LLR of
+// each edge's column, +inf padding), and for every ensemble member its serial schedule packed into steps
+// of 32 edges (k_steps): columns of one step touch disjoint checks and columns that share a check keep
+// their order, so the steps give the same floats as the serial order of Algorithm 1 (serial branch). The
+// dependency wavefronts, level(v) = 1 + max{level(u) : u before v in the member's order, u and v share a
+// check}, are found on request (member_levels).
 #include "vibe_internal.cuh"
 
 namespace vibe {
@@ -186,23 +186,39 @@ __global__ void k_levels(const uint32_t* __restrict__ perm, int n, int m, int K,
 // its size, and rounding each level up to whole warps leaves lanes idle. On random orders of the d=9
 // phenomenological problem the levels make 79 warps of edges and the steps 62 (E / 32 = 60.8); on
 // circuit-level d=11 4887 and 4407 (4371).
+// With a team of W > 1 warps (summary engine) W consecutive steps form a unit that shares no check, and
+// the steps are numbered so that a warp's steps of kStepChunk consecutive units are neighbours: their
+// records are copied together. Step u of the packing is number team_place(u); the count is rounded up to
+// whole groups of kStepChunk * W.
 // slot[v] = step << 5 | first lane, nstep = number of steps, off[s] = edges before step s (s <= nstep).
 // The search looks at 64 windows of 32 steps; past them it opens a new step at the end, which bounds the
 // work per column. lo (lane d - 1: degree d) skips the steps known to have no room for that degree.
 constexpr int kStepWindows = 64;
 
+__device__ __forceinline__ uint32_t team_place(uint32_t x, uint32_t W) {
+  if (W == 1u) return x;
+  const uint32_t unit = x / W;
+  return unit / kStepChunk * kStepChunk * W + (x % W) * kStepChunk + unit % kStepChunk;
+}
+__device__ __forceinline__ uint32_t team_unplace(uint32_t s, uint32_t W) {
+  if (W == 1u) return s;
+  const uint32_t group = kStepChunk * W, q = s % group;
+  return (s / group * kStepChunk + q % kStepChunk) * W + q / kStepChunk;
+}
+
 __global__ void k_steps(const uint32_t* __restrict__ perm, int n, int m, const int32_t* __restrict__ colptr,
                         const uint32_t* __restrict__ cpos, int room_in_smem, uint32_t* __restrict__ slot,
-                        uint32_t* __restrict__ off, int32_t* __restrict__ nstep, uint8_t* __restrict__ room_g) {
+                        uint32_t* __restrict__ off, int32_t* __restrict__ nstep, uint8_t* __restrict__ room_g, int cap,
+                        int off_pitch, uint32_t W) {
   extern __shared__ uint32_t sh[];
   uint32_t* nxt = sh;                       // m: first step allowed at each check
   uint32_t* stage = sh + m;                 // 32 x kMaxColDeg: checks of the 32 columns in work
   uint8_t* room = room_in_smem ? reinterpret_cast<uint8_t*>(stage + 32 * kMaxColDeg)
-                               : room_g + (size_t)blockIdx.x * n;   // free lanes of each step
+                               : room_g + (size_t)blockIdx.x * cap;   // free lanes of each step
   const int lane = threadIdx.x;
   perm += (size_t)blockIdx.x * n;
   slot += (size_t)blockIdx.x * n;
-  off += (size_t)blockIdx.x * (n + 1);
+  off += (size_t)blockIdx.x * off_pitch;
   for (int c = lane; c < m; c += 32) nxt[c] = 0u;
   uint32_t lo = 0u;
   uint32_t ns = 0u;
@@ -237,32 +253,36 @@ __global__ void k_steps(const uint32_t* __restrict__ perm, int n, int m, const i
           s += 32u;
         }
       }
-      if (!found) s = ns;
+      if (!found) s = max(ns, s0);
       else if (s0 <= lod && lane == (int)need - 1) lo = s;
       const uint32_t r = s < ns ? room[s] : 32u;
-      if (lane == j) mine = (s << 5) | (32u - r);
+      if (lane == j) mine = (team_place(s, W) << 5) | (32u - r);
       __syncwarp();
-      if (lane == 0) room[s] = (uint8_t)(r - need);
+      if (lane == 0) {
+        for (uint32_t x = ns; x < s; ++x) room[x] = 32u;   // the rest of a unit may stay empty
+        room[s] = (uint8_t)(r - need);
+      }
       ns = max(ns, s + 1u);
-      if (lane < dj) nxt[c] = s + 1u;
+      if (lane < dj) nxt[c] = (s / W + 1u) * W;
       __syncwarp();
     }
     if (lane < cnt) slot[v] = mine;
   }
   uint32_t run = 0u;
-  for (uint32_t s0 = 0; s0 <= ns; s0 += 32) {
-    const uint32_t x = s0 + lane;
-    const uint32_t u = x < ns ? 32u - room[x] : 0u;
+  const uint32_t group = kStepChunk * W, total = W == 1u ? ns : (ns + group - 1u) / group * group;
+  for (uint32_t s0 = 0; s0 <= total; s0 += 32) {
+    const uint32_t x = s0 + lane, px = team_unplace(x, W);
+    const uint32_t u = x < total && px < ns ? 32u - room[px] : 0u;
     uint32_t inc = u;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t y = __shfl_up_sync(kFull, inc, o);
       if (lane >= o) inc += y;
     }
-    if (x <= ns) off[x] = run + inc - u;
+    if (x <= total) off[x] = run + inc - u;
     run += __shfl_sync(kFull, inc, 31);
   }
-  if (lane == 0) nstep[blockIdx.x] = (int32_t)ns;
+  if (lane == 0) nstep[blockIdx.x] = (int32_t)total;
 }
 
 // Column of each edge slot (only the slots of first edges are written, and read).
@@ -482,10 +502,9 @@ __global__ void k_layers(const int32_t* __restrict__ rowptr, const int32_t* __re
 
 cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m, int n, int E, int K,
                          const uint32_t* d_perm, int RP, int DP, int msg_fp16, const float* d_lam, int32_t* d_colptr,
-                         int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init,
-                         uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, float4* d_xsum, int32_t* d_scratch,
-                         cudaStream_t s) {
-  // scratch layout: cnt[n] | fill[n]; later reused by k_levels (K*(m+3n+1))
+                         int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init, float4* d_xsum,
+                         int32_t* d_scratch, cudaStream_t s) {
+  // scratch layout: cnt[n] | fill[n]
   cudaError_t err;
   int32_t* cnt = d_scratch;
   int32_t* fill = cnt + n;
@@ -503,26 +522,42 @@ cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m
     k_msg_init<float><<<grid_for((long long)m * RP, 256), 256, 0, s>>>(d_rowptr, d_colidx, m, RP, d_lam,
                                                                       static_cast<float*>(d_msg_init));
   }
-  k_levels<<<(K + 31) / 32, 32, 0, s>>>(d_perm, n, m, K, d_colptr, d_rowidx, d_sched, d_lvl_off, d_nlev, d_scratch);
   return cudaGetLastError();
 }
 
-cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
-                        int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s) {
+cudaError_t member_levels(const uint32_t* d_perm, int n, int m, const int32_t* d_colptr, const int32_t* d_rowidx,
+                          uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, int32_t* d_scratch, cudaStream_t s) {
+  k_levels<<<1, 32, 0, s>>>(d_perm, n, m, 1, d_colptr, d_rowidx, d_sched, d_lvl_off, d_nlev, d_scratch);
+  return cudaGetLastError();
+}
+
+// Steps a member can have: one per column, in units of `team`, rounded up to whole groups.
+static int step_cap(int n, int team) {
+  const int group = kStepChunk * team;
+  return team == 1 ? n : (n * team + group - 1) / group * group;
+}
+
+cudaError_t build_steps(int m, int n, int K, int team, const uint32_t* d_perm, const int32_t* d_colptr,
+                        const uint32_t* d_cpos, int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s) {
+  const int cap = step_cap(n, team);
   uint32_t* slot = reinterpret_cast<uint32_t*>(d_scratch);
   uint32_t* off = slot + (size_t)K * n;
-  uint8_t* room = reinterpret_cast<uint8_t*>(off + (size_t)K * (n + 1));
+  uint8_t* room = reinterpret_cast<uint8_t*>(off + (size_t)K * (cap + 1));
   // m <= 16384 checks take 64 KB at most; the free-lane bytes follow when they fit too
-  const size_t fixed = 4 * ((size_t)m + 32 * kMaxColDeg), bytes = (size_t)n;
-  const bool room_in_smem = fixed + bytes <= 160u * 1024u;
-  const size_t smem = fixed + (room_in_smem ? bytes : 0);
+  const size_t fixed = 4 * ((size_t)m + 32 * kMaxColDeg);
+  const bool room_in_smem = fixed + (size_t)cap <= 160u * 1024u;
+  const size_t smem = fixed + (room_in_smem ? (size_t)cap : 0);
   cudaError_t err = ensure_dyn_smem<k_steps>(smem);
   if (err != cudaSuccess) return err;
-  k_steps<<<K, 32, smem, s>>>(d_perm, n, m, d_colptr, d_cpos, room_in_smem ? 1 : 0, slot, off, d_nstep, room);
+  k_steps<<<K, 32, smem, s>>>(d_perm, n, m, d_colptr, d_cpos, room_in_smem ? 1 : 0, slot, off, d_nstep, room, cap, cap + 1,
+                              (uint32_t)team);
   return cudaGetLastError();
 }
 
-size_t step_scratch_ints(int n, int K) { return (size_t)K * (2 * (size_t)n + 1) + ((size_t)K * n + 3) / 4; }
+size_t step_scratch_ints(int n, int K, int team) {
+  const size_t cap = step_cap(n, team);
+  return (size_t)K * (n + cap + 1) + ((size_t)K * cap + 3) / 4;
+}
 
 cudaError_t order_steps(int n, int SP, int K, int nstep, const int32_t* d_colptr, const uint32_t* d_cpos,
                         const int32_t* d_nstep, int32_t* d_scratch, uint32_t* d_tmp, cudaStream_t s) {
@@ -534,13 +569,13 @@ cudaError_t order_steps(int n, int SP, int K, int nstep, const int32_t* d_colptr
   return cudaGetLastError();
 }
 
-cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
+cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int team, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
                        const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
                        uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,
                        cudaStream_t s) {
   const uint32_t* slot = reinterpret_cast<const uint32_t*>(d_scratch);
   const uint32_t* off = slot + (size_t)K * n;
-  const int off_pitch = n + 1;
+  const int off_pitch = step_cap(n, team) + 1;
   k_step_offsets<<<grid_for((long long)K * pitch, 256), 256, 0, s>>>(off, off_pitch, d_nstep, K, pitch, d_soff);
   k_step_fill<<<grid_for((long long)K * n, 256), 256, 0, s>>>(slot, off, off_pitch, n, (long long)K * n, E, SP, d_rowptr,
                                                               d_colptr, d_cpos, d_lam, d_xrec, d_xlnk, d_xcolid, d_xrmap, DP > 16);

@@ -12,7 +12,7 @@
 namespace vibe {
 
 constexpr int kBpWarpsPerCta = 2;   // image engine: warps per CTA, one shot per warp
-constexpr int kBpxWarpsPerCta = 1;  // summary engine: warps per CTA, one shot per warp
+constexpr int kTeamClasses = 2;     // summary engine: teams of 1 or 8 warps (one CTA and one shot each)
 constexpr int kLsdThreads = 128;    // LSD kernel: default threads per CTA (64, 128 or 256), one shot per CTA
 constexpr int kMaxRowDeg = 255;     // position of an edge inside its check row fits in 8 bits
 constexpr int kMaxColDeg = 32;
@@ -25,7 +25,10 @@ constexpr uint32_t kInfBits = 0x7f800000u;
 // columns have more than 16 checks (DP 32, image engine only): first lane | k << 5 | degree - 1 << 10.
 constexpr int kLnkLastLane = 21;
 constexpr uint32_t kLnkLast = 1u << 30, kLnkEdge = 1u << 31;   // the record is the last edge's; it has a check
-constexpr int kStepPad = 66;            // step offsets kept past a member's last step (the kernels look ahead)
+constexpr int kTeam = 8;
+inline int team_class(int team) { return team > 1 ? 1 : 0; }
+constexpr int kStepChunk = 4;           // consecutive steps whose records are copied together
+constexpr int kStepPad = 8;             // step offsets kept past a member's last step (the kernels look ahead)
 
 // Position of slot `slot` of check row c inside the message image. A row is RP slots stored as
 // 16-byte chunks of `spc` slots (4 for float, 8 for half). When the row has 2, 4 or 8 chunks their
@@ -66,6 +69,7 @@ struct Tables {
   // the engine cannot run the problem), shared memory of one warp (the m check summaries, bytes) and the
   // parts of one warp's global scratch (bytes, 16-aligned)
   int XD, x_warp_smem;   // x_warp_smem: the m check summaries only
+  int team;              // warps that take a member's steps together
   int SP;                // edge slots of one member's sweep: E, and one per column without checks
   int nstep, soff_pitch; // largest step count of a member; entries per member of soff
   // xg_cpost = x_warp_scratch: the M*n candidate posteriors (soft output only) follow the fixed part
@@ -78,9 +82,6 @@ struct Tables {
   const float* lam;        // n prior LLRs
   const float* alpha_m;    // K scaling factors, member i's in alpha_m[i]
   const void* msg_init;    // m*RP messages (float or half): lambda of the edge's column, +inf padding
-  const uint32_t* sched;   // K*n: column | (degree << 24), grouped by wavefront level
-  const uint32_t* lvl_off; // K*(n+1): level offsets into sched
-  const int32_t* nlev;     // K level counts
   const int32_t* lrowptr;  // L CSR
   const int32_t* lcolidx;
   // layered schedule (only when n_layered > 0)
@@ -88,9 +89,10 @@ struct Tables {
   const int32_t* layer_chk;   // m checks grouped by layer, ascending within a layer
   const int32_t* layer_vptr;  // nlayer+1 offsets into layer_var
   const int32_t* layer_var;   // E: per layer, the columns of its checks in layer_chk order (each at most once)
-  // the steps of each member's sweep (k_steps). Step s of member i holds the edge slots
-  // soff[i][s] .. soff[i][s+1] (at most 32, one lane each; the checks of a step are distinct), the edges
-  // of a column in consecutive slots.
+  // the steps of each member's sweep (k_steps). Step s of member i holds the edge slots soff[i][s] ..
+  // soff[i][s+1] (at most 32, one lane each; the checks of a step are distinct), the edges of a column in
+  // consecutive slots. With a team of W > 1 warps the steps come in groups of kStepChunk * W, step
+  // kStepChunk * w + u of a group being warp w's part of the group's unit u; the checks of a unit are distinct.
   // xrec[i][slot] = (check << 18 | position of the edge in the check's CSR row, prior LLR), xlnk its links
   const int32_t* stepcnt;  // K step counts
   const uint32_t* soff;    // K * soff_pitch
@@ -107,8 +109,8 @@ struct Bounds {
   int RP;          // common row pitch if all problems share it, else 0
   int warp_smem;   // largest BP per-warp layout
   int lsd_order;   // largest LSD order
-  int x_warp_smem;    // summary-engine shared memory per warp: the step window and the largest problem's
-                      // check summaries (0 if no problem uses that engine)
+  int x_sums[kTeamClasses];   // largest check summaries of the summary-engine problems with that team size
+  int teams;          // bit per team class with a problem
   long long x_warp_scratch;   // largest summary-engine global scratch per warp, bytes
   int global_st;   // some image-engine problem keeps its step words in global scratch
   int engines;     // bit 0: some problem uses the image engine, bit 1: the summary engine
@@ -150,6 +152,8 @@ struct BpArgs {
   // summary engine, per-warp global scratch (Tables::xg_* offsets); pitch in bytes
   unsigned char* xscratch;
   long long xscratch_pitch;
+  int x_team_smem;             // shared memory of a team without the descriptors (set by launch_bpx)
+  int x_chunk;                 // steps whose records a warp copies together (set by launch_bpx)
   unsigned int* next_shot_x;   // the summary engine's own shot counter
   // pair mode (one warp per (shot, member) pair; see pair_epilogue): when pair_mode is set, pairs
   // q = shot * pair_K + member are taken from next_pair (image engine) or next_pair_x (summary
@@ -403,19 +407,22 @@ int set_error(int code, const char* msg);
 // check's CSR row.
 cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m, int n, int E, int K,
                          const uint32_t* d_perm, int RP, int DP, int msg_fp16, const float* d_lam, int32_t* d_colptr,
-                         int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init,
-                         uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, float4* d_xsum, int32_t* d_scratch,
-                         cudaStream_t s);
-// Packs each member's order into steps (K step counts in d_nstep); fill_steps then writes the resident
+                         int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init, float4* d_xsum,
+                         int32_t* d_scratch, cudaStream_t s);
+// The dependency levels of one member's order: columns grouped by level (column | degree << 24), n + 1
+// offsets, the level count; scratch: m + 3n + 1 ints.
+cudaError_t member_levels(const uint32_t* d_perm, int n, int m, const int32_t* d_colptr, const int32_t* d_rowidx,
+                          uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, int32_t* d_scratch, cudaStream_t s);
+// Packs each member's order into steps for teams of `team` warps (K step counts in d_nstep); fill_steps then writes the resident
 // tables from the same scratch (step_scratch_ints).
-size_t step_scratch_ints(int n, int K);
-cudaError_t build_steps(int m, int n, int K, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
+size_t step_scratch_ints(int n, int K, int team);
+cudaError_t build_steps(int m, int n, int K, int team, const uint32_t* d_perm, const int32_t* d_colptr, const uint32_t* d_cpos,
                         int32_t* d_nstep, int32_t* d_scratch, cudaStream_t s);
 // Orders the columns of each step over its lanes against bank conflicts (slot and off in the scratch;
 // tmp: K * SP words).
 cudaError_t order_steps(int n, int SP, int K, int nstep, const int32_t* d_colptr, const uint32_t* d_cpos,
                         const int32_t* d_nstep, int32_t* d_scratch, uint32_t* d_tmp, cudaStream_t s);
-cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
+cudaError_t fill_steps(int n, int E, int SP, int K, int DP, int team, int pitch, const int32_t* d_rowptr, const int32_t* d_colptr,
                        const uint32_t* d_cpos, const float* d_lam, const int32_t* d_nstep, const int32_t* d_scratch,
                        uint32_t* d_soff, uint2* d_xrec, uint32_t* d_xlnk, uint32_t* d_xcolid, uint32_t* d_xrmap,
                        cudaStream_t s);
@@ -437,12 +444,11 @@ cudaError_t bp_occupancy(const Bounds& b, int ndem, int msg_fp16, int* blocks_pe
 
 // K1': summary-engine BP + ensemble selection (vibe_bpx.cu)
 int bpx_degree_bucket(int maxcol);          // XD for a largest column degree (0: above 16)
-int bpx_window_bytes();                      // per-warp shared memory of the step window
 int bpx_summary_bytes(int m, int msg_fp16);  // shared memory of one warp's check summaries
 void bpx_layout(Tables* t, int msg_fp16);    // fills t's xg_* fields
-size_t bpx_cta_smem_bytes(const Bounds& b, int ndem);
-cudaError_t launch_bpx(const BpArgs& a, int msg_fp16, int grid, cudaStream_t s);
-cudaError_t bpx_occupancy(const Bounds& b, int ndem, int msg_fp16, int* blocks_per_sm);
+size_t bpx_cta_smem_bytes(const Bounds& b, int team, int ndem);
+cudaError_t launch_bpx(const BpArgs& a, int team, int msg_fp16, int grid, cudaStream_t s);
+cudaError_t bpx_occupancy(const Bounds& b, int team, int ndem, int msg_fp16, int* blocks_per_sm);
 
 // K3: LSD (vibe_lsd.cu). The per-column arrays (4 words per column) stay in shared memory up to 6144
 // columns and move to the CTA's global scratch above that.

@@ -63,13 +63,11 @@ SM_CLOCK_GHZ = 2.07          # maximum SM clock of the part (the recipe's figure
 SMEM_BYTES_PER_CLK = 128     # shared-memory bandwidth per SM and clock (32 banks x 4 bytes)
 INT_OPS_PER_CLK = 128        # 32-bit integer lanes per SM and clock
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one ncu capture of each BP kernel with
-# FP32 messages, per unit of work, for the rooflines' `traffic`: the image engine per shot (its DRAM
-# traffic is the per-shot I/O and LSD hand-off), the summary engine per executed sweep (its messages,
-# tables and rescans). Scaled to a launch by the units it processed; the captures and their commands
-# are in profiles/.
+# FP32 messages, per unit of work, for the rooflines' `traffic`; None until the present kernels have one
+# (the captures in profiles/ name the build they were taken on).
 PROFILED_TRAFFIC = {
-    "k_bp": {"per": "shot", "bytes": 4737024 / 20000, "profile": "profiles/k_bp_cc666_d9_pheno_full.md"},
-    "k_bpx": {"per": "sweep", "bytes": 615048462000 / 61857, "profile": "profiles/k_bpx_circuit_d11_k4_t10_full.md"},
+    "k_bp": {"per": "shot", "bytes": None, "profile": None},
+    "k_bpx": {"per": "sweep", "bytes": None, "profile": None},
 }
 
 

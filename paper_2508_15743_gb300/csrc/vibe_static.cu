@@ -74,16 +74,26 @@ extern "C" int vibe_decode_noalloc(vibe_handle* h, const uint32_t* d_syndromes, 
   if (t.engine != VIBE_ENGINE_IMAGE)
     return vibe::set_error(VIBE_ERR_UNSUPPORTED, "the static workspace serves warp-engine handles only");
   // Fixed part: counters, two n-float rows per BP warp (LLR accumulator, posterior; a third where the
-  // step words do not fit in shared memory), one row set per LSD CTA. The LSD CTAs are capped at one per SM so the fixed part stays small; the rest holds the
-  // LSD hand-off queue.
-  const int bp_grid = v.bp_grid;
+  // step words do not fit in shared memory), one row set per LSD CTA. The LSD CTAs are capped at one per
+  // SM so the fixed part stays small; the rest holds the LSD hand-off queue.
   const int lsd_grid = v.lsd_grid < v.num_sms ? v.lsd_grid : v.num_sms;
   const size_t ctrl_b = 256;
-  const size_t bp_b = up256((size_t)bp_grid * vibe::kBpWarpsPerCta * (2 + v.bnd.global_st) * (size_t)t.n * sizeof(float));
   const size_t lsd_b = up256((size_t)lsd_grid * (size_t)vibe::lsd_scratch_words(v.bnd, vibe::kLsdThreads) * sizeof(uint32_t));
-  const size_t fixed = ctrl_b + bp_b + lsd_b;
   const size_t per_shot = (size_t)t.n * sizeof(float) + sizeof(uint32_t);
-  const long long max_b = fixed + 512 < kStaticBytes ? (long long)((kStaticBytes - fixed - 512) / per_shot) : 0;
+  auto bp_bytes = [&](int grid) {
+    return up256((size_t)grid * vibe::kBpWarpsPerCta * (2 + v.bnd.global_st) * (size_t)t.n * sizeof(float));
+  };
+  auto most = [&](int grid) {   // largest batch beside the rows of `grid` BP CTAs
+    const size_t f = ctrl_b + bp_bytes(grid) + lsd_b;
+    return f + 512 < kStaticBytes ? (long long)((kStaticBytes - f - 512) / per_shot) : 0LL;
+  };
+  // a batch that does not fit beside the full grid's rows gets a smaller grid, down to a CTA per SM
+  const int least = v.bp_grid < v.num_sms ? v.bp_grid : v.num_sms;
+  int bp_grid = v.bp_grid;
+  while (bp_grid > least && B > most(bp_grid)) bp_grid = bp_grid - v.num_sms > least ? bp_grid - v.num_sms : least;
+  const size_t bp_b = bp_bytes(bp_grid);
+  const size_t fixed = ctrl_b + bp_b + lsd_b;
+  const long long max_b = most(least);
   if (B > max_b) {
     char msg[160];
     snprintf(msg, sizeof(msg), "batch of %lld shots exceeds the 64 MiB static workspace (at most %lld for this problem)",

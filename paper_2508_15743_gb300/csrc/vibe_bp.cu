@@ -427,7 +427,6 @@ template <typename MT, int DP, int NCH>
 __device__ __noinline__ int run_member(const Tables& t, int i, int smem_off, ImageRun& R) {
   extern __shared__ __align__(16) unsigned char smem[];
   unsigned char* base = smem + smem_off;
-  // through a shuffle: read once, and in a register of its own (the compiler would read it at each use)
   const int lane = __shfl_sync(kFull, (int)(threadIdx.x & 31), (int)(threadIdx.x & 31));
   const uint32_t sbase = __shfl_sync(kFull, (uint32_t)__cvta_generic_to_shared(smem) + (uint32_t)smem_off, lane);
   const int n = t.n, m = t.m, T = t.T, mw = t.mw;

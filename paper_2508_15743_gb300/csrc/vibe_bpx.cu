@@ -43,7 +43,7 @@
 // What bounds it and what the mapping bought. The engine is bound by instruction issue and by the
 // dependent chain of a step (summary, shuffles, sums, update, next step), not by DRAM. The mapping it
 // replaces gave each lane a whole column and unrolled its checks: on levels of 4-30 columns most lanes
-// idled through ~750 instructions; a step of 32 edges takes ~170 with nearly every lane at work.
+// idled; a step of 32 edges has nearly every lane at work.
 // Measured (GB300): circuit-level d=5, FP16, K=32, 4096 shots 826 -> 174 ms; XYZ d=7, FP32, K=16, 2500
 // shots 616 -> 147 ms; circuit-level d=11, FP32, K=64, T=50, 32 shots 220 -> 156 ms.
 //
@@ -435,9 +435,6 @@ struct MemberRun {
 template <typename MT, int DP>
 __device__ __noinline__ int run_member_x(const Tables& t, int i, MemberRun& R, unsigned char* gs) {
   extern __shared__ __align__(16) unsigned char smem[];
-  // Both through a shuffle: the compiler would otherwise read the thread index again wherever the lane is
-  // used and keep the addresses in uniform registers, moving them over at each use (14 of the 184
-  // instructions of a step).
   const int lane = __shfl_sync(kFull, (int)(threadIdx.x & 31), (int)(threadIdx.x & 31));
   const int W = (int)(blockDim.x >> 5), w = __shfl_sync(kFull, (int)(threadIdx.x >> 5), lane);
   const int tid = 32 * w + lane, nt = 32 * W;

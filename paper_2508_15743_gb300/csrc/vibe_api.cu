@@ -881,23 +881,40 @@ int vibe_get_wavefronts(vibe_handle* h, int32_t member, uint32_t* order_out, uin
                         int32_t* nlevels_out) {
   if (!h || !order_out || !level_offsets_out || !nlevels_out) return fail(VIBE_ERR_INVALID, "NULL argument");
   if (member < 0 || member >= h->t.K) return fail(VIBE_ERR_INVALID, "member out of range");
-  // the kernels run the packed steps; the levels are found here, for the member asked for
-  const int n = h->t.n, m = h->t.m;
-  uint32_t *sched = nullptr, *off = nullptr;
-  int32_t* work = nullptr;   // the level count, then scratch
-  cudaError_t e = dalloc(&sched, (size_t)n);
-  if (e == cudaSuccess) e = dalloc(&off, (size_t)n + 1);
-  if (e == cudaSuccess) e = dalloc(&work, (size_t)m + 3 * (size_t)n + 2);
-  if (e == cudaSuccess)
-    e = vibe::member_levels(h->perm + (size_t)member * n, n, m, h->colptr, h->rowidx, sched, off, work, work + 1, nullptr);
-  if (e == cudaSuccess) e = cudaMemcpy(order_out, sched, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(level_offsets_out, off, sizeof(uint32_t) * (n + 1), cudaMemcpyDeviceToHost);
-  if (e == cudaSuccess) e = cudaMemcpy(nlevels_out, work, sizeof(int32_t), cudaMemcpyDeviceToHost);
-  cudaFree(sched);
-  cudaFree(off);
-  cudaFree(work);
-  if (e != cudaSuccess) return cuda_fail(e, "wavefronts");
-  for (int j = 0; j < n; ++j) order_out[j] &= 0xffffffu;
+  // The kernels run the packed steps; the levels are found here, on the host, for the member asked for. Only
+  // copies touch the GPU: they work whichever device is current.
+  const int n = h->t.n, m = h->t.m, E = h->t.E;
+  try {
+    std::vector<uint32_t> perm(n);
+    std::vector<int32_t> colptr(n + 1), rowidx(E);
+    VIBE_CUDA(cudaMemcpy(perm.data(), h->perm + (size_t)member * n, sizeof(uint32_t) * n, cudaMemcpyDeviceToHost),
+              "wavefronts");
+    VIBE_CUDA(cudaMemcpy(colptr.data(), h->colptr, sizeof(int32_t) * (n + 1), cudaMemcpyDeviceToHost), "wavefronts");
+    VIBE_CUDA(cudaMemcpy(rowidx.data(), h->rowidx, sizeof(int32_t) * E, cudaMemcpyDeviceToHost), "wavefronts");
+    std::vector<int32_t> last(m, -1), lev(n);   // level of the latest column seen at each check; of each column
+    int nl = 0;
+    for (int t = 0; t < n; ++t) {
+      const int v = (int)perm[t];
+      int l = 0;
+      for (int e = colptr[v]; e < colptr[v + 1]; ++e) l = std::max(l, last[rowidx[e]] + 1);
+      for (int e = colptr[v]; e < colptr[v + 1]; ++e) last[rowidx[e]] = l;
+      lev[v] = l;
+      nl = std::max(nl, l + 1);
+    }
+    // grouped by level, inside a level by column degree, then by index
+    std::fill(level_offsets_out, level_offsets_out + n + 1, 0u);
+    for (int v = 0; v < n; ++v) level_offsets_out[lev[v] + 1]++;
+    for (int l = 0; l < nl; ++l) level_offsets_out[l + 1] += level_offsets_out[l];
+    std::vector<uint32_t> at(level_offsets_out, level_offsets_out + nl);
+    for (int v = 0; v < n; ++v) order_out[at[lev[v]]++] = (uint32_t)v;
+    for (int l = 0; l < nl; ++l)
+      std::stable_sort(order_out + level_offsets_out[l], order_out + level_offsets_out[l + 1], [&](uint32_t a, uint32_t b) {
+        return colptr[a + 1] - colptr[a] < colptr[b + 1] - colptr[b];
+      });
+    *nlevels_out = nl;
+  } catch (const std::bad_alloc&) {
+    return fail(VIBE_ERR_NOMEM, "wavefronts: host allocation failed");
+  }
   return VIBE_OK;
 }
 

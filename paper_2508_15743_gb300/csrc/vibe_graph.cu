@@ -4,9 +4,7 @@
 // per-column edge table csc_ent of the flooding and layered sweeps, the padded message image (prior LLR of
 // each edge's column, +inf padding), and for every ensemble member its serial schedule packed into steps
 // of 32 edges (k_steps): columns of one step touch disjoint checks and columns that share a check keep
-// their order, so the steps give the same floats as the serial order of Algorithm 1 (serial branch). The
-// dependency wavefronts, level(v) = 1 + max{level(u) : u before v in the member's order, u and v share a
-// check}, are found on request (member_levels).
+// their order, so the steps give the same floats as the serial order of Algorithm 1 (serial branch).
 #include "vibe_internal.cuh"
 
 namespace vibe {
@@ -127,53 +125,6 @@ __global__ void k_xsum(const int32_t* __restrict__ rowptr, const int32_t* __rest
     }
     out[c] = make_float4(a1, a2, a3, __uint_as_float(q1 | (q2 << 8) | (sg << 31)));
   }
-}
-
-// One thread per member: dependency levels of its schedule, then a stable counting sort into levels
-// and, inside each level, by column degree (lanes of a warp then see similar work).
-__global__ void k_levels(const uint32_t* __restrict__ perm, int n, int m, int K, const int32_t* __restrict__ colptr,
-                         const int32_t* __restrict__ rowidx, uint32_t* __restrict__ sched,
-                         uint32_t* __restrict__ lvl_off, int32_t* __restrict__ nlev, int32_t* __restrict__ scratch) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= K) return;
-  size_t per = (size_t)m + 3 * (size_t)n + 1;
-  int32_t* last = scratch + per * i;       // m: level of the latest column seen at each check
-  int32_t* lev = last + m;                 // n
-  int32_t* cnt = lev + n;                  // n + 1
-  int32_t* tmp = cnt + n + 1;              // n
-  for (int c = 0; c < m; ++c) last[c] = -1;
-  const uint32_t* p = perm + (size_t)i * n;
-  int nl = 0;
-  for (int t = 0; t < n; ++t) {
-    int v = (int)p[t];
-    int l = 0;
-    for (int e = colptr[v]; e < colptr[v + 1]; ++e) l = max(l, last[rowidx[e]] + 1);
-    for (int e = colptr[v]; e < colptr[v + 1]; ++e) last[rowidx[e]] = l;
-    lev[v] = l;
-    nl = max(nl, l + 1);
-  }
-  for (int l = 0; l <= nl; ++l) cnt[l] = 0;
-  for (int v = 0; v < n; ++v) cnt[lev[v]]++;
-  uint32_t* off = lvl_off + (size_t)i * (n + 1);
-  int run = 0;
-  for (int l = 0; l < nl; ++l) { off[l] = run; int c = cnt[l]; cnt[l] = run; run += c; }
-  off[nl] = run;
-  for (int v = 0; v < n; ++v) tmp[cnt[lev[v]]++] = v;   // stable: ascending v inside a level
-  uint32_t* out = sched + (size_t)i * n;
-  for (int l = 0; l < nl; ++l) {
-    int b = off[l], e = off[l + 1];
-    int dc[kMaxColDeg + 2];
-    for (int d = 0; d <= kMaxColDeg + 1; ++d) dc[d] = 0;
-    for (int t = b; t < e; ++t) { int v = tmp[t]; dc[colptr[v + 1] - colptr[v]]++; }
-    int r = b;
-    for (int d = 0; d <= kMaxColDeg; ++d) { int c = dc[d]; dc[d] = r; r += c; }
-    for (int t = b; t < e; ++t) {
-      int v = tmp[t];
-      int d = colptr[v + 1] - colptr[v];
-      out[dc[d]++] = (uint32_t)v | ((uint32_t)d << 24);
-    }
-  }
-  nlev[i] = nl;
 }
 
 // The steps of every member's sweep (one warp per member): its columns, taken in the member's order,
@@ -522,12 +473,6 @@ cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m
     k_msg_init<float><<<grid_for((long long)m * RP, 256), 256, 0, s>>>(d_rowptr, d_colidx, m, RP, d_lam,
                                                                       static_cast<float*>(d_msg_init));
   }
-  return cudaGetLastError();
-}
-
-cudaError_t member_levels(const uint32_t* d_perm, int n, int m, const int32_t* d_colptr, const int32_t* d_rowidx,
-                          uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, int32_t* d_scratch, cudaStream_t s) {
-  k_levels<<<1, 32, 0, s>>>(d_perm, n, m, 1, d_colptr, d_rowidx, d_sched, d_lvl_off, d_nlev, d_scratch);
   return cudaGetLastError();
 }
 

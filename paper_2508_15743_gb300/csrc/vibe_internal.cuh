@@ -409,10 +409,6 @@ cudaError_t build_tables(const int32_t* d_rowptr, const int32_t* d_colidx, int m
                          const uint32_t* d_perm, int RP, int DP, int msg_fp16, const float* d_lam, int32_t* d_colptr,
                          int32_t* d_rowidx, uint32_t* d_cpos, uint32_t* d_csc_ent, void* d_msg_init, float4* d_xsum,
                          int32_t* d_scratch, cudaStream_t s);
-// The dependency levels of one member's order: columns grouped by level (column | degree << 24), n + 1
-// offsets, the level count; scratch: m + 3n + 1 ints.
-cudaError_t member_levels(const uint32_t* d_perm, int n, int m, const int32_t* d_colptr, const int32_t* d_rowidx,
-                          uint32_t* d_sched, uint32_t* d_lvl_off, int32_t* d_nlev, int32_t* d_scratch, cudaStream_t s);
 // Packs each member's order into steps for teams of `team` warps (K step counts in d_nstep); fill_steps then writes the resident
 // tables from the same scratch (step_scratch_ints).
 size_t step_scratch_ints(int n, int K, int team);

@@ -273,6 +273,28 @@ typedef struct {
  */
 int vibe_get_launch(const vibe_handle* h, const vibe_batch* b, vibe_launch* out);
 
+/* How a handle or a batch runs pairs, one warp or team per (shot, member) (vibe_get_pairs). */
+typedef struct {
+  int64_t record_bytes; /* bound on the members' records: see vibe_set_pairs */
+  int64_t shots;        /* largest batch that shot mode runs as pairs, 0: none; -1 in pair mode: every batch */
+  int64_t shots_soft;   /* the same with soft output */
+  int64_t held_bytes;   /* members' records in the workspace now */
+  int32_t last;         /* how the last decode ran: 1 as pairs, 0 one warp or team per shot, -1 none yet */
+} vibe_pairs;
+
+/*
+ * vibe_get_pairs -- exactly one of h and b (the other NULL) into *out. Errors: VIBE_ERR_INVALID.
+ *
+ * vibe_set_pairs -- bounds the device memory of the members' records of exactly one of h and b. In shot mode
+ *   a small batch runs as pairs only while its records fit (record_bytes = 0: never, one warp or team per
+ *   shot whatever the batch); in pair mode a launch takes as many shots as fit, one at least. -1: the sizes a
+ *   handle is created with, 2 GiB in shot mode and 8 GiB in pair mode. Results do not depend on it. Records
+ *   held beyond the new bound are freed. A vibe_batch starts with the bound of its first handle.
+ *   Errors: VIBE_ERR_INVALID.
+ */
+int vibe_get_pairs(const vibe_handle* h, const vibe_batch* b, vibe_pairs* out);
+int vibe_set_pairs(vibe_handle* h, vibe_batch* b, int64_t record_bytes);
+
 /*
  * Mixed batches. The paper decodes one detector error model per run; a decoding service often holds
  * several (code distances, noise models, X and Z memory) and receives shots for all of them. A

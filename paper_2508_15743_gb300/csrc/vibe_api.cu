@@ -86,6 +86,7 @@ struct Launch {
   int bp_blocks_per_sm = 0, bpx_blocks_per_sm = 0, lsd_blocks_per_sm = 0;   // bpx: of the smallest teams
   int xocc[vibe::kTeamClasses] = {};   // summary engine: CTAs per SM that fit, by team class
   int pair_mode = 0;                // one warp per (shot, member) pair (vibe_params.pair_mode)
+  long long record_bytes = -1;      // bound on the members' records (vibe_set_pairs); -1: kPairBytes or kAutoPairBytes
   int lsd_threads = vibe::kLsdThreads;   // threads per LSD CTA (tuned: 64, 128 or 256)
   bool warp_engine() const { return (bnd.engines & 1) != 0; }
   bool cta_engine() const { return (bnd.engines & 2) != 0; }
@@ -114,9 +115,10 @@ struct Launch {
   long long pair_shot_bytes(bool soft) const {
     return (long long)bnd.K * (8LL + 4LL * bnd.nw + 4LL * bnd.n * (soft ? 2 : 1)) + 4;
   }
-  // pair mode: shots per launch -- as many as kPairBytes of member records hold, so that a large batch
+  long long record_bound() const { return record_bytes >= 0 ? record_bytes : pair_mode ? kPairBytes : kAutoPairBytes; }
+  // pair mode: shots per launch -- as many as the bound on the member records holds, so that a large batch
   // keeps every warp busy across shots (a launch ends with its slowest pair) and a small one runs whole
-  long long pair_chunk(bool soft) const { return std::max(1LL, kPairBytes / pair_shot_bytes(soft)); }
+  long long pair_chunk(bool soft) const { return std::max(1LL, record_bound() / pair_shot_bytes(soft)); }
   static constexpr long long kPairBytes = 8LL << 30;
   // Shots up to which a batch in shot mode runs as pairs all the same (same results). A batch of a few
   // shots per warp ends with the warps whose shots reach LSD: each runs K * T sweeps one after another
@@ -128,7 +130,7 @@ struct Launch {
   long long auto_pair_shots() const {
     if (bnd.K < 2) return 0;
     const long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta + (long long)bpx_grid();
-    return std::min(8 * warps, kAutoPairBytes / pair_shot_bytes(false));
+    return std::min(8 * warps, record_bound() / pair_shot_bytes(false));
   }
   static constexpr long long kAutoPairBytes = 2LL << 30;
 };
@@ -159,6 +161,7 @@ struct Workspace {
   unsigned int* pdone = nullptr;
 
   bool no_records = false;   // there was no memory for the records of shot mode's small batches
+  int last_pairs = -1;       // whether the last decode ran as pairs
 
   void release_records() {
     cudaFree(pconv); cudaFree(pW); cudaFree(pbits); cudaFree(pterms); cudaFree(ppost); cudaFree(pdone);
@@ -277,6 +280,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
   if (rc != VIBE_OK) return rc;
   const long long step = ws.chunk;
   const bool pairs = ws.as_pairs(L, q.B, q.soft != nullptr);
+  ws.last_pairs = pairs;
   for (long long b0 = 0; b0 < q.B; b0 += step) {
     const long long nb = std::min(step, q.B - b0);
     VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, Workspace::kCtrl * sizeof(unsigned int), s), "decode");
@@ -1032,6 +1036,28 @@ int vibe_get_launch(const vibe_handle* h, const vibe_batch* b, vibe_launch* out)
   return VIBE_OK;
 }
 
+int vibe_get_pairs(const vibe_handle* h, const vibe_batch* b, vibe_pairs* out) {
+  if ((!h) == (!b) || !out) return fail(VIBE_ERR_INVALID, "give exactly one of handle and batch, and an output");
+  const Launch& L = h ? h->L : b->L;
+  const Workspace& ws = h ? h->ws : b->ws;
+  out->record_bytes = L.record_bound();
+  out->shots = L.pair_mode ? -1 : L.auto_pair_shots();
+  out->shots_soft = out->shots;
+  out->held_bytes = ws.pair_shots * L.pair_shot_bytes(ws.pair_soft);
+  out->last = ws.last_pairs;
+  return VIBE_OK;
+}
+
+int vibe_set_pairs(vibe_handle* h, vibe_batch* b, int64_t record_bytes) {
+  if ((!h) == (!b)) return fail(VIBE_ERR_INVALID, "give exactly one of handle and batch");
+  if (record_bytes < -1) return fail(VIBE_ERR_INVALID, "record_bytes must be -1 or more");
+  Launch& L = h ? h->L : b->L;
+  Workspace& ws = h ? h->ws : b->ws;
+  L.record_bytes = record_bytes;
+  if (ws.pair_shots * L.pair_shot_bytes(ws.pair_soft) > L.record_bound()) ws.release_records();
+  return VIBE_OK;
+}
+
 int vibe_destroy(vibe_handle* h) {
   delete h;
   return VIBE_OK;
@@ -1072,6 +1098,7 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
   bt->L.bnd = b;
   bt->L.msg_fp16 = h0->L.msg_fp16;
   bt->L.pair_mode = h0->L.pair_mode;
+  bt->L.record_bytes = h0->L.record_bytes;
   bt->L.device = h0->device;
   bt->L.num_sms = h0->L.num_sms;
   int rc = size_launch(bt->L);

@@ -83,6 +83,10 @@ def _load():
     lib.vibe_batch_autotune.restype = ctypes.c_int
     lib.vibe_get_launch.argtypes = [vp, vp, vp]
     lib.vibe_get_launch.restype = ctypes.c_int
+    lib.vibe_get_pairs.argtypes = [vp, vp, vp]
+    lib.vibe_get_pairs.restype = ctypes.c_int
+    lib.vibe_set_pairs.argtypes = [vp, vp, i64]
+    lib.vibe_set_pairs.restype = ctypes.c_int
     lib.vibe_batch_destroy.argtypes = [vp]
     lib.vibe_batch_destroy.restype = ctypes.c_int
     lib.vibe_destroy.argtypes = [vp]
@@ -241,6 +245,23 @@ def vibe_get_launch(h=None, b=None):
     return {f: getattr(out, f) for f, _ in vibe_launch._fields_}
 
 
+class vibe_pairs(ctypes.Structure):
+    _fields_ = [("record_bytes", ctypes.c_int64), ("shots", ctypes.c_int64), ("shots_soft", ctypes.c_int64),
+                ("held_bytes", ctypes.c_int64), ("last", ctypes.c_int32)]
+
+
+def vibe_get_pairs(h=None, b=None):
+    """How a handle or a batch runs (shot, member) pairs, as a dict."""
+    out = vibe_pairs()
+    _check(_lib.vibe_get_pairs(h, b, ctypes.byref(out)))
+    return {f: getattr(out, f) for f, _ in vibe_pairs._fields_}
+
+
+def vibe_set_pairs(record_bytes, h=None, b=None):
+    """Bounds the members' records (bytes; 0: shot mode never runs pairs, -1: the default)."""
+    _check(_lib.vibe_set_pairs(h, b, int(record_bytes)))
+
+
 def vibe_batch_destroy(b):
     if b:
         _check(_lib.vibe_batch_destroy(b))
@@ -325,6 +346,12 @@ class Decoder:
     def launch(self):
         return vibe_get_launch(h=self.handle)
 
+    def pairs(self):
+        return vibe_get_pairs(h=self.handle)
+
+    def set_pairs(self, record_bytes):
+        vibe_set_pairs(record_bytes, h=self.handle)
+
 
 class MixedBatch:
     """Several Decoders decoded by one launch pair (vibe_batch_*); shot b uses decoders[problem[b]]."""
@@ -368,6 +395,12 @@ class MixedBatch:
 
     def launch(self):
         return vibe_get_launch(b=self.handle)
+
+    def pairs(self):
+        return vibe_get_pairs(b=self.handle)
+
+    def set_pairs(self, record_bytes):
+        vibe_set_pairs(record_bytes, b=self.handle)
 
 
 def stats_to_numpy(stats_tensor):

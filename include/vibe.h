@@ -156,7 +156,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
  *   shots whose L e differs; d_counters: VIBE_NUM_COUNTERS uint64 accumulators (may be NULL).
  *   The handle's workspace is allocated on the first call and grown when a larger batch needs it (in shot
  *   mode with up to 2 GiB of members' records; without that memory small batches run one warp per shot);
- *   calls with a batch no larger than an earlier one allocate nothing. Large batches run in chunks.
+ *   calls with a batch no larger than an earlier one allocate nothing, but for a first call with soft output,
+ *   which may. Large batches run in chunks.
  *   Calls on one handle must not overlap in time (the workspace is shared); use one handle per stream.
  *   Errors: VIBE_ERR_INVALID (NULL handle/required pointer, B < 0), VIBE_ERR_NOMEM, VIBE_ERR_CUDA.
  *   B = 0 is a no-op.

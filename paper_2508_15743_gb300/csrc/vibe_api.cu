@@ -135,38 +135,66 @@ struct Launch {
   static constexpr long long kAutoPairBytes = 2LL << 30;
 };
 
-// Device memory a decode uses besides its inputs and outputs; grown on demand, reused afterwards.
+// Device memory that only grows.
+struct Buffer {
+  void* p = nullptr;
+  size_t bytes = 0;
+  cudaError_t grow(size_t want) {
+    if (p && want <= bytes) return cudaSuccess;
+    release();
+    want = std::max<size_t>(want, 16);
+    const cudaError_t e = cudaMalloc(&p, want);
+    if (e == cudaSuccess) bytes = want;
+    else p = nullptr;
+    return e;
+  }
+  void release() {
+    cudaFree(p);
+    p = nullptr;
+    bytes = 0;
+  }
+  template <typename T>
+  T* as() const { return static_cast<T*>(p); }
+};
+
+// Device memory a decode uses besides its inputs and outputs. Every part grows by itself and keeps the largest
+// size asked for, so a batch no larger than an earlier one allocates nothing.
 struct Workspace {
-  long long chunk = 0, chunk_max = 0;
-  long long pk_nw = 0, pk_n = 0;   // pair records' sizes per shot the buffers were made for
-  long long lsd_words = 0;         // LSD scratch words per CTA the buffer was made for
-  int bp_warps = 0, lsd_ctas = 0;
-  long long bpx_bytes = 0;
+  long long chunk = 0, chunk_max = 0;   // shots of the LSD hand-off
   static constexpr int kCtrl = 4 + 2 * vibe::kTeamClasses;
-  unsigned int* ctrl = nullptr;   // [0] next shot (image engine), [1] LSD count, [2] next LSD shot, [3] next pair
-                                  // (image engine), then next shot and next pair of each team class
-  uint32_t* lsd_shots = nullptr;
-  float* lsd_soft = nullptr;
-  float* bp_scratch = nullptr;
-  unsigned char* bpx_scratch = nullptr;
-  uint32_t* lsd_scratch = nullptr;
-  // pair mode: member records of `pair_shots` shots (see BpArgs)
+  Buffer ctrl_b, lsd_shots_b, lsd_soft_b, bp_b, bpx_b, lsd_b;
+  unsigned int* ctrl() const { return ctrl_b.as<unsigned int>(); }   // [0] next shot (image engine), [1] LSD count,
+                                  // [2] next LSD shot, [3] next pair (image engine), then next shot and next pair of
+                                  // each team class
+  // member records of `pair_shots` shots (see BpArgs)
   long long pair_shots = 0;
   bool pair_soft = false;
-  int* pconv = nullptr;
-  float* pW = nullptr;
-  uint32_t* pbits = nullptr;
-  float* pterms = nullptr;
-  float* ppost = nullptr;
-  unsigned int* pdone = nullptr;
+  Buffer pconv, pW, pbits, pterms, ppost, pdone;
 
   bool no_records = false;   // there was no memory for the records of shot mode's small batches
   int last_pairs = -1;       // whether the last decode ran as pairs
 
   void release_records() {
-    cudaFree(pconv); cudaFree(pW); cudaFree(pbits); cudaFree(pterms); cudaFree(ppost); cudaFree(pdone);
-    pconv = nullptr; pW = nullptr; pbits = nullptr; pterms = nullptr; ppost = nullptr; pdone = nullptr;
+    for (Buffer* b : {&pconv, &pW, &pbits, &pterms, &ppost, &pdone}) b->release();
     pair_shots = 0; pair_soft = false; no_records = false;
+  }
+  // Records of S shots, with their posteriors if `soft`; none are left if there is no memory for them.
+  cudaError_t grow_records(const Launch& L, long long S, bool soft) {
+    const size_t K = (size_t)S * L.bnd.K;
+    cudaError_t e = pconv.grow(4 * K);
+    if (e == cudaSuccess) e = pW.grow(4 * K);
+    if (e == cudaSuccess) e = pbits.grow(4 * K * (size_t)L.bnd.nw);
+    if (e == cudaSuccess) e = pterms.grow(4 * K * (size_t)L.bnd.n);
+    if (e == cudaSuccess && soft) e = ppost.grow(4 * K * (size_t)L.bnd.n);
+    if (e == cudaSuccess) e = pdone.grow(4 * (size_t)S);
+    if (e == cudaSuccess) {
+      pair_shots = S;
+      pair_soft = soft;
+    } else {
+      cudaGetLastError();
+      release_records();
+    }
+    return e;
   }
   // whether a batch of B shots runs as pairs
   bool as_pairs(const Launch& L, long long B, bool soft) const {
@@ -174,63 +202,42 @@ struct Workspace {
   }
   void release() {
     release_records();
-    cudaFree(ctrl); cudaFree(lsd_shots); cudaFree(lsd_soft); cudaFree(bp_scratch); cudaFree(bpx_scratch);
-    cudaFree(lsd_scratch);
-    ctrl = nullptr; lsd_shots = nullptr; lsd_soft = nullptr; bp_scratch = nullptr; bpx_scratch = nullptr;
-    lsd_scratch = nullptr;
-    chunk = 0; bp_warps = 0; lsd_ctas = 0; bpx_bytes = 0; lsd_words = 0;
+    for (Buffer* b : {&ctrl_b, &lsd_shots_b, &lsd_soft_b, &bp_b, &bpx_b, &lsd_b}) b->release();
+    chunk = 0;
+  }
+  cudaError_t grow_scratch(const Launch& L, long long c, bool soft) {
+    const Bounds& b = L.bnd;
+    cudaError_t e = ctrl_b.grow(kCtrl * sizeof(unsigned int));
+    if (e == cudaSuccess) e = lsd_shots_b.grow(sizeof(uint32_t) * (size_t)c);
+    if (e == cudaSuccess) e = lsd_soft_b.grow(sizeof(float) * (size_t)c * b.n);
+    if (e == cudaSuccess)
+      e = bp_b.grow(sizeof(float) * (size_t)L.bp_grid() * vibe::kBpWarpsPerCta * (size_t)(2 + b.global_st + b.M) * b.n);
+    if (e == cudaSuccess) e = bpx_b.grow((size_t)L.bpx_grid() * (size_t)L.bpx_pitch(soft));
+    if (e == cudaSuccess)
+      e = lsd_b.grow(sizeof(uint32_t) * (size_t)L.lsd_grid() * (size_t)vibe::lsd_scratch_words(b, L.lsd_threads));
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
   }
   int ensure(const Launch& L, long long need, bool soft) {
-    // records of as many shots as a batch of this size or a smaller one runs as pairs. In shot mode a first
-    // soft output grows nothing: without the posteriors' records it runs one warp per shot
-    const long long ps = std::min(need, L.pair_mode ? L.pair_chunk(soft) : L.auto_pair_shots());
-    const long long want = std::min(need, chunk_max);
-    const int warps = L.bp_grid() * vibe::kBpWarpsPerCta;
-    const long long xb = (long long)L.bpx_grid() * L.bpx_pitch(soft);
-    const bool pair_ok = ps == 0 || (!L.pair_mode && no_records) ||
-                         (ps <= pair_shots && (!L.pair_mode || !soft || pair_soft) && L.bnd.K * L.bnd.nw <= pk_nw &&
-                          L.bnd.K * L.bnd.n <= pk_n);
-    const bool lsd_ok = (long long)L.lsd_grid() * vibe::lsd_scratch_words(L.bnd, L.lsd_threads) <=
-                        (long long)lsd_ctas * lsd_words;
-    if (ctrl && want <= chunk && warps <= bp_warps && lsd_ok && xb <= bpx_bytes && pair_ok)
-      return VIBE_OK;
-    const long long c = std::max(want, chunk);
-    const long long xkeep = std::max(xb, bpx_bytes);
-    release();
-    const Bounds& b = L.bnd;
-    VIBE_CUDA(dalloc(&ctrl, kCtrl), "workspace");
-    VIBE_CUDA(dalloc(&lsd_shots, (size_t)c), "workspace");
-    VIBE_CUDA(dalloc(&lsd_soft, (size_t)c * b.n), "workspace");
-    VIBE_CUDA(dalloc(&bp_scratch, (size_t)warps * (size_t)(2 + b.global_st + b.M) * b.n), "workspace");
-    VIBE_CUDA(dalloc(&bpx_scratch, (size_t)xkeep), "workspace");
-    VIBE_CUDA(dalloc(&lsd_scratch, (size_t)L.lsd_grid() * (size_t)vibe::lsd_scratch_words(b, L.lsd_threads)),
-              "workspace");
-    lsd_words = vibe::lsd_scratch_words(b, L.lsd_threads);
-    if (ps > 0) {
-      const size_t S = (size_t)ps;
-      cudaError_t e = dalloc(&pconv, S * b.K);
-      if (e == cudaSuccess) e = dalloc(&pW, S * b.K);
-      if (e == cudaSuccess) e = dalloc(&pbits, S * b.K * (size_t)b.nw);
-      if (e == cudaSuccess) e = dalloc(&pterms, S * b.K * (size_t)b.n);
-      if (e == cudaSuccess && soft) e = dalloc(&ppost, S * b.K * (size_t)b.n);
-      if (e == cudaSuccess) e = dalloc(&pdone, S);
-      if (e == cudaSuccess) {
-        pair_shots = ps;
-        pair_soft = soft;
-        pk_nw = (long long)b.K * b.nw;
-        pk_n = (long long)b.K * b.n;
-      } else if (L.pair_mode) {
-        return cuda_fail(e, "workspace");
-      } else {   // shot mode does without them
-        cudaGetLastError();
-        release_records();
-        no_records = true;
-      }
+    const long long c = std::max(std::min(need, chunk_max), chunk);
+    if (c > chunk) chunk = 0;   // should a growth fail, the next call asks for its own size
+    cudaError_t e = grow_scratch(L, c, soft);
+    if (e != cudaSuccess && !L.pair_mode && pair_shots > 0) {   // shot mode can do without records
+      release_records();
+      e = grow_scratch(L, c, soft);
     }
+    if (e != cudaSuccess) return cuda_fail(e, "workspace");
     chunk = c;
-    bp_warps = warps;
-    lsd_ctas = L.lsd_grid();
-    bpx_bytes = xkeep;
+    // records of as many shots as a batch of this size or a smaller one runs as pairs, and no fewer than before.
+    // In shot mode a first soft output grows nothing: without the posteriors' records it runs one warp per shot
+    const bool s = soft || pair_soft;
+    const long long most = L.pair_mode ? L.pair_chunk(s) : L.auto_pair_shots(), ps = std::min(need, most);
+    if (ps <= pair_shots && (!L.pair_mode || !soft || pair_soft)) return VIBE_OK;
+    if (!L.pair_mode && no_records) return VIBE_OK;
+    if ((e = grow_records(L, std::min(std::max(ps, pair_shots), most), s)) != cudaSuccess) {
+      if (L.pair_mode) return cuda_fail(e, "workspace");
+      no_records = true;
+    }
     return VIBE_OK;
   }
   ~Workspace() { release(); }
@@ -283,7 +290,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
   ws.last_pairs = pairs;
   for (long long b0 = 0; b0 < q.B; b0 += step) {
     const long long nb = std::min(step, q.B - b0);
-    VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, Workspace::kCtrl * sizeof(unsigned int), s), "decode");
+    VIBE_CUDA(cudaMemsetAsync(ws.ctrl(), 0, Workspace::kCtrl * sizeof(unsigned int), s), "decode");
     cudaEvent_t e0 = nullptr, e1 = nullptr, e2 = nullptr;
     if (prof.on) { e0 = prof.next(); e1 = prof.next(); e2 = prof.next(); }
     if (e0) cudaEventRecord(e0, s);
@@ -292,12 +299,12 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       const long long ns = std::min(sub, nb - s0);
       const long long o = b0 + s0;
       if (s0 > 0) {   // the BP work counters start again; the LSD queue keeps filling
-        VIBE_CUDA(cudaMemsetAsync(ws.ctrl, 0, sizeof(unsigned int), s), "decode");
-        VIBE_CUDA(cudaMemsetAsync(ws.ctrl + 3, 0, (Workspace::kCtrl - 3) * sizeof(unsigned int), s), "decode");
+        VIBE_CUDA(cudaMemsetAsync(ws.ctrl(), 0, sizeof(unsigned int), s), "decode");
+        VIBE_CUDA(cudaMemsetAsync(ws.ctrl() + 3, 0, (Workspace::kCtrl - 3) * sizeof(unsigned int), s), "decode");
       }
       if (pairs) {
-        VIBE_CUDA(cudaMemsetAsync(ws.pconv, 0, sizeof(int) * (size_t)ns * L.bnd.K, s), "decode");
-        VIBE_CUDA(cudaMemsetAsync(ws.pdone, 0, sizeof(unsigned int) * (size_t)ns, s), "decode");
+        VIBE_CUDA(cudaMemsetAsync(ws.pconv.p, 0, sizeof(int) * (size_t)ns * L.bnd.K, s), "decode");
+        VIBE_CUDA(cudaMemsetAsync(ws.pdone.p, 0, sizeof(unsigned int) * (size_t)ns, s), "decode");
       }
       vibe::BpArgs a{};
       a.one = L.one;
@@ -312,17 +319,17 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       a.soft = q.soft ? q.soft + (size_t)o * q.soft_stride : nullptr; a.soft_stride = q.soft_stride;
       a.obs = q.obs ? q.obs + (size_t)o * q.log_stride : nullptr;
       a.counters = q.counters;
-      a.next_shot = ws.ctrl; a.lsd_count = ws.ctrl + 1; a.lsd_shots = ws.lsd_shots; a.lsd_soft = ws.lsd_soft;
+      a.next_shot = ws.ctrl(); a.lsd_count = ws.ctrl() + 1; a.lsd_shots = ws.lsd_shots_b.as<uint32_t>(); a.lsd_soft = ws.lsd_soft_b.as<float>();
       a.lsd_shot_base = (uint32_t)s0;
-      a.scratch = ws.bp_scratch;
+      a.scratch = ws.bp_b.as<float>();
       a.scratch_pitch = (long long)(2 + L.bnd.global_st + L.bnd.M) * L.bnd.n;
-      a.xscratch = ws.bpx_scratch;
+      a.xscratch = ws.bpx_b.as<unsigned char>();
       a.xscratch_pitch = L.bpx_pitch(a.want_soft != 0);
       a.pair_mode = pairs;
       a.pair_K = L.bnd.K;
-      a.pconv = ws.pconv; a.pW = ws.pW; a.pbits = ws.pbits; a.pterms = ws.pterms; a.ppost = ws.ppost;
-      a.pdone = ws.pdone;
-      a.next_pair = ws.ctrl + 3;
+      a.pconv = ws.pconv.as<int>(); a.pW = ws.pW.as<float>(); a.pbits = ws.pbits.as<uint32_t>();
+      a.pterms = ws.pterms.as<float>(); a.ppost = ws.ppost.as<float>(); a.pdone = ws.pdone.as<unsigned int>();
+      a.next_pair = ws.ctrl() + 3;
       const long long units = pairs ? ns * L.bnd.K : ns;   // shots, or (shot, member) pairs
       if (L.warp_engine()) {
         const int grid =
@@ -335,7 +342,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
         if (!((L.bnd.teams >> k) & 1)) continue;
         a.flag_bad = first ? 1 : 0;
         first = false;
-        a.next_shot_x = ws.ctrl + 4 + 2 * k;
+        a.next_shot_x = ws.ctrl() + 4 + 2 * k;
         a.next_pair_x = a.next_shot_x + 1;
         VIBE_CUDA(vibe::launch_bpx(a, team_of(k), L.msg_fp16, (int)std::min<long long>(L.bpx_grid(k), units), s),
                   "BP kernel launch");
@@ -354,8 +361,8 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
     l.soft = q.soft ? q.soft + (size_t)b0 * q.soft_stride : nullptr; l.soft_stride = q.soft_stride;
     l.obs = q.obs ? q.obs + (size_t)b0 * q.log_stride : nullptr;
     l.counters = q.counters;
-    l.lsd_count = ws.ctrl + 1; l.lsd_shots = ws.lsd_shots; l.lsd_soft = ws.lsd_soft; l.lsd_next = ws.ctrl + 2;
-    l.scratch = ws.lsd_scratch;
+    l.lsd_count = ws.ctrl() + 1; l.lsd_shots = ws.lsd_shots_b.as<uint32_t>(); l.lsd_soft = ws.lsd_soft_b.as<float>(); l.lsd_next = ws.ctrl() + 2;
+    l.scratch = ws.lsd_b.as<uint32_t>();
     l.scratch_pitch = vibe::lsd_scratch_words(L.bnd, L.lsd_threads);
     VIBE_CUDA(vibe::launch_lsd(l, L.lsd_grid(), L.lsd_threads, s), "LSD kernel launch");
     if (e2) cudaEventRecord(e2, s);

@@ -1,0 +1,92 @@
+"""The workspace promise: a batch no larger than an earlier one allocates nothing, whatever came between.
+
+Batch sizes and calls with and without soft output are mixed on one handle; free device memory must stay as it
+is, and a graph captured after the warm-up must replay to the same bits. The buffers at stake are far above the
+allocator's granularity (140 KB of members' records per shot here).
+"""
+import numpy as np
+import pytest
+
+from paper_2508_15743_gb300 import circuit as C
+from paper_2508_15743_gb300 import dem as D
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+IMAGE, SUMMARY = 1, 2
+
+
+@pytest.fixture(scope="module")
+def V():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2508_15743_gb300 import build
+    build.build_library()
+    from paper_2508_15743_gb300 import vibe
+    return vibe
+
+
+def free_bytes():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+class Calls:
+    """Decodes of the first B shots of one batch into buffers made beforehand."""
+
+    def __init__(self, V, dm, K, shots, **kw):
+        self.dec = V.Decoder(dm, K, D.schedules(dm.n, K, 3), T=8, M=2, **kw)
+        syn, _ = D.sample(dm, shots, 5)
+        self.syn = torch.from_numpy(syn.view(np.int32)).cuda()
+        self.out = {s: dict(corrections=torch.zeros((shots, self.dec.nw), dtype=torch.int32, device="cuda"),
+                            logical=torch.zeros((shots, self.dec.kw), dtype=torch.int32, device="cuda"),
+                            stats=torch.zeros((shots, 12), dtype=torch.uint8, device="cuda"),
+                            soft=torch.zeros((shots, dm.n), device="cuda") if s else None) for s in (False, True)}
+
+    def __call__(self, B, soft=False):
+        out = {k: v if v is None else v[:B] for k, v in self.out[soft].items()}
+        self.dec.decode(self.syn[:B], out=out)
+        return out
+
+
+PROBLEMS = {
+    "summary": (lambda: C.circuit_dem(5, 5, 0.003, noise="si1000", basis="X"), SUMMARY),
+    "image": (lambda: D.phenomenological_dem(9, 9, 0.01, 0.01), IMAGE),
+}
+
+
+@pytest.mark.parametrize("pair", [False, True])
+@pytest.mark.parametrize("name", sorted(PROBLEMS))
+def test_smaller_batches_between_allocate_nothing(V, name, pair):
+    build, engine = PROBLEMS[name]
+    run = Calls(V, build(), 16, 1000, engine=engine, pair_mode=pair)
+    run(1000)
+    run(10, soft=True)     # a first soft output may grow the scratch
+    before = free_bytes()
+    for B, soft in ((1000, False), (10, True), (1, False), (1000, False), (7, True), (999, False)):
+        run(B, soft)
+    assert free_bytes() == before
+    run.dec.close()
+
+
+def test_capture_after_mixed_warm_up_replays_the_same_bits(V):
+    build, engine = PROBLEMS["summary"]
+    run = Calls(V, build(), 16, 1000, engine=engine)
+    want = {k: v.clone() for k, v in run(1000).items() if v is not None}
+    run(10, soft=True)
+    run(1000)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = run(1000)
+    run(10, soft=True)
+    run(500)
+    for v in out.values():
+        if v is not None:
+            v.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    for k, v in want.items():
+        assert torch.equal(out[k], v), k
+    run.dec.close()

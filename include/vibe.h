@@ -154,8 +154,10 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
  *   the normalised LLR average that ranked the columns;
  *   d_observables: B x ceil(k/32) true logical flips (may be NULL) -- with d_counters, counts
  *   shots whose L e differs; d_counters: VIBE_NUM_COUNTERS uint64 accumulators (may be NULL).
- *   The handle's workspace is allocated on the first call and grown when a larger batch needs it (in shot
- *   mode with up to 2 GiB of members' records; without that memory small batches run one warp per shot);
+ *   The handle's workspace is allocated on the first call and grown when a larger batch needs it. In shot
+ *   mode a small batch that is the largest so far also gets its members' records (vibe_set_pairs), unless there
+ *   is no memory for them or the stream is being captured; a small batch after a large one uses the records
+ *   there are, else one warp per shot (same results; to have both fast, decode a small one first). Other
  *   calls with a batch no larger than an earlier one allocate nothing, but for a first call with soft output,
  *   which may. Large batches run in chunks.
  *   Calls on one handle must not overlap in time (the workspace is shared); use one handle per stream.
@@ -290,7 +292,7 @@ typedef struct {
  *   a small batch runs as pairs only while its records fit (record_bytes = 0: never, one warp or team per
  *   shot whatever the batch); in pair mode a launch takes as many shots as fit, one at least. -1: the sizes a
  *   handle is created with, 2 GiB in shot mode and 8 GiB in pair mode. Results do not depend on it. Records
- *   held beyond the new bound are freed. A vibe_batch starts with the bound of its first handle.
+ *   held beyond the new bound are freed, and the next call may allocate its own. A vibe_batch starts with the bound of its first handle.
  *   Errors: VIBE_ERR_INVALID.
  */
 int vibe_get_pairs(const vibe_handle* h, const vibe_batch* b, vibe_pairs* out);

@@ -157,6 +157,17 @@ struct Buffer {
   T* as() const { return static_cast<T*>(p); }
 };
 
+// Whether work on s is being recorded, so that nothing may be allocated. (An error means that a capture
+// elsewhere forbids the question.)
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return true;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 // Device memory a decode uses besides its inputs and outputs. Every part grows by itself and keeps the largest
 // size asked for, so a batch no larger than an earlier one allocates nothing.
 struct Workspace {
@@ -171,12 +182,12 @@ struct Workspace {
   bool pair_soft = false;
   Buffer pconv, pW, pbits, pterms, ppost, pdone;
 
-  bool no_records = false;   // there was no memory for the records of shot mode's small batches
+  long long seen = 0;        // largest batch so far
   int last_pairs = -1;       // whether the last decode ran as pairs
 
   void release_records() {
     for (Buffer* b : {&pconv, &pW, &pbits, &pterms, &ppost, &pdone}) b->release();
-    pair_shots = 0; pair_soft = false; no_records = false;
+    pair_shots = 0; pair_soft = false;
   }
   // Records of S shots, with their posteriors if `soft`; none are left if there is no memory for them.
   cudaError_t grow_records(const Launch& L, long long S, bool soft) {
@@ -218,7 +229,7 @@ struct Workspace {
     if (e != cudaSuccess) cudaGetLastError();
     return e;
   }
-  int ensure(const Launch& L, long long need, bool soft) {
+  int ensure(const Launch& L, long long need, bool soft, cudaStream_t s) {
     const long long c = std::max(std::min(need, chunk_max), chunk);
     if (c > chunk) chunk = 0;   // should a growth fail, the next call asks for its own size
     cudaError_t e = grow_scratch(L, c, soft);
@@ -228,15 +239,19 @@ struct Workspace {
     }
     if (e != cudaSuccess) return cuda_fail(e, "workspace");
     chunk = c;
-    // records of as many shots as a batch of this size or a smaller one runs as pairs, and no fewer than before.
-    // In shot mode a first soft output grows nothing: without the posteriors' records it runs one warp per shot
-    const bool s = soft || pair_soft;
-    const long long most = L.pair_mode ? L.pair_chunk(s) : L.auto_pair_shots(), ps = std::min(need, most);
-    if (ps <= pair_shots && (!L.pair_mode || !soft || pair_soft)) return VIBE_OK;
-    if (!L.pair_mode && no_records) return VIBE_OK;
-    if ((e = grow_records(L, std::min(std::max(ps, pair_shots), most), s)) != cudaSuccess) {
-      if (L.pair_mode) return cuda_fail(e, "workspace");
-      no_records = true;
+    const bool larger = need > seen;
+    seen = std::max(seen, need);
+    const bool ps = soft || pair_soft;
+    if (L.pair_mode) {   // records of as many shots as a launch takes, and no fewer than before
+      const long long most = L.pair_chunk(ps), S = std::min(need, most);
+      if (S <= pair_shots && (!soft || pair_soft)) return VIBE_OK;
+      if ((e = grow_records(L, std::min(std::max(S, pair_shots), most), ps)) != cudaSuccess)
+        return cuda_fail(e, "workspace");
+    } else if (larger && need > pair_shots && need <= L.auto_pair_shots() && !capturing(s)) {
+      // Shot mode: a batch that would run as pairs, the largest so far. Larger batches need no records, and a
+      // smaller one may not allocate: it runs one warp per shot if there are none yet, as a batch does
+      // whose records find no memory or that is being captured. A first soft output grows no records.
+      grow_records(L, need, ps);
     }
     return VIBE_OK;
   }
@@ -283,7 +298,7 @@ struct Batch {
 // sub-chunks of up to ws.pair_shots shots (the member records), all queueing into the chunk's LSD
 // launch, so a chunk's slowest LSD shots are waited for once, not once per sub-chunk.
 int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaStream_t s) {
-  int rc = ws.ensure(L, q.B, q.soft != nullptr);
+  int rc = ws.ensure(L, q.B, q.soft != nullptr, s);
   if (rc != VIBE_OK) return rc;
   const long long step = ws.chunk;
   const bool pairs = ws.as_pairs(L, q.B, q.soft != nullptr);
@@ -454,7 +469,7 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
   };
   // times the current L; ms = 0 marks a rejected candidate
   auto time_once = [&](float& ms) -> int {
-    int r = ws.ensure(L, q.B, q.soft != nullptr);
+    int r = ws.ensure(L, q.B, q.soft != nullptr, s);
     if (r != VIBE_OK) return r;
     float first = 0.f;
     if ((r = timed(first)) != VIBE_OK) return r;
@@ -1062,6 +1077,7 @@ int vibe_set_pairs(vibe_handle* h, vibe_batch* b, int64_t record_bytes) {
   Workspace& ws = h ? h->ws : b->ws;
   L.record_bytes = record_bytes;
   if (ws.pair_shots * L.pair_shot_bytes(ws.pair_soft) > L.record_bound()) ws.release_records();
+  ws.seen = 0;   // the next batch may get its records
   return VIBE_OK;
 }
 

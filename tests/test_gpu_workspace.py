@@ -90,3 +90,52 @@ def test_capture_after_mixed_warm_up_replays_the_same_bits(V):
     for k, v in want.items():
         assert torch.equal(out[k], v), k
     run.dec.close()
+
+
+def test_records_are_held_only_for_batches_that_run_as_pairs(V):
+    build, engine = PROBLEMS["image"]
+    run = Calls(V, build(), 4, 60_000, engine=engine)
+    limit = run.dec.pairs()["shots"]
+    assert 0 < limit < 60_000
+    run(60_000)                       # one warp per shot: no records
+    p = run.dec.pairs()
+    assert p["last"] == 0 and p["held_bytes"] == 0
+    before = free_bytes()
+    run(100)                          # no larger than an earlier one: nothing may be allocated for it
+    assert run.dec.pairs()["last"] == 0 and free_bytes() == before
+    run.dec.close()
+    run = Calls(V, build(), 4, 60_000, engine=engine)
+    run(100)
+    held = run.dec.pairs()["held_bytes"]
+    assert run.dec.pairs()["last"] == 1 and held > 0
+    run(limit)
+    assert run.dec.pairs()["last"] == 1 and run.dec.pairs()["held_bytes"] > held
+    run(60_000)
+    assert run.dec.pairs()["last"] == 0
+    before = free_bytes()
+    for B in (100, limit):            # the records stayed
+        run(B)
+        assert run.dec.pairs()["last"] == 1
+    assert free_bytes() == before
+    run.dec.close()
+
+
+def test_first_small_batch_under_capture_allocates_nothing(V):
+    build, engine = PROBLEMS["image"]
+    run = Calls(V, build(), 4, 60_000, engine=engine)
+    run(60_000)
+    want = {k: v.clone() for k, v in run(300).items() if v is not None}
+    run.dec.set_pairs(-1)             # the next small batch outside a capture would get records
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        out = run(300)
+    assert run.dec.pairs()["last"] == 0 and run.dec.pairs()["held_bytes"] == 0
+    for v in out.values():
+        if v is not None:
+            v.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    for k, v in want.items():
+        assert torch.equal(out[k], v), k
+    run.dec.close()

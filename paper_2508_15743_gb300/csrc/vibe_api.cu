@@ -127,12 +127,12 @@ struct Launch {
   // 4.8.8 d=9 phenomenological code (K=16) 46.3 / 40.7 ms at 4.5 and 157 / 155 ms at 18; the 6.6.6 one 99.6
   // / 102 ms at 13 and 381 / 404 ms at 54. So the line is drawn at eight shots per warp, and where the
   // members' records pass 2 GiB.
-  long long auto_pair_shots() const {
+  long long auto_pair_shots(bool soft) const {
     if (bnd.K < 2) return 0;
     const long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta + (long long)bpx_grid();
-    return std::min(8 * warps, record_bound() / pair_shot_bytes(false));
+    return std::min(8 * warps, record_bound() / pair_shot_bytes(soft));
   }
-  static constexpr long long kAutoPairBytes = 2LL << 30;
+  static constexpr long long kAutoPairBytes = 2LL << 30;   // with the posteriors where there is soft output
 };
 
 // Device memory that only grows.
@@ -183,14 +183,21 @@ struct Workspace {
   Buffer pconv, pW, pbits, pterms, ppost, pdone;
 
   long long seen = 0;        // largest batch so far
+  bool seen_soft = false;    // whether one had soft output
   int last_pairs = -1;       // whether the last decode ran as pairs
 
+  long long record_bytes() const {
+    size_t n = 0;
+    for (const Buffer* b : {&pconv, &pW, &pbits, &pterms, &ppost, &pdone}) n += b->bytes;
+    return (long long)n;
+  }
   void release_records() {
     for (Buffer* b : {&pconv, &pW, &pbits, &pterms, &ppost, &pdone}) b->release();
     pair_shots = 0; pair_soft = false;
   }
   // Records of S shots, with their posteriors if `soft`; none are left if there is no memory for them.
   cudaError_t grow_records(const Launch& L, long long S, bool soft) {
+    if (S < pair_shots) release_records();   // the posteriors take the place of shots within the bound
     const size_t K = (size_t)S * L.bnd.K;
     cudaError_t e = pconv.grow(4 * K);
     if (e == cudaSuccess) e = pW.grow(4 * K);
@@ -209,7 +216,7 @@ struct Workspace {
   }
   // whether a batch of B shots runs as pairs
   bool as_pairs(const Launch& L, long long B, bool soft) const {
-    return L.pair_mode || (B <= std::min(pair_shots, L.auto_pair_shots()) && (!soft || pair_soft));
+    return L.pair_mode || (B <= std::min(pair_shots, L.auto_pair_shots(soft)) && (!soft || pair_soft));
   }
   void release() {
     release_records();
@@ -247,12 +254,14 @@ struct Workspace {
       if (S <= pair_shots && (!soft || pair_soft)) return VIBE_OK;
       if ((e = grow_records(L, std::min(std::max(S, pair_shots), most), ps)) != cudaSuccess)
         return cuda_fail(e, "workspace");
-    } else if (larger && need > pair_shots && need <= L.auto_pair_shots() && !capturing(s)) {
-      // Shot mode: a batch that would run as pairs, the largest so far. Larger batches need no records, and a
-      // smaller one may not allocate: it runs one warp per shot if there are none yet, as a batch does
-      // whose records find no memory or that is being captured. A first soft output grows no records.
-      grow_records(L, need, ps);
+    } else if ((larger || (soft && !seen_soft)) && (need > pair_shots || (soft && !pair_soft)) &&
+               need <= L.auto_pair_shots(ps) && !capturing(s)) {
+      // Shot mode: a batch that would run as pairs, the largest so far or the first with soft output. Larger
+      // batches need no records, and other ones may not allocate: they run one warp per shot if there are
+      // none, as a batch does whose records find no memory or that is being captured.
+      grow_records(L, std::min(std::max(need, pair_shots), L.auto_pair_shots(ps)), ps);
     }
+    seen_soft |= soft;
     return VIBE_OK;
   }
   ~Workspace() { release(); }
@@ -1063,9 +1072,9 @@ int vibe_get_pairs(const vibe_handle* h, const vibe_batch* b, vibe_pairs* out) {
   const Launch& L = h ? h->L : b->L;
   const Workspace& ws = h ? h->ws : b->ws;
   out->record_bytes = L.record_bound();
-  out->shots = L.pair_mode ? -1 : L.auto_pair_shots();
-  out->shots_soft = out->shots;
-  out->held_bytes = ws.pair_shots * L.pair_shot_bytes(ws.pair_soft);
+  out->shots = L.pair_mode ? -1 : L.auto_pair_shots(false);
+  out->shots_soft = L.pair_mode ? -1 : L.auto_pair_shots(true);
+  out->held_bytes = ws.record_bytes();
   out->last = ws.last_pairs;
   return VIBE_OK;
 }
@@ -1076,8 +1085,9 @@ int vibe_set_pairs(vibe_handle* h, vibe_batch* b, int64_t record_bytes) {
   Launch& L = h ? h->L : b->L;
   Workspace& ws = h ? h->ws : b->ws;
   L.record_bytes = record_bytes;
-  if (ws.pair_shots * L.pair_shot_bytes(ws.pair_soft) > L.record_bound()) ws.release_records();
+  if (ws.record_bytes() > L.record_bound()) ws.release_records();
   ws.seen = 0;   // the next batch may get its records
+  ws.seen_soft = false;
   return VIBE_OK;
 }
 

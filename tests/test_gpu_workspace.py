@@ -139,3 +139,36 @@ def test_first_small_batch_under_capture_allocates_nothing(V):
     for k, v in want.items():
         assert torch.equal(out[k], v), k
     run.dec.close()
+
+
+@pytest.mark.parametrize("name", sorted(PROBLEMS))
+def test_first_soft_output_of_a_small_batch_runs_as_pairs(V, name):
+    build, engine = PROBLEMS[name]
+    run = Calls(V, build(), 16, 1000, engine=engine)
+    run(1000)
+    run(50, soft=True)
+    assert run.dec.pairs()["last"] == 1
+    before = free_bytes()
+    for B, soft in ((1000, True), (1000, False), (3, True)):   # the posteriors' records are there for all of them
+        run(B, soft)
+        assert run.dec.pairs()["last"] == 1
+    assert free_bytes() == before
+    run.dec.close()
+
+
+@pytest.mark.parametrize("name", sorted(PROBLEMS))
+def test_posteriors_count_in_the_bound(V, name):
+    build, engine = PROBLEMS[name]
+    run = Calls(V, build(), 16, 1000, engine=engine)
+    run(500)
+    per_shot = run.dec.pairs()["held_bytes"] / 500
+    bound = int(per_shot * 800)
+    run.dec.set_pairs(bound)
+    p = run.dec.pairs()
+    assert p["shots"] == 800 and p["shots_soft"] < 500   # a posterior is as long as the term kept without it
+    for B, soft, as_pairs in ((800, False, 1), (1000, False, 0), (p["shots_soft"], True, 1), (500, True, 0)):
+        run(B, soft)
+        q = run.dec.pairs()
+        assert q["last"] == as_pairs, (B, soft)
+        assert q["held_bytes"] <= bound, (B, soft)
+    run.dec.close()

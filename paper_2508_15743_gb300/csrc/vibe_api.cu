@@ -101,15 +101,16 @@ struct Launch {
     if (!((bnd.teams >> k) & 1)) return 0;
     return std::max(1, xocc[k] * bpx_blocks_per_sm / std::max(1, xocc[first_team()])) * num_sms;
   }
-  int bpx_grid() const {   // the largest
-    int g = 0;
-    for (int k = 0; k < vibe::kTeamClasses; ++k) g = std::max(g, bpx_grid(k));
-    return g;
-  }
   int lsd_grid() const { return std::max(1, lsd_blocks_per_sm * num_sms); }
-  // per-warp global scratch of the summary engine, bytes; the candidate posteriors only with soft output
-  long long bpx_pitch(bool soft) const {
-    return (bnd.x_warp_scratch + (soft ? 4LL * bnd.M * bnd.n : 0LL) + 15) & ~15LL;
+  // global scratch of one of the summary engine's teams, bytes; the candidate posteriors only with soft output
+  long long bpx_pitch(int k, bool soft) const {
+    return (bnd.x_warp_scratch[k] + (soft ? 4LL * bnd.M * bnd.n : 0LL) + 15) & ~15LL;
+  }
+  // of all teams: the classes run one after another in the same memory
+  long long bpx_bytes(bool soft) const {
+    long long most = 0;
+    for (int k = 0; k < vibe::kTeamClasses; ++k) most = std::max(most, (long long)bpx_grid(k) * bpx_pitch(k, soft));
+    return most;
   }
   // pair mode: bytes of one shot's member records (iteration, weight, correction, LLR term, posterior)
   long long pair_shot_bytes(bool soft) const {
@@ -129,7 +130,9 @@ struct Launch {
   // members' records pass 2 GiB.
   long long auto_pair_shots(bool soft) const {
     if (bnd.K < 2) return 0;
-    const long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta + (long long)bpx_grid();
+    long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta, teams = 0;
+    for (int k = 0; k < vibe::kTeamClasses; ++k) teams = std::max(teams, (long long)bpx_grid(k));
+    warps += teams;
     return std::min(8 * warps, record_bound() / pair_shot_bytes(soft));
   }
   static constexpr long long kAutoPairBytes = 2LL << 30;   // with the posteriors where there is soft output
@@ -230,7 +233,7 @@ struct Workspace {
     if (e == cudaSuccess) e = lsd_soft_b.grow(sizeof(float) * (size_t)c * b.n);
     if (e == cudaSuccess)
       e = bp_b.grow(sizeof(float) * (size_t)L.bp_grid() * vibe::kBpWarpsPerCta * (size_t)(2 + b.global_st + b.M) * b.n);
-    if (e == cudaSuccess) e = bpx_b.grow((size_t)L.bpx_grid() * (size_t)L.bpx_pitch(soft));
+    if (e == cudaSuccess) e = bpx_b.grow((size_t)L.bpx_bytes(soft));
     if (e == cudaSuccess)
       e = lsd_b.grow(sizeof(uint32_t) * (size_t)L.lsd_grid() * (size_t)vibe::lsd_scratch_words(b, L.lsd_threads));
     if (e != cudaSuccess) cudaGetLastError();
@@ -348,7 +351,6 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
       a.scratch = ws.bp_b.as<float>();
       a.scratch_pitch = (long long)(2 + L.bnd.global_st + L.bnd.M) * L.bnd.n;
       a.xscratch = ws.bpx_b.as<unsigned char>();
-      a.xscratch_pitch = L.bpx_pitch(a.want_soft != 0);
       a.pair_mode = pairs;
       a.pair_K = L.bnd.K;
       a.pconv = ws.pconv.as<int>(); a.pW = ws.pW.as<float>(); a.pbits = ws.pbits.as<uint32_t>();
@@ -366,6 +368,7 @@ int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, c
         if (!((L.bnd.teams >> k) & 1)) continue;
         a.flag_bad = first ? 1 : 0;
         first = false;
+        a.xscratch_pitch = L.bpx_pitch(k, a.want_soft != 0);
         a.next_shot_x = ws.ctrl() + 4 + 2 * k;
         a.next_pair_x = a.next_shot_x + 1;
         VIBE_CUDA(vibe::launch_bpx(a, team_of(k), L.msg_fp16, (int)std::min<long long>(L.bpx_grid(k), units), s),
@@ -445,7 +448,7 @@ Bounds bounds_over(const Tables* ts, int count) {
       const int k = vibe::team_class(t.team);
       b.teams |= 1 << k;
       b.x_sums[k] = std::max(b.x_sums[k], t.x_warp_smem);
-      b.x_warp_scratch = std::max(b.x_warp_scratch, t.x_warp_scratch);
+      b.x_warp_scratch[k] = std::max(b.x_warp_scratch[k], t.x_warp_scratch);
     }
   }
   return b;

@@ -111,7 +111,7 @@ struct Bounds {
   int lsd_order;   // largest LSD order
   int x_sums[kTeamClasses];   // largest check summaries of the summary-engine problems with that team size
   int teams;          // bit per team class with a problem
-  long long x_warp_scratch;   // largest summary-engine global scratch per warp, bytes
+  long long x_warp_scratch[kTeamClasses];   // largest summary-engine global scratch per team of that size, bytes
   int global_st;   // some image-engine problem keeps its step words in global scratch
   int engines;     // bit 0: some problem uses the image engine, bit 1: the summary engine
   int XD;          // largest summary-engine column-degree bound

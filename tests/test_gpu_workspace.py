@@ -172,3 +172,37 @@ def test_posteriors_count_in_the_bound(V, name):
         assert q["last"] == as_pairs, (B, soft)
         assert q["held_bytes"] <= bound, (B, soft)
     run.dec.close()
+
+
+def test_mixed_scratch_is_sized_by_team(V):
+    """A batch of a narrow and a wide problem: the many one-warp teams don't get the wide problem's scratch."""
+    from test_gpu_shot_mode import team
+
+    def used(call):
+        before = free_bytes()
+        call()
+        return before - free_bytes()
+
+    decs, alone = [], 0
+    for dm in (PROBLEMS["summary"][0](), team()):
+        run = Calls(V, dm, 4, 1, engine=SUMMARY)
+        run.dec.set_pairs(0)
+        run(1)                # kernels are loaded now
+        run.dec.close()
+        run = Calls(V, dm, 4, 1, engine=SUMMARY)
+        run.dec.set_pairs(0)
+        alone += used(lambda: run(1))
+        decs.append(run.dec)
+    first = V.MixedBatch(decs)
+    syn = torch.zeros((2, first.mw), dtype=torch.int32, device="cuda")
+    pid = torch.arange(2, dtype=torch.int32, device="cuda")
+    first.decode(pid, syn)
+    first.close()
+    mb = V.MixedBatch(decs)
+    out = dict(corrections=torch.zeros((2, mb.nw), dtype=torch.int32, device="cuda"),
+               logical=torch.zeros((2, mb.kw), dtype=torch.int32, device="cuda"),
+               stats=torch.zeros((2, 12), dtype=torch.uint8, device="cuda"))
+    assert used(lambda: mb.decode(pid, syn, out=out)) <= alone + (64 << 20)   # its buffers are rounded up, too
+    mb.close()
+    for d in decs:
+        d.close()

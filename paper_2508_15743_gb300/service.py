@@ -145,7 +145,8 @@ class StreamingService:
 class GpuBackend:
     """Decodes micro-batches with vibe_batch_decode; outputs come back through pinned host memory."""
 
-    def __init__(self, decoders, max_batch: int, pipelines: int = 2):
+    def __init__(self, decoders, max_batch: int, pipelines: int = 2, record_bytes=None):
+        """record_bytes: bound on each pipeline's members' records (vibe_set_pairs), None: the library's."""
         import torch
 
         from . import vibe as V
@@ -156,6 +157,10 @@ class GpuBackend:
         self.nw = max(d.nw for d in decoders)
         self.kw = max(d.kw for d in decoders)
         self.handles = [V.vibe_batch_create([d.handle for d in decoders]) for _ in range(self.pipelines)]
+        if record_bytes is not None:
+            usual = V.vibe_get_pairs(b=self.handles[0])["record_bytes"]
+            for b in self.handles:
+                V.vibe_set_pairs(min(int(record_bytes), usual), b=b)
         self.streams = [torch.cuda.Stream() for _ in range(self.pipelines)]
         self.events = [torch.cuda.Event() for _ in range(self.pipelines)]
         B = self.max_batch
@@ -200,16 +205,37 @@ class GpuBackend:
         return (h["corr"].numpy()[:n].view(np.uint32).copy(), h["log"].numpy()[:n].view(np.uint32).copy(),
                 self.V.stats_to_numpy(h["st"][:n]).copy())
 
+    def warm_up(self):
+        """Grows every workspace to its final size: the largest batch that shot mode runs as pairs first (its
+        records stay, smaller batches use them), then the largest batch."""
+        limit = self.V.vibe_get_pairs(b=self.handles[0])["shots"]
+        sizes = [self.max_batch] if limit < 1 else [min(limit, self.max_batch), self.max_batch]
+        for n in sorted(set(sizes)):
+            for p in range(self.pipelines):
+                self.launch(p, np.zeros(n, np.int32), np.zeros((n, self.mw), np.uint32))
+                self.events[p].synchronize()
+
     def close(self):
         for b in self.handles:
             self.V.vibe_batch_destroy(b)
         self.handles = []
+        self.h = self.d = []
 
 
 def device_bytes_per_shot(mw: int, nw: int, kw: int, n_max: int) -> int:
     """Device memory one in-flight shot holds: the service's syndrome, problem id and output rows and
     the library's per-shot workspace (LSD queue entry and soft vector)."""
     return 4 * (mw + nw + kw) + 12 + 4 + 4 + 4 * n_max
+
+
+def split_budget(room: int, pipelines: int, per_shot: int, max_batch: int):
+    """(shots per batch, bytes of members' records) of each pipeline in shot mode, of `room` bytes for all of
+    them. Records make small batches faster (vibe_set_pairs): they get an eighth, and what the batch leaves. (Of the
+    circuit-level d=9 and d=13 mix, whose tables leave 5 GB of 8, that is 40 shots' records; one request at a
+    time takes 50 ms with them and seconds without.)"""
+    mine = max(room, 0) // pipelines
+    mb = min(max_batch, (mine - mine // 8) // per_shot)
+    return mb, mine - mb * per_shot
 
 
 # Problems the command line knows: name -> (DEM builder, K, T, M, natural order)
@@ -229,7 +255,7 @@ def build_service(names, budget_bytes: int, fp16: bool, max_batch: int, pipeline
     """Creates the resident problems, sizes the micro-batches to the device-memory budget, warms the
     pipelines up and returns (service, backend, decoders, dems). pair_mode decodes each shot's members
     at the same time on different warps (vibe_params.pair_mode): same outputs, lower latency per
-    request when the GPU is not saturated."""
+    request when the GPU is not saturated; its members' records come on top of the budget."""
     import torch
 
     from . import dem as D
@@ -248,22 +274,29 @@ def build_service(names, budget_bytes: int, fp16: bool, max_batch: int, pipeline
     kw = max(d.kw for d in decs)
     per_shot = device_bytes_per_shot(mw, nw, kw, max(d.n for d in decs))
     # fixed part: resident tables and the pipelines' shot-independent workspaces (measured)
-    probe = GpuBackend(decs, 1, pipelines)
-    for p in range(pipelines):
-        probe.launch(p, np.zeros(1, np.int32), np.zeros((1, mw), np.uint32))
-    torch.cuda.synchronize()
+    probe = GpuBackend(decs, 1, pipelines, record_bytes=None if pair_mode else 0)
+    probe.warm_up()
     free1, _ = torch.cuda.mem_get_info()
     probe.close()
     fixed = max(free0 - free1, 0)
-    fit = (budget_bytes - fixed) // (pipelines * per_shot)
-    if fit < 1:
-        raise MemoryError(f"budget {budget_bytes} B leaves no room for a shot (fixed part {fixed} B)")
-    mb = int(min(max_batch, fit))
-    backend = GpuBackend(decs, mb, pipelines)
-    for p in range(pipelines):   # grow every workspace to the batch size before serving
-        backend.launch(p, np.zeros(mb, np.int32), np.zeros((mb, mw), np.uint32))
-    torch.cuda.synchronize()
-    free2, _ = torch.cuda.mem_get_info()
+    # The sizes leave out what allocators round up; what shot mode uses in the end is measured, and the batch made
+    # smaller until it is within the budget.
+    room = budget_bytes - fixed
+    while True:
+        mb, records = split_budget(room, pipelines, per_shot, int(max_batch))
+        if pair_mode:
+            mb, records = min(int(max_batch), max(room, 0) // (pipelines * per_shot)), None
+        if mb < 1:
+            raise MemoryError(f"budget {budget_bytes} B leaves no room for a shot (fixed part {fixed} B)")
+        backend = GpuBackend(decs, mb, pipelines, record_bytes=records)
+        backend.warm_up()
+        free2, _ = torch.cuda.mem_get_info()
+        over = free0 - free2 - budget_bytes
+        if pair_mode or over <= 0:
+            break
+        backend.close()
+        torch.cuda.empty_cache()
+        room -= over
     svc = StreamingService(backend, capacity=pipelines * mb, max_batch=mb, max_wait_s=max_wait_s)
     svc.budget = dict(budget_bytes=int(budget_bytes), fixed_bytes=int(fixed), per_shot_bytes=int(per_shot),
                       max_batch=mb, pipelines=pipelines, used_bytes=int(max(free0 - free2, 0)),

@@ -243,8 +243,9 @@ int vibe_decode_noalloc(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, 
  * vibe_autotune -- times the decode of a sample batch (d_syndromes: B >= 1 shots, device) and keeps the
  * fastest launch configuration for this handle. For each BP engine the problem fits
  * (VIBE_ENGINE_IMAGE, VIBE_ENGINE_SUMMARY) it searches, one knob after the other: pair or shot mode
- * (one warp per (shot, member) pair, or one warp per shot -- the pair_mode given at creation is only
- * the starting point), the BP kernel's persistent grid (occupancy maximum, 3/4 and 1/2 CTAs per SM),
+ * (one warp per (shot, member) pair, or one warp per shot whatever the sample's size -- the pair_mode given
+ * at creation is only the starting point; where shot mode is kept on a sample that it would have run as
+ * pairs, it no longer does that with any batch), the BP kernel's persistent grid (occupancy maximum, 3/4 and 1/2 CTAs per SM),
  * and the LSD kernel's CTA size (64, 128 or 256 threads: warps that reduce the columns of different
  * clusters at the same time) with its grid (maximum and half). Every candidate is timed on a second
  * decode of the sample, unless its first decode took over twice the best time so far (a mode whose

@@ -86,6 +86,7 @@ struct Launch {
   int bp_blocks_per_sm = 0, bpx_blocks_per_sm = 0, lsd_blocks_per_sm = 0;   // bpx: of the smallest teams
   int xocc[vibe::kTeamClasses] = {};   // summary engine: CTAs per SM that fit, by team class
   int pair_mode = 0;                // one warp per (shot, member) pair (vibe_params.pair_mode)
+  bool auto_pairs = true;           // shot mode runs small batches as pairs; false: the tuner found that slower
   long long record_bytes = -1;      // bound on the members' records (vibe_set_pairs); -1: kPairBytes or kAutoPairBytes
   int lsd_threads = vibe::kLsdThreads;   // threads per LSD CTA (tuned: 64, 128 or 256)
   bool warp_engine() const { return (bnd.engines & 1) != 0; }
@@ -129,7 +130,7 @@ struct Launch {
   // / 102 ms at 13 and 381 / 404 ms at 54. So the line is drawn at eight shots per warp, and where the
   // members' records pass 2 GiB.
   long long auto_pair_shots(bool soft) const {
-    if (bnd.K < 2) return 0;
+    if (bnd.K < 2 || !auto_pairs) return 0;
     long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta, teams = 0;
     for (int k = 0; k < vibe::kTeamClasses; ++k) teams = std::max(teams, (long long)bpx_grid(k));
     warps += teams;
@@ -456,7 +457,7 @@ Bounds bounds_over(const Tables* ts, int count) {
 
 // Searches the launch knobs that leave every result unchanged (shots, and within a shot the members'
 // arithmetic, are fixed; only their placement on the GPU moves) for the fastest decode of the sample q:
-// pair or shot mode (one warp per (shot, member) pair, or one per shot), then each present BP engine's
+// pair or shot mode (one warp per (shot, member) pair, or one per shot whatever the sample's size), then each present BP engine's
 // persistent grid (occupancy maximum, 3/4, 1/2 CTAs per SM), then the LSD CTA size (64, 128, 256
 // threads) with its grid (maximum, half). A candidate is timed on a first decode (the workspace grown
 // beforehand) and, unless that took more than twice the best time so far, on a second one, which
@@ -513,6 +514,7 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
   for (int pm = 1; pm >= 0 && rc == VIBE_OK; --pm) {
     L = base;
     L.pair_mode = pm;
+    L.auto_pairs = false;   // one warp per shot whatever the sample's size
     bool dropped = false;
     if (L.warp_engine()) rc = grid_search(L.bp_blocks_per_sm, dropped);
     if (rc == VIBE_OK && !dropped && L.cta_engine()) rc = grid_search(L.bpx_blocks_per_sm, dropped);
@@ -537,8 +539,21 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   L = rc == VIBE_OK ? keep : base;
+  if (rc == VIBE_OK) {   // a sample too large to run as pairs by itself says nothing about small batches
+    Launch shot = base;
+    shot.pair_mode = 0;
+    L.auto_pairs = base.auto_pairs && q.B > shot.auto_pair_shots(q.soft != nullptr);
+  }
   best_ms = best;
   return rc;
+}
+
+// After a search that kept shot mode the records of the pair candidates go; the next batch may get its own.
+void settle(const Launch& L, Workspace& ws) {
+  if (L.pair_mode) return;
+  ws.release_records();
+  ws.seen = 0;
+  ws.seen_soft = false;
 }
 
 }  // namespace
@@ -1050,6 +1065,7 @@ int vibe_autotune(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, void* 
   }
   if ((rc = set_engine(h, best_engine)) != VIBE_OK) return rc;
   h->L = best_L;   // same engine, so the same problem descriptor and bounds
+  settle(h->L, h->ws);
   if (engine_out) *engine_out = best_engine;
   if (bp_blocks_per_sm) *bp_blocks_per_sm = h->L.warp_engine() ? h->L.bp_blocks_per_sm : h->L.bpx_blocks_per_sm;
   if (lsd_blocks_per_sm) *lsd_blocks_per_sm = h->L.lsd_blocks_per_sm;
@@ -1134,6 +1150,7 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
   bt->L.bnd = b;
   bt->L.msg_fp16 = h0->L.msg_fp16;
   bt->L.pair_mode = h0->L.pair_mode;
+  bt->L.auto_pairs = h0->L.auto_pairs;
   bt->L.record_bytes = h0->L.record_bytes;
   bt->L.device = h0->device;
   bt->L.num_sms = h0->L.num_sms;
@@ -1171,6 +1188,7 @@ int vibe_batch_autotune(vibe_batch* b, const int32_t* d_problem, const uint32_t*
   float ms = 0.f;
   const int rc = tune_launch(b->L, b->ws, b->prof, q, static_cast<cudaStream_t>(stream), ms);
   cudaFree(corr);
+  if (rc == VIBE_OK) settle(b->L, b->ws);
   return rc;
 }
 

@@ -128,7 +128,12 @@ struct Launch {
   // circuit-level d=5 (K=32, FP16) 202 / 73 ms at 1.1 shots per resident warp, 358 / 281 ms at 4.5; the
   // 4.8.8 d=9 phenomenological code (K=16) 46.3 / 40.7 ms at 4.5 and 157 / 155 ms at 18; the 6.6.6 one 99.6
   // / 102 ms at 13 and 381 / 404 ms at 54. So the line is drawn at eight shots per warp, and where the
-  // members' records pass 2 GiB.
+  // members' records pass 2 GiB. Below it pairs take 0.02 to 1.0 of the other's time over phenomenological d = 3, 5,
+  // 9 at p = 3e-4 to 1e-2 and circuit-level d = 3, 5, 7 at p = 1e-4 to 2e-3, K = 16 to 64, M = 1 to 8. Low noise is
+  // no exception, though all K members may run where M would do: a single shot that does not converge keeps its
+  // warp for K * T sweeps (circuit d=3, p = 1e-4, K=64, M=1, at the line: 169 / 15 ms). Pairs lose where no
+  // shot is like that and a sweep is as short as taking a pair from the counter, 0.7 ns each: d=3, p = 3e-4, K=64, M=1
+  // 0.52 / 1.04 ms at the line, 0.50 / 0.54 ms at half of it; and by up to 11 % at the line for d=5, p = 1e-2.
   long long auto_pair_shots(bool soft) const {
     if (bnd.K < 2 || !auto_pairs) return 0;
     long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta, teams = 0;

@@ -917,10 +917,12 @@ size_t bp_warp_smem_bytes(Tables* t, int msg_fp16) {
   t->off_par = (int)o;
   o = align16(o + words);
   // decision bytes and step words share their place: a member uses one of them. The words of a graph of
-  // long chains (few columns per step) that would take more than n + 2m bytes go to global scratch.
+  // long chains (few columns per step) go to global scratch where they would take the state beyond that of a
+  // byte per decision, per syndrome bit and per parity (which bounds the problems the engine takes).
   t->off_dec = t->off_st = (int)o;
+  const size_t bytes3 = align16(dec) + 2 * align16(((size_t)t->m + 3) / 4 * 4);
   size_t d = bytes ? dec : 0;
-  if (steps <= std::max<size_t>(d, (size_t)t->n + 2 * (size_t)t->m)) d = std::max(d, steps);
+  if (steps <= bytes3 - 2 * align16(words)) d = std::max(d, steps);
   else t->off_st = -1;
   o = align16(o + d);
   t->off_cand = (int)o;

@@ -802,13 +802,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     // not pay: d=11 with four 158 -> 153 ms, d=9 with two, in batches that fill the GPU, 92 -> 103 ms.
     if (t.XD > 0 && msg_bytes > kTeamImageBytes && t.SP >= 24 * vibe::kTeam * 32) {
       const long long single = t.nstep;
-      int optin = 0;
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
       VIBE_TRY(steps(vibe::kTeam), "step builder");
-      t.engine = VIBE_ENGINE_SUMMARY;
-      if (3 * t.nstep > 4 * single || vibe::bpx_cta_smem_bytes(bounds_over(&t, 1), vibe::kTeam, vibe::kMaxDems) > (size_t)optin)
-        VIBE_TRY(steps(1), "step builder");
-      t.engine = p->bp_engine;
+      if (3 * t.nstep > 4 * single) VIBE_TRY(steps(1), "step builder");
     }
     t.soff_pitch = t.nstep + vibe::kStepPad;
     VIBE_TRY(dalloc(&h->soff, (size_t)K * t.soff_pitch), "tables");

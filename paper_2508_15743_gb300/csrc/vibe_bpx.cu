@@ -966,7 +966,10 @@ static size_t team_smem(const Bounds& b, int team, int chunk) {
   return sizeof(TeamCmd) + (size_t)team * window_bytes(chunk) + (size_t)b.x_sums[team_class(team)];
 }
 
-// Steps per chunk: kChunk, or for single warps 2 where only that fits beside the summaries and descriptors.
+// Steps per chunk: kChunk, or for single warps 2 where only that fits beside the summaries and descriptors. That
+// takes m above 10,000, and LSD's shared memory ends at m = 4300, so 2 is not chosen at present. The choice
+// stays because the kernel without it measured slower with FP32 messages: XYZ d=7 49.9 -> 53.2 ms, circuit d=11 150 ->
+// 161 ms, the same in five forms of the code around the sweep.
 static int bpx_chunk(const Bounds& b, int team, int ndem) {
   const size_t limit = 227u * 1024u;   // shared memory of a CTA on sm_103a
   return team == 1 && team_smem(b, team, kChunk) + a16((size_t)ndem * sizeof(Tables)) > limit ? 2 : kChunk;

@@ -121,28 +121,53 @@ __device__ __forceinline__ bool is_finite_bits(float x) {
 // reads only its own slots, so the passes need no second image. Parity pass: (H e)_c XOR s_c from
 // the decisions (many columns touch a check in the column pass); returns whether the lane met an
 // unsatisfied check.
+// Its cost is instructions (18.4 G warp instructions for 60,000 shots of an all-flooding d=7 ensemble before, 13.2 G
+// in the form that read the tables from the parameter space): the row's swizzle is found once per row, from a row pitch
+// known at compile time, and a column's entries are one load. All flooding, d=7 phenomenological, K=8, T=20, 200,000
+// shots: FP32 86.1 -> 45.5 ms, FP16 (layer_sweep) 82.0 -> 59.2; all layered 199.9 -> 125.3 and 146.7 -> 106.1.
+// The csc_ent entries of column v (entries past its degree are not used). Where DP <= 4 every problem of the launch
+// has the pitch 4: one load.
+template <int DP>
+__device__ __forceinline__ void column_entries(const uint32_t* csc, size_t pitch, int v, int deg, uint32_t (&ent)[DP]) {
+  if constexpr (DP <= 4) {
+    const uint4 x = __ldg(reinterpret_cast<const uint4*>(csc) + v);
+    const uint32_t e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int k = 0; k < DP; ++k) ent[k] = e[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < DP; ++k) ent[k] = k < deg ? __ldg(csc + v * pitch + k) : 0u;
+  }
+}
+
 __device__ __forceinline__ uint32_t syn_bit(const uint32_t* s32, int c) { return (s32[c >> 5] >> (c & 31)) & 1u; }
 
-template <int DP>
+template <int DP, int NCH>
 __device__ __forceinline__ bool flood_sweep(const Tables& t, float alpha, float* msgs, uint8_t* dec8,
                                             const uint32_t* s32, float* lpost, int lane) {
   const int m = t.m, n = t.n;
-  const uint32_t RP = (uint32_t)t.RP;
+  // copies of t's fields: the stores below might alias t, which would make every use a load
+  const int32_t *rowptr = t.rowptr, *colidx = t.colidx, *colptr = t.colptr;
+  const uint32_t* csc = t.csc_ent;
+  const float* lam = t.lam;
+  const size_t pitch = (size_t)t.DP;
+  const uint32_t RP = NCH ? (uint32_t)(NCH * Msg<float>::kSpc) : (uint32_t)t.RP;
   for (int c = lane; c < m; c += 32) {
-    const int deg = __ldg(t.rowptr + c + 1) - __ldg(t.rowptr + c);
+    const int deg = __ldg(rowptr + c + 1) - __ldg(rowptr + c);
     float* row = msgs + (size_t)c * RP;
+    const uint32_t swz = row_position((uint32_t)c, 0u, (int)RP, 4);   // slot j is at j ^ swz
     float m1 = __int_as_float(0x7f800000), m2 = m1;
     int a1 = -1;
     uint32_t sx = 0;
     for (int j = 0; j < deg; ++j) {
-      const float x = row[row_position((uint32_t)c, (uint32_t)j, (int)RP, 4)];
+      const float x = row[(uint32_t)j ^ swz];
       const float ax = fabsf(x);
       sx ^= __float_as_uint(x) >> 31;
       if (ax < m1) { m2 = m1; m1 = ax; a1 = j; }
       else if (ax < m2) m2 = ax;
     }
     for (int j = 0; j < deg; ++j) {
-      const uint32_t pos = row_position((uint32_t)c, (uint32_t)j, (int)RP, 4);
+      const uint32_t pos = (uint32_t)j ^ swz;
       const float x = row[pos];
       const float mn = j == a1 ? m2 : m1;
       const uint32_t neg = (sx ^ (__float_as_uint(x) >> 31) ^ syn_bit(s32, c)) & 1u;
@@ -152,7 +177,9 @@ __device__ __forceinline__ bool flood_sweep(const Tables& t, float alpha, float*
   }
   __syncwarp();
   for (int v = lane; v < n; v += 32) {
-    const int deg = __ldg(t.colptr + v + 1) - __ldg(t.colptr + v);
+    const int deg = __ldg(colptr + v + 1) - __ldg(colptr + v);
+    uint32_t ent[DP];
+    column_entries<DP>(csc, pitch, v, deg, ent);
     float* slot[DP];
     float cv[DP];
 #pragma unroll
@@ -160,12 +187,11 @@ __device__ __forceinline__ bool flood_sweep(const Tables& t, float alpha, float*
       slot[k] = msgs;
       cv[k] = 0.0f;
       if (k < deg) {
-        const uint32_t ent = __ldg(t.csc_ent + (size_t)v * t.DP + k);
-        slot[k] = msgs + (size_t)(ent >> 9) * RP + (ent & 0xffu);
+        slot[k] = msgs + (size_t)(ent[k] >> 9) * RP + (ent[k] & 0xffu);
         cv[k] = *slot[k];
       }
     }
-    const float lamv = __ldg(t.lam + v);
+    const float lamv = __ldg(lam + v);
     float L = lamv;
 #pragma unroll
     for (int k = 0; k < DP; ++k)
@@ -189,7 +215,7 @@ __device__ __forceinline__ bool flood_sweep(const Tables& t, float alpha, float*
   bool bad = false;
   for (int c = lane; c < m; c += 32) {
     uint32_t p = syn_bit(s32, c);
-    for (int e = __ldg(t.rowptr + c); e < __ldg(t.rowptr + c + 1); ++e) p ^= dec8[__ldg(t.colidx + e)];
+    for (int e = __ldg(rowptr + c); e < __ldg(rowptr + c + 1); ++e) p ^= dec8[__ldg(colidx + e)];
     bad |= p != 0u;
   }
   __syncwarp();
@@ -209,31 +235,38 @@ __device__ __forceinline__ bool flood_sweep(const Tables& t, float alpha, float*
 // exclusion sums over the column's current cv entries, stored as its new variable-to-check messages).
 // Then every posterior (lambda plus the column's cv entries in ascending check order), decision and
 // check parity. cv holds zeros when a layered member starts (init in run_member).
-template <typename MT, int DP>
+template <typename MT, int DP, int NCH>
 __device__ __forceinline__ bool layer_sweep(const Tables& t, float alpha, bool flood, MT* msgs, float* cv,
                                             uint8_t* dec8, const uint32_t* s32, float* lpost, int lane) {
   const int m = t.m, n = t.n;
-  const uint32_t RP = (uint32_t)t.RP;
+  // copies of t's fields: the stores below might alias t, which would make every use a load
+  const int32_t *rowptr = t.rowptr, *colidx = t.colidx, *colptr = t.colptr, *layer_ptr = t.layer_ptr,
+                *layer_chk = t.layer_chk, *layer_vptr = t.layer_vptr, *layer_var = t.layer_var;
+  const uint32_t* csc = t.csc_ent;
+  const float* lam = t.lam;
+  const size_t pitch = (size_t)t.DP;
+  const uint32_t RP = NCH ? (uint32_t)(NCH * Msg<MT>::kSpc) : (uint32_t)t.RP;
   const int nl = flood ? 1 : t.nlayer;
   for (int l = 0; l < nl; ++l) {
-    const int c0 = flood ? 0 : __ldg(t.layer_ptr + l), c1 = flood ? m : __ldg(t.layer_ptr + l + 1);
+    const int c0 = flood ? 0 : __ldg(layer_ptr + l), c1 = flood ? m : __ldg(layer_ptr + l + 1);
     for (int q = c0 + lane; q < c1; q += 32) {
-      const int c = flood ? q : __ldg(t.layer_chk + q);
-      const int deg = __ldg(t.rowptr + c + 1) - __ldg(t.rowptr + c);
+      const int c = flood ? q : __ldg(layer_chk + q);
+      const int deg = __ldg(rowptr + c + 1) - __ldg(rowptr + c);
       const MT* row = msgs + (size_t)c * RP;
       float* crow = cv + (size_t)c * RP;
+      const uint32_t swz = row_position((uint32_t)c, 0u, (int)RP, Msg<MT>::kSpc);   // slot j is at j ^ swz
       float m1 = __int_as_float(0x7f800000), m2 = m1;
       int a1 = -1;
       uint32_t sx = 0;
       for (int j = 0; j < deg; ++j) {
-        const float x = Msg<MT>::value(row[row_position((uint32_t)c, (uint32_t)j, (int)RP, Msg<MT>::kSpc)]);
+        const float x = Msg<MT>::value(row[(uint32_t)j ^ swz]);
         const float ax = fabsf(x);
         sx ^= __float_as_uint(x) >> 31;
         if (ax < m1) { m2 = m1; m1 = ax; a1 = j; }
         else if (ax < m2) m2 = ax;
       }
       for (int j = 0; j < deg; ++j) {
-        const uint32_t pos = row_position((uint32_t)c, (uint32_t)j, (int)RP, Msg<MT>::kSpc);
+        const uint32_t pos = (uint32_t)j ^ swz;
         const float x = Msg<MT>::value(row[pos]);
         const uint32_t neg = (sx ^ (__float_as_uint(x) >> 31) ^ syn_bit(s32, c)) & 1u;
         const float mag = __fmul_rn(alpha, j == a1 ? m2 : m1);
@@ -241,23 +274,23 @@ __device__ __forceinline__ bool layer_sweep(const Tables& t, float alpha, bool f
       }
     }
     __syncwarp();
-    const int v0 = flood ? 0 : __ldg(t.layer_vptr + l), v1 = flood ? n : __ldg(t.layer_vptr + l + 1);
+    const int v0 = flood ? 0 : __ldg(layer_vptr + l), v1 = flood ? n : __ldg(layer_vptr + l + 1);
     for (int q = v0 + lane; q < v1; q += 32) {
-      const int v = flood ? q : __ldg(t.layer_var + q);
-      const int deg = __ldg(t.colptr + v + 1) - __ldg(t.colptr + v);
-      uint32_t slot[DP];
+      const int v = flood ? q : __ldg(layer_var + q);
+      const int deg = __ldg(colptr + v + 1) - __ldg(colptr + v);
+      uint32_t slot[DP], ent[DP];
+      column_entries<DP>(csc, pitch, v, deg, ent);
       float c2v[DP];
 #pragma unroll
       for (int k = 0; k < DP; ++k) {
         slot[k] = 0u;
         c2v[k] = 0.0f;
         if (k < deg) {
-          const uint32_t ent = __ldg(t.csc_ent + (size_t)v * t.DP + k);
-          slot[k] = (ent >> 9) * RP + (ent & 0xffu);
+          slot[k] = (ent[k] >> 9) * RP + (ent[k] & 0xffu);
           c2v[k] = cv[slot[k]];
         }
       }
-      float pre = __ldg(t.lam + v);   // lambda + m_0 + ... + m_{k-1}, the shared head of every exclusion sum
+      float pre = __ldg(lam + v);   // lambda + m_0 + ... + m_{k-1}, the shared head of every exclusion sum
 #pragma unroll
       for (int k = 0; k < DP; ++k) {
         if (k < deg) {
@@ -273,14 +306,13 @@ __device__ __forceinline__ bool layer_sweep(const Tables& t, float alpha, bool f
     __syncwarp();
   }
   for (int v = lane; v < n; v += 32) {
-    const int deg = __ldg(t.colptr + v + 1) - __ldg(t.colptr + v);
-    float L = __ldg(t.lam + v);
+    const int deg = __ldg(colptr + v + 1) - __ldg(colptr + v);
+    float L = __ldg(lam + v);
+    uint32_t ent[DP];
+    column_entries<DP>(csc, pitch, v, deg, ent);
 #pragma unroll
     for (int k = 0; k < DP; ++k)
-      if (k < deg) {
-        const uint32_t ent = __ldg(t.csc_ent + (size_t)v * t.DP + k);
-        L = __fadd_rn(L, cv[(ent >> 9) * RP + (ent & 0xffu)]);
-      }
+      if (k < deg) L = __fadd_rn(L, cv[(ent[k] >> 9) * RP + (ent[k] & 0xffu)]);
     dec8[v] = L <= 0.0f ? 1u : 0u;
     if (lpost) lpost[v] = L;
   }
@@ -288,7 +320,7 @@ __device__ __forceinline__ bool layer_sweep(const Tables& t, float alpha, bool f
   bool bad = false;
   for (int c = lane; c < m; c += 32) {
     uint32_t p = syn_bit(s32, c);
-    for (int e = __ldg(t.rowptr + c); e < __ldg(t.rowptr + c + 1); ++e) p ^= dec8[__ldg(t.colidx + e)];
+    for (int e = __ldg(rowptr + c); e < __ldg(rowptr + c + 1); ++e) p ^= dec8[__ldg(colidx + e)];
     bad |= p != 0u;
   }
   __syncwarp();
@@ -472,9 +504,9 @@ __device__ __noinline__ int run_member(const Tables& t, int i, int smem_off, Ima
       MT* msgs = reinterpret_cast<MT*>(base + t.off_msg);
       uint8_t* dec8 = base + t.off_dec;
       if (std::is_same<MT, float>::value && flood)
-        bad = flood_sweep<DP>(t, alpha, reinterpret_cast<float*>(msgs), dec8, s32, lp, lane);
+        bad = flood_sweep<DP, NCH>(t, alpha, reinterpret_cast<float*>(msgs), dec8, s32, lp, lane);
       else
-        bad = layer_sweep<MT, DP>(t, alpha, flood, msgs, cv, dec8, s32, lp, lane);
+        bad = layer_sweep<MT, DP, NCH>(t, alpha, flood, msgs, cv, dec8, s32, lp, lane);
     } else {
       if (lp)
         step_sweep<MT, DP, NCH, true>(t, soff, ns, first, alpha, sbase + t.off_msg, sbase + t.off_s, sbase + t.off_par,

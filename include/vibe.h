@@ -134,7 +134,7 @@ typedef struct vibe_batch vibe_batch; /* opaque: several handles decoded in one 
  *   (member i: SplitMix64 started at seed + (i+1)*0xD1B54A32D192ED03, Durstenfeld shuffle taking
  *   j = high 64 bits of next()*(k+1) for k = n-1 down to 1).
  *   Uses the current CUDA device. Copies everything it is given; the device tables (CSR/CSC of H,
- *   per-member packed steps, message images) stay resident until vibe_destroy.
+ *   per-member packed steps -- two sets for wide graphs --, message images) stay resident until vibe_destroy.
  *   Limits of this build (VIBE_ERR_UNSUPPORTED beyond them): n < 2^24, m < 2^24, every row of H has
  *   at most 255 entries, every column at most 32, and one shot's BP state (messages, posteriors,
  *   syndrome) must fit in 200 KB of shared memory.
@@ -284,6 +284,8 @@ typedef struct {
   int64_t shots_soft;   /* the same with soft output */
   int64_t held_bytes;   /* members' records in the workspace now */
   int32_t last;         /* how the last decode ran: 1 as pairs, 0 one warp or team per shot, -1 none yet */
+  int32_t team;         /* most warps that took a member's steps together in it: 1, or 8 where a wide problem
+                           (summary engine) is in a batch that does not fill the GPU; 0 none yet */
 } vibe_pairs;
 
 /*

@@ -132,8 +132,8 @@ struct Launch {
   // 9 at p = 3e-4 to 1e-2 and circuit-level d = 3, 5, 7 at p = 1e-4 to 2e-3, K = 16 to 64, M = 1 to 8. Low noise is
   // no exception, though all K members may run where M would do: a single shot that does not converge keeps its
   // warp for K * T sweeps (circuit d=3, p = 1e-4, K=64, M=1, at the line: 169 / 15 ms). Pairs lose where no
-  // shot is like that and a sweep is as short as taking a pair from the counter, 0.7 ns each: d=3, p = 3e-4, K=64, M=1
-  // 0.52 / 1.04 ms at the line, 0.50 / 0.54 ms at half of it; and by up to 11 % at the line for d=5, p = 1e-2.
+  // shot is like that and a sweep is as short as taking a pair from the counter, 0.7 ns each: d=3, p = 3e-4, M=1 at the
+  // line 0.52 / 1.04 ms with K=64 and 0.5 / 4.1 ms with K=255; and by up to 13 % at the line for d=5, p = 1e-2.
   long long auto_pair_shots(bool soft) const {
     if (bnd.K < 2 || !auto_pairs) return 0;
     long long warps = (long long)bp_grid() * vibe::kBpWarpsPerCta, teams = 0;
@@ -143,6 +143,15 @@ struct Launch {
   }
   static constexpr long long kAutoPairBytes = 2LL << 30;   // with the posteriors where there is soft output
 };
+
+// The launch of a batch of `units` shots or (shot, member) pairs. LT, if there is one, packs the wide problems for
+// teams of eight warps: a member takes less time, but its lanes are used less well and its barriers cost, so that pays
+// only while the GPU is not full. Circuit-level d=13, pairs, team / one warp: 512 pairs FP32 71 / 77 ms, FP16 67
+// / 79; 1200 pairs 133 / 129 and 124 / 80; 2048 pairs 234 / 160 and 223 / 147; one shot a team, 4000 shots
+// 1677 / 1091 and 1552 / 884. The line lies at twice the teams that are resident (608).
+const Launch& pick_launch(const Launch& L, const Launch* LT, long long units) {
+  return LT && units <= 2LL * LT->bpx_grid(1) ? *LT : L;
+}
 
 // Device memory that only grows.
 struct Buffer {
@@ -193,6 +202,7 @@ struct Workspace {
 
   long long seen = 0;        // largest batch so far
   bool seen_soft = false;    // whether one had soft output
+  int last_team = 0;         // largest team of the last decode
   int last_pairs = -1;       // whether the last decode ran as pairs
 
   long long record_bytes() const {
@@ -245,23 +255,17 @@ struct Workspace {
     if (e != cudaSuccess) cudaGetLastError();
     return e;
   }
-  int ensure(const Launch& L, long long need, bool soft, cudaStream_t s) {
-    const long long c = std::max(std::min(need, chunk_max), chunk);
-    if (c > chunk) chunk = 0;   // should a growth fail, the next call asks for its own size
-    cudaError_t e = grow_scratch(L, c, soft);
-    if (e != cudaSuccess && !L.pair_mode && pair_shots > 0) {   // shot mode can do without records
-      release_records();
-      e = grow_scratch(L, c, soft);
-    }
-    if (e != cudaSuccess) return cuda_fail(e, "workspace");
-    chunk = c;
+  // Makes room for a batch of `need` shots and picks its launch and mode (see pick_launch).
+  int ensure(const Launch& L, const Launch* LT, long long need, bool soft, cudaStream_t s, const Launch** use,
+             bool* pairs) {
     const bool larger = need > seen;
     seen = std::max(seen, need);
     const bool ps = soft || pair_soft;
+    cudaError_t e;
     if (L.pair_mode) {   // records of as many shots as a launch takes, and no fewer than before
       const long long most = L.pair_chunk(ps), S = std::min(need, most);
-      if (S <= pair_shots && (!soft || pair_soft)) return VIBE_OK;
-      if ((e = grow_records(L, std::min(std::max(S, pair_shots), most), ps)) != cudaSuccess)
+      if ((S > pair_shots || (soft && !pair_soft)) &&
+          (e = grow_records(L, std::min(std::max(S, pair_shots), most), ps)) != cudaSuccess)
         return cuda_fail(e, "workspace");
     } else if ((larger || (soft && !seen_soft)) && (need > pair_shots || (soft && !pair_soft)) &&
                need <= L.auto_pair_shots(ps) && !capturing(s)) {
@@ -271,6 +275,16 @@ struct Workspace {
       grow_records(L, std::min(std::max(need, pair_shots), L.auto_pair_shots(ps)), ps);
     }
     seen_soft |= soft;
+    const long long c = std::max(std::min(need, chunk_max), chunk);
+    if (c > chunk) chunk = 0;   // should a growth fail, the next call asks for its own size
+    for (;;) {
+      *pairs = as_pairs(L, need, soft);
+      *use = &pick_launch(L, LT, *pairs ? need * L.bnd.K : need);
+      if ((e = grow_scratch(**use, c, soft)) == cudaSuccess) break;
+      if (L.pair_mode || pair_shots == 0) return cuda_fail(e, "workspace");
+      release_records();   // shot mode can do without
+    }
+    chunk = c;
     return VIBE_OK;
   }
   ~Workspace() { release(); }
@@ -315,12 +329,15 @@ struct Batch {
 // then one LSD launch over the shots they queued. In pair mode the BP part of a chunk runs in
 // sub-chunks of up to ws.pair_shots shots (the member records), all queueing into the chunk's LSD
 // launch, so a chunk's slowest LSD shots are waited for once, not once per sub-chunk.
-int run_decode(const Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaStream_t s) {
-  int rc = ws.ensure(L, q.B, q.soft != nullptr, s);
+int run_decode(const Launch& L1, const Launch* LT, Workspace& ws, Profiler& prof, const Batch& q, cudaStream_t s) {
+  const Launch* use = &L1;
+  bool pairs = false;
+  int rc = ws.ensure(L1, LT, q.B, q.soft != nullptr, s, &use, &pairs);
   if (rc != VIBE_OK) return rc;
+  const Launch& L = *use;
   const long long step = ws.chunk;
-  const bool pairs = ws.as_pairs(L, q.B, q.soft != nullptr);
   ws.last_pairs = pairs;
+  ws.last_team = L.bnd.teams & 2 ? vibe::kTeam : 1;
   for (long long b0 = 0; b0 < q.B; b0 += step) {
     const long long nb = std::min(step, q.B - b0);
     VIBE_CUDA(cudaMemsetAsync(ws.ctrl(), 0, Workspace::kCtrl * sizeof(unsigned int), s), "decode");
@@ -468,17 +485,17 @@ Bounds bounds_over(const Tables* ts, int count) {
 // beforehand) and, unless that took more than twice the best time so far, on a second one, which
 // counts; a mode whose first candidate is rejected that way is dropped. L keeps the fastest; best_ms
 // its time.
-int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaStream_t s, float& best_ms) {
+int tune_launch(Launch& L1, Launch* LT, Workspace& ws, Profiler& prof, const Batch& q, cudaStream_t s, float& best_ms) {
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   VIBE_CUDA(cudaEventCreate(&e0), "autotune");
   if (cudaEventCreate(&e1) != cudaSuccess) { cudaEventDestroy(e0); return cuda_fail(cudaGetLastError(), "autotune"); }
-  const Launch base = L;
-  Launch keep = base;
+  Launch L = L1, keep = L1;   // the candidate, the best one
+  bool team = false, keep_team = false;   // whether it is LT's
   float best = 1e30f;
   int rc = VIBE_OK;
   auto timed = [&](float& ms) -> int {
     cudaEventRecord(e0, s);
-    const int r = run_decode(L, ws, prof, q, s);
+    const int r = run_decode(L, nullptr, ws, prof, q, s);
     if (r != VIBE_OK) return r;
     cudaEventRecord(e1, s);
     VIBE_CUDA(cudaEventSynchronize(e1), "autotune");
@@ -487,13 +504,15 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
   };
   // times the current L; ms = 0 marks a rejected candidate
   auto time_once = [&](float& ms) -> int {
-    int r = ws.ensure(L, q.B, q.soft != nullptr, s);
+    const Launch* use;
+    bool pairs;
+    int r = ws.ensure(L, nullptr, q.B, q.soft != nullptr, s, &use, &pairs);
     if (r != VIBE_OK) return r;
     float first = 0.f;
     if ((r = timed(first)) != VIBE_OK) return r;
     if (first > 2.f * best) { ms = 0.f; return VIBE_OK; }
     if ((r = timed(ms)) != VIBE_OK) return r;
-    if (ms < best) { best = ms; keep = L; }
+    if (ms < best) { best = ms; keep = L; keep_team = team; }
     return VIBE_OK;
   };
   // one BP grid knob: the occupancy maximum and two fractions of it; leaves the fastest in cfg.
@@ -517,7 +536,9 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
     return VIBE_OK;
   };
   for (int pm = 1; pm >= 0 && rc == VIBE_OK; --pm) {
+    const Launch& base = pick_launch(L1, LT, pm ? q.B * L1.bnd.K : q.B);
     L = base;
+    team = &base != &L1;
     L.pair_mode = pm;
     L.auto_pairs = false;   // one warp per shot whatever the sample's size
     bool dropped = false;
@@ -527,6 +548,7 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
   const int nts[] = {64, 128, 256};
   for (int ni = 0; ni < 3 && rc == VIBE_OK; ++ni) {
     L = keep;
+    team = keep_team;
     L.lsd_threads = nts[ni];
     int mx = 0;
     if (vibe::lsd_occupancy(L.bnd, L.ndem, nts[ni], &mx) != cudaSuccess || mx < 1) {
@@ -543,14 +565,24 @@ int tune_launch(Launch& L, Workspace& ws, Profiler& prof, const Batch& q, cudaSt
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
-  L = rc == VIBE_OK ? keep : base;
-  if (rc == VIBE_OK) {   // a sample too large to run as pairs by itself says nothing about small batches
-    Launch shot = base;
-    shot.pair_mode = 0;
-    L.auto_pairs = base.auto_pairs && q.B > shot.auto_pair_shots(q.soft != nullptr);
-  }
   best_ms = best;
-  return rc;
+  if (rc != VIBE_OK) return rc;
+  Launch shot = L1;
+  shot.pair_mode = 0;
+  // a sample too large to run as pairs by itself says nothing about small batches
+  keep.auto_pairs = L1.auto_pairs && q.B > shot.auto_pair_shots(q.soft != nullptr);
+  for (Launch* o : {&L1, LT}) {   // the mode and LSD's shape are for all batches, the BP grids for batches like this one
+    if (!o) continue;
+    if ((o == LT) == keep_team) {
+      *o = keep;
+    } else {
+      o->pair_mode = keep.pair_mode;
+      o->auto_pairs = keep.auto_pairs;
+      o->lsd_threads = keep.lsd_threads;
+      o->lsd_blocks_per_sm = keep.lsd_blocks_per_sm;
+    }
+  }
+  return VIBE_OK;
 }
 
 // After a search that kept shot mode the records of the pair candidates go; the next batch may get its own.
@@ -566,8 +598,10 @@ void settle(const Launch& L, Workspace& ws) {
 struct vibe_handle {
   int device = 0;
   Tables t{};                 // host copy of the problem descriptor
-  Tables* d_desc = nullptr;   // device copy
-  Launch L;
+  bool wide = false;          // there is a second packing of the steps, for teams of eight warps
+  Tables tt{};                // descriptor with that packing
+  Tables* d_desc = nullptr;   // device copies of both
+  Launch L, LT;
   Workspace ws;
   Profiler prof;
   // resident tables
@@ -577,9 +611,12 @@ struct vibe_handle {
   float* lam = nullptr;
   float* alpha_m = nullptr;
   void* msg_init = nullptr;
-  uint32_t *cpos = nullptr, *soff = nullptr, *xlnk = nullptr, *xcolid = nullptr, *xrmap = nullptr;
-  int32_t* stepcnt = nullptr;
-  uint2* xrec = nullptr;
+  uint32_t* cpos = nullptr;
+  struct Steps {
+    uint32_t *soff = nullptr, *xlnk = nullptr, *xcolid = nullptr, *xrmap = nullptr;
+    int32_t* stepcnt = nullptr;
+    uint2* xrec = nullptr;
+  } steps[2];   // of single warps, of teams (wide)
   int32_t *layer_ptr = nullptr, *layer_chk = nullptr, *layer_vptr = nullptr, *layer_var = nullptr,
           *nlayer_d = nullptr;
   float4* xsum = nullptr;
@@ -593,6 +630,7 @@ struct vibe_handle {
     cudaFree(st_syn); cudaFree(st_corr); cudaFree(st_log); cudaFree(st_obs); cudaFree(st_stats);
     st_syn = st_corr = st_log = st_obs = nullptr; st_stats = nullptr; stage_cap = 0;
   }
+  const Launch* team_launch() const { return wide ? &LT : nullptr; }
   ~vibe_handle() {
     int prev = 0;
     cudaGetDevice(&prev);
@@ -602,8 +640,10 @@ struct vibe_handle {
     cudaFree(tmp_counters);
     cudaFree(rowptr); cudaFree(colidx); cudaFree(colptr); cudaFree(rowidx); cudaFree(lrowptr); cudaFree(lcolidx);
     cudaFree(csc_ent); cudaFree(perm); cudaFree(lam); cudaFree(alpha_m);
-    cudaFree(msg_init); cudaFree(cpos); cudaFree(soff); cudaFree(stepcnt); cudaFree(xrec); cudaFree(xlnk); cudaFree(xcolid);
-    cudaFree(xrmap); cudaFree(xsum); cudaFree(d_desc);
+    cudaFree(msg_init); cudaFree(cpos); cudaFree(xsum); cudaFree(d_desc);
+    for (Steps& p : steps) {
+      cudaFree(p.soff); cudaFree(p.stepcnt); cudaFree(p.xrec); cudaFree(p.xlnk); cudaFree(p.xcolid); cudaFree(p.xrmap);
+    }
     cudaFree(layer_ptr); cudaFree(layer_chk); cudaFree(layer_vptr); cudaFree(layer_var); cudaFree(nlayer_d);
     cudaSetDevice(prev);
   }
@@ -612,10 +652,12 @@ struct vibe_handle {
 struct vibe_batch {
   int device = 0;
   std::vector<vibe_handle*> hs;
-  Tables* d_desc = nullptr;
-  Launch L;
+  Tables* d_desc = nullptr;   // the problems, then the same with teams where they have that packing
+  bool wide = false;          // some have
+  Launch L, LT;
   Workspace ws;
   Profiler prof;
+  const Launch* team_launch() const { return wide ? &LT : nullptr; }
   ~vibe_batch() {
     int prev = 0;
     cudaGetDevice(&prev);
@@ -644,6 +686,26 @@ int handle_view(const vibe_handle* h, HandleView* v) {
 int set_error(int code, const char* msg) { return fail(code, "%s", msg); }
 
 }  // namespace vibe
+
+namespace {
+
+// d's steps become those of `packed`.
+void with_packing(Tables& d, const Tables& packed) {
+  d.team = packed.team; d.nstep = packed.nstep; d.soff_pitch = packed.soff_pitch;
+  d.stepcnt = packed.stepcnt; d.soff = packed.soff;
+  d.xrec = packed.xrec; d.xlnk = packed.xlnk; d.xcolid = packed.xcolid; d.xrmap = packed.xrmap;
+}
+
+// The launch of the team packing beside h->L.
+int size_team_launch(vibe_handle* h) {
+  h->LT = h->L;
+  h->LT.one = h->tt;
+  h->LT.d_desc = h->d_desc + 1;
+  h->LT.bnd = bounds_over(&h->tt, 1);
+  return size_launch(h->LT);
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -753,9 +815,8 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   VIBE_TRY(dalloc(&h->alpha_m, K), "tables");
   VIBE_TRY(cudaMalloc(&h->msg_init, std::max<size_t>(msg_bytes, 16)), "tables");
   VIBE_TRY(dalloc(&h->cpos, E), "tables");
-  VIBE_TRY(dalloc(&h->stepcnt, K), "tables");
   VIBE_TRY(dalloc(&h->xsum, m), "tables");
-  VIBE_TRY(dalloc(&h->d_desc, 1), "tables");
+  VIBE_TRY(dalloc(&h->d_desc, 2), "tables");
   if (p->n_layered > 0) {
     VIBE_TRY(dalloc(&h->layer_ptr, (size_t)m + 1), "tables");
     VIBE_TRY(dalloc(&h->layer_chk, (size_t)m), "tables");
@@ -784,40 +845,43 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
            "graph builder");
   {
     std::vector<int32_t> cnt(K);
-    auto steps = [&](int team) -> cudaError_t {
-      cudaError_t er = vibe::build_steps(m, n, K, team, h->perm, h->colptr, h->cpos, h->stepcnt, scratch, s);
+    // The steps of teams of `team` warps into packing P; with `wanted`, unless their count does not suit it.
+    auto pack = [&](int team, vibe_handle::Steps& P, Tables& d, auto&& wanted) -> cudaError_t {
+      cudaError_t er = P.stepcnt ? cudaSuccess : dalloc(&P.stepcnt, K);
+      if (er == cudaSuccess) er = vibe::build_steps(m, n, K, team, h->perm, h->colptr, h->cpos, P.stepcnt, scratch, s);
       if (er == cudaSuccess)
-        er = cudaMemcpyAsync(cnt.data(), h->stepcnt, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, s);
+        er = cudaMemcpyAsync(cnt.data(), P.stepcnt, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, s);
       if (er == cudaSuccess) er = cudaStreamSynchronize(s);
-      t.team = team;
-      t.nstep = er == cudaSuccess ? *std::max_element(cnt.begin(), cnt.end()) : 0;
+      if (er != cudaSuccess) return er;
+      d.team = team;
+      d.nstep = *std::max_element(cnt.begin(), cnt.end());
+      d.soff_pitch = d.nstep + vibe::kStepPad;
+      if (!wanted(d.nstep)) return cudaSuccess;
+      er = dalloc(&P.soff, (size_t)K * d.soff_pitch);
+      if (er == cudaSuccess) er = dalloc(&P.xrec, (size_t)K * d.SP + 4);   // copied in groups of four slots
+      if (er == cudaSuccess) er = dalloc(&P.xlnk, (size_t)K * d.SP + 4);
+      if (er == cudaSuccess) er = dalloc(&P.xcolid, (size_t)K * d.SP);
+      if (er == cudaSuccess && d.XD > 0) er = dalloc(&P.xrmap, (size_t)K * E);
+      // the lanes' order pays where the image engine runs (xcolid serves as its scratch: it is filled next)
+      if (er == cudaSuccess && team == 1 && msg_bytes <= kTeamImageBytes)
+        er = vibe::order_steps(n, d.SP, K, d.nstep, h->colptr, h->cpos, P.stepcnt, scratch, P.xcolid, s);
+      if (er == cudaSuccess)
+        er = vibe::fill_steps(n, E, d.SP, K, d.DP, team, d.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, P.stepcnt,
+                              scratch, P.soff, P.xrec, P.xlnk, P.xcolid, P.xrmap, s);
+      d.stepcnt = P.stepcnt; d.soff = P.soff; d.xrec = P.xrec; d.xlnk = P.xlnk; d.xcolid = P.xcolid; d.xrmap = P.xrmap;
       return er;
     };
-    VIBE_TRY(steps(1), "step builder");
-    // Wide graphs get a team of eight warps per member, where only the summary engine can run them and
-    // units of 8 x 32 edges keep at least 3/4 of their lanes at work (random orders: circuit-level d=13 7674
-    // steps with one warp, 1066 units with eight; d=11 4407 and 998: no). A member then takes that much less
-    // time, and its check summaries, which leave one-warp members 7 (FP32) or 12 warps on an SM at d=13,
-    // serve all eight. Measured, 4 shots of d=9 and d=13 (K=32, T=50): 182 -> 99 ms. Smaller teams did
-    // not pay: d=11 with four 158 -> 153 ms, d=9 with two, in batches that fill the GPU, 92 -> 103 ms.
+    VIBE_TRY(pack(1, h->steps[0], t, [](int) { return true; }), "step builder");
+    // Wide graphs get a second packing for teams of eight warps per member, which small batches use (pick_launch),
+    // where only the summary engine can run them and units of 8 x 32 edges keep at least 3/4 of their lanes at
+    // work (random orders: circuit-level d=13 7674 steps with one warp, 1066 units with eight; d=11 4407 and
+    // 998: no). Measured, 4 shots of d=9 and d=13 (K=32, T=50): 182 -> 99 ms. Smaller teams did not pay: d=11
+    // with four 158 -> 153 ms, d=9 with two, in batches that fill the GPU, 92 -> 103 ms.
     if (t.XD > 0 && msg_bytes > kTeamImageBytes && t.SP >= 24 * vibe::kTeam * 32) {
-      const long long single = t.nstep;
-      VIBE_TRY(steps(vibe::kTeam), "step builder");
-      if (3 * t.nstep > 4 * single) VIBE_TRY(steps(1), "step builder");
-    }
-    t.soff_pitch = t.nstep + vibe::kStepPad;
-    VIBE_TRY(dalloc(&h->soff, (size_t)K * t.soff_pitch), "tables");
-    VIBE_TRY(dalloc(&h->xrec, (size_t)K * t.SP + 4), "tables");   // copied in groups of four slots
-    VIBE_TRY(dalloc(&h->xlnk, (size_t)K * t.SP + 4), "tables");
-    VIBE_TRY(dalloc(&h->xcolid, (size_t)K * t.SP), "tables");
-    if (t.XD > 0) VIBE_TRY(dalloc(&h->xrmap, (size_t)K * E), "tables");
-    // the lanes' order pays where the image engine runs (xcolid serves as its scratch: it is filled next)
-    if (t.team == 1 && msg_bytes <= kTeamImageBytes)
-      VIBE_TRY(vibe::order_steps(n, t.SP, K, t.nstep, h->colptr, h->cpos, h->stepcnt, scratch, h->xcolid, s),
+      h->tt = t;
+      VIBE_TRY(pack(vibe::kTeam, h->steps[1], h->tt, [&](int ns) { return h->wide = 3LL * ns <= 4LL * t.nstep; }),
                "step builder");
-    VIBE_TRY(vibe::fill_steps(n, E, t.SP, K, t.DP, t.team, t.soff_pitch, h->rowptr, h->colptr, h->cpos, h->lam, h->stepcnt, scratch,
-                              h->soff, h->xrec, h->xlnk, h->xcolid, h->xrmap, s),
-             "step builder");
+    }
   }
   vibe::bpx_layout(&t, p->msg_fp16);
   vibe::bp_warp_smem_bytes(&t, p->msg_fp16);
@@ -850,8 +914,15 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   t.rowptr = h->rowptr; t.colidx = h->colidx; t.colptr = h->colptr; t.rowidx = h->rowidx;
   t.csc_ent = h->csc_ent; t.lam = h->lam; t.alpha_m = h->alpha_m; t.msg_init = h->msg_init;
   t.lrowptr = h->lrowptr; t.lcolidx = h->lcolidx;
-  t.stepcnt = h->stepcnt; t.soff = h->soff; t.xrec = h->xrec; t.xlnk = h->xlnk; t.xcolid = h->xcolid; t.xrmap = h->xrmap; t.xsum = h->xsum;
-  VIBE_TRY(cudaMemcpyAsync(h->d_desc, &t, sizeof(Tables), cudaMemcpyHostToDevice, s), "upload");
+  t.xsum = h->xsum;
+  if (h->wide) {
+    const Tables packed = h->tt;
+    h->tt = t;
+    with_packing(h->tt, packed);
+    vibe::bpx_layout(&h->tt, p->msg_fp16);
+  }
+  const Tables desc[2] = {t, h->wide ? h->tt : t};
+  VIBE_TRY(cudaMemcpyAsync(h->d_desc, desc, sizeof(desc), cudaMemcpyHostToDevice, s), "upload");
   VIBE_TRY(cudaStreamSynchronize(s), "graph builder");
   cudaFree(scratch);
   scratch = nullptr;
@@ -863,6 +934,7 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
   h->L.ndem = 1;
   h->L.bnd = bounds_over(&t, 1);
   if ((rc = size_launch(h->L)) != VIBE_OK) return bail(rc);
+  if (h->wide && (rc = size_team_launch(h)) != VIBE_OK) return bail(rc);
   h->ws.chunk_max = std::max<long long>(1, (long long)(kWorkspaceBytes / ((size_t)n * 4 + 8)));
   *out = h;
   return VIBE_OK;
@@ -879,7 +951,7 @@ int vibe_decode(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, uint32_t
   const Tables& t = h->t;
   Batch q{nullptr, d_syndromes, t.mw, B, d_corrections, t.nw, d_logical, t.kw, d_stats, d_soft, t.n,
           d_observables, reinterpret_cast<unsigned long long*>(d_counters)};
-  return run_decode(h->L, h->ws, h->prof, q, static_cast<cudaStream_t>(stream));
+  return run_decode(h->L, h->team_launch(), h->ws, h->prof, q, static_cast<cudaStream_t>(stream));
 }
 
 int vibe_decode_host(vibe_handle* h, const uint32_t* h_syndromes, int64_t B, uint32_t* h_corrections,
@@ -911,7 +983,7 @@ int vibe_decode_host(vibe_handle* h, const uint32_t* h_syndromes, int64_t B, uin
                                   cudaMemcpyHostToDevice, s), "H2D");
       Batch q{nullptr, h->st_syn, t.mw, nb, h->st_corr, t.nw, h->st_log, t.kw, h->st_stats, nullptr, t.n,
               h_observables ? h->st_obs : nullptr, h_counters ? h->tmp_counters : nullptr};
-      int rc = run_decode(h->L, h->ws, h->prof, q, s);
+      int rc = run_decode(h->L, h->team_launch(), h->ws, h->prof, q, s);
       if (rc != VIBE_OK) return rc;
       VIBE_CUDA(cudaMemcpyAsync(h_corrections + (size_t)b0 * t.nw, h->st_corr, sizeof(uint32_t) * nb * t.nw,
                                 cudaMemcpyDeviceToHost, s), "D2H");
@@ -1030,7 +1102,7 @@ static int set_engine(vibe_handle* h, int engine) {
   int rc = size_launch(L);
   if (rc != VIBE_OK) return rc;
   VIBE_CUDA(cudaMemcpy(h->d_desc, &t, sizeof(Tables), cudaMemcpyHostToDevice), "engine switch");
-  h->t = t;
+  h->t = t;   // a wide problem runs on the summary engine only: its team packing stays as it is
   h->L = L;
   return VIBE_OK;
 }
@@ -1040,30 +1112,33 @@ int vibe_autotune(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, void* 
   if (!h || !d_syndromes || B < 1) return fail(VIBE_ERR_INVALID, "NULL handle/syndromes or empty sample");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int start_engine = h->t.engine;
-  const Launch start = h->L;
+  const Launch start = h->L, start_team = h->LT;
   uint32_t* corr = nullptr;
   VIBE_CUDA(dalloc(&corr, (size_t)B * h->t.nw), "autotune");
   int rc = VIBE_OK;
   float best = 1e30f;
   int best_engine = start_engine;
-  Launch best_L = start;
+  Launch best_L = start, best_team = start_team;
   const int cand_engine[] = {VIBE_ENGINE_IMAGE, VIBE_ENGINE_SUMMARY};
   for (int ci = 0; ci < 2 && rc == VIBE_OK; ++ci) {
     h->L = start;
+    h->LT = start_team;
     if (set_engine(h, cand_engine[ci]) != VIBE_OK) continue;   // the problem does not fit this engine
     const Tables& t = h->t;
     Batch q{nullptr, d_syndromes, t.mw, B, corr, t.nw, nullptr, t.kw, nullptr, nullptr, t.n, nullptr, nullptr};
     float ms = 0.f;
-    if ((rc = tune_launch(h->L, h->ws, h->prof, q, s, ms)) != VIBE_OK) break;
-    if (ms < best) { best = ms; best_engine = cand_engine[ci]; best_L = h->L; }
+    if ((rc = tune_launch(h->L, h->wide ? &h->LT : nullptr, h->ws, h->prof, q, s, ms)) != VIBE_OK) break;
+    if (ms < best) { best = ms; best_engine = cand_engine[ci]; best_L = h->L; best_team = h->LT; }
   }
   cudaFree(corr);
   h->L = start;
+  h->LT = start_team;
   if (rc != VIBE_OK) {
     set_engine(h, start_engine);
     return rc;
   }
   if ((rc = set_engine(h, best_engine)) != VIBE_OK) return rc;
+  h->LT = best_team;
   h->L = best_L;   // same engine, so the same problem descriptor and bounds
   settle(h->L, h->ws);
   if (engine_out) *engine_out = best_engine;
@@ -1095,6 +1170,7 @@ int vibe_get_pairs(const vibe_handle* h, const vibe_batch* b, vibe_pairs* out) {
   out->shots_soft = L.pair_mode ? -1 : L.auto_pair_shots(true);
   out->held_bytes = ws.record_bytes();
   out->last = ws.last_pairs;
+  out->team = ws.last_team;
   return VIBE_OK;
 }
 
@@ -1104,6 +1180,7 @@ int vibe_set_pairs(vibe_handle* h, vibe_batch* b, int64_t record_bytes) {
   Launch& L = h ? h->L : b->L;
   Workspace& ws = h ? h->ws : b->ws;
   L.record_bytes = record_bytes;
+  (h ? h->LT : b->LT).record_bytes = record_bytes;
   if (ws.record_bytes() > L.record_bound()) ws.release_records();
   ws.seen = 0;   // the next batch may get its records
   ws.seen_soft = false;
@@ -1123,12 +1200,15 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
   for (int i = 0; i < count; ++i)
     if (!handles[i]) return fail(VIBE_ERR_INVALID, "handle %d is NULL", i);
   const vibe_handle* h0 = handles[0];
-  std::vector<Tables> desc(count);
+  std::vector<Tables> desc(2 * count);   // with single warps, with teams where a problem has that packing
+  bool wide = false;
   for (int i = 0; i < count; ++i) {
     const vibe_handle* h = handles[i];
     if (h->device != h0->device) return fail(VIBE_ERR_INVALID, "handles live on different devices");
     if (h->L.msg_fp16 != h0->L.msg_fp16) return fail(VIBE_ERR_INVALID, "handles mix FP16 and FP32 messages");
     desc[i] = h->t;
+    desc[count + i] = h->wide ? h->tt : h->t;
+    wide |= h->wide;
   }
   const Bounds b = bounds_over(desc.data(), count);
   int cur = -1;
@@ -1139,8 +1219,8 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
   bt->device = h0->device;
   bt->hs.assign(handles, handles + count);
   cudaError_t e;
-  if ((e = dalloc(&bt->d_desc, count)) != cudaSuccess) { delete bt; return cuda_fail(e, "batch"); }
-  if ((e = cudaMemcpy(bt->d_desc, desc.data(), sizeof(Tables) * count, cudaMemcpyHostToDevice)) != cudaSuccess) {
+  if ((e = dalloc(&bt->d_desc, 2 * (size_t)count)) != cudaSuccess) { delete bt; return cuda_fail(e, "batch"); }
+  if ((e = cudaMemcpy(bt->d_desc, desc.data(), sizeof(Tables) * 2 * count, cudaMemcpyHostToDevice)) != cudaSuccess) {
     delete bt;
     return cuda_fail(e, "batch");
   }
@@ -1155,6 +1235,13 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
   bt->L.device = h0->device;
   bt->L.num_sms = h0->L.num_sms;
   int rc = size_launch(bt->L);
+  if (rc == VIBE_OK && wide) {
+    bt->wide = true;
+    bt->LT = bt->L;
+    bt->LT.d_desc = bt->d_desc + count;
+    bt->LT.bnd = bounds_over(desc.data() + count, count);
+    rc = size_launch(bt->LT);
+  }
   if (rc != VIBE_OK) { delete bt; return rc; }
   bt->ws.chunk_max = std::max<long long>(1, (long long)(kWorkspaceBytes / ((size_t)b.n * 4 + 8)));
   *out = bt;
@@ -1173,7 +1260,7 @@ int vibe_batch_decode(vibe_batch* b, const int32_t* d_problem, const uint32_t* d
     return fail(VIBE_ERR_INVALID, "strides smaller than the largest problem's words");
   Batch q{d_problem, d_syndromes, syn_stride, B, d_corrections, corr_stride, d_logical, log_stride, d_stats, nullptr,
           b->L.bnd.n, d_observables, reinterpret_cast<unsigned long long*>(d_counters)};
-  return run_decode(b->L, b->ws, b->prof, q, static_cast<cudaStream_t>(stream));
+  return run_decode(b->L, b->team_launch(), b->ws, b->prof, q, static_cast<cudaStream_t>(stream));
 }
 
 int vibe_batch_autotune(vibe_batch* b, const int32_t* d_problem, const uint32_t* d_syndromes, int32_t syn_stride,
@@ -1186,7 +1273,7 @@ int vibe_batch_autotune(vibe_batch* b, const int32_t* d_problem, const uint32_t*
   Batch q{d_problem, d_syndromes, syn_stride, B, corr, b->L.bnd.nw, nullptr, b->L.bnd.kw, nullptr, nullptr,
           b->L.bnd.n, nullptr, nullptr};
   float ms = 0.f;
-  const int rc = tune_launch(b->L, b->ws, b->prof, q, static_cast<cudaStream_t>(stream), ms);
+  const int rc = tune_launch(b->L, b->wide ? &b->LT : nullptr, b->ws, b->prof, q, static_cast<cudaStream_t>(stream), ms);
   cudaFree(corr);
   if (rc == VIBE_OK) settle(b->L, b->ws);
   return rc;

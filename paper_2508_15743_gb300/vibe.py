@@ -247,7 +247,7 @@ def vibe_get_launch(h=None, b=None):
 
 class vibe_pairs(ctypes.Structure):
     _fields_ = [("record_bytes", ctypes.c_int64), ("shots", ctypes.c_int64), ("shots_soft", ctypes.c_int64),
-                ("held_bytes", ctypes.c_int64), ("last", ctypes.c_int32)]
+                ("held_bytes", ctypes.c_int64), ("last", ctypes.c_int32), ("team", ctypes.c_int32)]
 
 
 def vibe_get_pairs(h=None, b=None):

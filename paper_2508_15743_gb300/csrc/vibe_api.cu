@@ -80,6 +80,7 @@ struct Launch {
   bool mixed = false;               // shots name their problems (vibe_batch)
   const Tables* d_desc = nullptr;   // ndem problem descriptors on the device
   int ndem = 0;
+  int wide = 0;                     // of them with the team packing (a team launch)
   Bounds bnd{};
   int msg_fp16 = 0;
   int device = 0, num_sms = 0;
@@ -148,9 +149,11 @@ struct Launch {
 // teams of eight warps: a member takes less time, but its lanes are used less well and its barriers cost, so that pays
 // only while the GPU is not full. Circuit-level d=13, pairs, team / one warp: 512 pairs FP32 71 / 77 ms, FP16 67
 // / 79; 1200 pairs 133 / 129 and 124 / 80; 2048 pairs 234 / 160 and 223 / 147; one shot a team, 4000 shots
-// 1677 / 1091 and 1552 / 884. The line lies at twice the teams that are resident (608).
+// 1677 / 1091 and 1552 / 884. The line lies at twice the teams that are resident (608). Where the shots' problems are
+// not known here, as many units are taken to be the wide ones' as of the problems are wide: their launch runs by
+// itself. (1000 shots of d=9 and d=13 in equal parts, one shot a team or warp, K=32, T=50: 5.4 / 6.8 s.)
 const Launch& pick_launch(const Launch& L, const Launch* LT, long long units) {
-  return LT && units <= 2LL * LT->bpx_grid(1) ? *LT : L;
+  return LT && units * LT->wide <= 2LL * LT->bpx_grid(1) * LT->ndem ? *LT : L;
 }
 
 // Device memory that only grows.
@@ -701,6 +704,7 @@ int size_team_launch(vibe_handle* h) {
   h->LT = h->L;
   h->LT.one = h->tt;
   h->LT.d_desc = h->d_desc + 1;
+  h->LT.wide = 1;
   h->LT.bnd = bounds_over(&h->tt, 1);
   return size_launch(h->LT);
 }
@@ -1201,14 +1205,14 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
     if (!handles[i]) return fail(VIBE_ERR_INVALID, "handle %d is NULL", i);
   const vibe_handle* h0 = handles[0];
   std::vector<Tables> desc(2 * count);   // with single warps, with teams where a problem has that packing
-  bool wide = false;
+  int wide = 0;
   for (int i = 0; i < count; ++i) {
     const vibe_handle* h = handles[i];
     if (h->device != h0->device) return fail(VIBE_ERR_INVALID, "handles live on different devices");
     if (h->L.msg_fp16 != h0->L.msg_fp16) return fail(VIBE_ERR_INVALID, "handles mix FP16 and FP32 messages");
     desc[i] = h->t;
     desc[count + i] = h->wide ? h->tt : h->t;
-    wide |= h->wide;
+    wide += h->wide ? 1 : 0;
   }
   const Bounds b = bounds_over(desc.data(), count);
   int cur = -1;
@@ -1239,6 +1243,7 @@ int vibe_batch_create(vibe_handle* const* handles, int32_t count, vibe_batch** o
     bt->wide = true;
     bt->LT = bt->L;
     bt->LT.d_desc = bt->d_desc + count;
+    bt->LT.wide = wide;
     bt->LT.bnd = bounds_over(desc.data() + count, count);
     rc = size_launch(bt->LT);
   }

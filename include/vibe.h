@@ -69,11 +69,12 @@ typedef struct {
                         mixing heuristics (Sec. V); results, ranking and LLR average are otherwise
                         unchanged. Both engines, all schedules and storage precisions */
   int32_t pair_mode; /* 0: one warp per shot runs the shot's members one after another (throughput), except
-                        that a batch of at most eight shots per resident warp, whose members' records
-                        fit in 2 GiB, runs as in pair mode, which ends sooner; 1: one warp per (shot, member) pair, so a shot's members run at the same time
-                        and its BP latency is that of its slowest member, not the sum (latency). The
-                        outputs are identical; pair mode does more sweeps in total (members run until
-                        they see M earlier candidates) and keeps every member's record per shot */
+                        that a batch of at most eight shots per resident warp whose members' records fit
+                        (vibe_set_pairs) runs as in pair mode, which ends sooner; 1: one warp per (shot,
+                        member) pair, so a shot's members run at the same time and its BP latency is that of
+                        its slowest member, not the sum (latency). The outputs are identical; pairs do more
+                        sweeps in total (members run until they see M earlier candidates) and keep every
+                        member's record per shot */
   int32_t n_layered; /* members n_flood .. n_flood+n_layered-1 use a layered schedule (Sec. V names
                         layered schedules between serial and parallel without defining one; read as
                         row-layered min-sum): the checks are split into layers by greedy colouring in
@@ -87,7 +88,8 @@ typedef struct {
                         only, FP32 or FP16 storage (only the variable-to-check messages are rounded) */
 } vibe_params;
 
-/* BP engines; both run one warp per shot (per (shot, member) pair in pair mode) and give the same bits.
+/* BP engines; both give the same bits and run one warp per shot, or per (shot, member) pair (the summary engine a
+ * team of eight warps where a wide graph is in a batch that does not fill the GPU).
  * IMAGE: the member's whole message image in shared memory; fast for problems whose image is small
  * (code capacity, phenomenological). SUMMARY: the messages in global memory in schedule order and,
  * per check, a summary in shared memory (smallest and second-smallest magnitude with their holders, a
@@ -114,7 +116,9 @@ typedef struct {
 #define VIBE_CNT_SHOTS 0       /* shots decoded */
 #define VIBE_CNT_FAILURES 1    /* shots whose L*e differs from the given observables */
 #define VIBE_CNT_LSD 2         /* shots sent to LSD */
-#define VIBE_CNT_PAIR_ITERS 3  /* BP sweeps executed, summed over (shot, member) pairs */
+#define VIBE_CNT_PAIR_ITERS 3  /* BP sweeps executed, summed over (shot, member) pairs; where pairs run (also for
+                                  shot mode's small batches) those of members that turn out not to count are in
+                                  it, as many as their timing allows */
 #define VIBE_CNT_UNSOLVABLE 4
 #define VIBE_CNT_BAD_PROBLEM 5 /* vibe_batch_decode shots with an out-of-range problem index */
 #define VIBE_CNT_RESCANS 6     /* summary engine: check rows rescanned (a summary could not answer) */
@@ -135,9 +139,11 @@ typedef struct vibe_batch vibe_batch; /* opaque: several handles decoded in one 
  *   j = high 64 bits of next()*(k+1) for k = n-1 down to 1).
  *   Uses the current CUDA device. Copies everything it is given; the device tables (CSR/CSC of H,
  *   per-member packed steps -- two sets for wide graphs --, message images) stay resident until vibe_destroy.
- *   Limits of this build (VIBE_ERR_UNSUPPORTED beyond them): n < 2^24, m < 2^24, every row of H has
- *   at most 255 entries, every column at most 32, and one shot's BP state (messages, posteriors,
- *   syndrome) must fit in 200 KB of shared memory.
+ *   Limits of this build (VIBE_ERR_UNSUPPORTED beyond them): n < 2^23, m <= 16384, every row of H has
+ *   at most 255 entries, every column at most 32 (16 for the summary engine), and the states must fit in the
+ *   227 KB of shared memory of a CTA: LSD's, about 54 bytes per check and, up to 6144 columns, 16 per column
+ *   (which ends at about 4300 checks), and the BP engine's, two members' message images (image engine) or 16
+ *   bytes per check, 8 with FP16 messages (summary engine).
  *   Errors: VIBE_ERR_INVALID (NULL pointers, malformed CSR, a row with no entry, priors outside
  *   (0, 0.5), bad K/params, schedules not permutations), VIBE_ERR_NOMEM, VIBE_ERR_CUDA.
  *   On error *out is set to NULL and nothing is leaked.
@@ -202,7 +208,7 @@ int vibe_get_layers(vibe_handle* h, int32_t* layer_of_check_out, int32_t* nlayer
  * vibe_decode launches on the caller's stream; clears the totals. vibe_profile_read waits for the
  * last recorded event and returns the summed device time (ms) of the BP ensemble kernel and of the
  * LSD kernel since the last vibe_profile call, and how many of each were launched. A decode runs in
- * chunks, each one LSD launch after its BP launches; in pair mode a chunk's BP part is several
+ * chunks, each one LSD launch after its BP launches; where pairs run a chunk's BP part is several
  * launches (sized by the member records), timed together as the chunk's BP time.
  */
 int vibe_profile(vibe_handle* h, int32_t enable);
@@ -213,14 +219,14 @@ int vibe_profile_read(vibe_handle* h, double* bp_ms, double* lsd_ms, int64_t* bp
  * decode: a control loop that has to keep a fixed memory footprint once running, a process sharing
  * the GPU under a hard memory budget, or code running where the CUDA allocator may not be entered.
  * The paper has no counterpart; this is an operational variant of vibe_decode.
- *   It runs the same BP ensemble and LSD kernels but takes all of their scratch from one static
+ *   It runs the same BP ensemble and LSD kernels, one warp per shot, but takes all of their scratch from one static
  *   device array of 64 MiB that every GPU loading the library holds until the process exits. It
  *   calls no cudaMalloc/cudaFree and allocates nothing on the host; the handle must already exist.
  *   Inputs and outputs are as for vibe_decode (d_logical and d_stats may be NULL); no soft output,
  *   observables or counters.
  *   Limit: B shots need B*(4n+4) bytes beside a fixed part that depends on the problem
- *   (counters, one n-float accumulator per BP warp, one row set per LSD CTA); a batch that does not
- *   fit returns VIBE_ERR_UNSUPPORTED with the largest batch that does (about 15,000 shots for the
+ *   (counters, two or three rows of n floats per BP warp, one row set per LSD CTA); a batch that does not
+ *   fit returns VIBE_ERR_UNSUPPORTED with the largest batch that does (about 17,000 shots for the
  *   d=9 phenomenological problem) -- split larger batches into several calls.
  *   CUDA loads device code lazily by default (CUDA_MODULE_LOADING=EAGER changes that), so the array is
  *   placed on a device, and its address looked up (cudaGetSymbolAddress, with the handle's device
@@ -245,8 +251,8 @@ int vibe_decode_noalloc(vibe_handle* h, const uint32_t* d_syndromes, int64_t B, 
  * (VIBE_ENGINE_IMAGE, VIBE_ENGINE_SUMMARY) it searches, one knob after the other: pair or shot mode
  * (one warp per (shot, member) pair, or one warp per shot whatever the sample's size -- the pair_mode given
  * at creation is only the starting point; where shot mode is kept on a sample that it would have run as
- * pairs, it no longer does that with any batch), the BP kernel's persistent grid (occupancy maximum, 3/4 and 1/2 CTAs per SM),
- * and the LSD kernel's CTA size (64, 128 or 256 threads: warps that reduce the columns of different
+ * pairs, it no longer does that with any batch), the BP kernel's persistent grid (occupancy maximum, 3/4 and
+ * 1/2 CTAs per SM), and the LSD kernel's CTA size (64, 128 or 256 threads: warps that reduce the columns of different
  * clusters at the same time) with its grid (maximum and half). Every candidate is timed on a second
  * decode of the sample, unless its first decode took over twice the best time so far (a mode whose
  * first candidate fails that way is dropped). Decoding results do not depend on any of these knobs (shots are
@@ -295,7 +301,8 @@ typedef struct {
  *   a small batch runs as pairs only while its records fit (record_bytes = 0: never, one warp or team per
  *   shot whatever the batch); in pair mode a launch takes as many shots as fit, one at least. -1: the sizes a
  *   handle is created with, 2 GiB in shot mode and 8 GiB in pair mode. Results do not depend on it. Records
- *   held beyond the new bound are freed, and the next call may allocate its own. A vibe_batch starts with the bound of its first handle.
+ *   held beyond the new bound are freed, and the next call may allocate its own. A vibe_batch starts with the
+ *   bound of its first handle.
  *   Errors: VIBE_ERR_INVALID.
  */
 int vibe_get_pairs(const vibe_handle* h, const vibe_batch* b, vibe_pairs* out);

@@ -372,7 +372,8 @@ int run_decode(const Launch& L1, const Launch* LT, Workspace& ws, Profiler& prof
       a.soft = q.soft ? q.soft + (size_t)o * q.soft_stride : nullptr; a.soft_stride = q.soft_stride;
       a.obs = q.obs ? q.obs + (size_t)o * q.log_stride : nullptr;
       a.counters = q.counters;
-      a.next_shot = ws.ctrl(); a.lsd_count = ws.ctrl() + 1; a.lsd_shots = ws.lsd_shots_b.as<uint32_t>(); a.lsd_soft = ws.lsd_soft_b.as<float>();
+      a.next_shot = ws.ctrl(); a.lsd_count = ws.ctrl() + 1;
+      a.lsd_shots = ws.lsd_shots_b.as<uint32_t>(); a.lsd_soft = ws.lsd_soft_b.as<float>();
       a.lsd_shot_base = (uint32_t)s0;
       a.scratch = ws.bp_b.as<float>();
       a.scratch_pitch = (long long)(2 + L.bnd.global_st + L.bnd.M) * L.bnd.n;
@@ -414,7 +415,8 @@ int run_decode(const Launch& L1, const Launch* LT, Workspace& ws, Profiler& prof
     l.soft = q.soft ? q.soft + (size_t)b0 * q.soft_stride : nullptr; l.soft_stride = q.soft_stride;
     l.obs = q.obs ? q.obs + (size_t)b0 * q.log_stride : nullptr;
     l.counters = q.counters;
-    l.lsd_count = ws.ctrl() + 1; l.lsd_shots = ws.lsd_shots_b.as<uint32_t>(); l.lsd_soft = ws.lsd_soft_b.as<float>(); l.lsd_next = ws.ctrl() + 2;
+    l.lsd_count = ws.ctrl() + 1; l.lsd_next = ws.ctrl() + 2;
+    l.lsd_shots = ws.lsd_shots_b.as<uint32_t>(); l.lsd_soft = ws.lsd_soft_b.as<float>();
     l.scratch = ws.lsd_b.as<uint32_t>();
     l.scratch_pitch = vibe::lsd_scratch_words(L.bnd, L.lsd_threads);
     VIBE_CUDA(vibe::launch_lsd(l, L.lsd_grid(), L.lsd_threads, s), "LSD kernel launch");
@@ -482,8 +484,8 @@ Bounds bounds_over(const Tables* ts, int count) {
 
 // Searches the launch knobs that leave every result unchanged (shots, and within a shot the members'
 // arithmetic, are fixed; only their placement on the GPU moves) for the fastest decode of the sample q:
-// pair or shot mode (one warp per (shot, member) pair, or one per shot whatever the sample's size), then each present BP engine's
-// persistent grid (occupancy maximum, 3/4, 1/2 CTAs per SM), then the LSD CTA size (64, 128, 256
+// pair or shot mode (one warp per (shot, member) pair, or one per shot whatever the sample's size), then each
+// present BP engine's persistent grid (occupancy maximum, 3/4, 1/2 CTAs per SM), then the LSD CTA size (64, 128, 256
 // threads) with its grid (maximum, half). A candidate is timed on a first decode (the workspace grown
 // beforehand) and, unless that took more than twice the best time so far, on a second one, which
 // counts; a mode whose first candidate is rejected that way is dropped. L keeps the fastest; best_ms

@@ -354,10 +354,11 @@ constexpr int kRecSteps = 2;   // steps fetched together, one group ahead
 // stores the new message in its slot. Decisions are one
 // word per step (on the lane of the column's last edge); check parities are flipped, and the word
 // stored, only when one changes.
-// What bounds it: shared-memory wavefronts (94 % of their peak). The lanes' rows are random; the order of a
-// step's columns (k_step_order) brings a 16-byte row load of 32 lanes from ~9.5 wavefronts to ~8 (ideal 4).
-// With one lane per column a sweep of the d=9 phenomenological problem took 42 chunks of 187 instructions
-// and 2800 wavefronts; its 62 steps take 90 instructions each. Measured, 32768 shots of it (K=16, T=30):
+// What bounds it: shared-memory wavefronts (90 % of their peak with FP32 messages; with FP16 77 %, and issue at
+// 67 %). The lanes' rows are random; the order of a step's columns (k_step_order) brings a 16-byte row load of 32
+// lanes from ~9.5 wavefronts to ~8 (ideal 4). With one lane per column a sweep of the d=9 phenomenological problem
+// took 42 chunks of 187 warp instructions and 2800 wavefronts in all; its 62 steps take 95 (FP16 84) and 33
+// wavefronts (FP16 20) each, by the profiler's counters. Measured, 32768 shots of it (K=16, T=30):
 // 96.7 -> 61.7 ms with FP32 messages (73.1 before the order and without the dropped slot), 78.1 -> 48.0 ms with
 // FP16; the 4.8.8 code, whose rows of 10 now take three chunks instead of four, 40 -> 13 ms.
 // NCH: 16-byte chunks of a row (0: from the tables). par32 holds the check parities.

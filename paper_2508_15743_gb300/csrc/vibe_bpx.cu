@@ -3,10 +3,10 @@
 // results as the image engine (vibe_bp.cu), which keeps a member's whole message image in shared
 // memory; a different layout.
 //
-// Mapping: one warp, or for wide graphs a team of 8 (a CTA either way), per (shot, member), one lane per
-// edge. A sweep runs the
-// member's steps (k_steps in vibe_graph.cu): up to 32 edges per warp of columns that share no check, packed
-// in the member's order. A lane asks its check's summary for the check-to-variable message of its edge,
+// Mapping: one warp, or for wide graphs in batches that do not fill the GPU a team of 8 (a CTA either way), per
+// (shot, member), one lane per edge. A sweep runs the member's steps (k_steps in vibe_graph.cu): up to 32 edges per
+// warp of columns that share no check, packed in the member's order. A lane asks its check's summary for the
+// check-to-variable message of its edge,
 // the lanes of a column pass each other these messages with shuffles, and every lane forms its own
 // exclusion sum and updates its own check. A team takes a unit of as many steps as it has warps at a
 // time, no two of which share a check, with a barrier after each unit. In shot mode each team decodes one
@@ -40,12 +40,15 @@
 // l's edge; the decision on the lane of the column's last edge). Messages are read only by rescans,
 // through a per-member map from each CSR entry of H to its message slot.
 //
-// What bounds it and what the mapping bought. The engine is bound by instruction issue and by the
-// dependent chain of a step (summary, shuffles, sums, update, next step), not by DRAM. The mapping it
-// replaces gave each lane a whole column and unrolled its checks: on levels of 4-30 columns most lanes
-// idled; a step of 32 edges has nearly every lane at work.
-// Measured (GB300): circuit-level d=5, FP16, K=32, 4096 shots 826 -> 174 ms; XYZ d=7, FP32, K=16, 2500
-// shots 616 -> 147 ms; circuit-level d=11, FP32, K=64, T=50, 32 shots 220 -> 156 ms.
+// What bounds it and what the mapping bought. A sweep is a dependent chain of steps (summary, shuffles, sums,
+// update, next step); in a member's first sweeps, which rescan most, the rescans' message rows come on top: on
+// circuit-level d=11 (1672 members of 10 sweeps in flight, 565 rescans a sweep) issue is active 22 % of the time, the
+// long scoreboard is the main stall and DRAM runs at 39 % of its peak, 10.2 MB a sweep for 1.1 MB of messages. The
+// mapping it replaces gave each lane a whole column and unrolled its checks: on levels of 4-30 columns most
+// lanes idled (88.4 G warp instructions for that launch, 52.2 G now: 191 a step, rescans included); a step of 32
+// edges has nearly every lane at work (31.2 lanes an instruction).
+// Measured (GB300), column / edge per lane, one warp per shot: circuit-level d=5, K=8, T=20, 100,000 shots FP32 1898
+// / 491 ms, FP16 2313 / 512; d=9, 6000 shots 1087 / 619 and 1235 / 603. As pairs: d=11, FP32, K=64, T=50, 32 shots 223 / 153.
 //
 // Arithmetic equals the oracle's bit for bit: same per-node operation order (__fadd_rn/__fmul_rn), min
 // and sign exact, FP16 storage with -0 stored as +0.

@@ -12,7 +12,7 @@
 namespace vibe {
 
 constexpr int kBpWarpsPerCta = 2;   // image engine: warps per CTA, one shot per warp
-constexpr int kTeamClasses = 2;     // summary engine: teams of 1 or 8 warps (one CTA and one shot each)
+constexpr int kTeamClasses = 2;     // summary engine: teams of 1 or 8 warps (one CTA and one shot or pair each)
 constexpr int kLsdThreads = 128;    // LSD kernel: default threads per CTA (64, 128 or 256), one shot per CTA
 constexpr int kMaxRowDeg = 255;     // position of an edge inside its check row fits in 8 bits
 constexpr int kMaxColDeg = 32;
@@ -50,7 +50,7 @@ __host__ __device__ inline uint32_t csc_entry(uint32_t c, uint32_t slot, int RP,
 // of one warp, and the device-resident tables (owned by the handle). Plain data, copied to the device.
 struct Tables {
   int m, n, k, E, K;
-  int RP;        // row pitch of the padded message image: max row degree rounded up to 8
+  int RP;        // row pitch of the padded message image: max row degree in whole 16-byte chunks (4 FP32, 8 FP16 slots)
   int DP;        // column pitch of csc_ent: max column degree rounded up to 4 (4, 8, 16 or 32)
   int CD;        // column-degree bound of the image engine: 3, or DP
   int mw, nw, kw;
@@ -69,7 +69,7 @@ struct Tables {
   // the engine cannot run the problem), shared memory of one warp (the m check summaries, bytes) and the
   // parts of one warp's global scratch (bytes, 16-aligned)
   int XD, x_warp_smem;   // x_warp_smem: the m check summaries only
-  int team;              // warps that take a member's steps together
+  int team;              // warps that take a member's steps together (a wide problem has a descriptor for each packing)
   int SP;                // edge slots of one member's sweep: E, and one per column without checks
   int nstep, soff_pitch; // largest step count of a member; entries per member of soff
   // xg_cpost = x_warp_scratch: the M*n candidate posteriors (soft output only) follow the fixed part

@@ -63,11 +63,13 @@ SM_CLOCK_GHZ = 2.07          # maximum SM clock of the part (the recipe's figure
 SMEM_BYTES_PER_CLK = 128     # shared-memory bandwidth per SM and clock (32 banks x 4 bytes)
 INT_OPS_PER_CLK = 128        # 32-bit integer lanes per SM and clock
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one ncu capture of each BP kernel with
-# FP32 messages, per unit of work, for the rooflines' `traffic`; None until the present kernels have one
-# (the captures in profiles/ name the build they were taken on).
+# FP32 messages, per unit of work, for the rooflines' `traffic`: the image engine per shot (its DRAM
+# traffic is the per-shot I/O and LSD hand-off), the summary engine per executed sweep (its messages,
+# tables and rescans). Scaled to a launch by the units it processed; the captures and their commands
+# are in profiles/.
 PROFILED_TRAFFIC = {
-    "k_bp": {"per": "shot", "bytes": None, "profile": None},
-    "k_bpx": {"per": "sweep", "bytes": None, "profile": None},
+    "k_bp": {"per": "shot", "bytes": 46869760 / 40000, "profile": "profiles/k_bp_edges_cc666_d9_pheno.md"},
+    "k_bpx": {"per": "sweep", "bytes": 630915047936 / 61970, "profile": "profiles/k_bpx_edges_circuit_d11_k4_t10.md"},
 }
 
 
@@ -646,7 +648,8 @@ def run_vibe(args):
         total_ms = max_over_ranks(sum(step_ms))
         results[label] = dict(step_ms=step_ms, total_ms=total_ms, prof=prof, counters=c, clocks=clk, wall=wall,
                               corr=out["corrections"].clone(), logical=out["logical"].clone(), tune=tune,
-                              RP=int(np.diff(dm.H.rowptr).max() + 7) // 8 * 8)
+                              # row pitch of the message image: whole 16-byte chunks
+                              RP=-(-int(np.diff(dm.H.rowptr).max()) // (8 if fp16 else 4)) * (8 if fp16 else 4))
         # end to end through the host-buffer entry point (H2D + decode + D2H every step)
         if label == "f32":
             hsyn = torch.from_numpy(syn.view(np.int32)).pin_memory()
@@ -689,8 +692,8 @@ def run_vibe(args):
                              traffic=profiled_traffic("k_bp" if image else "k_bpx", label, B, sweeps))
         entry["launch"] = r["tune"]["chosen"]
         if image:
-            # shared-memory view: each column update scans the whole padded row of each of its checks
-            # (RP slots of b bytes) and writes its messages back
+            # shared-memory view: every edge's update scans its check's whole padded row (RP slots of b bytes)
+            # and writes its message back
             smem_bytes = sweeps * E * (r["RP"] + 1) * b
             smem_peak = SM_COUNT_NOMINAL * SMEM_BYTES_PER_CLK * SM_CLOCK_GHZ   # GB/s
             smem_ach = smem_bytes / (ms / 1000.0) / 1e9

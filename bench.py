@@ -69,7 +69,7 @@ INT_OPS_PER_CLK = 128        # 32-bit integer lanes per SM and clock
 # are in profiles/.
 PROFILED_TRAFFIC = {
     "k_bp": {"per": "shot", "bytes": 46869760 / 40000, "profile": "profiles/k_bp_edges_cc666_d9_pheno.md"},
-    "k_bpx": {"per": "sweep", "bytes": 630915047936 / 61970, "profile": "profiles/k_bpx_edges_circuit_d11_k4_t10.md"},
+    "k_bpx": {"per": "sweep", "bytes": 188516016896 / 56083, "profile": "profiles/k_bpx_edges_circuit_d11_k4_t10.md"},
 }
 
 

@@ -621,6 +621,10 @@ struct vibe_handle {
     uint32_t *soff = nullptr, *xlnk = nullptr, *xcolid = nullptr, *xrmap = nullptr;
     int32_t* stepcnt = nullptr;
     uint2* xrec = nullptr;
+    void release() {
+      cudaFree(soff); cudaFree(stepcnt); cudaFree(xrec); cudaFree(xlnk); cudaFree(xcolid); cudaFree(xrmap);
+      *this = Steps();
+    }
   } steps[2];   // of single warps, of teams (wide)
   int32_t *layer_ptr = nullptr, *layer_chk = nullptr, *layer_vptr = nullptr, *layer_var = nullptr,
           *nlayer_d = nullptr;
@@ -646,9 +650,7 @@ struct vibe_handle {
     cudaFree(rowptr); cudaFree(colidx); cudaFree(colptr); cudaFree(rowidx); cudaFree(lrowptr); cudaFree(lcolidx);
     cudaFree(csc_ent); cudaFree(perm); cudaFree(lam); cudaFree(alpha_m);
     cudaFree(msg_init); cudaFree(cpos); cudaFree(xsum); cudaFree(d_desc);
-    for (Steps& p : steps) {
-      cudaFree(p.soff); cudaFree(p.stepcnt); cudaFree(p.xrec); cudaFree(p.xlnk); cudaFree(p.xcolid); cudaFree(p.xrmap);
-    }
+    for (Steps& p : steps) p.release();
     cudaFree(layer_ptr); cudaFree(layer_chk); cudaFree(layer_vptr); cudaFree(layer_var); cudaFree(nlayer_d);
     cudaSetDevice(prev);
   }
@@ -885,8 +887,14 @@ int vibe_create(const vibe_csr* H, const vibe_csr* L, const double* priors, int3
     // with four 158 -> 153 ms, d=9 with two, in batches that fill the GPU, 92 -> 103 ms.
     if (t.XD > 0 && msg_bytes > kTeamImageBytes && t.SP >= 24 * vibe::kTeam * 32) {
       h->tt = t;
-      VIBE_TRY(pack(vibe::kTeam, h->steps[1], h->tt, [&](int ns) { return h->wide = 3LL * ns <= 4LL * t.nstep; }),
-               "step builder");
+      e = pack(vibe::kTeam, h->steps[1], h->tt, [&](int ns) { return h->wide = 3LL * ns <= 4LL * t.nstep; });
+      if (e == cudaErrorMemoryAllocation) {   // single warps do without
+        cudaGetLastError();
+        h->wide = false;
+        e = cudaSuccess;
+      }
+      VIBE_TRY(e, "step builder");
+      if (!h->wide) h->steps[1].release();
     }
   }
   vibe::bpx_layout(&t, p->msg_fp16);

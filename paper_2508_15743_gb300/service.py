@@ -231,8 +231,8 @@ def device_bytes_per_shot(mw: int, nw: int, kw: int, n_max: int) -> int:
 def split_budget(room: int, pipelines: int, per_shot: int, max_batch: int):
     """(shots per batch, bytes of members' records) of each pipeline in shot mode, of `room` bytes for all of
     them. Records make small batches faster (vibe_set_pairs): they get an eighth, and what the batch leaves. (Of the
-    circuit-level d=9 and d=13 mix, whose tables leave 5 GB of 8, that is 40 shots' records; one request at a
-    time takes 50 ms with them and seconds without.)"""
+    circuit-level d=9 and d=13 mix in 8 GiB that is a few tens of shots' records; one request at a time takes 50 ms
+    with them and seconds without.)"""
     mine = max(room, 0) // pipelines
     mb = min(max_batch, (mine - mine // 8) // per_shot)
     return mb, mine - mb * per_shot
